@@ -150,7 +150,7 @@ lqcd_status lqcd_gauge_load(lqcd_ctx* ctx, const double* links);
  * from the loaded links: four-leaf Fhat, two 6x6 Hermitian blocks per site,
  * computed and inverted in FP64 (Gauss-Jordan with partial pivoting), then
  * rounded into every held precision.  csw = 0 gives A = 1 (nothing stored
- * is read).  Returns LQCD_ERR_CLOVER_SINGULAR if some block is singular. */
+ * is read).  Uses the solver vectors of the workspace as scratch.  Returns LQCD_ERR_CLOVER_SINGULAR if some block is singular. */
 lqcd_status lqcd_clover_compute(lqcd_ctx* ctx, double kappa, double csw);
 
 /* Canonical FP64 spinor(s) (host or device) <-> internal field(s) of one

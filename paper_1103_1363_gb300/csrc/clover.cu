@@ -9,228 +9,175 @@
 namespace lqcd {
 
 // 3x3 complex matrices as 18 doubles, row-major, (re, im) interleaved.
-__device__ __forceinline__ void m3_mul(const double* a, const double* b, double* out)  // out = a b
+// Entry (i, j) of a, or of a^dag.
+template <bool DAGGER>
+__device__ __forceinline__ void m3_entry(const double a[18], int i, int j, double& re, double& im)
 {
-    double t[18];
+    const int k = DAGGER ? 2 * (3 * j + i) : 2 * (3 * i + j);
+    re = a[k];
+    im = DAGGER ? -a[k + 1] : a[k + 1];
+}
+
+// out (+)= s op(a) op(b), op = dagger where the flag says so, s = +1 or -1;
+// one multiply-add per real product.
+template <bool DA, bool DB, bool ACC, int S>
+__device__ __forceinline__ void m3_mul(const double a[18], const double b[18], double out[18])
+{
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            double re = 0, im = 0;
+            double re = ACC ? out[2 * (3 * i + j)] : 0.0, im = ACC ? out[2 * (3 * i + j) + 1] : 0.0;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const double ar = a[2 * (3 * i + k)], ai = a[2 * (3 * i + k) + 1];
-                const double br = b[2 * (3 * k + j)], bi = b[2 * (3 * k + j) + 1];
-                re += ar * br - ai * bi;
-                im += ar * bi + ai * br;
+                double ar, ai, br, bi;
+                m3_entry<DA>(a, i, k, ar, ai);
+                m3_entry<DB>(b, k, j, br, bi);
+                re += S * ar * br;
+                re -= S * ai * bi;
+                im += S * ar * bi;
+                im += S * ai * br;
             }
-            t[2 * (3 * i + j)] = re;
-            t[2 * (3 * i + j) + 1] = im;
-        }
-#pragma unroll
-    for (int k = 0; k < 18; ++k) out[k] = t[k];
-}
-
-__device__ __forceinline__ void m3_dag(const double* a, double* out)
-{
-    double t[18];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            t[2 * (3 * i + j)] = a[2 * (3 * j + i)];
-            t[2 * (3 * i + j) + 1] = -a[2 * (3 * j + i) + 1];
-        }
-#pragma unroll
-    for (int k = 0; k < 18; ++k) out[k] = t[k];
-}
-
-__device__ __forceinline__ void link_at(const Geom& g, const void* gauge, const int c[4], int mu, double u[18])
-{
-    const int full = full_index(g, c);
-    const int par = (c[0] + c[1] + c[2] + c[3]) & 1;
-    GaugeIO<P64, 18>::load(gauge, g.stride, par, mu, full >> 1, u);
-}
-
-__device__ __forceinline__ void shifted(const Geom& g, const int c[4], int mu, int d, int out[4])
-{
-    out[0] = c[0]; out[1] = c[1]; out[2] = c[2]; out[3] = c[3];
-    out[mu] = (out[mu] + d + g.L[mu]) % g.L[mu];
-}
-
-// Sum of the four plaquette leaves in the mu-nu plane, all circulating mu -> nu.
-__device__ void leaves(const Geom& g, const void* gauge, const int c[4], int mu, int nu, double Q[18])
-{
-    int pm[4], mm[4], pn[4], mn[4], mm_pn[4], mm_mn[4], pm_mn[4];
-    shifted(g, c, mu, +1, pm);
-    shifted(g, c, mu, -1, mm);
-    shifted(g, c, nu, +1, pn);
-    shifted(g, c, nu, -1, mn);
-    shifted(g, mm, nu, +1, mm_pn);
-    shifted(g, mm, nu, -1, mm_mn);
-    shifted(g, pm, nu, -1, pm_mn);
-    double a[18], b[18], t[18];
-#pragma unroll
-    for (int k = 0; k < 18; ++k) Q[k] = 0;
-    // U_mu(x) U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-    link_at(g, gauge, c, mu, a);
-    link_at(g, gauge, pm, nu, b);
-    m3_mul(a, b, t);
-    link_at(g, gauge, pn, mu, a);
-    m3_dag(a, a);
-    m3_mul(t, a, t);
-    link_at(g, gauge, c, nu, a);
-    m3_dag(a, a);
-    m3_mul(t, a, t);
-#pragma unroll
-    for (int k = 0; k < 18; ++k) Q[k] += t[k];
-    // U_nu(x) U_mu(x-mu+nu)^dag U_nu(x-mu)^dag U_mu(x-mu)
-    link_at(g, gauge, c, nu, a);
-    link_at(g, gauge, mm_pn, mu, b);
-    m3_dag(b, b);
-    m3_mul(a, b, t);
-    link_at(g, gauge, mm, nu, a);
-    m3_dag(a, a);
-    m3_mul(t, a, t);
-    link_at(g, gauge, mm, mu, a);
-    m3_mul(t, a, t);
-#pragma unroll
-    for (int k = 0; k < 18; ++k) Q[k] += t[k];
-    // U_mu(x-mu)^dag U_nu(x-mu-nu)^dag U_mu(x-mu-nu) U_nu(x-nu)
-    link_at(g, gauge, mm, mu, a);
-    m3_dag(a, a);
-    link_at(g, gauge, mm_mn, nu, b);
-    m3_dag(b, b);
-    m3_mul(a, b, t);
-    link_at(g, gauge, mm_mn, mu, a);
-    m3_mul(t, a, t);
-    link_at(g, gauge, mn, nu, a);
-    m3_mul(t, a, t);
-#pragma unroll
-    for (int k = 0; k < 18; ++k) Q[k] += t[k];
-    // U_nu(x-nu)^dag U_mu(x-nu) U_nu(x+mu-nu) U_mu(x)^dag
-    link_at(g, gauge, mn, nu, a);
-    m3_dag(a, a);
-    link_at(g, gauge, mn, mu, b);
-    m3_mul(a, b, t);
-    link_at(g, gauge, pm_mn, nu, a);
-    m3_mul(t, a, t);
-    link_at(g, gauge, c, mu, a);
-    m3_dag(a, a);
-    m3_mul(t, a, t);
-#pragma unroll
-    for (int k = 0; k < 18; ++k) Q[k] += t[k];
-}
-
-// sigma_{mu nu} restricted to the two chiral blocks of the DeGrand-Rossi
-// basis (upper: spins 0,1; lower: spins 2,3), planes xy, xz, xt, yz, yt, zt.
-// Entries are (re, im) of the 2x2 block, row-major.  Worked out from
-// sigma = (i/2)[g_mu, g_nu]; every sigma_{mu nu} commutes with g5 here.
-__constant__ double SIGMA_BLK[6][2][8] = {
-    {{1, 0, 0, 0, 0, 0, -1, 0}, {1, 0, 0, 0, 0, 0, -1, 0}},    // xy: diag(1,-1), diag(1,-1)
-    {{0, 0, 0, -1, 0, 1, 0, 0}, {0, 0, 0, -1, 0, 1, 0, 0}},    // xz: [[0,-i],[i,0]] both
-    {{0, 0, -1, 0, -1, 0, 0, 0}, {0, 0, 1, 0, 1, 0, 0, 0}},    // xt: [[0,-1],[-1,0]], [[0,1],[1,0]]
-    {{0, 0, 1, 0, 1, 0, 0, 0}, {0, 0, 1, 0, 1, 0, 0, 0}},      // yz: [[0,1],[1,0]] both
-    {{0, 0, 0, -1, 0, 1, 0, 0}, {0, 0, 0, 1, 0, -1, 0, 0}},    // yt: [[0,-i],[i,0]], [[0,i],[-i,0]]
-    {{-1, 0, 0, 0, 0, 0, 1, 0}, {1, 0, 0, 0, 0, 0, -1, 0}},    // zt: diag(-1,1), diag(1,-1)
-};
-
-// Pack a 6x6 Hermitian block m[r][s][re/im] into 36 reals.
-__device__ __forceinline__ void pack_herm6(const double m[6][6][2], double c[36])
-{
-#pragma unroll
-    for (int r = 0; r < 6; ++r) c[r] = m[r][r][0];
-    int k = 6;
-#pragma unroll
-    for (int r = 1; r < 6; ++r)
-#pragma unroll
-        for (int s = 0; s < r; ++s) {
-            c[k++] = m[r][s][0];
-            c[k++] = m[r][s][1];
+            out[2 * (3 * i + j)] = re;
+            out[2 * (3 * i + j) + 1] = im;
         }
 }
 
-__device__ __forceinline__ void unpack_herm6(const double c[36], double m[6][6][2])
+// g = a b - (a b)^dag as 9 reals: the imaginary diagonal, then the complex
+// entries (1,0), (2,0), (2,1).
+__device__ __forceinline__ void m3_mul_anti(const double a[18], const double b[18], double g[9])
 {
-    for (int r = 0; r < 6; ++r) {
-        m[r][r][0] = c[r];
-        m[r][r][1] = 0.0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        double im = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            im += a[2 * (3 * i + k)] * b[2 * (3 * k + i) + 1];
+            im += a[2 * (3 * i + k) + 1] * b[2 * (3 * k + i)];
+        }
+        g[i] = 2.0 * im;
     }
-    int k = 6;
-    for (int r = 1; r < 6; ++r)
-        for (int s = 0; s < r; ++s) {
-            m[r][s][0] = c[k];
-            m[r][s][1] = c[k + 1];
-            m[s][r][0] = c[k];
-            m[s][r][1] = -c[k + 1];
-            k += 2;
+    int q = 3;
+#pragma unroll
+    for (int i = 1; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < i; ++j) {
+            double re = 0.0, im = 0.0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const double ur = a[2 * (3 * i + k)], ui = a[2 * (3 * i + k) + 1];
+                const double vr = b[2 * (3 * k + j)], vi = b[2 * (3 * k + j) + 1];
+                const double sr = a[2 * (3 * j + k)], si = a[2 * (3 * j + k) + 1];
+                const double tr = b[2 * (3 * k + i)], ti = b[2 * (3 * k + i) + 1];
+                re += ur * vr;  // (a b)_ij - conj((a b)_ji)
+                re -= ui * vi;
+                re -= sr * tr;
+                re += si * ti;
+                im += ur * vi;
+                im += ui * vr;
+                im += sr * ti;
+                im += si * tr;
+            }
+            g[q++] = re;
+            g[q++] = im;
         }
 }
 
-// One thread per site of parity blockIdx.y: A blocks in FP64.
-__global__ void clover_build_kernel(Geom g, const void* gauge, double kc, char* A64, size_t par_bytes)
+// Checkerboard index of the site DM steps along MU and DN along NU from c (each -1, 0 or 1).
+template <int MU, int DM, int NU, int DN>
+__device__ __forceinline__ int cb_shift(const Geom& g, const int c[4])
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int par = blockIdx.y;
-    if (i >= g.Vh) return;
+    int d[4] = {c[0], c[1], c[2], c[3]};
+    if (DM > 0) d[MU] = d[MU] == g.L[MU] - 1 ? 0 : d[MU] + 1;
+    if (DM < 0) d[MU] = d[MU] == 0 ? g.L[MU] - 1 : d[MU] - 1;
+    if (DN > 0) d[NU] = d[NU] == g.L[NU] - 1 ? 0 : d[NU] + 1;
+    if (DN < 0) d[NU] = d[NU] == 0 ? g.L[NU] - 1 : d[NU] - 1;
+    return full_index(g, d) >> 1;
+}
+
+// Field strength.  With the staples of the link (x, mu) in the mu-nu plane,
+//   T(x) = U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag - U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu),
+// the sum Q of the four plaquette leaves at x (all circulating mu -> nu) has
+//   Q - Q^dag = anti(U_mu(x) T(x)) + anti(T(x-mu) U_mu(x-mu)),  anti(X) = X - X^dag:
+// a leaf and its adjoint have opposite anti-parts, so the lower staple enters
+// with a minus sign, and the two leaves behind x hold the staples of x - mu.
+// This kernel forms both terms at the link's own site, for one plane and
+// site a thread: six 3x3 products (four whole, two of which only the
+// anti-Hermitian part is formed) where the four leaves took twelve, and six
+// times the threads of a thread per site, which small lattices need.
+//
+// The bound is the FP64 pipe (1.256 TFLOP/s measured: a warp's multiply-add
+// occupies it for 15 cycles), so the count of FP64 instructions is what
+// matters: about 650 a plane and site here.  The terms go through scratch
+// (2 x 9 doubles a plane and site, 864 bytes written and read a site, a
+// tenth of the time).  At 16^3 x 32: 810 us; the four leaves per site,
+// with their twelve products and arrays in local memory, took 3218 us.
+enum { CLOVER_PLANES = 6, CLOVER_TERM = 9 };
+
+// element q of term `which` (0: at x, 1: for x + mu) of a plane, at site i of parity par
+__device__ __forceinline__ size_t term_at(const Geom& g, int plane, int which, int q, int par, int i)
+{
+    return ((size_t)((plane * 2 + which) * CLOVER_TERM + q) * 2 + par) * g.stride + i;
+}
+
+template <int MU, int NU>
+__device__ __forceinline__ void plane_terms(const Geom& g, const void* gauge, int plane, int par, int i, double* terms)
+{
+    typedef GaugeIO<P64, 18> IO;
     int c[4];
     cb_coords(g, i, par, c);
-    double blk[2][6][6][2];
-    for (int b = 0; b < 2; ++b)
-        for (int r = 0; r < 6; ++r)
-            for (int s = 0; s < 6; ++s) {
-                blk[b][r][s][0] = (r == s) ? 1.0 : 0.0;
-                blk[b][r][s][1] = 0.0;
-            }
-    const int PL[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
-    for (int p = 0; p < 6; ++p) {
-        double Q[18], F[18];
-        leaves(g, gauge, c, PL[p][0], PL[p][1], Q);
-        // Fhat = (Q - Q^dag) / 8, traceless
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) {
-                F[2 * (3 * a + b)] = (Q[2 * (3 * a + b)] - Q[2 * (3 * b + a)]) * 0.125;
-                F[2 * (3 * a + b) + 1] = (Q[2 * (3 * a + b) + 1] + Q[2 * (3 * b + a) + 1]) * 0.125;
-            }
-        const double tri = (F[1] + F[9] + F[17]) / 3.0;  // trace is imaginary
-        F[1] -= tri;
-        F[9] -= tri;
-        F[17] -= tri;
-        // block += i kc sigma (x) F
-        for (int b = 0; b < 2; ++b)
-            for (int s = 0; s < 2; ++s)
-                for (int r = 0; r < 2; ++r) {
-                    const double sr = SIGMA_BLK[p][b][2 * (2 * s + r)], si = SIGMA_BLK[p][b][2 * (2 * s + r) + 1];
-                    if (sr == 0.0 && si == 0.0) continue;
-                    for (int a = 0; a < 3; ++a)
-                        for (int cc = 0; cc < 3; ++cc) {
-                            const double fr = F[2 * (3 * a + cc)], fi = F[2 * (3 * a + cc) + 1];
-                            const double zr = sr * fr - si * fi, zi = sr * fi + si * fr;
-                            blk[b][3 * s + a][3 * r + cc][0] += -kc * zi;
-                            blk[b][3 * s + a][3 * r + cc][1] += kc * zr;
-                        }
-                }
-    }
-    for (int b = 0; b < 2; ++b) {
-        double pk[36];
-        pack_herm6(blk[b], pk);
-        CloverIO<P64>::store_block(A64 + par * par_bytes, g.stride, i, b, pk);
+    double u[18], v[18], m[18], t[18], q[9];
+    // upper staple
+    IO::load(gauge, g.stride, par, NU, i, u);
+    IO::load(gauge, g.stride, 1 - par, MU, cb_shift<MU, 0, NU, 1>(g, c), v);
+    m3_mul<false, false, false, 1>(u, v, m);
+    IO::load(gauge, g.stride, 1 - par, NU, cb_shift<MU, 1, NU, 0>(g, c), u);
+    m3_mul<false, true, false, 1>(u, m, t);
+    // minus the lower one
+    IO::load(gauge, g.stride, 1 - par, MU, cb_shift<MU, 0, NU, -1>(g, c), u);
+    IO::load(gauge, g.stride, par, NU, cb_shift<MU, 1, NU, -1>(g, c), v);
+    m3_mul<false, false, false, 1>(u, v, m);
+    IO::load(gauge, g.stride, 1 - par, NU, cb_shift<MU, 0, NU, -1>(g, c), u);
+    m3_mul<true, false, true, -1>(m, u, t);
+    IO::load(gauge, g.stride, par, MU, i, u);
+    m3_mul_anti(u, t, q);
+#pragma unroll
+    for (int k = 0; k < CLOVER_TERM; ++k) terms[term_at(g, plane, 0, k, par, i)] = q[k];
+    m3_mul_anti(t, u, q);
+#pragma unroll
+    for (int k = 0; k < CLOVER_TERM; ++k) terms[term_at(g, plane, 1, k, par, i)] = q[k];
+}
+
+// blockIdx.y: plane (xy, xz, xt, yz, yt, zt); blockIdx.z: parity.
+__global__ void __launch_bounds__(64) clover_terms_kernel(Geom g, const void* gauge, double* terms)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int plane = blockIdx.y, par = blockIdx.z;
+    if (i >= g.Vh) return;
+    switch (plane) {
+    case 0: plane_terms<0, 1>(g, gauge, 0, par, i, terms); break;
+    case 1: plane_terms<0, 2>(g, gauge, 1, par, i, terms); break;
+    case 2: plane_terms<0, 3>(g, gauge, 2, par, i, terms); break;
+    case 3: plane_terms<1, 2>(g, gauge, 3, par, i, terms); break;
+    case 4: plane_terms<1, 3>(g, gauge, 4, par, i, terms); break;
+    default: plane_terms<2, 3>(g, gauge, 5, par, i, terms); break;
     }
 }
 
-// One thread per (site, chiral block) of parity blockIdx.y: Gauss-Jordan
-// inversion with partial pivoting in FP64.
-__global__ void clover_invert_kernel(Geom g, const char* A64, char* Ainv64, size_t par_bytes, int* errw)
+// Packed position of the real part of entry (r, s), r > s, of a 6x6 Hermitian block.
+__host__ __device__ constexpr int herm6_at(int r, int s) { return 6 + r * (r - 1) + 2 * s; }
+
+// Inverse of a packed Hermitian block by Gauss-Jordan with partial pivoting
+// (rows); false if a pivot is below 1e-12.  The general case: indexed rows
+// live in local memory.
+__device__ __noinline__ bool invert_pivoting(const double c[36], double out[36])
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int par = blockIdx.y;
-    if (t >= 2 * g.Vh) return;
-    const int i = t >> 1, b = t & 1;
-    double pk[36], m[6][6][2], inv[6][6][2];
-    CloverIO<P64>::load_block(A64 + par * par_bytes, g.stride, i, b, pk);
-    unpack_herm6(pk, m);
+    double m[6][6][2], inv[6][6][2];
     for (int r = 0; r < 6; ++r)
         for (int s = 0; s < 6; ++s) {
+            const int k = r > s ? herm6_at(r, s) : herm6_at(s, r);
+            m[r][s][0] = r == s ? c[r] : c[k];
+            m[r][s][1] = r == s ? 0.0 : r > s ? c[k + 1] : -c[k + 1];
             inv[r][s][0] = (r == s) ? 1.0 : 0.0;
             inv[r][s][1] = 0.0;
         }
@@ -272,62 +219,229 @@ __global__ void clover_invert_kernel(Geom g, const char* A64, char* Ainv64, size
             }
         }
     }
-    if (!ok) atomicOr(errw, ERRW_CLOVER_SINGULAR);
-    pack_herm6(inv, pk);
-    CloverIO<P64>::store_block(Ainv64 + par * par_bytes, g.stride, i, b, pk);
+    for (int r = 0; r < 6; ++r) {
+        out[r] = inv[r][r][0];
+        for (int s = 0; s < r; ++s) {
+            out[herm6_at(r, s)] = inv[r][s][0];
+            out[herm6_at(r, s) + 1] = inv[r][s][1];
+        }
+    }
+    return ok;
 }
 
-// FP64 clover -> precision P, both parities (blockIdx.y).
-template <int P>
-__global__ void clover_round_kernel(Geom g, const char* src, size_t src_pb, char* dst, size_t dst_pb)
+// The same elimination where no row has to be exchanged: the pivots are the
+// diagonal entries.  Swept in place the matrix stays Hermitian up to the sign
+// of the entries between swept and unswept rows (M_kj = -conj(M_jk)), so the
+// lower triangle in registers is enough: 60 multiply-adds and one division a
+// pivot, against 290 and the pivot search's square roots.  False, with c
+// destroyed, as soon as partial pivoting would exchange rows or the pivot is
+// below 1e-12: the caller then takes invert_pivoting.
+__device__ __forceinline__ bool invert_in_place(double c[36])
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const double dk = c[k], d2 = dk * dk;
+        double vr[6], vi[6];  // column k of the matrix
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            if (i > k) {
+                vr[i] = c[herm6_at(i, k)];
+                vi[i] = c[herm6_at(i, k) + 1];
+                ok = ok && d2 >= vr[i] * vr[i] + vi[i] * vi[i];
+            } else if (i < k) {
+                vr[i] = -c[herm6_at(k, i)];
+                vi[i] = c[herm6_at(k, i) + 1];
+            }
+        }
+        ok = ok && d2 >= 1e-24;
+        const double p = 1.0 / dk;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            if (i == k) continue;
+            const double tr = p * vr[i], ti = p * vi[i];
+            // M_ij -= p v_i M_kj, M_kj = conj(v_j) for j > k and -conj(v_j) for j < k
+#pragma unroll
+            for (int j = 0; j < i; ++j) {
+                if (j == k) continue;
+                const int e = herm6_at(i, j);
+                if (j > k) {
+                    c[e] -= tr * vr[j];
+                    c[e] -= ti * vi[j];
+                    c[e + 1] += tr * vi[j];
+                    c[e + 1] -= ti * vr[j];
+                } else {
+                    c[e] += tr * vr[j];
+                    c[e] += ti * vi[j];
+                    c[e + 1] -= tr * vi[j];
+                    c[e + 1] += ti * vr[j];
+                }
+            }
+            if (i > k) {
+                c[i] -= tr * vr[i];
+                c[i] -= ti * vi[i];
+                c[herm6_at(i, k)] = -tr;
+                c[herm6_at(i, k) + 1] = -ti;
+            } else {
+                c[i] += tr * vr[i];
+                c[i] += ti * vi[i];
+                c[herm6_at(k, i)] = -tr;  // p M_ki, M_ki = -conj(v_i)
+                c[herm6_at(k, i) + 1] = ti;
+            }
+        }
+        c[k] = p;
+    }
+    return ok;
+}
+
+// Where the blocks of A and A^{-1} go: per storage precision the field of
+// both parities (nullptr: not held) and the bytes of one parity.
+struct CloverOut {
+    char* a[4];
+    char* inv[4];
+    size_t pb[4];
+};
+
+// Block b of site i, rounded to each held precision (through FP32 for the
+// 16-bit ones, whose 36 halves a block are nine 8-byte pieces of the uint4 chunks).
+__device__ __forceinline__ void store_rounded(char* const dst[4], const size_t pb[4], int stride, int par, int i, int b,
+                                              const double c[36])
+{
+    CloverIO<P64>::store_block(dst[P64] + par * pb[P64], stride, i, b, c);
+    float f[36];
+#pragma unroll
+    for (int k = 0; k < 36; ++k) f[k] = (float)c[k];
+    if (dst[P32]) CloverIO<P32>::store_block(dst[P32] + par * pb[P32], stride, i, b, f);
+#pragma unroll
+    for (int P = P16; P <= PB16; ++P) {
+        if (!dst[P]) continue;
+        uint2* p = reinterpret_cast<uint2*>(dst[P] + par * pb[P]);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int piece = 9 * b + k;  // of the site's 18; two to a chunk
+            p[((size_t)(piece >> 1) * stride + i) * 2 + (piece & 1)] =
+                make_uint2(f2h(f[4 * k], f[4 * k + 1], P == PB16), f2h(f[4 * k + 2], f[4 * k + 3], P == PB16));
+        }
+    }
+}
+
+// Field strength terms -> A = 1 + i kc sum sigma Fhat, its inverse, and both
+// in every held precision, in one pass.  Thread = (site, chiral block):
+// threads 0..31 of a block of 64 take block 0 of 32 sites, 32..63 block 1
+// (the second read of the terms hits L1).  sigma in the DeGrand-Rossi basis,
+// worked out from (i/2)[g_mu, g_nu] (every sigma_{mu nu} commutes with g5):
+// xy and zt are diagonal, diag(1,-1) and -+diag(1,-1) in the two blocks; xz
+// and yt have (1,0) entries i and +-i; xt and yz have -+1 and 1.
+// kc = kappa csw; Fhat = (Q - Q^dag)/8 made traceless.  FP64-bound like the
+// terms: about 630 instructions a block.  At 16^3 x 32: 335 us; the
+// inversion from memory (1570 us, local memory and pivot search) and the
+// rounding passes (47 us) were kernels of their own.
+__global__ void __launch_bounds__(64) clover_finish_kernel(Geom g, const double* __restrict__ terms, double kc,
+                                                           CloverOut o, int* errw)
+{
+    const int b = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + (threadIdx.x & 31);
     const int par = blockIdx.y;
     if (i >= g.Vh) return;
-    double a[36], b[36];
-    CloverIO<P64>::load_block(src + par * src_pb, g.stride, i, 0, a);
-    CloverIO<P64>::load_block(src + par * src_pb, g.stride, i, 1, b);
-    if constexpr (P == P32) {
-        float fa[36], fb[36];
-        for (int k = 0; k < 36; ++k) { fa[k] = (float)a[k]; fb[k] = (float)b[k]; }
-        CloverIO<P32>::store_block(dst + par * dst_pb, g.stride, i, 0, fa);
-        CloverIO<P32>::store_block(dst + par * dst_pb, g.stride, i, 1, fb);
-    } else {
-        float f[72];
-        for (int k = 0; k < 36; ++k) { f[k] = (float)a[k]; f[36 + k] = (float)b[k]; }
-        CloverIO<P>::store_all(dst + par * dst_pb, g.stride, i, f);
+    int c[4];
+    cb_coords(g, i, par, c);
+    const int back[3] = {cb_shift<0, -1, 1, 0>(g, c), cb_shift<1, -1, 0, 0>(g, c), cb_shift<2, -1, 0, 0>(g, c)};
+    auto field = [&](int plane, int mu, double f[9]) {
+#pragma unroll
+        for (int q = 0; q < CLOVER_TERM; ++q)
+            f[q] = terms[term_at(g, plane, 0, q, par, i)] + terms[term_at(g, plane, 1, q, 1 - par, back[mu])];
+    };
+    // e = F_xy + s F_zt, pp = F_yz + s F_xt, rr = F_xz - s F_yt with s = -1, +1 in the two blocks
+    const double s = b ? 1.0 : -1.0;
+    double e[9], pp[9], rr[9], f[9];
+    field(0, 0, e);
+    field(5, 2, f);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) e[q] += s * f[q];
+    field(3, 1, pp);
+    field(2, 0, f);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) pp[q] += s * f[q];
+    field(1, 0, rr);
+    field(4, 1, f);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) rr[q] -= s * f[q];
+    const double k8 = 0.125 * kc;
+    auto scale = [&](double v[9]) {  // times k8, traceless
+        const double tr = (v[0] + v[1] + v[2]) * (1.0 / 3.0);
+#pragma unroll
+        for (int q = 0; q < 9; ++q) v[q] = k8 * (q < 3 ? v[q] - tr : v[q]);
+    };
+    scale(e);
+    scale(pp);
+    scale(rr);
+    double blk[36];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        // diagonal spin blocks 1 +- i e: the diagonal of e is imaginary
+        blk[a] = 1.0 - e[a];
+        blk[3 + a] = 1.0 + e[a];
+#pragma unroll
+        for (int q = 0; q < a; ++q) {
+            const int l = a == 1 ? 3 : 5 + 2 * q;  // entry (a, q) of the 9 reals
+            blk[herm6_at(a, q)] = -e[l + 1];
+            blk[herm6_at(a, q) + 1] = e[l];
+            blk[herm6_at(3 + a, 3 + q)] = e[l + 1];
+            blk[herm6_at(3 + a, 3 + q) + 1] = -e[l];
+        }
+        // spin (1, 0): i pp - rr, with entry (c, a) = -conj of entry (a, c)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int hi = a > q ? a : q, lo = a > q ? q : a;
+            const int l = hi == 1 ? 3 : 5 + 2 * lo;
+            double re, im;
+            if (a == q) {
+                re = -pp[a];
+                im = -rr[a];
+            } else if (a > q) {
+                re = -pp[l + 1] - rr[l];
+                im = pp[l] - rr[l + 1];
+            } else {
+                re = rr[l] - pp[l + 1];
+                im = -pp[l] - rr[l + 1];
+            }
+            blk[herm6_at(3 + a, q)] = re;
+            blk[herm6_at(3 + a, q) + 1] = im;
+        }
     }
+    store_rounded(o.a, o.pb, g.stride, par, i, b, blk);
+    if (!invert_in_place(blk)) {
+        double src[36];
+        const double2* p = reinterpret_cast<const double2*>(o.a[P64] + par * o.pb[P64]) + (size_t)(18 * b) * g.stride + i;
+        for (int k = 0; k < 18; ++k) {  // the block that this thread has just stored
+            const double2 v = p[(size_t)k * g.stride];
+            src[2 * k] = v.x;
+            src[2 * k + 1] = v.y;
+        }
+        if (!invert_pivoting(src, blk)) atomicOr(errw, ERRW_CLOVER_SINGULAR);
+    }
+    store_rounded(o.inv, o.pb, g.stride, par, i, b, blk);
 }
 
 lqcd_status clover_build(lqcd_ctx* c, double kappa, double csw)
 {
+    // the field strength terms go through the solver vectors: 2 parities x 108 doubles a site
+    static_assert(2 * CLOVER_PLANES * 2 * CLOVER_TERM * sizeof(double) <= NV64 * 2 * 192, "terms exceed the solver vectors");
+    double* terms = reinterpret_cast<double*>(c->vec64);
     const int block = 64;
-    dim3 grid((c->g.Vh + block - 1) / block, 2);
-    const size_t pb64 = c->clov_parity_bytes(P64);
-    clover_build_kernel<<<grid, block, 0, c->stream>>>(c->g, c->gauge[P64], kappa * csw,
-                                                       static_cast<char*>(c->clov[P64]), pb64);
+    clover_terms_kernel<<<dim3((c->g.Vh + block - 1) / block, CLOVER_PLANES, 2), block, 0, c->stream>>>(
+        c->g, c->gauge[P64], terms);
     LQ_CUDA(cudaGetLastError());
     c->launches++;
-    dim3 grid2((2 * c->g.Vh + block - 1) / block, 2);
-    clover_invert_kernel<<<grid2, block, 0, c->stream>>>(c->g, static_cast<const char*>(c->clov[P64]),
-                                                         static_cast<char*>(c->clovinv[P64]), pb64, c->errw);
-    LQ_CUDA(cudaGetLastError());
-    c->launches++;
-    for (int P = P32; P <= PB16; ++P) {
-        if (!c->holds(P)) continue;
-        const size_t pb = c->clov_parity_bytes(P);
-        for (int which = 0; which < 2; ++which) {
-            const char* src = static_cast<const char*>(which ? c->clovinv[P64] : c->clov[P64]);
-            char* dst = static_cast<char*>(which ? c->clovinv[P] : c->clov[P]);
-            switch (P) {
-            case P32: clover_round_kernel<P32><<<grid, block, 0, c->stream>>>(c->g, src, pb64, dst, pb); break;
-            case P16: clover_round_kernel<P16><<<grid, block, 0, c->stream>>>(c->g, src, pb64, dst, pb); break;
-            default: clover_round_kernel<PB16><<<grid, block, 0, c->stream>>>(c->g, src, pb64, dst, pb); break;
-            }
-            LQ_CUDA(cudaGetLastError());
-            c->launches++;
-        }
+    CloverOut o;
+    for (int P = 0; P < 4; ++P) {
+        o.a[P] = c->holds(P) ? static_cast<char*>(c->clov[P]) : nullptr;
+        o.inv[P] = c->holds(P) ? static_cast<char*>(c->clovinv[P]) : nullptr;
+        o.pb[P] = c->clov_parity_bytes(P);
     }
+    clover_finish_kernel<<<dim3((c->g.Vh + 31) / 32, 2), block, 0, c->stream>>>(c->g, terms, kappa * csw, o, c->errw);
+    LQ_CUDA(cudaGetLastError());
+    c->launches++;
     return LQCD_OK;
 }
 
