@@ -100,12 +100,31 @@ static double launch_bytes_per_site(const lqcd_ctx* c, const DslashArgs& A, int 
     return nrhs * per_rhs + 8 * L + (epi == EPI_NONE ? 0.0 : Cl);
 }
 
+// Does the warp-per-direction kernel take a launch of `sites` (sites per
+// parity times right-hand sides) by default?  Measured, gathering kernel
+// against it (schur / CG iteration in plain launches, us): FP32 2048 sites
+// 8.0 / 32.4 against 5.8 / 24.9, 10368 13.9 / 35.3 against 6.8 / 31.2, 16384
+// 14.1 / 44.5 (32.8 as a graph) against 9.9 / 38.4 (41.5), 32768 15.0 / 50.7
+// against 13.8 / 55.4.  So the plain launches change over at 16384 sites,
+// about where each SM holds its three blocks of 32 sites, and the reducing
+// ones, whose blocks all end in the reduction, below that.  FP64 (bound by
+// its pipe, which the idle warps at the barrier leave unused once the SMs
+// are full): 2048 sites 83 / 189 against 31 / 83, 6144 134 / 237 against 60 /
+// 145, 10368 86 / 188 against 89 / 210.
+static bool wide_default(int mode, bool reducing, long sites)
+{
+    return sites <= (mode == P64 ? 8192 : reducing ? 12288 : 16384);
+}
+
 lqcd_status launch_dslash(lqcd_ctx* c, const DslashArgs& A0, int P, bool dag, int epi, bool red, int nrhs)
 {
     DslashArgs A = A0;
     if (red || epi == EPI_CG) A.sites_per_thread = c->tuned_spt[P][dag ? 1 : 0];
     int block = c->tuned_block[P][dag ? 1 : 0][red ? 1 : 0];
     if (block <= 0) block = c->block;
+    const bool reducing = red || epi == EPI_CG;
+    if (block == DSLASH_MAX_BLOCK && A.sites_per_thread == 0 && wide_default(P, reducing, (long)c->g.Vh * nrhs + own_capture.other_sites))
+        block = DSLASH_WIDE;
     const int rc = c->recon_of(mode_pg(P));
     Profiler* pr = c->prof;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;

@@ -72,6 +72,7 @@ __global__ void cg_p_kernel(Geom g, char* p, size_t p_rb, const char* r, size_t 
     typedef typename RealT<PP>::type RP;
     typedef typename RealT<PR>::type RR;
     const int rhs = blockIdx.y;
+    pdl_wait();
     if (skip && skip[rhs]) return;
     const double* sc = scal + rhs * SC_PER_RHS;
     const double bden = sc[den] + sc[den + 1];  // 0 once the residual has vanished
@@ -87,6 +88,7 @@ __global__ void cg_p_kernel(Geom g, char* p, size_t p_rb, const char* r, size_t 
             for (int k = 0; k < 24; ++k) vp[k] = (RP)(vr[k] + beta * (RR)vp[k]);
             SpinorIO<PP>::store(p + rhs * p_rb + f * fp, g.stride, i, vp);
         }
+    pdl_start_next();
 }
 
 // xhi += xlo; xlo = 0
@@ -125,10 +127,13 @@ __global__ void zero_kernel(Geom g, char* x, size_t rb, int nf)
         for (int f = 0; f < nf; ++f) SpinorIO<P>::store(x + rhs * rb + f * fb, g.stride, i, v);
 }
 
-__global__ void copy_scalar_kernel(double* scal, int dst, int src, int nrhs)
+// the (even, odd) pair of slots dst, dst + 1 = src, src + 1 of each right-hand side
+__global__ void copy_scalar_pair_kernel(double* scal, int dst, int src, int nrhs)
 {
-    const int r = threadIdx.x;
-    if (r < nrhs) scal[r * SC_PER_RHS + dst] = scal[r * SC_PER_RHS + src];
+    const int r = threadIdx.x >> 1, k = threadIdx.x & 1;
+    pdl_start_next();
+    pdl_wait();
+    if (r < nrhs) scal[r * SC_PER_RHS + dst + k] = scal[r * SC_PER_RHS + src + k];
 }
 
 #define LQ_SWITCH_P(P, CALL)                 \
@@ -171,15 +176,15 @@ lqcd_status blas_cg_p_update(lqcd_ctx* c, void* p, int Pp, const void* r, int Pr
     dim3 grid(blas_grid(c, block), nrhs);
     char* pp = static_cast<char*>(p);
     const char* rr = static_cast<const char*>(r);
+    const bool small = (long)c->g.Vh * nrhs + own_capture.other_sites <= 12288;  // as the iteration's reducing hops
     if (Pr == P64) {
         if (Pp != P64) return fail(LQCD_ERR_INVALID, "cg_p_update: FP64 r needs FP64 p");
-        cg_p_kernel<P64, P64><<<grid, block, 0, c->stream>>>(c->g, pp, p_rb, rr, r_rb, nf, c->scal, s_num, s_den,
-                                                             c->skip);
+        LQ_CUDA(launch_dependent(cg_p_kernel<P64, P64>, small, grid, block, c->stream, c->g, pp, p_rb, rr, r_rb, nf,
+                                 c->scal, s_num, s_den, c->skip));
     } else {
-        LQ_SWITCH_P(Pp, (cg_p_kernel<PT, P32><<<grid, block, 0, c->stream>>>(c->g, pp, p_rb, rr, r_rb, nf, c->scal,
-                                                                               s_num, s_den, c->skip)));
+        LQ_SWITCH_P(Pp, LQ_CUDA(launch_dependent(cg_p_kernel<PT, P32>, small, grid, block, c->stream, c->g, pp, p_rb, rr,
+                                                 r_rb, nf, c->scal, s_num, s_den, c->skip)));
     }
-    LQ_CUDA(cudaGetLastError());
     c->launches++;
     return LQCD_OK;
 }
@@ -207,10 +212,10 @@ lqcd_status blas_zero(lqcd_ctx* c, void* x, int P, int nrhs, size_t rb, int nf)
     return LQCD_OK;
 }
 
-lqcd_status blas_copy_scalar(lqcd_ctx* c, int dst, int src, int nrhs)
+lqcd_status blas_copy_scalar_pair(lqcd_ctx* c, int dst, int src, int nrhs)
 {
-    copy_scalar_kernel<<<1, 32 * ((nrhs + 31) / 32), 0, c->stream>>>(c->scal, dst, src, nrhs);
-    LQ_CUDA(cudaGetLastError());
+    LQ_CUDA(launch_dependent(copy_scalar_pair_kernel, false, dim3(1), dim3(64 * ((nrhs + 31) / 32)), c->stream, c->scal,
+                             dst, src, nrhs));
     c->launches++;
     return LQCD_OK;
 }

@@ -93,6 +93,57 @@ __device__ __forceinline__ uint32_t f2h(float a, float b, int isbf)
     return u;
 }
 
+// ---- programmatic dependent launch
+// A kernel launched with launch_dependent() may start while its predecessor
+// in the stream finishes: it computes its indices, then pdl_wait() holds it
+// until the predecessor has completed and its writes are visible.  Before
+// pdl_wait() it reads kernel parameters only, and every thread calls it, so
+// that a kernel's completion implies its predecessor's.  pdl_start_next()
+// stands where a block has done its sites, before the reduction: called at
+// the top, the next kernel's blocks fill the slots that happen to be free
+// and share SMs unevenly (CG iteration at 16^4, FP32: 50.9 us, as without;
+// called late 39.0; schur at 8^4 12.3 -> 5.7 us, hop at 32^3 x 64 96.6 -> 94.2).
+//
+// Captured launches have no such gaps to hide: on lattices that fill the GPU
+// the iteration block is 2 to 4 % slower with programmatic edges (16^4 38.5
+// -> 39.7 us an iteration), on small ones 4 to 8 % faster (8^4 27.3 -> 25.1).
+// So a launch under capture takes the attribute only where the library
+// captures its own block and the caller says that the launch is small; a
+// user's capture sees plain launches.
+__device__ __forceinline__ void pdl_start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// What this thread is capturing: an iteration block of the library, and the
+// sites (times right-hand sides) of the other lattices on parallel branches
+// of it.  Branches share the GPU, so whether a launch counts as small goes by
+// the sum (the uneven 8^4 + 12^4 + 16^3 x 32 batch lost 2 % when its small
+// lattices' launches spread over all SMs beside the large one's).
+struct OwnCapture {
+    bool on = false;
+    long other_sites = 0;
+};
+inline thread_local OwnCapture own_capture;
+
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), bool small, dim3 grid, dim3 block, cudaStream_t s, A... args)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (s) {  // (the legacy stream is never captured)
+        const cudaError_t e = cudaStreamIsCapturing(s, &cap);
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = cap == cudaStreamCaptureStatusNone || (own_capture.on && small) ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ------------------------------------------------------------ spinor fields
 // 24 reals per site: index 2*(spin*3 + colour) + {0: re, 1: im}.
 
@@ -116,6 +167,25 @@ template <> struct SpinorIO<P64> {
 #pragma unroll
         for (int k = 0; k < 12; ++k) p[(size_t)k * stride + i] = make_double2(v[2 * k], v[2 * k + 1]);
     }
+    // spins 2 B and 2 B + 1 (the 12 reals from 12 B)
+    template <int B>
+    __device__ __forceinline__ static void load_half(const void* base, int stride, int i, double v[12])
+    {
+        const double2* p = static_cast<const double2*>(base) + (size_t)(6 * B) * stride + i;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            double2 c = __ldg(p + (size_t)k * stride);
+            v[2 * k] = c.x;
+            v[2 * k + 1] = c.y;
+        }
+    }
+    template <int B>
+    __device__ __forceinline__ static void store_half(void* base, int stride, int i, const double v[12])
+    {
+        double2* p = static_cast<double2*>(base) + (size_t)(6 * B) * stride + i;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) p[(size_t)k * stride] = make_double2(v[2 * k], v[2 * k + 1]);
+    }
 };
 
 template <> struct SpinorIO<P32> {
@@ -138,6 +208,27 @@ template <> struct SpinorIO<P32> {
 #pragma unroll
         for (int k = 0; k < 6; ++k)
             p[(size_t)k * stride + i] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+    }
+    template <int B>
+    __device__ __forceinline__ static void load_half(const void* base, int stride, int i, float v[12])
+    {
+        const float4* p = static_cast<const float4*>(base) + (size_t)(3 * B) * stride + i;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            float4 c = __ldg(p + (size_t)k * stride);
+            v[4 * k] = c.x;
+            v[4 * k + 1] = c.y;
+            v[4 * k + 2] = c.z;
+            v[4 * k + 3] = c.w;
+        }
+    }
+    template <int B>
+    __device__ __forceinline__ static void store_half(void* base, int stride, int i, const float v[12])
+    {
+        float4* p = static_cast<float4*>(base) + (size_t)(3 * B) * stride + i;
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            p[(size_t)k * stride] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
     }
 };
 
@@ -179,6 +270,36 @@ template <int ISBF> struct SpinorHalfIO {
             p[(size_t)k * stride + i] = c;
         }
         reinterpret_cast<float*>(p + (size_t)3 * stride)[i] = n;
+    }
+    // spins 2 B and 2 B + 1: one whole chunk and half of the middle one
+    template <int B>
+    __device__ __forceinline__ static void load_half(const void* base, int stride, int i, float v[12])
+    {
+        const uint4* p = static_cast<const uint4*>(base);
+        const float n = __ldg(reinterpret_cast<const float*>(p + (size_t)3 * stride) + i);
+        const uint4 c = __ldg(p + (size_t)(2 * B) * stride + i);
+        const uint2 m = __ldg(reinterpret_cast<const uint2*>(p + (size_t)stride + i) + B);
+        const uint32_t w[6] = {B ? m.x : c.x, B ? m.y : c.y, B ? c.x : c.z, B ? c.y : c.w, B ? c.z : m.x, B ? c.w : m.y};
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const float2 a = h2f(w[k], ISBF);
+            v[2 * k] = a.x * n;
+            v[2 * k + 1] = a.y * n;
+        }
+    }
+    // n: the largest component of the whole site (half 0 stores the norm)
+    template <int B>
+    __device__ __forceinline__ static void store_half(void* base, int stride, int i, const float v[12], float n)
+    {
+        uint4* p = static_cast<uint4*>(base);
+        if (n < 1.17549435e-38f) n = 0.f;
+        const float s = n > 0.f ? 1.f / n : 0.f;
+        uint32_t w[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) w[k] = f2h(v[2 * k] * s, v[2 * k + 1] * s, ISBF);
+        p[(size_t)(2 * B) * stride + i] = B ? make_uint4(w[2], w[3], w[4], w[5]) : make_uint4(w[0], w[1], w[2], w[3]);
+        reinterpret_cast<uint2*>(p + (size_t)stride + i)[B] = B ? make_uint2(w[0], w[1]) : make_uint2(w[4], w[5]);
+        if (B == 0) reinterpret_cast<float*>(p + (size_t)3 * stride)[i] = n;
     }
 };
 template <> struct SpinorIO<P16> : SpinorHalfIO<0> {};
@@ -403,6 +524,18 @@ template <int ISBF> struct CloverHalfIO {
             float2 a = h2f(v.x, ISBF), b = h2f(v.y, ISBF), d = h2f(v.z, ISBF), e = h2f(v.w, ISBF);
             c[8 * k] = a.x; c[8 * k + 1] = a.y; c[8 * k + 2] = b.x; c[8 * k + 3] = b.y;
             c[8 * k + 4] = d.x; c[8 * k + 5] = d.y; c[8 * k + 6] = e.x; c[8 * k + 7] = e.y;
+        }
+    }
+    // block b alone: nine 8-byte pieces, two to a chunk
+    __device__ __forceinline__ static void load_block(const void* base, int stride, int i, int b, float c[36])
+    {
+        const uint2* p = static_cast<const uint2*>(base);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int piece = 9 * b + k;
+            const uint2 v = __ldg(p + ((size_t)(piece >> 1) * stride + i) * 2 + (piece & 1));
+            const float2 x = h2f(v.x, ISBF), y = h2f(v.y, ISBF);
+            c[4 * k] = x.x; c[4 * k + 1] = x.y; c[4 * k + 2] = y.x; c[4 * k + 3] = y.y;
         }
     }
     __device__ __forceinline__ static void store_all(void* base, int stride, int i, const float c[72])

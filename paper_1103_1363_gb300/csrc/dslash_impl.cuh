@@ -197,10 +197,10 @@ __device__ __forceinline__ void su3_mul_half(const R u[18], const R h[12], R w[1
 // swapped by DAG); the link is U_mu at checkerboard index lidx of parity
 // lpar; flip: the hop crosses the antiperiodic t boundary.
 template <int PG, int RECON, int MU, bool DAG, bool BWD, bool PACK, class R>
-__device__ __forceinline__ void hop_term(const DslashArgs& A, const R v[24], bool flip, int lpar, int lidx, R acc[24])
+__device__ __forceinline__ void hop_product(const DslashArgs& A, const R v[24], bool flip, int lpar, int lidx, R w[12])
 {
     constexpr int S = (BWD != DAG) ? +1 : -1;
-    R h[12], u[18], w[12];
+    R h[12], u[18];
     project<MU, S>(v, h);
     if (flip) {
 #pragma unroll
@@ -208,7 +208,13 @@ __device__ __forceinline__ void hop_term(const DslashArgs& A, const R v[24], boo
     }
     GaugeIO<PG, RECON>::load(A.gauge, A.g.stride, lpar, MU, lidx, u);
     su3_mul_half<BWD, PACK>(u, h, w);
-    accumulate<MU, S>(acc, w);
+}
+template <int PG, int RECON, int MU, bool DAG, bool BWD, bool PACK, class R>
+__device__ __forceinline__ void hop_term(const DslashArgs& A, const R v[24], bool flip, int lpar, int lidx, R acc[24])
+{
+    R w[12];
+    hop_product<PG, RECON, MU, DAG, BWD, PACK>(A, v, flip, lpar, lidx, w);
+    accumulate<MU, (BWD != DAG) ? +1 : -1>(acc, w);
 }
 
 // PG: storage of links and clover; PS: storage of spinor fields; the
@@ -280,9 +286,9 @@ __device__ __forceinline__ void load_half_hop(const char* in, const void* gauge,
 }
 
 template <int ISBF, int RECON, int MU, bool BWD, bool DAG, bool PACK>
-__device__ __forceinline__ void compute_half_hop(const HalfHopRaw<RECON>& r, bool flip, float acc[24])
+__device__ __forceinline__ void half_hop_product(const HalfHopRaw<RECON>& r, bool flip, float w[12])
 {
-    float v[24], h[12], u[18], w[12];
+    float v[24], h[12], u[18];
     // decode without the norm: the projection is linear, so the norm (and the
     // boundary sign) scale the 12 projected values instead of the 24 inputs
 #pragma unroll
@@ -305,7 +311,13 @@ __device__ __forceinline__ void compute_half_hop(const HalfHopRaw<RECON>& r, boo
 #pragma unroll
     for (int k = 0; k < 12; ++k) h[k] *= scale;
     su3_mul_half<BWD, PACK>(u, h, w);
-    accumulate<MU, S>(acc, w);
+}
+template <int ISBF, int RECON, int MU, bool BWD, bool DAG, bool PACK>
+__device__ __forceinline__ void compute_half_hop(const HalfHopRaw<RECON>& r, bool flip, float acc[24])
+{
+    float w[12];
+    half_hop_product<ISBF, RECON, MU, BWD, DAG, PACK>(r, flip, w);
+    accumulate<MU, (BWD != DAG) ? +1 : -1>(acc, w);
 }
 
 template <int ISBF, int RECON, bool DAG, bool PACK, int H>
@@ -351,6 +363,7 @@ __device__ __forceinline__ void hop_all_half(const DslashArgs& A, const char* in
 #define LQCD_DSLASH_MINB 4  // <= 128 registers; 4, 5, 6 measured within 5% on 32^3x64
 #endif
 #define DSLASH_MAX_BLOCK 128
+#define DSLASH_WIDE 2    // internal: the warp-per-direction kernel
 #define DSLASH_STAGED 1  // a "block size" that selects the shared-memory staged kernel (LQCD_BLOCK_STAGED)
 // Epilogue at output site i of right-hand side rhs for the hopping term
 // acc; nrm accumulates |out|^2 (|r|^2 for EPI_CG).
@@ -476,6 +489,7 @@ __global__ void __launch_bounds__(DSLASH_MAX_BLOCK, (PG == P64 ? 1 : LQCD_DSLASH
 {
     const int rhs = (int)(blockIdx.x % (unsigned)A.nrhs);
     const int sb = (int)(blockIdx.x / (unsigned)A.nrhs), nsb = (int)(gridDim.x / (unsigned)A.nrhs);
+    pdl_wait();
     if (A.skip && A.skip[rhs]) return;  // uniform over the rhs: no block of it reduces
     double nrm = 0.0;
     if constexpr (RED || EPI == EPI_CG) {
@@ -483,11 +497,13 @@ __global__ void __launch_bounds__(DSLASH_MAX_BLOCK, (PG == P64 ? 1 : LQCD_DSLASH
         // block's partial sum covers many sites
         for (int i = sb * blockDim.x + threadIdx.x; i < A.g.Vh; i += nsb * blockDim.x)
             dslash_site<PG, PS, RECON, DAG, EPI, RED>(A, rhs, i, nrm);
+        pdl_start_next();
         double v[1] = {nrm};
         block_reduce_finalize<1>(v, A.partials + rhs * A.part_rs, A.tickets + rhs, A.red + rhs * A.red_rs, sb, nsb);
     } else {
         const int i = sb * blockDim.x + threadIdx.x;
         if (i < A.g.Vh) dslash_site<PG, PS, RECON, DAG, EPI, RED>(A, rhs, i, nrm);
+        pdl_start_next();
     }
 }
 
@@ -524,8 +540,269 @@ cudaError_t launch_dslash_t(const DslashArgs& A, int nrhs, int block, cudaStream
     if ((long)gx * nrhs > 0x7fffffffL) return cudaErrorInvalidConfiguration;
     DslashArgs Ar = A;
     Ar.nrhs = nrhs;
-    dslash_kernel<PG, PS, RECON, DAG, EPI, RED><<<gx * nrhs, block, 0, s>>>(Ar);
-    return cudaGetLastError();
+    return launch_dependent(dslash_kernel<PG, PS, RECON, DAG, EPI, RED>, false, gx * nrhs, block, s, Ar);
+}
+
+// ---------------------------------------------------------------------------
+// The hopping term with a warp per direction (launches of few sites, see
+// wide_default).  A block takes 32 sites of one right-hand side: warps 0 to 3
+// each form the products U P v of both hops of one direction and put their
+// two colour vectors into shared memory; warp 4 (spins 0, 1) and warp 5
+// (spins 2, 3) meanwhile load the epilogue's operands (and form Cl y), then
+// add the eight products in the gathering kernel's order and run the epilogue
+// on their chiral half.
+//
+// Why: with few sites nothing is bound by bandwidth.  A thread per site runs
+// the loads and products of its eight hops one after another (registers keep
+// it from having all loads in flight), a chain that is mostly L2 latency, on
+// a GPU that is nearly empty; in FP64 the chain is 1100 instructions at one
+// per 64 cycles and scheduler.  Here the chain is two hops, one barrier and
+// the epilogue, over six times the warps.  Every sum runs over the same terms
+// in the same order, so that the fields are those of the gathering kernel bit
+// for bit (the norms' grid sums are grouped per 32 sites).  A warp per hop
+// (320 threads) was as fast below 2048 sites and 20 to 30 % slower at 10368;
+// four hops a warp slower below 4096.
+enum { WIDE_SITES = 32, WIDE_THREADS = 192 };
+
+template <class R> struct Pair;
+template <> struct Pair<float> { typedef float2 type; };
+template <> struct Pair<double> { typedef double2 type; };
+
+// The product of hop H (2 mu + backward) at site i into ws[6 H + q][lane].
+template <int PG, int PS, int RECON, bool DAG, bool PACK, int H>
+__device__ __forceinline__ void wide_hop(const DslashArgs& A, const char* in, int i, int full, const int c[4],
+                                         typename Pair<typename RealT<PS>::type>::type* ws)
+{
+    typedef typename RealT<PS>::type R;
+    constexpr int MU = H / 2;
+    constexpr bool BWD = (H & 1) != 0;
+    const int L = A.g.L[MU];
+    const int step = (MU > 0 ? A.g.L[0] : 1) * (MU > 1 ? A.g.L[1] : 1) * (MU > 2 ? A.g.L[2] : 1);
+    const bool edge = BWD ? c[MU] == 0 : c[MU] == L - 1;
+    const int nb = BWD ? (edge ? full + (L - 1) * step : full - step) : (edge ? full - (L - 1) * step : full + step);
+    const int j = nb >> 1;
+    const bool flip = MU == 3 && A.g.tanti && edge;
+    R w[12];
+    if constexpr ((PS == P16 || PS == PB16) && PG == PS) {
+        HopPlan hp;
+        hp.nb[H] = j;
+        hp.lidx[H] = BWD ? j : i;
+        HalfHopRaw<RECON> raw;
+        load_half_hop<RECON>(in, A.gauge, A.g.stride, A.par, hp, H, raw);
+        half_hop_product<PS == PB16 ? 1 : 0, RECON, MU, BWD, DAG, PACK>(raw, flip, w);
+    } else {
+        R v[24];
+        SpinorIO<PS>::load(in, A.g.stride, j, v);
+        hop_product<PG, RECON, MU, DAG, BWD, PACK>(A, v, flip, BWD ? 1 - A.par : A.par, BWD ? j : i, w);
+    }
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        ws[(6 * H + q) * 32 + lane].x = w[2 * q];
+        ws[(6 * H + q) * 32 + lane].y = w[2 * q + 1];
+    }
+}
+
+// both hops of direction MU
+template <int PG, int PS, int RECON, bool DAG, bool PACK, int MU>
+__device__ __forceinline__ void wide_hops(const DslashArgs& A, const char* in, int i, int full, const int c[4],
+                                          typename Pair<typename RealT<PS>::type>::type* ws)
+{
+    wide_hop<PG, PS, RECON, DAG, PACK, 2 * MU>(A, in, i, full, c, ws);
+    wide_hop<PG, PS, RECON, DAG, PACK, 2 * MU + 1>(A, in, i, full, c, ws);
+}
+
+template <bool DAG, int B, int H, class R>
+__device__ __forceinline__ void wide_sum(const typename Pair<R>::type* ws, R acc[24])
+{
+    const int lane = threadIdx.x & 31;
+    R w[12];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        const typename Pair<R>::type t = ws[(6 * H + q) * 32 + lane];
+        w[2 * q] = t.x;
+        w[2 * q + 1] = t.y;
+    }
+    accumulate<H / 2, (((H & 1) != 0) != DAG) ? +1 : -1>(acc, w);  // (the other half is dead code)
+    if constexpr (H < 7) wide_sum<DAG, B, H + 1>(ws, acc);
+}
+
+// What an epilogue warp holds before the barrier, for its half B of the site.
+template <int PS, int EPI>
+struct WideOperands {
+    typedef typename RealT<PS>::type R;
+    typedef typename RealT<AccumP<PS>::value>::type RA;
+    R t[EPI >= EPI_XPAY ? 12 : 1];            // Cl y
+    R cl[EPI == EPI_CLOVINV ? 36 : 1];        // block of Cl
+    R p[EPI == EPI_CG ? 12 : 1];
+    RA x[EPI == EPI_CG ? 12 : 1], r[EPI == EPI_CG ? 12 : 1], alpha;
+};
+
+template <int PG, int PS, int EPI, int B>
+__device__ __forceinline__ void wide_operands(const DslashArgs& A, int rhs, int i, WideOperands<PS, EPI>& o)
+{
+    typedef typename RealT<PS>::type R;
+    if constexpr (EPI == EPI_CLOVINV) {
+        if (A.clov) CloverIO<PG>::load_block(A.clov, A.g.stride, i, B, o.cl);
+    }
+    if constexpr (EPI >= EPI_XPAY) {
+        R yv[12];
+        SpinorIO<PS>::template load_half<B>(static_cast<const char*>(A.y) + rhs * A.y_rb, A.g.stride, i, yv);
+        if (A.clov) {
+            R cl[36];
+            CloverIO<PG>::load_block(A.clov, A.g.stride, i, B, cl);
+            hermitian6_apply<R>(cl, yv, o.t);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) o.t[k] = yv[k];
+        }
+    }
+    if constexpr (EPI == EPI_CG) {
+        typedef typename RealT<AccumP<PS>::value>::type RA;
+        constexpr int PA = AccumP<PS>::value;
+        const double* sc = A.scal + rhs * A.scal_rs;
+        const double den = sc[A.s_den] + sc[A.s_den2];
+        o.alpha = den > 0.0 ? (RA)((sc[A.s_num] + sc[A.s_num2]) / den) : (RA)0;
+        SpinorIO<PS>::template load_half<B>(static_cast<const char*>(A.p) + rhs * A.p_rb, A.g.stride, i, o.p);
+        SpinorIO<PA>::template load_half<B>(static_cast<const char*>(A.x) + rhs * A.acc_rb, A.g.stride, i, o.x);
+        SpinorIO<PA>::template load_half<B>(static_cast<const char*>(A.r) + rhs * A.acc_rb, A.g.stride, i, o.r);
+    }
+}
+
+// Sum, epilogue and store of half B; both epilogue warps run this together
+// (they exchange the half's norm and largest component through ex[2][32]).
+// Returns the site's |out|^2 (|r|^2) in the thread of half 1: its FP32 sum
+// runs over the 24 components in order, so half 1 continues from half 0's.
+template <int PG, int PS, bool DAG, int EPI, bool RED, int B>
+__device__ __forceinline__ double wide_finish(const DslashArgs& A, int rhs, int i, bool live,
+                                              const typename Pair<typename RealT<PS>::type>::type* ws,
+                                              WideOperands<PS, EPI>& o, typename RealT<PS>::type (*ex)[32])
+{
+    typedef typename RealT<PS>::type R;
+    typedef typename RealT<AccumP<PS>::value>::type RA;
+    constexpr bool HALF = PS == P16 || PS == PB16;
+    constexpr bool NORM = RED || EPI == EPI_CG;
+    const int lane = threadIdx.x & 31;
+    R full[24], out[12];
+#pragma unroll
+    for (int k = 0; k < 24; ++k) full[k] = 0;
+    wide_sum<DAG, B, 0, R>(ws, full);
+    const R* acc = full + 12 * B;
+    const R a = (R)A.a;
+    if constexpr (EPI == EPI_NONE) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) out[k] = acc[k] * a;
+    } else if constexpr (EPI == EPI_CLOVINV) {
+        if (A.clov) {
+            R t[12];
+            hermitian6_apply<R>(o.cl, acc, t);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) out[k] = a * t[k];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) out[k] = acc[k] * a;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) out[k] = o.t[k] + a * acc[k];
+    }
+    if constexpr (EPI == EPI_CG) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            o.x[k] += o.alpha * (RA)o.p[k];
+            o.r[k] -= o.alpha * (RA)out[k];
+        }
+        if (live) {
+            constexpr int PA = AccumP<PS>::value;
+            SpinorIO<PA>::template store_half<B>(static_cast<char*>(A.x) + rhs * A.acc_rb, A.g.stride, i, o.x);
+            SpinorIO<PA>::template store_half<B>(static_cast<char*>(A.r) + rhs * A.acc_rb, A.g.stride, i, o.r);
+        }
+    } else if constexpr (!HALF) {
+        if (live) SpinorIO<PS>::template store_half<B>(static_cast<char*>(A.out) + rhs * A.out_rb, A.g.stride, i, out);
+    }
+    R big = 0, n = 0;
+    if constexpr (HALF && EPI != EPI_CG) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) big = fmaxf(big, fabsf(out[k]));
+        ex[B][lane] = big;
+    }
+    if constexpr (NORM) {
+        if (B == 0) {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) n += EPI == EPI_CG ? (R)o.r[k] * (R)o.r[k] : out[k] * out[k];
+            ex[2][lane] = n;
+        }
+    }
+    if constexpr ((HALF && EPI != EPI_CG) || NORM) asm volatile("bar.sync 1, 64;" ::: "memory");
+    if constexpr (HALF && EPI != EPI_CG) {
+        big = fmaxf(big, ex[1 - B][lane]);
+        if (live)
+            SpinorIO<PS>::template store_half<B>(static_cast<char*>(A.out) + rhs * A.out_rb, A.g.stride, i, out, big);
+    }
+    if constexpr (NORM) {
+        if (B == 1) {
+            n = ex[2][lane];
+#pragma unroll
+            for (int k = 0; k < 12; ++k) n += EPI == EPI_CG ? (R)o.r[k] * (R)o.r[k] : out[k] * out[k];
+        }
+    }
+    return B == 1 && live ? (double)n : 0.0;
+}
+
+// One-dimensional grid as in dslash_kernel: block b serves right-hand side
+// b % nrhs and site block b / nrhs.
+template <int PG, int PS, int RECON, bool DAG, int EPI, bool RED>
+__global__ void __launch_bounds__(WIDE_THREADS, (PG == P64 ? 1 : 3)) dslash_wide_kernel(const DslashArgs A)
+{
+    typedef typename RealT<PS>::type R;
+    typedef typename Pair<R>::type R2;
+    __shared__ R2 ws[8 * 6 * 32];
+    __shared__ R ex[3][32];
+    const int rhs = (int)(blockIdx.x % (unsigned)A.nrhs);
+    const int sb = (int)(blockIdx.x / (unsigned)A.nrhs), nsb = (int)(gridDim.x / (unsigned)A.nrhs);
+    constexpr bool PACK = !(RED || EPI == EPI_CG);  // the gathering kernel's choice per launch class
+    const int warp = threadIdx.x >> 5;
+    const int i = sb * WIDE_SITES + (threadIdx.x & 31);
+    const bool live = i < A.g.Vh;
+    int c[4];
+    cb_coords(A.g, i, A.par, c);
+    const int full = full_index(A.g, c);
+    pdl_wait();
+    if (A.skip && A.skip[rhs]) return;  // uniform over the rhs: no block of it reduces
+    WideOperands<PS, EPI> o;
+    if (warp < 4) {
+        if (live) {
+            const char* in = static_cast<const char*>(A.in) + rhs * A.in_rb;
+            switch (warp) {
+            case 0: wide_hops<PG, PS, RECON, DAG, PACK, 0>(A, in, i, full, c, ws); break;
+            case 1: wide_hops<PG, PS, RECON, DAG, PACK, 1>(A, in, i, full, c, ws); break;
+            case 2: wide_hops<PG, PS, RECON, DAG, PACK, 2>(A, in, i, full, c, ws); break;
+            default: wide_hops<PG, PS, RECON, DAG, PACK, 3>(A, in, i, full, c, ws); break;
+            }
+        }
+    } else if (live) {
+        if (warp == 4) wide_operands<PG, PS, EPI, 0>(A, rhs, i, o);
+        else wide_operands<PG, PS, EPI, 1>(A, rhs, i, o);
+    }
+    __syncthreads();
+    double nrm = 0.0;
+    if (warp == 4) nrm = wide_finish<PG, PS, DAG, EPI, RED, 0>(A, rhs, i, live, ws, o, ex);
+    else if (warp == 5) nrm = wide_finish<PG, PS, DAG, EPI, RED, 1>(A, rhs, i, live, ws, o, ex);
+    pdl_start_next();
+    if constexpr (RED || EPI == EPI_CG) {
+        double v[1] = {nrm};
+        block_reduce_finalize<1>(v, A.partials + rhs * A.part_rs, A.tickets + rhs, A.red + rhs * A.red_rs, sb, nsb);
+    }
+}
+
+template <int PG, int PS, int RECON, bool DAG, int EPI, bool RED>
+cudaError_t launch_wide_t(const DslashArgs& A, int nrhs, cudaStream_t s)
+{
+    const long blocks = (long)((A.g.Vh + WIDE_SITES - 1) / WIDE_SITES) * nrhs;
+    if (blocks > 0x7fffffffL) return cudaErrorInvalidConfiguration;
+    DslashArgs Ar = A;
+    Ar.nrhs = nrhs;
+    return launch_dependent(dslash_wide_kernel<PG, PS, RECON, DAG, EPI, RED>, true, (unsigned)blocks, WIDE_THREADS, s, Ar);
 }
 
 // ---------------------------------------------------------------------------
@@ -780,7 +1057,8 @@ cudaError_t dispatch_dslash_p(const DslashArgs& A, int recon, bool dag, int epi,
     }
 #define LQ_CASE(RC, DG, EP, RD)                                                              \
     if (recon == RC && dag == DG && epi == EP && red == RD)                                 \
-        return launch_dslash_t<PG, PS, RC, DG, EP, RD>(A, nrhs, block, s);
+        return block == DSLASH_WIDE ? launch_wide_t<PG, PS, RC, DG, EP, RD>(A, nrhs, s)       \
+                                    : launch_dslash_t<PG, PS, RC, DG, EP, RD>(A, nrhs, block, s);
 #define LQ_EPIS(RC, DG)                  \
     LQ_CASE(RC, DG, EPI_NONE, false)     \
     LQ_CASE(RC, DG, EPI_CLOVINV, false)  \

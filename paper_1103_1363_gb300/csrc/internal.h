@@ -257,7 +257,7 @@ lqcd_status blas_cg_p_update(lqcd_ctx* c, void* p, int Pp, const void* r, int Pr
 lqcd_status blas_accumulate_x(lqcd_ctx* c, void* xhi, const void* xlo, int Plo, int nrhs, size_t hi_rb,
                               size_t lo_rb, int nf);
 lqcd_status blas_zero(lqcd_ctx* c, void* x, int P, int nrhs, size_t rb, int nf);
-lqcd_status blas_copy_scalar(lqcd_ctx* c, int dst_slot, int src_slot, int nrhs);
+lqcd_status blas_copy_scalar_pair(lqcd_ctx* c, int dst_slot, int src_slot, int nrhs);
 lqcd_status clover_apply_launch(lqcd_ctx* c, void* out, const void* in, int parity, int inverse, int P,
                                 int nrhs, size_t rb);
 // operators (api.cu)

@@ -233,9 +233,7 @@ lqcd_status run_block(Cg& s, int n, bool ru_at_end)
         LQ_TRY(blas_cg_p_update(s.c, s.Pv + s.oi, mode_ps(s.Pi), s.RV + s.oa, s.PA, s.R, s.rbi, s.rba, s.nf, rr_slot(j + 1),
                                 rr_slot(j)));
     }
-    LQ_TRY(blas_copy_scalar(s.c, rr_slot(0), rr_slot(n), s.R));
-    LQ_TRY(blas_copy_scalar(s.c, rr_slot(0) + 1, rr_slot(n) + 1, s.R));
-    return LQCD_OK;
+    return blas_copy_scalar_pair(s.c, rr_slot(0), rr_slot(n), s.R);
 }
 
 lqcd_status read_scalars(lqcd_ctx* c, int R, std::vector<double>& h)
@@ -646,10 +644,7 @@ lqcd_status run_block_persistent(std::vector<CgRun*>& runs, unsigned long long m
             LQ_TRY(reliable_update(s, jn));
             LQ_TRY(blas_cg_p_update(s.c, s.Pv + s.oi, mode_ps(s.Pi), s.RV + s.oa, s.PA, s.R, s.rbi, s.rba, s.nf,
                                     rr_slot(jn), rr_slot(jp)));
-            if (jn) {
-                LQ_TRY(blas_copy_scalar(s.c, rr_slot(0), rr_slot(1), s.R));
-                LQ_TRY(blas_copy_scalar(s.c, rr_slot(0) + 1, rr_slot(1) + 1, s.R));
-            }
+            if (jn) LQ_TRY(blas_copy_scalar_pair(s.c, rr_slot(0), rr_slot(1), s.R));
         }
     }
     return LQCD_OK;
@@ -748,6 +743,10 @@ lqcd_status iterate(std::vector<CgRun*>& runs, const lqcd_solver_params* p)
                 LQ_CUDA(cudaStreamBeginCapture(c0->stream, cudaStreamCaptureModeThreadLocal));
                 lqcd_status cs = LQCD_OK;
                 cudaError_t fe = cudaSuccess;
+                auto sites_of = [](const CgRun& r) { return (long)r.c->g.Vh * r.s.R; };
+                long total_sites = 0;  // of the block's parallel branches
+                for (size_t i = 0; i < runs.size(); ++i)
+                    if (mask >> i & 1) total_sites += sites_of(*runs[i]);
                 if (branches) fe = cudaEventRecord(fork.events[0], c0->stream);
                 for (size_t i = 0; i < runs.size() && cs == LQCD_OK && fe == cudaSuccess; ++i) {
                     if (!(mask >> i & 1)) continue;
@@ -759,7 +758,9 @@ lqcd_status iterate(std::vector<CgRun*>& runs, const lqcd_solver_params* p)
                         c->stream = fork.streams[i];
                     }
                     const long d0 = c->dslash_count, l0 = c->launches;
+                    own_capture = OwnCapture{true, branches ? total_sites - sites_of(*runs[i]) : 0};
                     cs = run_block(runs[i]->s, n, ru);
+                    own_capture = OwnCapture();
                     e.dslash[i] = c->dslash_count - d0;
                     e.launches[i] = c->launches - l0;
                     c->dslash_count = d0;

@@ -5,7 +5,7 @@ import pytest
 
 import oracle
 import synth
-from tests.gpu_helpers import require_cuda
+from tests.gpu_helpers import hop_ref, rel, require_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -70,3 +70,75 @@ def test_clover_build_and_inverse(lq, dims, kind, kappa, csw):
                 # per site: against the size of the operator times the input
                 err = np.linalg.norm(g - w, axis=-1) / (size * np.linalg.norm(psi.reshape(par.shape + (12,))[par == p], axis=-1))
                 assert err.max() < tol, (prec, inverse, p, err.max(), tol)
+
+
+@pytest.mark.parametrize("dims,nrhs,recon", [
+    ((2, 2, 2, 2), 1, 12),      # 8 sites per parity: most lanes idle, every neighbour wraps
+    ((4, 2, 6, 6), 3, 18),      # 144 sites: a last block of 16
+    ((8, 8, 8, 8), 1, 12),
+    ((6, 10, 14, 4), 5, 12),    # 8400 site-rhs: past the FP64 line, below the reducing one
+    ((8, 16, 16, 16), 1, 12),   # 16384: the last size of the plain launches
+    ((8, 16, 16, 18), 1, 12),   # the first past it
+])
+@pytest.mark.parametrize("prec", ["f64", "f32", "f16", "bf16links", "f16spinors", "bf16"])
+def test_small_launch_kernel_is_bit_identical(lq, dims, nrhs, recon, prec):
+    """The warp-per-direction kernel of small launches against the gathering
+    kernel (selected by a block of 96 threads): every operator, both
+    directions, with and without a clover term, bit for bit; the hopping term
+    against the oracle as well."""
+    import torch
+    U = synth.gauge_field(dims, "smooth", 5, eps=0.5)
+    psi = np.stack([synth.gaussian_spinor(dims, 6 + r) for r in range(nrhs)])
+    lat = lq.Lattice(dims, precisions=("f64", "f32", prec), recon=recon, max_nrhs=nrhs)
+    lat.gauge_load(on_device(U))
+    for csw in (0.0, 1.0):
+        lat.clover_compute(0.13, csw)
+        for op in (lq.OP_HOP, lq.OP_SCHUR, lq.OP_FULL):
+            full = op == lq.OP_FULL
+            fin = lat.new_field(prec, nrhs, full)
+            lat.pack(fin, on_device(psi), -1 if full else 1, prec, nrhs)
+            for dag in (False, True):
+                out = []
+                for block in (128, 96):
+                    lq.lqcd_tune_set(lat.ctx, prec, (block,) * 4)
+                    f = torch.zeros_like(fin)
+                    lat.dslash(f, fin, 1 if op == lq.OP_SCHUR else 0, 0.13, csw, op, dag, prec, nrhs)
+                    lat.sync()
+                    out.append(f)
+                assert torch.equal(*out), (csw, op, dag)
+    if prec == "f64" and nrhs > 1:
+        fin, fout = lat.new_field(prec, nrhs), lat.new_field(prec, nrhs)
+        lat.pack(fin, on_device(psi), 1, prec, nrhs)
+        lq.lqcd_tune_set(lat.ctx, prec, (128,) * 4)
+        lat.dslash(fout, fin, 0, prec=prec, nrhs=nrhs)
+        got = lat.canonical_spinor(nrhs)
+        lat.unpack(got, fout, 0, prec, nrhs)
+        lat.sync()
+        for r in range(nrhs):
+            assert rel(got[r].cpu().numpy(), hop_ref(U, psi[r], dims, 0)) < 1e-13
+
+
+@pytest.mark.parametrize("dims,inner", [((2, 2, 2, 2), "f64"), ((4, 2, 6, 6), "f32"), ((8, 8, 8, 8), "f16spinors"),
+                                        ((8, 16, 16, 12), "f32")])
+@pytest.mark.parametrize("graph", [0, 1])
+def test_small_solves(lq, dims, inner, graph):
+    """Solves whose every launch is small (reducing epilogues, captured and
+    not): the oracle's true residual, and the iterates of the gathering
+    kernel's solve (fields bit-identical, global sums regrouped)."""
+    import torch
+    U = synth.gauge_field(dims, "smooth", 7, eps=0.5)
+    b = synth.gaussian_spinor(dims, 8)
+    lat = lq.Lattice(dims, precisions=("f64", "f32"), stream=torch.cuda.Stream())
+    lat.gauge_load(on_device(U))
+    lat.clover_compute(0.12, 1.0)
+    A = oracle.clover(U, 0.12, 1.0)
+    xs = []
+    for block in (128, 96):
+        for prec in {"f64", "f32", inner}:
+            lq.lqcd_tune_set(lat.ctx, prec, (block,) * 4)
+        x, bd = lat.canonical_spinor(), on_device(b)
+        torch.cuda.synchronize()
+        _, st = lat.solve(x, bd, 1e-10, inner_prec=inner, use_graph=graph)
+        xs.append(x.cpu().numpy())
+        assert oracle.true_residual(U, A, 0.12, b, xs[-1]) <= 1e-10
+    assert rel(xs[0], xs[1]) < 1e-8  # both within 1e-10 residual of the solution, |M^-1| |M| well below 100
