@@ -179,10 +179,10 @@ lqcd_status blas_cg_p_update(lqcd_ctx* c, void* p, int Pp, const void* r, int Pr
     const bool small = (long)c->g.Vh * nrhs + own_capture.other_sites <= 12288;  // as the iteration's reducing hops
     if (Pr == P64) {
         if (Pp != P64) return fail(LQCD_ERR_INVALID, "cg_p_update: FP64 r needs FP64 p");
-        LQ_CUDA(launch_dependent(cg_p_kernel<P64, P64>, small, grid, block, c->stream, c->g, pp, p_rb, rr, r_rb, nf,
+        LQ_CUDA(launch_dependent(cg_p_kernel<P64, P64>, small, grid, block, c->stream, 0, c->g, pp, p_rb, rr, r_rb, nf,
                                  c->scal, s_num, s_den, c->skip));
     } else {
-        LQ_SWITCH_P(Pp, LQ_CUDA(launch_dependent(cg_p_kernel<PT, P32>, small, grid, block, c->stream, c->g, pp, p_rb, rr,
+        LQ_SWITCH_P(Pp, LQ_CUDA(launch_dependent(cg_p_kernel<PT, P32>, small, grid, block, c->stream, 0, c->g, pp, p_rb, rr,
                                                  r_rb, nf, c->scal, s_num, s_den, c->skip)));
     }
     c->launches++;
@@ -214,7 +214,7 @@ lqcd_status blas_zero(lqcd_ctx* c, void* x, int P, int nrhs, size_t rb, int nf)
 
 lqcd_status blas_copy_scalar_pair(lqcd_ctx* c, int dst, int src, int nrhs)
 {
-    LQ_CUDA(launch_dependent(copy_scalar_pair_kernel, false, dim3(1), dim3(64 * ((nrhs + 31) / 32)), c->stream, c->scal,
+    LQ_CUDA(launch_dependent(copy_scalar_pair_kernel, false, dim3(1), dim3(64 * ((nrhs + 31) / 32)), c->stream, 0, c->scal,
                              dst, src, nrhs));
     c->launches++;
     return LQCD_OK;

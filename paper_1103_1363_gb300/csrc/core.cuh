@@ -125,7 +125,7 @@ struct OwnCapture {
 inline thread_local OwnCapture own_capture;
 
 template <class... P, class... A>
-inline cudaError_t launch_dependent(void (*kernel)(P...), bool small, dim3 grid, dim3 block, cudaStream_t s, A... args)
+inline cudaError_t launch_dependent(void (*kernel)(P...), bool small, dim3 grid, dim3 block, cudaStream_t s, size_t smem, A... args)
 {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (s) {  // (the legacy stream is never captured)
@@ -138,6 +138,7 @@ inline cudaError_t launch_dependent(void (*kernel)(P...), bool small, dim3 grid,
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = &attr;
     cfg.numAttrs = cap == cudaStreamCaptureStatusNone || (own_capture.on && small) ? 1 : 0;

@@ -540,7 +540,7 @@ cudaError_t launch_dslash_t(const DslashArgs& A, int nrhs, int block, cudaStream
     if ((long)gx * nrhs > 0x7fffffffL) return cudaErrorInvalidConfiguration;
     DslashArgs Ar = A;
     Ar.nrhs = nrhs;
-    return launch_dependent(dslash_kernel<PG, PS, RECON, DAG, EPI, RED>, false, gx * nrhs, block, s, Ar);
+    return launch_dependent(dslash_kernel<PG, PS, RECON, DAG, EPI, RED>, false, gx * nrhs, block, s, 0, Ar);
 }
 
 // ---------------------------------------------------------------------------
@@ -802,7 +802,7 @@ cudaError_t launch_wide_t(const DslashArgs& A, int nrhs, cudaStream_t s)
     if (blocks > 0x7fffffffL) return cudaErrorInvalidConfiguration;
     DslashArgs Ar = A;
     Ar.nrhs = nrhs;
-    return launch_dependent(dslash_wide_kernel<PG, PS, RECON, DAG, EPI, RED>, true, (unsigned)blocks, WIDE_THREADS, s, Ar);
+    return launch_dependent(dslash_wide_kernel<PG, PS, RECON, DAG, EPI, RED>, true, (unsigned)blocks, WIDE_THREADS, s, 0, Ar);
 }
 
 // ---------------------------------------------------------------------------

@@ -238,7 +238,7 @@ lqcd_status solve_fgcr(lqcd_ctx* c, lqcd_net* net, double* x, const double* b, d
     // the elementwise update: one thread per (parity, float4 chunk, site), at most 8 blocks per SM
     const long nupd = (12L * c->g.Vh + block - 1) / block;
     const int gu = (int)(nupd < 8 * 152 ? nupd : 8 * 152);
-    bool sap = !net && c->sap_on;
+    bool sap = !net && c->sap_on, sap_ready = false;
     if (sap) LQ_TRY(sap_check(c, c->sap_bs));
     int iters = 0, restarts = 0, fallback = 0;
     double res = 1.0, res_prev = 0.0;
@@ -293,8 +293,9 @@ lqcd_status solve_fgcr(lqcd_ctx* c, lqcd_net* net, double* x, const double* b, d
             char* wk = Wb + (size_t)k * fld;
             if (net) LQ_TRY(net_apply_internal(net, zk, R32, fld));
             else if (sap) LQ_TRY(sap_apply(c, zk, R32, c->sap_bs, c->sap_ncycle, c->sap_nmr, vec64_field(c, 4, 0),
-                                           vec64_field(c, 5, 0)));
+                                           vec64_field(c, 5, 0), sap_ready));
             else LQ_TRY(convert_field(c, zk, P32, R32, P32, 1, fld, fld, 2, -1));
+            sap_ready = sap;
             LQ_TRY(op_full(c, wk, zk, mode, false, 1, fld));
             // classical Gram-Schmidt, a second pass when the first cancels
             std::vector<cd> ck(k, cd(0.0, 0.0)), cj(k);

@@ -232,7 +232,7 @@ lqcd_status solve_fgmres_dr(lqcd_ctx* c, lqcd_net* net, double* x, const double*
     LQ_TRY(read(c->scal, h, SC_PER_RHS));
     const double bn2 = h[SC_TMP + 0];
     const double bn = std::sqrt(bn2);
-    bool sap = !net && c->sap_on;
+    bool sap = !net && c->sap_on, sap_ready = false;
     if (sap) LQ_TRY(sap_check(c, c->sap_bs));
 
     auto vec = [&](int j) { return Vb + (size_t)j * fld; };
@@ -371,8 +371,9 @@ lqcd_status solve_fgmres_dr(lqcd_ctx* c, lqcd_net* net, double* x, const double*
             char* w = vec(nv);
             if (net) LQ_TRY(net_apply_internal(net, zj, vec(j), fld));
             else if (sap) LQ_TRY(sap_apply(c, zj, vec(j), c->sap_bs, c->sap_ncycle, c->sap_nmr, vec64_field(c, 4, 0),
-                                           vec64_field(c, 5, 0)));
+                                           vec64_field(c, 5, 0), sap_ready));
             else LQ_TRY(convert_field(c, zj, P32, vec(j), P32, 1, fld, fld, 2, -1));
+            sap_ready = sap;
             LQ_TRY(op_full(c, w, zj, mode, false, 1, fld));
             std::vector<cd> hcol;
             double wn = 0.0;

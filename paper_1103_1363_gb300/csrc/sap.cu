@@ -21,10 +21,11 @@
 // colour, so the gather needs no atomics.
 //
 // Blocks of at most SAP_THREADS sites run one site per thread with q and
-// delta in registers and the block's links staged in shared memory once per
-// block solve; larger blocks (up to 1024 sites, e.g. the paper's 8x4x8x4)
-// stride over the sites with q in shared memory, delta accumulated in dlt
-// and the links read through L1/L2.
+// delta in registers, the block's links staged in shared memory once per
+// block solve and the clover term read from a copy in block order; larger
+// blocks (up to 1024 sites, e.g. the paper's 8x4x8x4) stride over the sites
+// with q in shared memory, delta accumulated in dlt and the links read
+// through L1/L2.
 #include <cmath>
 #include <cstring>
 
@@ -45,6 +46,7 @@ struct SapArgs {
     const void* gauge;  // FP32 links
     const char* clov;   // FP32 clover A, parity p at clov + p * clov_pb; nullptr: A = 1
     size_t clov_pb;
+    const float4* clovb;  // the clover term in block order (one thread per site)
     float kappa;
     const char* rho_in; // residual on the solved sites before the neighbours' last correction
     char* rho_out;      // final block residual on the solved sites (may equal rho_in)
@@ -121,75 +123,6 @@ __device__ __forceinline__ void sap_hop(const SapArgs& a, const float4* rs, cons
     }
 }
 
-// The block's links in shared memory, [mu][plane][site]: recon-12 keeps rows
-// 0 and 1 as three float4 planes (row 2 rebuilt on use), recon-18 all nine
-// complex entries as float2 planes.  The link of x - mu that a backward hop
-// needs is the forward link of a site inside the block.
-template <int RECON> struct SmemLinks;
-template <> struct SmemLinks<12> {
-    static constexpr int bytes = 48;
-    __device__ __forceinline__ static void store(char* base, int vol, int mu, int l, const float u[18])
-    {
-        float4* p = reinterpret_cast<float4*>(base) + mu * 3 * vol + l;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) p[k * vol] = make_float4(u[4 * k], u[4 * k + 1], u[4 * k + 2], u[4 * k + 3]);
-    }
-    __device__ __forceinline__ static void load(const char* base, int vol, int mu, int l, float u[18])
-    {
-        const float4* p = reinterpret_cast<const float4*>(base) + mu * 3 * vol + l;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const float4 t = p[k * vol];
-            u[4 * k] = t.x;
-            u[4 * k + 1] = t.y;
-            u[4 * k + 2] = t.z;
-            u[4 * k + 3] = t.w;
-        }
-        reconstruct_row2(u);
-    }
-};
-template <> struct SmemLinks<18> {
-    static constexpr int bytes = 72;
-    __device__ __forceinline__ static void store(char* base, int vol, int mu, int l, const float u[18])
-    {
-        float2* p = reinterpret_cast<float2*>(base) + mu * 9 * vol + l;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) p[k * vol] = make_float2(u[2 * k], u[2 * k + 1]);
-    }
-    __device__ __forceinline__ static void load(const char* base, int vol, int mu, int l, float u[18])
-    {
-        const float2* p = reinterpret_cast<const float2*>(base) + mu * 9 * vol + l;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const float2 t = p[k * vol];
-            u[2 * k] = t.x;
-            u[2 * k + 1] = t.y;
-        }
-    }
-};
-
-// sap_hop with the links taken from shared memory
-template <int RECON, int MU>
-__device__ __forceinline__ void sap_hop_staged(const SapArgs& a, const float4* rs, const char* lk, const SapSite& s,
-                                               int l, int lstride, float acc[24])
-{
-    float v[24], h[12], u[18], w[12];
-    if (s.l[MU] + 1 < a.bs[MU]) {
-        smem_load(rs, a.vol, l + lstride, v);
-        project<MU, -1>(v, h);
-        SmemLinks<RECON>::load(lk, a.vol, MU, l, u);
-        su3_mul_half<false, true>(u, h, w);
-        accumulate<MU, -1>(acc, w);
-    }
-    if (s.l[MU] > 0) {
-        smem_load(rs, a.vol, l - lstride, v);
-        project<MU, +1>(v, h);
-        SmemLinks<RECON>::load(lk, a.vol, MU, l - lstride, u);
-        su3_mul_half<true, true>(u, h, w);
-        accumulate<MU, +1>(acc, w);
-    }
-}
-
 // acc += the hops of direction MU that reach site s from outside its block,
 // applied to the neighbours' corrections (lattice wrap-around and the
 // antiperiodic t phase included, as in the full operator).
@@ -249,27 +182,17 @@ __device__ __forceinline__ void sap_residual_site(const SapArgs& a, const SapSit
 
 // q = M_B rho at site s (rho of the whole block in shared memory), with the
 // site's contributions to |q|^2 and <q, rho>.
-// lk: the block's links in shared memory, or nullptr to read them from the
-// global FP32 copy.
-template <int RECON, bool STAGED>
-__device__ __forceinline__ void sap_block_op_site(const SapArgs& a, const float4* rs, const char* lk,
-                                                  const SapSite& s, int l, const int ls[4], float q[24], float& qq,
-                                                  float& qr_re, float& qr_im)
+template <int RECON>
+__device__ __forceinline__ void sap_block_op_site(const SapArgs& a, const float4* rs, const SapSite& s, int l,
+                                                  const int ls[4], float q[24], float& qq, float& qr_re, float& qr_im)
 {
     float acc[24], rho[24];
 #pragma unroll
     for (int k = 0; k < 24; ++k) acc[k] = 0.f;
-    if (STAGED) {
-        sap_hop_staged<RECON, 0>(a, rs, lk, s, l, ls[0], acc);
-        sap_hop_staged<RECON, 1>(a, rs, lk, s, l, ls[1], acc);
-        sap_hop_staged<RECON, 2>(a, rs, lk, s, l, ls[2], acc);
-        sap_hop_staged<RECON, 3>(a, rs, lk, s, l, ls[3], acc);
-    } else {
-        sap_hop<RECON, 0>(a, rs, s, l, ls[0], acc);
-        sap_hop<RECON, 1>(a, rs, s, l, ls[1], acc);
-        sap_hop<RECON, 2>(a, rs, s, l, ls[2], acc);
-        sap_hop<RECON, 3>(a, rs, s, l, ls[3], acc);
-    }
+    sap_hop<RECON, 0>(a, rs, s, l, ls[0], acc);
+    sap_hop<RECON, 1>(a, rs, s, l, ls[1], acc);
+    sap_hop<RECON, 2>(a, rs, s, l, ls[2], acc);
+    sap_hop<RECON, 3>(a, rs, s, l, ls[3], acc);
     smem_load(rs, a.vol, l, rho);
     if (a.clov) {
         clover_apply_site<P32>(a.clov + s.par * a.clov_pb, a.g.stride, s.cb, rho, q);
@@ -314,56 +237,233 @@ __device__ __forceinline__ void cta_sum3(float& a, float& b, float& c, float* re
     __syncthreads();  // red may be overwritten by the next call
 }
 
-__device__ __forceinline__ bool sap_block_coords(const SapArgs& a, int bc[4])
+// Coordinates of this CTA's block: the grid runs over the blocks of the
+// launch's colour (half of each row along x; the blocks per direction are even).
+__device__ __forceinline__ void sap_block_coords(const SapArgs& a, int bc[4])
 {
     int b = blockIdx.x;
-    bc[0] = b % a.nb[0];
-    b /= a.nb[0];
+    const int half = a.nb[0] >> 1;
+    const int xh = b % half;
+    b /= half;
     bc[1] = b % a.nb[1];
     b /= a.nb[1];
     bc[2] = b % a.nb[2];
     bc[3] = b / a.nb[2];
-    return ((bc[0] + bc[1] + bc[2] + bc[3]) & 1) == a.colour;
+    bc[0] = 2 * xh + ((bc[1] + bc[2] + bc[3] + a.colour) & 1);
 }
 
-// One site per thread (vol <= blockDim.x): q and delta in registers, the
-// block's links staged in shared memory behind rho.
-template <int RECON>
+// Extents of a block as the kernels see them: B in every direction, so that
+// neighbours and planes lie at constant distances, or read from the arguments (0).
+template <int B>
+struct SapShape {
+    __device__ __forceinline__ static int vol(const SapArgs& a) { return B ? B * B * B * B : a.vol; }
+    template <int MU>
+    __device__ __forceinline__ static int extent(const SapArgs& a) { return B ? B : a.bs[MU]; }
+    template <int MU>
+    __device__ __forceinline__ static int step(const SapArgs& a)
+    {
+        if (B) return MU == 0 ? 1 : MU == 1 ? B : MU == 2 ? B * B : B * B * B;
+        return (MU > 0 ? a.bs[0] : 1) * (MU > 1 ? a.bs[1] : 1) * (MU > 2 ? a.bs[2] : 1);
+    }
+};
+
+// The block's links in shared memory, [mu][plane][site]: recon-12 keeps rows
+// 0 and 1 as three float4 planes (row 2 rebuilt on use), recon-18 all nine
+// complex entries as float2 planes.  The link of x - mu that a backward hop
+// needs is the forward link of a site inside the block.
+template <int RECON> struct SmemLinks;
+template <> struct SmemLinks<12> {
+    static constexpr int bytes = 48;
+    __device__ __forceinline__ static void store(char* base, int vol, int mu, int l, const float u[18])
+    {
+        float4* p = reinterpret_cast<float4*>(base) + mu * 3 * vol + l;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) p[k * vol] = make_float4(u[4 * k], u[4 * k + 1], u[4 * k + 2], u[4 * k + 3]);
+    }
+    __device__ __forceinline__ static void load(const char* base, int vol, int mu, int l, float u[18])
+    {
+        const float4* p = reinterpret_cast<const float4*>(base) + mu * 3 * vol + l;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float4 t = p[k * vol];
+            u[4 * k] = t.x;
+            u[4 * k + 1] = t.y;
+            u[4 * k + 2] = t.z;
+            u[4 * k + 3] = t.w;
+        }
+        reconstruct_row2(u);
+    }
+};
+template <> struct SmemLinks<18> {
+    static constexpr int bytes = 72;
+    __device__ __forceinline__ static void store(char* base, int vol, int mu, int l, const float u[18])
+    {
+        float2* p = reinterpret_cast<float2*>(base) + mu * 9 * vol + l;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) p[k * vol] = make_float2(u[2 * k], u[2 * k + 1]);
+    }
+    __device__ __forceinline__ static void load(const char* base, int vol, int mu, int l, float u[18])
+    {
+        const float2* p = reinterpret_cast<const float2*>(base) + mu * 9 * vol + l;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const float2 t = p[k * vol];
+            u[2 * k] = t.x;
+            u[2 * k + 1] = t.y;
+        }
+    }
+};
+
+// ---------------------------------------------------------------------------
+// One thread per site (blocks of at most SAP_THREADS sites): q and delta in
+// registers, the block's links staged in shared memory behind rho, two CTAs
+// an SM, so that one block's loads and barriers hide behind the other's
+// arithmetic.  The clover term is read in every MR step, from a copy in block
+// order: in the field's order the pieces of a warp's load lie in sixteen
+// places (two sites of a parity side by side), and those lookups took 4.6 M
+// of L1's 7.8 M wavefronts a launch at 16^3 x 32, more than shared memory's
+// 3.2 M; from the copy they take 0.6 M.  What is left is bound by L1 and
+// shared memory (6.0 M wavefronts, two thirds of the time) and the issue of
+// 2000 instructions a site and step (40 %).  One application (4^4 blocks, 5
+// cycles of 4 steps): 16^4 391 -> 248 us, 16^3 x 32 436 -> 374, 32^3 x 64
+// 5.85 -> 5.40 ms, of which the copy is 8 us at 16^3 x 32.
+// Two threads a site (a colour vector each, the clover block in registers,
+// one CTA of 512 threads an SM) took 222 us at 16^4, 493 at 16^3 x 32 and 7.4
+// ms at 32^3 x 64: each reads every link for itself.
+template <int RECON, int MU, int B>
+__device__ __forceinline__ void sap_hop_staged(const SapArgs& a, const float4* rs, const char* lk, const int xl[4],
+                                               int l, float acc[24])
+{
+    typedef SapShape<B> Shape;
+    const int vol = Shape::vol(a), step = Shape::template step<MU>(a);
+    float v[24], h[12], u[18], w[12];
+    if (xl[MU] + 1 < Shape::template extent<MU>(a)) {
+        smem_load(rs, vol, l + step, v);
+        project<MU, -1>(v, h);
+        SmemLinks<RECON>::load(lk, vol, MU, l, u);
+        su3_mul_half<false, true>(u, h, w);
+        accumulate<MU, -1>(acc, w);
+    }
+    if (xl[MU] > 0) {
+        smem_load(rs, vol, l - step, v);
+        project<MU, +1>(v, h);
+        SmemLinks<RECON>::load(lk, vol, MU, l - step, u);
+        su3_mul_half<true, true>(u, h, w);
+        accumulate<MU, +1>(acc, w);
+    }
+}
+
+// A in block order: float4 chunk k (18 a site) of site l of block b at [(b 18 + k) vol + l].
+__global__ void sap_clover_kernel(const SapArgs a, float4* out)
+{
+    const int b = blockIdx.x;
+    const int bc[4] = {b % a.nb[0], b / a.nb[0] % a.nb[1], b / (a.nb[0] * a.nb[1]) % a.nb[2],
+                       b / (a.nb[0] * a.nb[1] * a.nb[2])};
+    for (int l = threadIdx.x; l < a.vol; l += blockDim.x) {
+        const SapSite s = sap_site(a, bc, l);
+        const float4* src = reinterpret_cast<const float4*>(a.clov + s.par * a.clov_pb) + s.cb;
+#pragma unroll
+        for (int k = 0; k < 18; ++k) out[((size_t)b * 18 + k) * a.vol + l] = __ldg(src + (size_t)k * a.g.stride);
+    }
+}
+
+template <int RECON, int B>
 __global__ void __launch_bounds__(SAP_THREADS, 2) sap_block_kernel_one(const SapArgs a)
 {
     extern __shared__ float4 sap_smem[];
-    __shared__ float red[3 * (SAP_THREADS / 32)];
-    float4* rs = sap_smem;                                     // block residual rho [6][vol]
-    char* lk = reinterpret_cast<char*>(sap_smem + 6 * a.vol);  // links [4][planes][vol]
+    __shared__ float red[2][3 * (SAP_THREADS / 32)];
+    const int vol = SapShape<B>::vol(a);
+    float4* rs = sap_smem;                                   // block residual rho [6][vol]
+    char* lk = reinterpret_cast<char*>(sap_smem + 6 * vol);  // links [4][planes][vol]
     int bc[4];
-    if (!sap_block_coords(a, bc)) return;  // whole CTA
-    const int ls[4] = {1, a.bs[0], a.bs[0] * a.bs[1], a.bs[0] * a.bs[1] * a.bs[2]};
+    sap_block_coords(a, bc);
     const int l = threadIdx.x;
-    const bool live = l < a.vol;
-    const SapSite s = sap_site(a, bc, live ? l : 0);
+    const bool live = B ? true : l < vol;
+    SapSite s = sap_site(a, bc, live ? l : 0);
+    if (B) {
+        s.l[0] = l % B; s.l[1] = l / B % B; s.l[2] = l / (B * B) % B; s.l[3] = l / (B * B * B);
+    }
+    const float4* clb = a.clovb + (size_t)(((bc[3] * a.nb[2] + bc[2]) * a.nb[1] + bc[1]) * a.nb[0] + bc[0]) * 18 * vol + l;
     float delta[24];
 #pragma unroll
     for (int k = 0; k < 24; ++k) delta[k] = 0.f;
-    if (live) {
-        float rho[24], u[18];
+    if (live) {  // links: complete since before the chain of launches (it starts with an ordinary one)
+        float u[18];
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
             GaugeIO<P32, RECON>::load(a.gauge, a.g.stride, s.par, mu, s.cb, u);
-            SmemLinks<RECON>::store(lk, a.vol, mu, l, u);
+            SmemLinks<RECON>::store(lk, vol, mu, l, u);
         }
+    }
+    pdl_wait();
+    if (live) {
+        float rho[24];
         sap_residual_site<RECON>(a, s, rho);
-        smem_store(rs, a.vol, l, rho);
+        smem_store(rs, vol, l, rho);
     }
     __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int it = 0; it < a.nmr; ++it) {
-        float q[24], qq = 0.f, qr_re = 0.f, qr_im = 0.f;
-        if (live) sap_block_op_site<RECON, true>(a, rs, lk, s, l, ls, q, qq, qr_re, qr_im);
-        cta_sum3(qq, qr_re, qr_im, red);  // also orders every read of rho before the update
-        if (!(qq > 0.f)) break;           // same totals in every thread: uniform
-        const float ar = qr_re / qq, ai = qr_im / qq;
+        float q[24], rho[24], qq = 0.f, qr = 0.f, qi = 0.f;
+        if (live) {
+            float acc[24];
+#pragma unroll
+            for (int k = 0; k < 24; ++k) acc[k] = 0.f;
+            sap_hop_staged<RECON, 0, B>(a, rs, lk, s.l, l, acc);
+            sap_hop_staged<RECON, 1, B>(a, rs, lk, s.l, l, acc);
+            sap_hop_staged<RECON, 2, B>(a, rs, lk, s.l, l, acc);
+            sap_hop_staged<RECON, 3, B>(a, rs, lk, s.l, l, acc);
+            smem_load(rs, vol, l, rho);
+            if (a.clov) {
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    float c[36];
+#pragma unroll
+                    for (int k = 0; k < 9; ++k) {
+                        const float4 v = __ldg(clb + (9 * b + k) * vol);
+                        c[4 * k] = v.x; c[4 * k + 1] = v.y; c[4 * k + 2] = v.z; c[4 * k + 3] = v.w;
+                    }
+                    hermitian6_apply<float>(c, rho + 12 * b, q + 12 * b);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 24; ++k) q[k] = rho[k];
+            }
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                const float qa = q[2 * k] - a.kappa * acc[2 * k];
+                const float qb = q[2 * k + 1] - a.kappa * acc[2 * k + 1];
+                q[2 * k] = qa;
+                q[2 * k + 1] = qb;
+                qq += qa * qa + qb * qb;
+                qr += qa * rho[2 * k] + qb * rho[2 * k + 1];  // <q, rho> = sum conj(q) rho
+                qi += qa * rho[2 * k + 1] - qb * rho[2 * k];
+            }
+        }
+        // CTA sums (two sets of partials in turn: one barrier, which also orders
+        // every read of rho before the update); every thread gets the same totals
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            qq += __shfl_xor_sync(0xffffffffu, qq, o);
+            qr += __shfl_xor_sync(0xffffffffu, qr, o);
+            qi += __shfl_xor_sync(0xffffffffu, qi, o);
+        }
+        float* const rd = red[it & 1];
+        if (lane == 0) {
+            rd[3 * warp] = qq;
+            rd[3 * warp + 1] = qr;
+            rd[3 * warp + 2] = qi;
+        }
+        __syncthreads();
+        qq = qr = qi = 0.f;
+        for (int w = 0; w < nw; ++w) {
+            qq += rd[3 * w];
+            qr += rd[3 * w + 1];
+            qi += rd[3 * w + 2];
+        }
+        if (!(qq > 0.f)) break;  // uniform
+        const float ar = qr / qq, ai = qi / qq;
         if (live) {  // delta += alpha rho, rho -= alpha q
-            float rho[24];
-            smem_load(rs, a.vol, l, rho);
 #pragma unroll
             for (int k = 0; k < 12; ++k) {
                 const float rr = rho[2 * k], ri = rho[2 * k + 1];
@@ -372,13 +472,14 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) sap_block_kernel_one(const Sap
                 rho[2 * k] = rr - (ar * q[2 * k] - ai * q[2 * k + 1]);
                 rho[2 * k + 1] = ri - (ar * q[2 * k + 1] + ai * q[2 * k]);
             }
-            smem_store(rs, a.vol, l, rho);
+            smem_store(rs, vol, l, rho);
         }
         __syncthreads();
     }
+    pdl_start_next();
     if (live) {
         float rho[24], zv[24];
-        smem_load(rs, a.vol, l, rho);
+        smem_load(rs, vol, l, rho);
         SpinorIO<P32>::store(a.rho_out + s.par * a.fb, a.g.stride, s.cb, rho);
         SpinorIO<P32>::store(a.dlt + s.par * a.fb, a.g.stride, s.cb, delta);
         char* zp = a.z + s.par * a.fb;
@@ -399,7 +500,7 @@ __global__ void __launch_bounds__(SAP_THREADS) sap_block_kernel_strided(const Sa
     float4* rs = sap_smem;              // block residual rho [6][vol]
     float4* qs = sap_smem + 6 * a.vol;  // q = M_B rho      [6][vol]
     int bc[4];
-    if (!sap_block_coords(a, bc)) return;  // whole CTA
+    sap_block_coords(a, bc);
     const int ls[4] = {1, a.bs[0], a.bs[0] * a.bs[1], a.bs[0] * a.bs[1] * a.bs[2]};
     const float zero[24] = {};
     for (int l = threadIdx.x; l < a.vol; l += blockDim.x) {
@@ -418,7 +519,7 @@ __global__ void __launch_bounds__(SAP_THREADS) sap_block_kernel_strided(const Sa
         for (int l = threadIdx.x; l < a.vol; l += blockDim.x) {
             const SapSite s = sap_site(a, bc, l);
             float q[24];
-            sap_block_op_site<RECON, false>(a, rs, nullptr, s, l, ls, q, qq, qr_re, qr_im);
+            sap_block_op_site<RECON>(a, rs, s, l, ls, q, qq, qr_re, qr_im);
             smem_store(qs, a.vol, l, q);
         }
         cta_sum3(qq, qr_re, qr_im, red);
@@ -475,7 +576,7 @@ lqcd_status sap_check(const lqcd_ctx* c, const int bs[4])
 }
 
 lqcd_status sap_apply(lqcd_ctx* c, void* z, const void* r, const int bs[4], int ncycle, int nmr, char* rho_buf,
-                      char* dlt_buf)
+                      char* dlt_buf, bool have_clover)
 {
     LQ_TRY(sap_check(c, bs));
     const size_t fb = c->field_bytes(P32), fld = 2 * fb;
@@ -500,15 +601,28 @@ lqcd_status sap_apply(lqcd_ctx* c, void* z, const void* r, const int bs[4], int 
     a.dlt = dlt_buf;
     a.z = static_cast<char*>(z);
     a.fb = fb;
-    const bool one = a.vol <= SAP_THREADS;
-    const int threads = one ? (a.vol + 31) / 32 * 32 : SAP_THREADS;
-    const size_t link_bytes = c->cfg.recon == 12 ? SmemLinks<12>::bytes : SmemLinks<18>::bytes;
-    const size_t smem = one ? (size_t)a.vol * (6 * sizeof(float4) + 4 * link_bytes)
-                            : (size_t)a.vol * 2 * 6 * sizeof(float4);
+    const bool small = a.vol <= SAP_THREADS;
     const bool r12 = c->cfg.recon == 12;
-    const void* fn = one ? (r12 ? (const void*)sap_block_kernel_one<12> : (const void*)sap_block_kernel_one<18>)
-                         : (r12 ? (const void*)sap_block_kernel_strided<12> : (const void*)sap_block_kernel_strided<18>);
-    LQ_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int threads = small ? (a.vol + 31) / 32 * 32 : SAP_THREADS;
+    const size_t link_bytes = r12 ? SmemLinks<12>::bytes : SmemLinks<18>::bytes;
+    const size_t smem = small ? (size_t)a.vol * (6 * sizeof(float4) + 4 * link_bytes)
+                              : (size_t)a.vol * 2 * 6 * sizeof(float4);
+    const bool cube = bs[0] == 4 && bs[1] == 4 && bs[2] == 4 && bs[3] == 4;
+    typedef void (*Kernel)(const SapArgs);
+    const Kernel fn = !small ? (r12 ? sap_block_kernel_strided<12> : sap_block_kernel_strided<18>)
+                      : cube ? (r12 ? sap_block_kernel_one<12, 4> : sap_block_kernel_one<18, 4>)
+                             : (r12 ? sap_block_kernel_one<12, 0> : sap_block_kernel_one<18, 0>);
+    LQ_CUDA(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (small && a.clov) {  // CG's inner vectors are free here: 576 bytes a site, of which the copy takes 288
+        static_assert(NVLO * 192 >= 288, "the block-ordered clover term exceeds the inner vectors");
+        float4* copy = reinterpret_cast<float4*>(c->veclo);
+        if (!have_clover) {
+            sap_clover_kernel<<<nblocks, threads, 0, c->stream>>>(a, copy);
+            LQ_CUDA(cudaGetLastError());
+            c->launches++;
+        }
+        a.clovb = copy;
+    }
     for (int cy = 0; cy < ncycle; ++cy)
         for (int colour = 0; colour < 2; ++colour) {
             // the first cycle starts from r on both colours (z = 0 there before
@@ -516,10 +630,8 @@ lqcd_status sap_apply(lqcd_ctx* c, void* z, const void* r, const int bs[4], int 
             a.rho_in = cy == 0 ? static_cast<const char*>(r) : rho_buf;
             a.has_prev = !(cy == 0 && colour == 0);
             a.colour = colour;
-            if (one && r12) sap_block_kernel_one<12><<<nblocks, threads, smem, c->stream>>>(a);
-            else if (one) sap_block_kernel_one<18><<<nblocks, threads, smem, c->stream>>>(a);
-            else if (r12) sap_block_kernel_strided<12><<<nblocks, threads, smem, c->stream>>>(a);
-            else sap_block_kernel_strided<18><<<nblocks, threads, smem, c->stream>>>(a);
+            if (small) LQ_CUDA(launch_dependent(fn, false, dim3(nblocks / 2), dim3(threads), c->stream, smem, a));
+            else fn<<<nblocks / 2, threads, smem, c->stream>>>(a);
             LQ_CUDA(cudaGetLastError());
             c->launches++;
         }
@@ -559,7 +671,7 @@ lqcd_status lqcd_sap_apply(lqcd_ctx* c, void* z, const void* r, const int block[
     if (ncycle < 1 || nmr < 1) return fail(LQCD_ERR_INVALID, "lqcd_sap_apply: ncycle and nmr must be >= 1");
     DeviceScope dev_scope;
     LQ_TRY(dev_scope.enter(c->device));
-    return sap_apply(c, z, r, block, ncycle, nmr, vec64_field(c, 4, 0), vec64_field(c, 5, 0));
+    return sap_apply(c, z, r, block, ncycle, nmr, vec64_field(c, 4, 0), vec64_field(c, 5, 0), false);
 }
 
 }  // extern "C"

@@ -142,3 +142,54 @@ def test_small_solves(lq, dims, inner, graph):
         xs.append(x.cpu().numpy())
         assert oracle.true_residual(U, A, 0.12, b, xs[-1]) <= 1e-10
     assert rel(xs[0], xs[1]) < 1e-8  # both within 1e-10 residual of the solution, |M^-1| |M| well below 100
+
+
+@pytest.mark.parametrize("dims,block,recon,csw", [
+    ((8, 8, 8, 8), (4, 4, 4, 4), 18, 1.0),    # the constant-extent kernel
+    ((8, 8, 8, 8), (4, 4, 4, 2), 12, 1.0),    # extents from the arguments
+    ((4, 12, 8, 4), (2, 6, 4, 2), 12, 1.0),   # 96 sites a block: a whole number of warps, fewer than the CTA's most
+    ((12, 12, 4, 4), (6, 6, 2, 2), 18, 1.0),  # 144: idle lanes
+    ((8, 8, 8, 8), (4, 4, 4, 4), 12, 0.0),    # no clover term
+])
+def test_sap_block_kernel(lq, dims, block, recon, csw):
+    """SAP of blocks of at most 256 sites against the oracle (FP32 sums of
+    about 2000 products a site, 6e-8 each, through nmr ncycle steps: 1e-5
+    bounds it generously), after other fields went through the same context."""
+    U = [synth.gauge_field(dims, "smooth", 11 + k, eps=0.5) for k in range(2)]
+    r = synth.gaussian_spinor(dims, 12)
+    lat = lq.Lattice(dims, precisions=("f64", "f32"), recon=recon)
+    for u in U:  # the second field's clover term must be the one that is used
+        lat.gauge_load(on_device(u))
+        lat.clover_compute(0.13, csw)
+        fr, fz = lat.new_field("f32", full=True), lat.new_field("f32", full=True)
+        lat.pack(fr, on_device(r), -1, "f32")
+        lat.sap_apply(fz, fr, block, 2, 3)
+        z = lat.canonical_spinor()
+        lat.unpack(z, fz, -1, "f32")
+        lat.sync()
+    A = oracle.clover(U[1], 0.13, csw) if csw else None
+    assert rel(z.cpu().numpy(), oracle.sap(U[1], A, 0.13, r, block, 2, 3)) < 1e-5
+
+
+def test_sap_solves_in_turn(lq):
+    """Flexible solves with SAP one after the other on one context, the block
+    shape, the field and the solver changing between them: each takes the
+    iterations of a fresh context."""
+    import torch
+    dims = (8, 8, 8, 8)
+    b = synth.gaussian_spinor(dims, 13)
+    old = lq.Lattice(dims, precisions=("f64", "f32"), gcr_nkrylov=20)
+    for seed, block, solver in ((14, (4, 4, 4, 4), lq.SOLVER_FGCR), (15, (4, 4, 4, 4), lq.SOLVER_FGMRES_DR),
+                                (15, (4, 4, 2, 4), lq.SOLVER_FGCR), (14, (4, 4, 4, 4), lq.SOLVER_FGCR)):
+        U = synth.gauge_field(dims, "smooth", seed, eps=0.5)
+        A = oracle.clover(U, 0.13, 1.0)
+        its = []
+        for lat in (old, lq.Lattice(dims, precisions=("f64", "f32"), gcr_nkrylov=20)):
+            lat.gauge_load(on_device(U))
+            lat.clover_compute(0.13, 1.0)
+            lat.set_sap(block, 2, 4)
+            x = lat.canonical_spinor()
+            _, st = lat.solve(x, on_device(b), 1e-10, solver=solver, inner_prec="f32", nkrylov=20)
+            its.append(st["iterations"])
+            assert oracle.true_residual(U, A, 0.13, b, x.cpu().numpy()) <= 1e-10
+        assert its[0] == its[1]
