@@ -382,6 +382,76 @@ __device__ __forceinline__ void load_act(const void* act, int bf, int V, int ch,
     else load_channel(reinterpret_cast<const float*>(item), V, ci, y, p);
 }
 
+// ---- transport of one BF16 channel at one site (multi-channel layers)
+// raw[k]: complex k = 3 spin + colour as two BF16 (real low).  The hop's link
+// times the boundary sign is staged as nine (u_r, u_r, -u_i, u_i) per site, so
+// that the two packed multiply-adds of a complex product,
+//   (re, im) += (u_r, u_r) (p_r, p_i),   (re, im) += (-u_i, u_i) (p_i, p_r),
+// take their operands as they come from shared memory and from the BF16
+// words: 72 packed instructions a channel instead of 144 scalar ones, with
+// the same products in the same order per lane (same bits).  Spins are done
+// one after the other, which keeps six decoded pairs live instead of 24 values.
+enum { LINK_PAIRS = 9 };
+
+__device__ __forceinline__ void load_raw_bf16(const void* act, int V, int ch, int b, int ci, int y, uint32_t raw[12])
+{
+    if (y >= 0) {
+        const uint4* src = reinterpret_cast<const uint4*>(static_cast<const char*>(act) + (size_t)b * V * ch * 48) +
+                           (size_t)ci * 3 * V + y;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const uint4 v = __ldg(src + (size_t)q * V);
+            raw[4 * q] = v.x; raw[4 * q + 1] = v.y; raw[4 * q + 2] = v.z; raw[4 * q + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 12; ++q) raw[q] = 0u;
+    }
+}
+
+__device__ __forceinline__ void stage_link_pairs(float4* dst, const float u[18], float sign)
+{
+#pragma unroll
+    for (int k = 0; k < LINK_PAIRS; ++k) {
+        const float ur = sign * u[2 * k], ui = sign * u[2 * k + 1];
+        dst[k] = make_float4(ur, ur, -ui, ui);
+    }
+}
+
+// w[colour][spin] = the transported channel, rounded to BF16
+__device__ __forceinline__ void transport_bf16(const uint32_t raw[12], const float4 link[LINK_PAIRS], bool identity,
+                                               uint32_t w[3][4])
+{
+    if (identity) {
+#pragma unroll
+        for (int ca = 0; ca < 3; ++ca)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) w[ca][r] = raw[3 * r + ca];
+        return;
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        float2 p[3], q[3];
+#pragma unroll
+        for (int cb = 0; cb < 3; ++cb) {  // BF16 is the upper half of FP32
+            const float re = __uint_as_float(raw[3 * r + cb] << 16), im = __uint_as_float(raw[3 * r + cb] & 0xffff0000u);
+            p[cb] = make_float2(re, im);
+            q[cb] = make_float2(im, re);
+        }
+#pragma unroll
+        for (int ca = 0; ca < 3; ++ca) {
+            float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int cb = 0; cb < 3; ++cb) {
+                const float4 u = link[3 * ca + cb];
+                acc = __ffma2_rn(make_float2(u.x, u.y), p[cb], acc);
+                acc = __ffma2_rn(make_float2(u.z, u.w), q[cb], acc);
+            }
+            w[ca][r] = pack_bf16x2(acc.x, acc.y);
+        }
+    }
+}
+
 // Default bound of a wait on the kernels' own MMAs and copies (a hop's MMAs
 // take microseconds); an expired wait sets ERRW_TIMEOUT and the CTA stops,
 // after waiting (with this bound) for its own operations in flight and
@@ -391,8 +461,8 @@ __device__ __forceinline__ void load_act(const void* act, int bf, int V, int ch,
 // BF16 forward of one layer on the tensor cores.  Shared memory: two
 // operand stages, each X (3 colour blocks of 128 sites x K2p) and B_h
 // (N2p x K2p), both BF16 in core-matrix order; two link stages (per site
-// the hop's link times the boundary sign in 18 floats, plus one float of
-// padding: the odd stride makes the reads conflict-free); then four
+// the hop's link as nine pairs of pairs: 36 words a site, so that the eight
+// lanes of a 16-byte read phase hit different banks); then four
 // mbarriers (MMAs of stage s done, B_h of stage s landed) and the
 // tensor-memory address.  Thread (site sl = tid % 128, group grp = tid /
 // 128): group 0 stages hop h+1's links while groups 1-3 gather hop h
@@ -411,8 +481,8 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_layer_tc_kernel(const NetL
     const int K2p = a.K2p, N2p = a.N2p;
     const uint32_t blk = (uint32_t)NTC_TS * K2p * 2;  // one colour block of X
     const uint32_t xbytes = 3 * blk, bbytes = (uint32_t)N2p * K2p * 2;
-    float* lbuf = reinterpret_cast<float*>(smem + 2 * xbytes + 2 * bbytes);              // [2][NTC_TS][19]
-    uint64_t* mma_bar = reinterpret_cast<uint64_t*>(lbuf + 2 * NTC_TS * 19);              // [2]
+    float4* lbuf = reinterpret_cast<float4*>(smem + 2 * xbytes + 2 * bbytes);             // [2][NTC_TS][LINK_PAIRS]
+    uint64_t* mma_bar = reinterpret_cast<uint64_t*>(lbuf + 2 * NTC_TS * LINK_PAIRS);      // [2]
     uint64_t* b_bar = mma_bar + 2;                                                     // [2]
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mma_bar + 4);
     const uint32_t sbo = (uint32_t)(K2p / 8) * 128;  // 8-row groups; K-adjacent core matrices are 128 B apart
@@ -442,10 +512,10 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_layer_tc_kernel(const NetL
     // previous item is transported (across the hop barrier and into the next tile).
     const int cfirst = grp - 1;
     const int nj = (grp > 0 && cfirst < a.cin) ? (a.cin - cfirst + TG - 1) / TG : 0;
-    float nxt[24];
+    uint32_t nxt[12];
     if ((int)blockIdx.x < total && nj > 0) {
         const int t = blockIdx.x, b = t / ntiles, x0 = (t - b * ntiles) * NTC_TS + sl;
-        load_act(a.in, a.in_bf16, a.V, a.cin, b, cfirst, x0 < a.V ? x0 : -1, nxt);
+        load_raw_bf16(a.in, a.V, a.cin, b, cfirst, x0 < a.V ? x0 : -1, nxt);
     }
     bool wait_failed = false;
     for (int t = blockIdx.x; t < total; t += gridDim.x) {
@@ -470,20 +540,18 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_layer_tc_kernel(const NetL
 #pragma unroll
                     for (int k = 0; k < 18; ++k) un[k] = 0.f;
                 }
-                float* ls = lbuf + (((h + 1) & 1) * NTC_TS + sl) * 19;
-#pragma unroll
-                for (int k = 0; k < 18; ++k) ls[k] = sign * un[k];
+                stage_link_pairs(lbuf + (((h + 1) & 1) * NTC_TS + sl) * LINK_PAIRS, un, sign);
             }
             if (tid == 0) {  // B_h, stored in core-matrix order: one contiguous bulk copy
                 tc::mbar_arrive_expect_tx(&b_bar[s], bbytes);
                 tc::bulk_g2s(Bst, a.Bh + (size_t)h * N2p * K2p, bbytes, &b_bar[s]);
             }
             ++copies;
-            float u[18];  // link of the hop times the boundary sign (staged at hop h - 1)
+            float4 u[LINK_PAIRS];  // link of the hop times the boundary sign (staged at hop h - 1)
             if (h > 0 && nj > 0) {
-                const float* ls = lbuf + ((h & 1) * NTC_TS + sl) * 19;
+                const float4* ls = lbuf + ((h & 1) * NTC_TS + sl) * LINK_PAIRS;
 #pragma unroll
-                for (int k = 0; k < 18; ++k) u[k] = ls[k];
+                for (int k = 0; k < LINK_PAIRS; ++k) u[k] = ls[k];
             }
             const int yh = x < a.V ? hop_neighbour(a, x, c0, c1, c2, c3, h) : -1;
             unsigned char* xrow = Xst + (sl >> 3) * sbo + (sl & 7) * 16;
@@ -491,45 +559,23 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_layer_tc_kernel(const NetL
             for (int j = 0; j < CPT; ++j) {
                 if (j >= nj) break;
                 const int ci = cfirst + TG * j;
-                float cur[24];
+                uint32_t cur[12], w[3][4];
 #pragma unroll
-                for (int q = 0; q < 24; ++q) cur[q] = nxt[q];
+                for (int q = 0; q < 12; ++q) cur[q] = nxt[q];
                 if (j + 1 < nj) {
-                    load_act(a.in, a.in_bf16, a.V, a.cin, b, ci + TG, yh, nxt);
+                    load_raw_bf16(a.in, a.V, a.cin, b, ci + TG, yh, nxt);
                 } else if (h + 1 < a.nhops) {
-                    load_act(a.in, a.in_bf16, a.V, a.cin, b, cfirst,
+                    load_raw_bf16(a.in, a.V, a.cin, b, cfirst,
                              x < a.V ? hop_neighbour(a, x, c0, c1, c2, c3, h + 1) : -1, nxt);
                 } else if (tn < total) {
                     const int bn = tn / ntiles, xn = (tn - bn * ntiles) * NTC_TS + sl;
-                    load_act(a.in, a.in_bf16, a.V, a.cin, bn, cfirst, xn < a.V ? xn : -1, nxt);
+                    load_raw_bf16(a.in, a.V, a.cin, bn, cfirst, xn < a.V ? xn : -1, nxt);
                 }
+                transport_bf16(cur, u, h == 0, w);
+                // k2 = 8 ci .. 8 ci + 7: one 16-byte row of core matrix (site group, ci)
 #pragma unroll
-                for (int ca = 0; ca < 3; ++ca) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        float re, im;
-                        if (h == 0) {
-                            re = cur[2 * (3 * r + ca)];
-                            im = cur[2 * (3 * r + ca) + 1];
-                        } else {
-                            re = 0.f;
-                            im = 0.f;
-#pragma unroll
-                            for (int cb = 0; cb < 3; ++cb) {  // one multiply-add per real product
-                                const float ur = u[2 * (3 * ca + cb)], ui = u[2 * (3 * ca + cb) + 1];
-                                const float pr = cur[2 * (3 * r + cb)], pi = cur[2 * (3 * r + cb) + 1];
-                                re += ur * pr;
-                                re -= ui * pi;
-                                im += ur * pi;
-                                im += ui * pr;
-                            }
-                        }
-                        w[r] = pack_bf16x2(re, im);
-                    }
-                    // k2 = 8 ci .. 8 ci + 7: one 16-byte row of core matrix (site group, ci)
-                    *reinterpret_cast<uint4*>(xrow + ca * blk + ci * 128) = make_uint4(w[0], w[1], w[2], w[3]);
-                }
+                for (int ca = 0; ca < 3; ++ca)
+                    *reinterpret_cast<uint4*>(xrow + ca * blk + ci * 128) = make_uint4(w[ca][0], w[ca][1], w[ca][2], w[ca][3]);
             }
             tc::fence_proxy_async();
             if (!wait_failed) wait_failed = !tc::mbar_wait(&b_bar[s], (g >> 1) & 1u, a.wait_ns);
@@ -1156,8 +1202,8 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_hg_kernel(const NetL
     const uint32_t blkx = (uint32_t)WG_TS * K2p * 2, blkg = (uint32_t)WG_TS * WG_MN * 2;
     unsigned char* const Xs = smem;                  // [2][3][blkx]
     unsigned char* const Gs = smem + 6 * blkx;       // [2][3][blkg]
-    float* lbuf = reinterpret_cast<float*>(Gs + 6 * blkg);                        // [2][WG_TS][19]
-    uint64_t* mma_bar = reinterpret_cast<uint64_t*>(lbuf + 2 * WG_TS * 19);       // [2]
+    float4* lbuf = reinterpret_cast<float4*>(Gs + 6 * blkg);                         // [2][WG_TS][LINK_PAIRS]
+    uint64_t* mma_bar = reinterpret_cast<uint64_t*>(lbuf + 2 * WG_TS * LINK_PAIRS);  // [2]
     uint32_t* tslot = reinterpret_cast<uint32_t*>(mma_bar + 2);
     const uint32_t idesc = tc::idesc_bf16_f32(WG_MN, K2p) | (1u << 15) | (1u << 16);  // A and B MN-major
     const uint32_t ncols = (uint32_t)a.tmem_cols;
@@ -1186,15 +1232,13 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_hg_kernel(const NetL
 #pragma unroll
             for (int q = 0; q < 18; ++q) un[q] = 0.f;
         }
-        float* ls = lbuf + (slot * WG_TS + sl) * 19;
-#pragma unroll
-        for (int q = 0; q < 18; ++q) ls[q] = sign * un[q];
+        stage_link_pairs(lbuf + (slot * WG_TS + sl) * LINK_PAIRS, un, sign);
     };
-    float nxt[24];
+    uint32_t nxt[12];
     if ((int)blockIdx.x < total) {
         const int t = blockIdx.x, b = t / ntiles, x = (t - b * ntiles) * WG_TS + sl;
         if (grp == 0) stage_links(x, h0, 0);
-        if (nj > 0) load_act(a.in, a.in_bf16, a.V, a.cin, b, cfirst, x < a.V ? site_neighbour(a, x, h0) : -1, nxt);
+        if (nj > 0) load_raw_bf16(a.in, a.V, a.cin, b, cfirst, x < a.V ? site_neighbour(a, x, h0) : -1, nxt);
     }
     tc::fence_before();
     __syncthreads();
@@ -1220,23 +1264,19 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_hg_kernel(const NetL
             unsigned char* const Gb = Gs + (q & 1) * 3 * blkg;
             if (hl == 0) {  // the output gradient at the tile's sites, once per tile
                 for (int co = grp; co < a.cout; co += NG) {
-                    float p[24];
-                    load_act(gout, a.gout_bf16, a.V, a.cout, b, co, x < a.V ? x : -1, p);
+                    uint32_t p[12];
+                    load_raw_bf16(gout, a.V, a.cout, b, co, x < a.V ? x : -1, p);
 #pragma unroll
-                    for (int ca = 0; ca < 3; ++ca) {
-                        uint32_t w[4];
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) w[r] = pack_bf16x2(p[2 * (3 * r + ca)], p[2 * (3 * r + ca) + 1]);
+                    for (int ca = 0; ca < 3; ++ca)
                         *reinterpret_cast<uint4*>(Gb + ca * blkg + (sl >> 3) * sbog + co * 128 + rowoff) =
-                            make_uint4(w[0], w[1], w[2], w[3]);
-                    }
+                            make_uint4(p[ca], p[3 + ca], p[6 + ca], p[9 + ca]);
                 }
             }
-            float u[18];
+            float4 u[LINK_PAIRS];
             if (nj > 0) {
-                const float* ls = lbuf + (s * WG_TS + sl) * 19;
+                const float4* ls = lbuf + (s * WG_TS + sl) * LINK_PAIRS;
 #pragma unroll
-                for (int k = 0; k < 18; ++k) u[k] = ls[k];
+                for (int k = 0; k < LINK_PAIRS; ++k) u[k] = ls[k];
             }
             const int yh = x < a.V ? site_neighbour(a, x, h) : -1;
             unsigned char* const Xb = Xs + s * 3 * blkx;
@@ -1244,42 +1284,20 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_hg_kernel(const NetL
             for (int j = 0; j < CPT; ++j) {
                 if (j >= nj) break;
                 const int ci = cfirst + TG * j;
-                float cur[24];
+                uint32_t cur[12], w[3][4];
 #pragma unroll
-                for (int k = 0; k < 24; ++k) cur[k] = nxt[k];
+                for (int k = 0; k < 12; ++k) cur[k] = nxt[k];
                 if (j + 1 < nj) {
-                    load_act(a.in, a.in_bf16, a.V, a.cin, b, ci + TG, yh, nxt);
+                    load_raw_bf16(a.in, a.V, a.cin, b, ci + TG, yh, nxt);
                 } else if (more) {
-                    load_act(a.in, a.in_bf16, a.V, a.cin, last ? bn : b, cfirst,
+                    load_raw_bf16(a.in, a.V, a.cin, last ? bn : b, cfirst,
                              xs < a.V ? site_neighbour(a, xs, hs) : -1, nxt);
                 }
+                transport_bf16(cur, u, h == 0, w);
 #pragma unroll
-                for (int ca = 0; ca < 3; ++ca) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        float re, im;
-                        if (h == 0) {
-                            re = cur[2 * (3 * r + ca)];
-                            im = cur[2 * (3 * r + ca) + 1];
-                        } else {
-                            re = 0.f;
-                            im = 0.f;
-#pragma unroll
-                            for (int cb = 0; cb < 3; ++cb) {  // one multiply-add per real product
-                                const float ur = u[2 * (3 * ca + cb)], ui = u[2 * (3 * ca + cb) + 1];
-                                const float pr = cur[2 * (3 * r + cb)], pi = cur[2 * (3 * r + cb) + 1];
-                                re += ur * pr;
-                                re -= ui * pi;
-                                im += ur * pi;
-                                im += ui * pr;
-                            }
-                        }
-                        w[r] = pack_bf16x2(re, im);
-                    }
+                for (int ca = 0; ca < 3; ++ca)
                     *reinterpret_cast<uint4*>(Xb + ca * blkx + (sl >> 3) * sbox + ci * 128 + rowoff) =
-                        make_uint4(w[0], w[1], w[2], w[3]);
-                }
+                        make_uint4(w[ca][0], w[ca][1], w[ca][2], w[ca][3]);
             }
             tc::fence_proxy_async();
             if (__syncthreads_or(wait_failed)) {
@@ -1781,7 +1799,7 @@ NetLayerArgs layer_args(const lqcd_net* n, int l, bool adjoint, const float* in,
 // that one CTA runs per SM and its tensor-memory allocation never waits.
 size_t layer_smem_tc(const NetLayerArgs& a)
 {
-    const size_t need = 2 * ((size_t)3 * NTC_TS * a.K2p * 2 + (size_t)a.N2p * a.K2p * 2) + 2 * NTC_TS * 19 * 4 + 4 * 8 + 16;
+    const size_t need = 2 * ((size_t)3 * NTC_TS * a.K2p * 2 + (size_t)a.N2p * a.K2p * 2) + 2 * NTC_TS * LINK_PAIRS * 16 + 4 * 8 + 16;
     return need > (size_t)NTC_MIN_SMEM ? need : (size_t)NTC_MIN_SMEM;
 }
 
@@ -1979,7 +1997,7 @@ lqcd_status run_wgrad(lqcd_net* n, int layer, const float* in, const float* gout
             if (n->max_ctas > 0 && gx > n->max_ctas) gx = n->max_ctas;
             NetLayerArgs w = a;
             w.tmem_cols = 512;
-            const size_t smw = (size_t)6 * WG_TS * (a.K2p + WG_MN) * 2 + (size_t)2 * WG_TS * 19 * 4 + 2 * 8 + 16;
+            const size_t smw = (size_t)6 * WG_TS * (a.K2p + WG_MN) * 2 + (size_t)2 * WG_TS * LINK_PAIRS * 16 + 2 * 8 + 16;
             dim3 gw(gx, 2);
             if (c->cfg.recon == 12) {
                 LQ_CUDA(cudaFuncSetAttribute(net_wgrad_hg_kernel<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw));
