@@ -79,16 +79,10 @@ __device__ __forceinline__ size_t planar_c(int V, int ci, int k, int site)
 // Link for hop h at canonical site x: V (3x3 complex, 18 floats) and the
 // fermion sign; returns the neighbour site.
 template <int RECON>
-__device__ __forceinline__ int hop_link(const NetLayerArgs& a, int x, int h, float u[18], float& sign)
+__device__ __forceinline__ int hop_link(const NetLayerArgs& a, int x, int c0, int c1, int c2, int c3, int h, float u[18],
+                                        float& sign)
 {
     const int L0 = a.L[0], L1 = a.L[1], L2 = a.L[2], L3 = a.L[3];
-    int s = x;
-    const int c0 = s % L0;
-    s /= L0;
-    const int c1 = s % L1;
-    s /= L1;
-    const int c2 = s % L2;
-    const int c3 = s / L2;
     sign = 1.f;
     if (h == 0) return x;
     const int mu = (h - 1) / 2;
@@ -118,6 +112,17 @@ __device__ __forceinline__ int hop_link(const NetLayerArgs& a, int x, int h, flo
             }
     }
     return y;
+}
+
+template <int RECON>
+__device__ __forceinline__ int hop_link(const NetLayerArgs& a, int x, int h, float u[18], float& sign)
+{
+    int s = x;
+    const int c0 = s % a.L[0];
+    s /= a.L[0];
+    const int c1 = s % a.L[1];
+    s /= a.L[1];
+    return hop_link<RECON>(a, x, c0, c1, s % a.L[2], s / a.L[2], h, u, sign);
 }
 
 __device__ __forceinline__ uint16_t f2bf(float f)
@@ -451,6 +456,47 @@ __device__ __forceinline__ void transport_bf16(const uint32_t raw[12], const flo
         }
     }
 }
+
+// Position of a thread's loads in its sequence of items: tiles
+// t, t + gridDim.x, ..., hops h0 .. h1 - 1, channels cfirst + step j (j < nj).
+// The neighbour is worked out once a hop and the coordinates once a tile (a
+// division by each extent): the weight gradient spent 150 of its 410
+// instructions an item on them.
+struct ItemCursor {
+    int t, h, j;
+    int b, x, y;  // batch item, site (>= V: none), neighbour (-1: none)
+    int c0, c1, c2, c3;
+    __device__ __forceinline__ void set_tile(const NetLayerArgs& a, int ntiles, int ts, int sl)
+    {
+        b = t / ntiles;
+        x = (t - b * ntiles) * ts + sl;
+        int s = x;
+        c0 = s % a.L[0];
+        s /= a.L[0];
+        c1 = s % a.L[1];
+        s /= a.L[1];
+        c2 = s % a.L[2];
+        c3 = s / a.L[2];
+    }
+    __device__ __forceinline__ void set_hop(const NetLayerArgs& a)
+    {
+        y = x < a.V ? hop_neighbour(a, x, c0, c1, c2, c3, h) : -1;
+    }
+    // the next item's first hop of a tile: total tiles in all, ts sites each
+    __device__ __forceinline__ void advance(const NetLayerArgs& a, int nj, int h0, int h1, int total, int ntiles, int ts,
+                                            int sl)
+    {
+        if (++j < nj) return;
+        j = 0;
+        if (++h == h1) {
+            h = h0;
+            t += gridDim.x;
+            if (t < total) set_tile(a, ntiles, ts, sl);
+        }
+        if (t < total) set_hop(a);
+        else y = -1;
+    }
+};
 
 // Default bound of a wait on the kernels' own MMAs and copies (a hop's MMAs
 // take microseconds); an expired wait sets ERRW_TIMEOUT and the CTA stops,
@@ -1181,13 +1227,6 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_o1_kernel(const NetL
 // group 0 while groups 1-7 gather this stage's channels one item ahead.
 enum { WG_TS = 64, WG_HOPS = 5, WG_MN = 128 };
 
-__device__ __forceinline__ int site_neighbour(const NetLayerArgs& a, int x, int h)
-{
-    const int c0 = x % a.L[0], c1 = (x / a.L[0]) % a.L[1], c2 = (x / (a.L[0] * a.L[1])) % a.L[2],
-              c3 = x / (a.L[0] * a.L[1] * a.L[2]);
-    return hop_neighbour(a, x, c0, c1, c2, c3, h);
-}
-
 template <int RECON>
 __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_hg_kernel(const NetLayerArgs a, const float* gout, float* gW)
 {
@@ -1223,22 +1262,31 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_hg_kernel(const NetL
     const int cfirst = grp - 1;
     const int nj = (grp > 0 && cfirst < a.cin) ? (a.cin - cfirst + TG - 1) / TG : 0;
     // links of hop h at site x into slot `slot` (group 0): times the boundary sign, zero past V or for h = 0
-    auto stage_links = [&](int x, int h, int slot) {
+    auto stage_links = [&](const ItemCursor& p, int slot) {
         float un[18];
         float sign = 1.f;
-        if (x < a.V && h > 0) {
-            hop_link<RECON>(a, x, h, un, sign);
+        if (p.x < a.V && p.h > 0) {
+            hop_link<RECON>(a, p.x, p.c0, p.c1, p.c2, p.c3, p.h, un, sign);
         } else {
 #pragma unroll
             for (int q = 0; q < 18; ++q) un[q] = 0.f;
         }
         stage_link_pairs(lbuf + (slot * WG_TS + sl) * LINK_PAIRS, un, sign);
     };
+    const int h1 = h0 + nh;
     uint32_t nxt[12];
-    if ((int)blockIdx.x < total) {
-        const int t = blockIdx.x, b = t / ntiles, x = (t - b * ntiles) * WG_TS + sl;
-        if (grp == 0) stage_links(x, h0, 0);
-        if (nj > 0) load_raw_bf16(a.in, a.V, a.cin, b, cfirst, x < a.V ? site_neighbour(a, x, h0) : -1, nxt);
+    ItemCursor at;  // group 0: the stage whose links are staged next; others: the next load
+    at.t = blockIdx.x;
+    at.h = h0;
+    at.j = 0;
+    at.set_tile(a, ntiles, WG_TS, sl);
+    at.set_hop(a);
+    if (grp == 0) {
+        if ((int)blockIdx.x < total) stage_links(at, 0);
+        at.advance(a, 1, h0, h1, total, ntiles, WG_TS, sl);
+    } else if (nj > 0) {
+        load_raw_bf16(a.in, a.V, a.cin, at.b, cfirst, at.y, nxt);
+        at.advance(a, nj, h0, h1, total, ntiles, WG_TS, sl);
     }
     tc::fence_before();
     __syncthreads();
@@ -1250,17 +1298,14 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_hg_kernel(const NetL
     bool wait_failed = false, failed = false;
     for (int t = blockIdx.x; t < total && !failed; t += gridDim.x, ++q) {
         const int b = t / ntiles, x = (t - b * ntiles) * WG_TS + sl;
-        const int tn = t + gridDim.x;
-        const int bn = tn / ntiles, xn = (tn - bn * ntiles) * WG_TS + sl;
         for (int hl = 0; hl < nh; ++hl) {
             const int h = h0 + hl, s = g & 1;
             // X stage s (and the G buffer of this tile's parity) is free once stage g - 2's MMAs completed
             if (g >= 2 && !wait_failed) wait_failed = !tc::mbar_wait(&mma_bar[s], ((g - 2) >> 1) & 1u, a.wait_ns);
-            // the next stage: hop h + 1 of this tile, else the first hop of the next tile
-            const bool last = hl + 1 == nh;
-            const int xs = last ? xn : x, hs = last ? h0 : h + 1;
-            const bool more = !last || tn < total;
-            if (grp == 0 && more) stage_links(xs, hs, (g + 1) & 1);
+            if (grp == 0 && at.t < total) {  // the next stage's links
+                stage_links(at, (g + 1) & 1);
+                at.advance(a, 1, h0, h1, total, ntiles, WG_TS, sl);
+            }
             unsigned char* const Gb = Gs + (q & 1) * 3 * blkg;
             if (hl == 0) {  // the output gradient at the tile's sites, once per tile
                 for (int co = grp; co < a.cout; co += NG) {
@@ -1278,7 +1323,6 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_hg_kernel(const NetL
 #pragma unroll
                 for (int k = 0; k < LINK_PAIRS; ++k) u[k] = ls[k];
             }
-            const int yh = x < a.V ? site_neighbour(a, x, h) : -1;
             unsigned char* const Xb = Xs + s * 3 * blkx;
 #pragma unroll
             for (int j = 0; j < CPT; ++j) {
@@ -1287,12 +1331,8 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_hg_kernel(const NetL
                 uint32_t cur[12], w[3][4];
 #pragma unroll
                 for (int k = 0; k < 12; ++k) cur[k] = nxt[k];
-                if (j + 1 < nj) {
-                    load_raw_bf16(a.in, a.V, a.cin, b, ci + TG, yh, nxt);
-                } else if (more) {
-                    load_raw_bf16(a.in, a.V, a.cin, last ? bn : b, cfirst,
-                             xs < a.V ? site_neighbour(a, xs, hs) : -1, nxt);
-                }
+                load_raw_bf16(a.in, a.V, a.cin, at.b, cfirst + TG * at.j, at.y, nxt);
+                at.advance(a, nj, h0, h1, total, ntiles, WG_TS, sl);
                 transport_bf16(cur, u, h == 0, w);
 #pragma unroll
                 for (int ca = 0; ca < 3; ++ca)
@@ -2392,10 +2432,315 @@ lqcd_status lqcd_net_train_step(lqcd_net* n, const float* r, const float* e, int
     // loss and its gradient
     const int nb = 256;
     dim3 g1(NET_PARTIALS, batch);
-    net_loss_reduce_kernel<<<g1, nb, 0, c->stream>>>(n->act[n->nlayers], ep, n_per, n->partials, 2 * NET_PARTIALS,
-                                                     n->tickets, n->red);
     LQ_CUDA(cudaGetLastError());
-    net_loss_grad_kernel<<<g1, nb, 0, c->stream>>>(n->act[n->nlayers], ep, n_per, n->red, batch, n->gact[0]);
+    c->launches += 2;
+    return LQCD_OK;
+}
+
+}  // namespace lqcd
+
+extern "C" {
+
+lqcd_status lqcd_net_create(lqcd_ctx* c, int nlayers, const int* channels, int bf16, int max_batch, lqcd_net** out)
+{
+    try {
+        if (!c || !channels || !out) return fail(LQCD_ERR_INVALID, "lqcd_net_create: null argument");
+        if (nlayers < 1 || nlayers > 8) return fail(LQCD_ERR_INVALID, "lqcd_net_create: 1..8 layers");
+        if (channels[0] != 1 || channels[nlayers] != 1)
+            return fail(LQCD_ERR_INVALID, "lqcd_net_create: the first and last widths must be 1 (spinor in, spinor out)");
+        for (int l = 0; l <= nlayers; ++l)
+            if (channels[l] < 1 || channels[l] > NET_MAXC) return fail(LQCD_ERR_INVALID, "lqcd_net_create: widths in [1, 12]");
+        if (max_batch < 1) return fail(LQCD_ERR_INVALID, "lqcd_net_create: max_batch >= 1");
+        if (!c->holds(P32)) return fail(LQCD_ERR_STATE, "lqcd_net_create: the context must hold F32 links");
+        if (c->cut()) return fail(LQCD_ERR_STATE, "lqcd_net_create: not on a sub-domain of a cut lattice");
+        lqcd_net* n = new lqcd_net();
+        memset(n, 0, sizeof(*n));
+        n->ctx = c;
+        n->nlayers = nlayers;
+        for (int l = 0; l <= nlayers; ++l) n->ch[l] = channels[l];
+        n->bf16 = bf16 ? 1 : 0;
+        n->max_batch = max_batch;
+        size_t w = 0;
+        for (int l = 0; l < nlayers; ++l) {
+            n->woff[l] = w;
+            w += (size_t)9 * 4 * channels[l + 1] * 4 * channels[l] * 2;
+        }
+        n->woff[nlayers] = w;
+        size_t off = 0;
+        auto take = [&](size_t bytes) { size_t o = off; off += a256(bytes); return o; };
+        size_t oW = take(w * 4), ogW = take(w * 4), om1 = take(w * 4), om2 = take(w * 4);
+        size_t oB[8], oBh[8], oBA[8], oBhA[8];
+        for (int l = 0; l < nlayers; ++l) {
+            const int K2p = pad16(8 * channels[l]), N2p = pad16(8 * channels[l + 1]);
+            const int K2pa = pad16(8 * channels[l + 1]), N2pa = pad16(8 * channels[l]);
+            oB[l] = take((size_t)9 * K2p * N2p * 4);
+            oBh[l] = take((size_t)9 * K2p * N2p * 2);
+            oBA[l] = take((size_t)9 * K2pa * N2pa * 4);
+            oBhA[l] = take((size_t)9 * K2pa * N2pa * 2);
+        }
+        size_t oS[8] = {0, 0, 0, 0, 0, 0, 0, 0}, oZ = 0;
+        bool any_stack = false;
+        for (int l = 0; l < nlayers; ++l) {
+            n->stacked[l] = n->bf16 && channels[l + 1] == 1 && channels[l] > 1;
+            if (n->stacked[l]) {
+                oS[l] = take((size_t)80 * pad16(8 * channels[l]) * 2);
+                any_stack = true;
+            }
+        }
+        if (any_stack) oZ = take((size_t)max_batch * 2 * c->g.Vh * 9 * 48);
+        size_t oA[9];
+        int cmax = 1;
+        for (int l = 0; l <= nlayers; ++l) {
+            oA[l] = take((size_t)max_batch * act_floats(n, channels[l]) * 4);
+            cmax = channels[l] > cmax ? channels[l] : cmax;
+        }
+        size_t oG0 = take((size_t)max_batch * act_floats(n, cmax) * 4);
+        size_t oG1 = take((size_t)max_batch * act_floats(n, cmax) * 4);
+        size_t oR = take((size_t)max_batch * 2 * sizeof(double));
+        size_t oP = take((size_t)max_batch * 2 * NET_PARTIALS * sizeof(double));  // 2 sums per block
+        size_t oT = take((size_t)max_batch * sizeof(unsigned));
+        n->need = off;
+        // stash offsets in the pointer fields until the workspace arrives
+        n->W = reinterpret_cast<float*>(oW);
+        n->gW = reinterpret_cast<float*>(ogW);
+        n->m1 = reinterpret_cast<float*>(om1);
+        n->m2 = reinterpret_cast<float*>(om2);
+        for (int l = 0; l < nlayers; ++l) {
+            n->Bf[l] = reinterpret_cast<float*>(oB[l]);
+            n->Bh[l] = reinterpret_cast<uint16_t*>(oBh[l]);
+            n->BfA[l] = reinterpret_cast<float*>(oBA[l]);
+            n->BhA[l] = reinterpret_cast<uint16_t*>(oBhA[l]);
+        }
+        for (int l = 0; l <= nlayers; ++l) n->act[l] = reinterpret_cast<float*>(oA[l]);
+        for (int l = 0; l < nlayers; ++l) n->BhS[l] = reinterpret_cast<uint16_t*>(oS[l]);
+        n->zbuf = reinterpret_cast<float*>(oZ);
+        n->gact[0] = reinterpret_cast<float*>(oG0);
+        n->gact[1] = reinterpret_cast<float*>(oG1);
+        n->red = reinterpret_cast<double*>(oR);
+        n->partials = reinterpret_cast<double*>(oP);
+        n->tickets = reinterpret_cast<unsigned*>(oT);
+        *out = n;
+        return LQCD_OK;
+    } catch (...) {
+        return fail(LQCD_ERR_NOMEM, "lqcd_net_create: host allocation failed");
+    }
+}
+
+lqcd_status lqcd_net_destroy(lqcd_net* n)
+{
+    if (n) delete n->prof;
+    delete n;
+    return LQCD_OK;
+}
+
+lqcd_status lqcd_net_profile_enable(lqcd_net* n, int enable)
+{
+    try {
+        if (!n) return fail(LQCD_ERR_INVALID, "lqcd_net_profile_enable: null network");
+        if (!n->prof) n->prof = new NetProfiler();
+        n->prof->on = enable != 0;
+        return LQCD_OK;
+    } catch (...) {
+        return fail(LQCD_ERR_NOMEM, "lqcd_net_profile_enable: host allocation failed");
+    }
+}
+
+lqcd_status lqcd_net_profile_read(lqcd_net* n, lqcd_profile_entry* out, int nentries)
+{
+    if (!n || !out) return fail(LQCD_ERR_INVALID, "lqcd_net_profile_read: null argument");
+    if (nentries < 3 * n->nlayers) return fail(LQCD_ERR_INVALID, "lqcd_net_profile_read: needs 3 x nlayers entries");
+    for (int i = 0; i < nentries; ++i) out[i] = lqcd_profile_entry{0, 0.0, 0.0, 0.0};
+    if (!n->prof) return LQCD_OK;
+    DeviceScope dev_scope;
+    LQ_TRY(dev_scope.enter(n->ctx->device));
+    LQ_CUDA(cudaStreamSynchronize(n->ctx->stream));
+    for (auto& r : n->prof->pending) {
+        float ms = 0.f;
+        LQ_CUDA(cudaEventElapsedTime(&ms, r.a, r.b));
+        out[r.idx].launches += 1;
+        out[r.idx].ms += ms;
+        out[r.idx].bytes += r.bytes;
+        out[r.idx].flops += r.flops;
+        n->prof->pool.push_back(r.a);
+        n->prof->pool.push_back(r.b);
+    }
+    n->prof->pending.clear();
+    return LQCD_OK;
+}
+
+lqcd_status lqcd_net_workspace_size(const lqcd_net* n, size_t* bytes)
+{
+    if (!n || !bytes) return fail(LQCD_ERR_INVALID, "lqcd_net_workspace_size: null argument");
+    *bytes = n->need;
+    return LQCD_OK;
+}
+
+lqcd_status lqcd_net_set_workspace(lqcd_net* n, void* ptr, size_t bytes)
+{
+    if (!n || !ptr) return fail(LQCD_ERR_INVALID, "lqcd_net_set_workspace: null argument");
+    if (n->ws) return fail(LQCD_ERR_STATE, "lqcd_net_set_workspace: workspace already set");
+    if (bytes < n->need) return fail(LQCD_ERR_NOMEM, "lqcd_net_set_workspace: too small");
+    if (reinterpret_cast<uintptr_t>(ptr) & 255) return fail(LQCD_ERR_INVALID, "lqcd_net_set_workspace: 256-byte alignment");
+    DeviceScope dev_scope;
+    LQ_TRY(dev_scope.enter(n->ctx->device));
+    char* base = static_cast<char*>(ptr);
+    auto fix = [&](auto*& p) { p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(base + reinterpret_cast<uintptr_t>(p)); };
+    fix(n->W); fix(n->gW); fix(n->m1); fix(n->m2);
+    for (int l = 0; l < n->nlayers; ++l) { fix(n->Bf[l]); fix(n->Bh[l]); fix(n->BfA[l]); fix(n->BhA[l]); }
+    for (int l = 0; l <= n->nlayers; ++l) fix(n->act[l]);
+    bool any_stack = false;
+    for (int l = 0; l < n->nlayers; ++l)
+        if (n->stacked[l]) {
+            fix(n->BhS[l]);
+            any_stack = true;
+        }
+    if (any_stack) fix(n->zbuf);
+    fix(n->gact[0]); fix(n->gact[1]); fix(n->red); fix(n->partials); fix(n->tickets);
+    n->ws = base;
+    n->ws_bytes = bytes;
+    lqcd_ctx* c = n->ctx;
+    LQ_CUDA(cudaMemsetAsync(n->W, 0, n->nW() * 4, c->stream));
+    LQ_CUDA(cudaMemsetAsync(n->tickets, 0, (size_t)n->max_batch * sizeof(unsigned), c->stream));
+    LQ_CUDA(cudaMemsetAsync(n->m1, 0, n->nW() * 4, c->stream));
+    LQ_CUDA(cudaMemsetAsync(n->m2, 0, n->nW() * 4, c->stream));
+    n->adam_t = 0;
+    return prep_weights(n);
+}
+
+// Transport with another context's links from now on (same lattice).
+lqcd_status lqcd_net_bind(lqcd_net* n, lqcd_ctx* c)
+{
+    if (!n || !c) return fail(LQCD_ERR_INVALID, "lqcd_net_bind: null argument");
+    const lqcd_ctx* o = n->ctx;
+    for (int m = 0; m < 4; ++m)
+        if (c->g.L[m] != o->g.L[m]) return fail(LQCD_ERR_INVALID, "lqcd_net_bind: lattice extents differ");
+    if (c->g.tanti != o->g.tanti || c->cfg.recon != o->cfg.recon)
+        return fail(LQCD_ERR_INVALID, "lqcd_net_bind: boundary condition or link storage differs");
+    if (c->device != o->device) return fail(LQCD_ERR_INVALID, "lqcd_net_bind: contexts on different GPUs");
+    if (!c->ws || !c->holds(P32) || !c->gauge_loaded)
+        return fail(LQCD_ERR_STATE, "lqcd_net_bind: the context needs a workspace and loaded F32 links");
+    n->ctx = c;
+    return LQCD_OK;
+}
+
+// At most max_ctas CTAs per launch of the persistent layer kernel and per hop
+// of the weight-gradient kernels (0: the default, one per SM).
+lqcd_status lqcd_net_set_max_ctas(lqcd_net* n, int max_ctas)
+{
+    if (!n) return fail(LQCD_ERR_INVALID, "lqcd_net_set_max_ctas: null network");
+    if (max_ctas < 0) return fail(LQCD_ERR_INVALID, "lqcd_net_set_max_ctas: max_ctas must be >= 0");
+    n->max_ctas = max_ctas;
+    return LQCD_OK;
+}
+
+lqcd_status lqcd_net_set_wait(lqcd_net* n, unsigned long long limit_ns, int expire_test)
+{
+    if (!n) return fail(LQCD_ERR_INVALID, "lqcd_net_set_wait: null network");
+    n->wait_ns = limit_ns > 0 ? limit_ns : NTC_WAIT_NS;
+    n->expire_test = expire_test ? 1 : 0;
+    return LQCD_OK;
+}
+
+// Weights: complex FP32, layer after layer, each [9][4 cout][4 cin] (re, im).
+lqcd_status lqcd_net_num_weights(const lqcd_net* n, size_t* count)
+{
+    if (!n || !count) return fail(LQCD_ERR_INVALID, "null argument");
+    *count = n->nW() / 2;
+    return LQCD_OK;
+}
+
+lqcd_status lqcd_net_set_weights(lqcd_net* n, const float* w)
+{
+    if (!n || !w || !n->ws) return fail(LQCD_ERR_INVALID, "lqcd_net_set_weights: null argument or no workspace");
+    DeviceScope dev_scope;
+    LQ_TRY(dev_scope.enter(n->ctx->device));
+    LQ_CUDA(cudaMemcpyAsync(n->W, w, n->nW() * 4, cudaMemcpyDefault, n->ctx->stream));
+    LQ_CUDA(cudaMemsetAsync(n->m1, 0, n->nW() * 4, n->ctx->stream));
+    LQ_CUDA(cudaMemsetAsync(n->m2, 0, n->nW() * 4, n->ctx->stream));
+    n->adam_t = 0;
+    return prep_weights(n);
+}
+
+lqcd_status lqcd_net_get_weights(const lqcd_net* n, float* w, float* grad)
+{
+    if (!n || !n->ws) return fail(LQCD_ERR_INVALID, "lqcd_net_get_weights: no workspace");
+    DeviceScope dev_scope;
+    LQ_TRY(dev_scope.enter(n->ctx->device));
+    if (w) LQ_CUDA(cudaMemcpyAsync(w, n->W, n->nW() * 4, cudaMemcpyDefault, n->ctx->stream));
+    if (grad) LQ_CUDA(cudaMemcpyAsync(grad, n->gW, n->nW() * 4, cudaMemcpyDefault, n->ctx->stream));
+    LQ_CUDA(cudaStreamSynchronize(n->ctx->stream));
+    return LQCD_OK;
+}
+
+// One layer forward (adjoint = 0) or its adjoint (adjoint = 1: input
+// gradient) on caller-provided device activations of `batch` items.
+lqcd_status lqcd_net_layer_apply(lqcd_net* n, int layer, int adjoint, float* out, const float* in, int batch)
+{
+    if (!n || !n->ws || !out || !in) return fail(LQCD_ERR_INVALID, "lqcd_net_layer_apply: bad argument");
+    if (layer < 0 || layer >= n->nlayers || batch < 1 || batch > n->max_batch)
+        return fail(LQCD_ERR_INVALID, "lqcd_net_layer_apply: bad layer/batch");
+    DeviceScope dev_scope;
+    LQ_TRY(dev_scope.enter(n->ctx->device));
+    const NetLayerArgs a = layer_args(n, layer, adjoint != 0, n->gact[0], n->gact[1]);
+    LQ_TRY(convert_layout(n, in, n->gact[0], a.cin, batch, true));
+    LQ_TRY(run_layer(n, a, batch, 3 * layer + (adjoint ? 1 : 0)));
+    return convert_layout(n, n->gact[1], out, a.cout, batch, false);
+}
+
+// Weight gradient of one layer (accumulated into the net's gradient buffer
+// after zeroing it when `zero`): G_W += sum over batch and sites.
+lqcd_status lqcd_net_layer_wgrad(lqcd_net* n, int layer, const float* in, const float* gout, int batch, int zero)
+{
+    if (!n || !n->ws || !in || !gout) return fail(LQCD_ERR_INVALID, "lqcd_net_layer_wgrad: bad argument");
+    if (layer < 0 || layer >= n->nlayers || batch < 1 || batch > n->max_batch)
+        return fail(LQCD_ERR_INVALID, "lqcd_net_layer_wgrad: bad layer/batch");
+    DeviceScope dev_scope;
+    LQ_TRY(dev_scope.enter(n->ctx->device));
+    LQ_TRY(convert_layout(n, in, n->gact[0], n->ch[layer], batch, true));
+    LQ_TRY(convert_layout(n, gout, n->gact[1], n->ch[layer + 1], batch, true));
+    return run_wgrad(n, layer, n->gact[0], n->gact[1], batch, zero);
+}
+
+// Whole-net forward on canonical FP32 complex spinors (batch items):
+// out, in: [batch][site][spin][colour] complex (device).
+lqcd_status lqcd_net_forward(lqcd_net* n, float* out, const float* in, int batch)
+{
+    NvtxRange nvtx_range("lqcd_net_forward");
+    if (!n || !n->ws || !out || !in) return fail(LQCD_ERR_INVALID, "lqcd_net_forward: bad argument");
+    if (batch < 1 || batch > n->max_batch) return fail(LQCD_ERR_INVALID, "lqcd_net_forward: batch out of range");
+    DeviceScope dev_scope;
+    LQ_TRY(dev_scope.enter(n->ctx->device));
+    LQ_TRY(convert_layout(n, in, n->act[0], 1, batch, true));
+    LQ_TRY(net_forward_all(n, batch));
+    return convert_layout(n, n->act[n->nlayers], out, 1, batch, false);
+}
+
+// One training step on `batch` pairs (r, e) of canonical FP32 complex
+// spinors: forward, loss L = mean |N(r) - e|^2 / |e|^2, backward through
+// every layer, Adam (lr, beta1, beta2, eps).  *loss receives L (FP64) and
+// the call synchronises the stream to read it.
+lqcd_status lqcd_net_train_step(lqcd_net* n, const float* r, const float* e, int batch, double lr, double beta1,
+                                double beta2, double eps, double* loss)
+{
+    NvtxRange nvtx_range("lqcd_net_train_step");
+    if (!n || !n->ws || !r || !e) return fail(LQCD_ERR_INVALID, "lqcd_net_train_step: bad argument");
+    if (batch < 1 || batch > n->max_batch) return fail(LQCD_ERR_INVALID, "lqcd_net_train_step: batch out of range");
+    DeviceScope dev_scope;
+    LQ_TRY(dev_scope.enter(n->ctx->device));
+    lqcd_ctx* c = n->ctx;
+    const size_t n_per = act_floats(n, 1);
+    LQ_TRY(convert_layout(n, r, n->act[0], 1, batch, true));
+    LQ_TRY(convert_layout(n, e, n->gact[1], 1, batch, true));  // planar target; gact[1] is free until the backward
+    LQ_TRY(net_forward_all(n, batch));
+    const float* ep = n->gact[1];
+    // loss and its gradient
+    const int nb = 256;
+    dim3 g1(NET_PARTIALS, batch);
+    const float4* y4 = reinterpret_cast<const float4*>(n->act[n->nlayers]);
+    const float4* e4 = reinterpret_cast<const float4*>(ep);
+    net_loss_reduce_kernel<<<g1, nb, 0, c->stream>>>(y4, e4, n_per / 4, n->partials, 2 * NET_PARTIALS, n->tickets, n->red);
+    LQ_CUDA(cudaGetLastError());
+    net_loss_grad_kernel<<<g1, nb, 0, c->stream>>>(y4, e4, n_per / 4, n->red, batch, reinterpret_cast<float4*>(n->gact[0]));
     LQ_CUDA(cudaGetLastError());
     c->launches += 2;
     // backward
