@@ -1691,30 +1691,63 @@ __global__ void net_layout_bf16_kernel(const void* src, void* dst, int V, int ch
     }
 }
 
+// Running sum in two FP32 words (value hi + lo), good to about 2^-46: FP64
+// additions would be bound by the FP64 pipe (five of its instructions an
+// element took 211 us for 16 spinors of 16^4, at 1/63 of the FP32 rate).
+// Components whose square FP32 cannot hold to its last bit (and infinities,
+// NaN) go to an FP64 sum as before.
+struct TwoFloat {
+    float hi = 0.f, lo = 0.f;
+    double rest = 0.0;
+    // + a^2, the square exact as s + fma(a, a, -s) (sum of Knuth: the error of hi + s is exact)
+    __device__ __forceinline__ void add_square(float a)
+    {
+        const float m = fabsf(a);
+        if (!(m >= 0x1p-48f && m <= 0x1p50f)) {
+            if (a != 0.f) rest += (double)a * a;
+            return;
+        }
+        const float s = __fmul_rn(a, a), e = __fmaf_rn(a, a, -s);
+        const float t = __fadd_rn(hi, s), z = __fadd_rn(t, -hi);
+        const float r = __fadd_rn(__fadd_rn(hi, -__fadd_rn(t, -z)), __fadd_rn(s, -z));
+        hi = t;
+        lo = __fadd_rn(lo, __fadd_rn(r, e));
+    }
+    __device__ __forceinline__ double value() const { return rest + ((double)hi + (double)lo); }
+};
+
 // Loss L = (1/B) sum_b |y_b - e_b|^2 / |e_b|^2; gout_b = 2 (y_b - e_b) / (B |e_b|^2).
 // Pass 1 reduces |y - e|^2 and |e|^2 per batch item (deterministic two-stage).
-__global__ void net_loss_reduce_kernel(const float* y, const float* e, size_t n_per, double* partials, size_t part_rs,
+__global__ void net_loss_reduce_kernel(const float4* y, const float4* e, size_t n_per, double* partials, size_t part_rs,
                                        unsigned* tickets, double* red)
 {
     const int b = blockIdx.y;
-    double d2 = 0.0, e2 = 0.0;
-    const float* yb = y + (size_t)b * n_per;
-    const float* eb = e + (size_t)b * n_per;
+    TwoFloat d2, e2;
+    const float4* yb = y + (size_t)b * n_per;
+    const float4* eb = e + (size_t)b * n_per;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_per; i += (size_t)gridDim.x * blockDim.x) {
-        const float d = yb[i] - eb[i];
-        d2 += (double)d * d;
-        e2 += (double)eb[i] * eb[i];
+        const float4 p = yb[i], q = eb[i];
+        d2.add_square(p.x - q.x);
+        d2.add_square(p.y - q.y);
+        d2.add_square(p.z - q.z);
+        d2.add_square(p.w - q.w);
+        e2.add_square(q.x);
+        e2.add_square(q.y);
+        e2.add_square(q.z);
+        e2.add_square(q.w);
     }
-    double v[2] = {d2, e2};
+    double v[2] = {d2.value(), e2.value()};
     block_reduce_finalize<2>(v, partials + b * part_rs, tickets + b, red + b * 2);
 }
 
-__global__ void net_loss_grad_kernel(const float* y, const float* e, size_t n_per, const double* red, int nb, float* g)
+__global__ void net_loss_grad_kernel(const float4* y, const float4* e, size_t n_per, const double* red, int nb, float4* g)
 {
     const int b = blockIdx.y;
     const float s = (float)(2.0 / (nb * red[2 * b + 1]));
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_per; i += (size_t)gridDim.x * blockDim.x)
-        g[(size_t)b * n_per + i] = s * (y[(size_t)b * n_per + i] - e[(size_t)b * n_per + i]);
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_per; i += (size_t)gridDim.x * blockDim.x) {
+        const float4 p = y[(size_t)b * n_per + i], q = e[(size_t)b * n_per + i];
+        g[(size_t)b * n_per + i] = make_float4(s * (p.x - q.x), s * (p.y - q.y), s * (p.z - q.z), s * (p.w - q.w));
+    }
 }
 
 // Adam on real parameters (re and im of W separately).
@@ -2128,310 +2161,6 @@ lqcd_status net_apply_internal(lqcd_net* n, void* z, const void* r, size_t rb)
     LQ_CUDA(cudaGetLastError());
     LQ_TRY(net_forward_all(n, 1));
     net_to_internal_kernel<<<grid, 128, 0, c->stream>>>(c->g, static_cast<char*>(z), rb, n->act[n->nlayers], 1);
-    LQ_CUDA(cudaGetLastError());
-    c->launches += 2;
-    return LQCD_OK;
-}
-
-}  // namespace lqcd
-
-extern "C" {
-
-lqcd_status lqcd_net_create(lqcd_ctx* c, int nlayers, const int* channels, int bf16, int max_batch, lqcd_net** out)
-{
-    try {
-        if (!c || !channels || !out) return fail(LQCD_ERR_INVALID, "lqcd_net_create: null argument");
-        if (nlayers < 1 || nlayers > 8) return fail(LQCD_ERR_INVALID, "lqcd_net_create: 1..8 layers");
-        if (channels[0] != 1 || channels[nlayers] != 1)
-            return fail(LQCD_ERR_INVALID, "lqcd_net_create: the first and last widths must be 1 (spinor in, spinor out)");
-        for (int l = 0; l <= nlayers; ++l)
-            if (channels[l] < 1 || channels[l] > NET_MAXC) return fail(LQCD_ERR_INVALID, "lqcd_net_create: widths in [1, 12]");
-        if (max_batch < 1) return fail(LQCD_ERR_INVALID, "lqcd_net_create: max_batch >= 1");
-        if (!c->holds(P32)) return fail(LQCD_ERR_STATE, "lqcd_net_create: the context must hold F32 links");
-        if (c->cut()) return fail(LQCD_ERR_STATE, "lqcd_net_create: not on a sub-domain of a cut lattice");
-        lqcd_net* n = new lqcd_net();
-        memset(n, 0, sizeof(*n));
-        n->ctx = c;
-        n->nlayers = nlayers;
-        for (int l = 0; l <= nlayers; ++l) n->ch[l] = channels[l];
-        n->bf16 = bf16 ? 1 : 0;
-        n->max_batch = max_batch;
-        size_t w = 0;
-        for (int l = 0; l < nlayers; ++l) {
-            n->woff[l] = w;
-            w += (size_t)9 * 4 * channels[l + 1] * 4 * channels[l] * 2;
-        }
-        n->woff[nlayers] = w;
-        size_t off = 0;
-        auto take = [&](size_t bytes) { size_t o = off; off += a256(bytes); return o; };
-        size_t oW = take(w * 4), ogW = take(w * 4), om1 = take(w * 4), om2 = take(w * 4);
-        size_t oB[8], oBh[8], oBA[8], oBhA[8];
-        for (int l = 0; l < nlayers; ++l) {
-            const int K2p = pad16(8 * channels[l]), N2p = pad16(8 * channels[l + 1]);
-            const int K2pa = pad16(8 * channels[l + 1]), N2pa = pad16(8 * channels[l]);
-            oB[l] = take((size_t)9 * K2p * N2p * 4);
-            oBh[l] = take((size_t)9 * K2p * N2p * 2);
-            oBA[l] = take((size_t)9 * K2pa * N2pa * 4);
-            oBhA[l] = take((size_t)9 * K2pa * N2pa * 2);
-        }
-        size_t oS[8] = {0, 0, 0, 0, 0, 0, 0, 0}, oZ = 0;
-        bool any_stack = false;
-        for (int l = 0; l < nlayers; ++l) {
-            n->stacked[l] = n->bf16 && channels[l + 1] == 1 && channels[l] > 1;
-            if (n->stacked[l]) {
-                oS[l] = take((size_t)80 * pad16(8 * channels[l]) * 2);
-                any_stack = true;
-            }
-        }
-        if (any_stack) oZ = take((size_t)max_batch * 2 * c->g.Vh * 9 * 48);
-        size_t oA[9];
-        int cmax = 1;
-        for (int l = 0; l <= nlayers; ++l) {
-            oA[l] = take((size_t)max_batch * act_floats(n, channels[l]) * 4);
-            cmax = channels[l] > cmax ? channels[l] : cmax;
-        }
-        size_t oG0 = take((size_t)max_batch * act_floats(n, cmax) * 4);
-        size_t oG1 = take((size_t)max_batch * act_floats(n, cmax) * 4);
-        size_t oR = take((size_t)max_batch * 2 * sizeof(double));
-        size_t oP = take((size_t)max_batch * 2 * NET_PARTIALS * sizeof(double));  // 2 sums per block
-        size_t oT = take((size_t)max_batch * sizeof(unsigned));
-        n->need = off;
-        // stash offsets in the pointer fields until the workspace arrives
-        n->W = reinterpret_cast<float*>(oW);
-        n->gW = reinterpret_cast<float*>(ogW);
-        n->m1 = reinterpret_cast<float*>(om1);
-        n->m2 = reinterpret_cast<float*>(om2);
-        for (int l = 0; l < nlayers; ++l) {
-            n->Bf[l] = reinterpret_cast<float*>(oB[l]);
-            n->Bh[l] = reinterpret_cast<uint16_t*>(oBh[l]);
-            n->BfA[l] = reinterpret_cast<float*>(oBA[l]);
-            n->BhA[l] = reinterpret_cast<uint16_t*>(oBhA[l]);
-        }
-        for (int l = 0; l <= nlayers; ++l) n->act[l] = reinterpret_cast<float*>(oA[l]);
-        for (int l = 0; l < nlayers; ++l) n->BhS[l] = reinterpret_cast<uint16_t*>(oS[l]);
-        n->zbuf = reinterpret_cast<float*>(oZ);
-        n->gact[0] = reinterpret_cast<float*>(oG0);
-        n->gact[1] = reinterpret_cast<float*>(oG1);
-        n->red = reinterpret_cast<double*>(oR);
-        n->partials = reinterpret_cast<double*>(oP);
-        n->tickets = reinterpret_cast<unsigned*>(oT);
-        *out = n;
-        return LQCD_OK;
-    } catch (...) {
-        return fail(LQCD_ERR_NOMEM, "lqcd_net_create: host allocation failed");
-    }
-}
-
-lqcd_status lqcd_net_destroy(lqcd_net* n)
-{
-    if (n) delete n->prof;
-    delete n;
-    return LQCD_OK;
-}
-
-lqcd_status lqcd_net_profile_enable(lqcd_net* n, int enable)
-{
-    try {
-        if (!n) return fail(LQCD_ERR_INVALID, "lqcd_net_profile_enable: null network");
-        if (!n->prof) n->prof = new NetProfiler();
-        n->prof->on = enable != 0;
-        return LQCD_OK;
-    } catch (...) {
-        return fail(LQCD_ERR_NOMEM, "lqcd_net_profile_enable: host allocation failed");
-    }
-}
-
-lqcd_status lqcd_net_profile_read(lqcd_net* n, lqcd_profile_entry* out, int nentries)
-{
-    if (!n || !out) return fail(LQCD_ERR_INVALID, "lqcd_net_profile_read: null argument");
-    if (nentries < 3 * n->nlayers) return fail(LQCD_ERR_INVALID, "lqcd_net_profile_read: needs 3 x nlayers entries");
-    for (int i = 0; i < nentries; ++i) out[i] = lqcd_profile_entry{0, 0.0, 0.0, 0.0};
-    if (!n->prof) return LQCD_OK;
-    DeviceScope dev_scope;
-    LQ_TRY(dev_scope.enter(n->ctx->device));
-    LQ_CUDA(cudaStreamSynchronize(n->ctx->stream));
-    for (auto& r : n->prof->pending) {
-        float ms = 0.f;
-        LQ_CUDA(cudaEventElapsedTime(&ms, r.a, r.b));
-        out[r.idx].launches += 1;
-        out[r.idx].ms += ms;
-        out[r.idx].bytes += r.bytes;
-        out[r.idx].flops += r.flops;
-        n->prof->pool.push_back(r.a);
-        n->prof->pool.push_back(r.b);
-    }
-    n->prof->pending.clear();
-    return LQCD_OK;
-}
-
-lqcd_status lqcd_net_workspace_size(const lqcd_net* n, size_t* bytes)
-{
-    if (!n || !bytes) return fail(LQCD_ERR_INVALID, "lqcd_net_workspace_size: null argument");
-    *bytes = n->need;
-    return LQCD_OK;
-}
-
-lqcd_status lqcd_net_set_workspace(lqcd_net* n, void* ptr, size_t bytes)
-{
-    if (!n || !ptr) return fail(LQCD_ERR_INVALID, "lqcd_net_set_workspace: null argument");
-    if (n->ws) return fail(LQCD_ERR_STATE, "lqcd_net_set_workspace: workspace already set");
-    if (bytes < n->need) return fail(LQCD_ERR_NOMEM, "lqcd_net_set_workspace: too small");
-    if (reinterpret_cast<uintptr_t>(ptr) & 255) return fail(LQCD_ERR_INVALID, "lqcd_net_set_workspace: 256-byte alignment");
-    DeviceScope dev_scope;
-    LQ_TRY(dev_scope.enter(n->ctx->device));
-    char* base = static_cast<char*>(ptr);
-    auto fix = [&](auto*& p) { p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(base + reinterpret_cast<uintptr_t>(p)); };
-    fix(n->W); fix(n->gW); fix(n->m1); fix(n->m2);
-    for (int l = 0; l < n->nlayers; ++l) { fix(n->Bf[l]); fix(n->Bh[l]); fix(n->BfA[l]); fix(n->BhA[l]); }
-    for (int l = 0; l <= n->nlayers; ++l) fix(n->act[l]);
-    bool any_stack = false;
-    for (int l = 0; l < n->nlayers; ++l)
-        if (n->stacked[l]) {
-            fix(n->BhS[l]);
-            any_stack = true;
-        }
-    if (any_stack) fix(n->zbuf);
-    fix(n->gact[0]); fix(n->gact[1]); fix(n->red); fix(n->partials); fix(n->tickets);
-    n->ws = base;
-    n->ws_bytes = bytes;
-    lqcd_ctx* c = n->ctx;
-    LQ_CUDA(cudaMemsetAsync(n->W, 0, n->nW() * 4, c->stream));
-    LQ_CUDA(cudaMemsetAsync(n->tickets, 0, (size_t)n->max_batch * sizeof(unsigned), c->stream));
-    LQ_CUDA(cudaMemsetAsync(n->m1, 0, n->nW() * 4, c->stream));
-    LQ_CUDA(cudaMemsetAsync(n->m2, 0, n->nW() * 4, c->stream));
-    n->adam_t = 0;
-    return prep_weights(n);
-}
-
-// Transport with another context's links from now on (same lattice).
-lqcd_status lqcd_net_bind(lqcd_net* n, lqcd_ctx* c)
-{
-    if (!n || !c) return fail(LQCD_ERR_INVALID, "lqcd_net_bind: null argument");
-    const lqcd_ctx* o = n->ctx;
-    for (int m = 0; m < 4; ++m)
-        if (c->g.L[m] != o->g.L[m]) return fail(LQCD_ERR_INVALID, "lqcd_net_bind: lattice extents differ");
-    if (c->g.tanti != o->g.tanti || c->cfg.recon != o->cfg.recon)
-        return fail(LQCD_ERR_INVALID, "lqcd_net_bind: boundary condition or link storage differs");
-    if (c->device != o->device) return fail(LQCD_ERR_INVALID, "lqcd_net_bind: contexts on different GPUs");
-    if (!c->ws || !c->holds(P32) || !c->gauge_loaded)
-        return fail(LQCD_ERR_STATE, "lqcd_net_bind: the context needs a workspace and loaded F32 links");
-    n->ctx = c;
-    return LQCD_OK;
-}
-
-// At most max_ctas CTAs per launch of the persistent layer kernel and per hop
-// of the weight-gradient kernels (0: the default, one per SM).
-lqcd_status lqcd_net_set_max_ctas(lqcd_net* n, int max_ctas)
-{
-    if (!n) return fail(LQCD_ERR_INVALID, "lqcd_net_set_max_ctas: null network");
-    if (max_ctas < 0) return fail(LQCD_ERR_INVALID, "lqcd_net_set_max_ctas: max_ctas must be >= 0");
-    n->max_ctas = max_ctas;
-    return LQCD_OK;
-}
-
-lqcd_status lqcd_net_set_wait(lqcd_net* n, unsigned long long limit_ns, int expire_test)
-{
-    if (!n) return fail(LQCD_ERR_INVALID, "lqcd_net_set_wait: null network");
-    n->wait_ns = limit_ns > 0 ? limit_ns : NTC_WAIT_NS;
-    n->expire_test = expire_test ? 1 : 0;
-    return LQCD_OK;
-}
-
-// Weights: complex FP32, layer after layer, each [9][4 cout][4 cin] (re, im).
-lqcd_status lqcd_net_num_weights(const lqcd_net* n, size_t* count)
-{
-    if (!n || !count) return fail(LQCD_ERR_INVALID, "null argument");
-    *count = n->nW() / 2;
-    return LQCD_OK;
-}
-
-lqcd_status lqcd_net_set_weights(lqcd_net* n, const float* w)
-{
-    if (!n || !w || !n->ws) return fail(LQCD_ERR_INVALID, "lqcd_net_set_weights: null argument or no workspace");
-    DeviceScope dev_scope;
-    LQ_TRY(dev_scope.enter(n->ctx->device));
-    LQ_CUDA(cudaMemcpyAsync(n->W, w, n->nW() * 4, cudaMemcpyDefault, n->ctx->stream));
-    LQ_CUDA(cudaMemsetAsync(n->m1, 0, n->nW() * 4, n->ctx->stream));
-    LQ_CUDA(cudaMemsetAsync(n->m2, 0, n->nW() * 4, n->ctx->stream));
-    n->adam_t = 0;
-    return prep_weights(n);
-}
-
-lqcd_status lqcd_net_get_weights(const lqcd_net* n, float* w, float* grad)
-{
-    if (!n || !n->ws) return fail(LQCD_ERR_INVALID, "lqcd_net_get_weights: no workspace");
-    DeviceScope dev_scope;
-    LQ_TRY(dev_scope.enter(n->ctx->device));
-    if (w) LQ_CUDA(cudaMemcpyAsync(w, n->W, n->nW() * 4, cudaMemcpyDefault, n->ctx->stream));
-    if (grad) LQ_CUDA(cudaMemcpyAsync(grad, n->gW, n->nW() * 4, cudaMemcpyDefault, n->ctx->stream));
-    LQ_CUDA(cudaStreamSynchronize(n->ctx->stream));
-    return LQCD_OK;
-}
-
-// One layer forward (adjoint = 0) or its adjoint (adjoint = 1: input
-// gradient) on caller-provided device activations of `batch` items.
-lqcd_status lqcd_net_layer_apply(lqcd_net* n, int layer, int adjoint, float* out, const float* in, int batch)
-{
-    if (!n || !n->ws || !out || !in) return fail(LQCD_ERR_INVALID, "lqcd_net_layer_apply: bad argument");
-    if (layer < 0 || layer >= n->nlayers || batch < 1 || batch > n->max_batch)
-        return fail(LQCD_ERR_INVALID, "lqcd_net_layer_apply: bad layer/batch");
-    DeviceScope dev_scope;
-    LQ_TRY(dev_scope.enter(n->ctx->device));
-    const NetLayerArgs a = layer_args(n, layer, adjoint != 0, n->gact[0], n->gact[1]);
-    LQ_TRY(convert_layout(n, in, n->gact[0], a.cin, batch, true));
-    LQ_TRY(run_layer(n, a, batch, 3 * layer + (adjoint ? 1 : 0)));
-    return convert_layout(n, n->gact[1], out, a.cout, batch, false);
-}
-
-// Weight gradient of one layer (accumulated into the net's gradient buffer
-// after zeroing it when `zero`): G_W += sum over batch and sites.
-lqcd_status lqcd_net_layer_wgrad(lqcd_net* n, int layer, const float* in, const float* gout, int batch, int zero)
-{
-    if (!n || !n->ws || !in || !gout) return fail(LQCD_ERR_INVALID, "lqcd_net_layer_wgrad: bad argument");
-    if (layer < 0 || layer >= n->nlayers || batch < 1 || batch > n->max_batch)
-        return fail(LQCD_ERR_INVALID, "lqcd_net_layer_wgrad: bad layer/batch");
-    DeviceScope dev_scope;
-    LQ_TRY(dev_scope.enter(n->ctx->device));
-    LQ_TRY(convert_layout(n, in, n->gact[0], n->ch[layer], batch, true));
-    LQ_TRY(convert_layout(n, gout, n->gact[1], n->ch[layer + 1], batch, true));
-    return run_wgrad(n, layer, n->gact[0], n->gact[1], batch, zero);
-}
-
-// Whole-net forward on canonical FP32 complex spinors (batch items):
-// out, in: [batch][site][spin][colour] complex (device).
-lqcd_status lqcd_net_forward(lqcd_net* n, float* out, const float* in, int batch)
-{
-    NvtxRange nvtx_range("lqcd_net_forward");
-    if (!n || !n->ws || !out || !in) return fail(LQCD_ERR_INVALID, "lqcd_net_forward: bad argument");
-    if (batch < 1 || batch > n->max_batch) return fail(LQCD_ERR_INVALID, "lqcd_net_forward: batch out of range");
-    DeviceScope dev_scope;
-    LQ_TRY(dev_scope.enter(n->ctx->device));
-    LQ_TRY(convert_layout(n, in, n->act[0], 1, batch, true));
-    LQ_TRY(net_forward_all(n, batch));
-    return convert_layout(n, n->act[n->nlayers], out, 1, batch, false);
-}
-
-// One training step on `batch` pairs (r, e) of canonical FP32 complex
-// spinors: forward, loss L = mean |N(r) - e|^2 / |e|^2, backward through
-// every layer, Adam (lr, beta1, beta2, eps).  *loss receives L (FP64) and
-// the call synchronises the stream to read it.
-lqcd_status lqcd_net_train_step(lqcd_net* n, const float* r, const float* e, int batch, double lr, double beta1,
-                                double beta2, double eps, double* loss)
-{
-    NvtxRange nvtx_range("lqcd_net_train_step");
-    if (!n || !n->ws || !r || !e) return fail(LQCD_ERR_INVALID, "lqcd_net_train_step: bad argument");
-    if (batch < 1 || batch > n->max_batch) return fail(LQCD_ERR_INVALID, "lqcd_net_train_step: batch out of range");
-    DeviceScope dev_scope;
-    LQ_TRY(dev_scope.enter(n->ctx->device));
-    lqcd_ctx* c = n->ctx;
-    const size_t n_per = act_floats(n, 1);
-    LQ_TRY(convert_layout(n, r, n->act[0], 1, batch, true));
-    LQ_TRY(convert_layout(n, e, n->gact[1], 1, batch, true));  // planar target; gact[1] is free until the backward
-    LQ_TRY(net_forward_all(n, batch));
-    const float* ep = n->gact[1];
-    // loss and its gradient
-    const int nb = 256;
-    dim3 g1(NET_PARTIALS, batch);
     LQ_CUDA(cudaGetLastError());
     c->launches += 2;
     return LQCD_OK;

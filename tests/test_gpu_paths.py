@@ -193,3 +193,34 @@ def test_sap_solves_in_turn(lq):
             its.append(st["iterations"])
             assert oracle.true_residual(U, A, 0.13, b, x.cpu().numpy()) <= 1e-10
         assert its[0] == its[1]
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-18, 1e17, "mixed"])
+@pytest.mark.parametrize("batch", [1, 3])
+def test_training_loss(lq, scale, batch):
+    """The loss against FP64 sums over the network's own output, for
+    components whose squares FP32 holds and for ones that it does not (2^-46
+    for each sum; the division and the mean stay in FP64)."""
+    import torch
+    dims, channels = (4, 2, 6, 6), (1, 3, 1)
+    lat = lq.Lattice(dims, precisions=("f64", "f32"))
+    lat.gauge_load(on_device(synth.gauge_field(dims, "smooth", 21, eps=0.5)))
+    net = lq.Net(lat, channels, bf16=True, max_batch=batch)
+    rng = np.random.default_rng(22)
+    net.set_weights((0.1 * (rng.standard_normal(net.num_weights) + 1j * rng.standard_normal(net.num_weights))).astype(np.complex64))
+    shape = (batch, dims[3], dims[2], dims[1], dims[0], 4, 3)
+    r, e = ((rng.standard_normal(shape) + 1j * rng.standard_normal(shape)) for _ in range(2))
+    if scale == "mixed":  # zeros, and sixteen orders of magnitude on both sides of one
+        s = 10.0 ** rng.integers(-16, 17, size=shape)
+        s[rng.random(shape) < 0.2] = 0.0
+        r, e = r * s, e * s
+    else:
+        r, e = r * scale, e * scale
+    r, e = on_device(r.astype(np.complex64)), on_device(e.astype(np.complex64))
+    y = torch.empty_like(r)
+    net.forward(y, r, batch)
+    lat.sync()
+    flat = lambda t: torch.view_as_real(t).reshape(batch, -1).cpu().numpy()
+    d = (flat(y) - flat(e)).astype(np.float64)  # the difference is taken in FP32
+    want = np.mean((d ** 2).sum(1) / (flat(e).astype(np.float64) ** 2).sum(1))
+    assert abs(net.train_step(r, e, batch, lr=0.0) / want - 1.0) < 1e-12
