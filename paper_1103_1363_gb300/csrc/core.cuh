@@ -70,15 +70,40 @@ struct Geom {
 
 // ----------------------------------------------------------------- helpers
 
-__device__ __forceinline__ float2 h2f(uint32_t u, int isbf)
+// FP32 c + a or a - c for half HI (0: low) of the packed pair w: the
+// mixed-precision add of sm_100 and later reads the 16-bit operand exactly, in
+// one instruction where a conversion and an add are two (the conversion on the
+// half of the FMA pipe that the packed products need).
+template <int ISBF, int HI>
+__device__ __forceinline__ float add_half(uint32_t w, float c)
 {
-    if (isbf) {
-        __nv_bfloat162 b = *reinterpret_cast<__nv_bfloat162*>(&u);
-        return __bfloat1622float2(b);
-    }
-    __half2 h = *reinterpret_cast<__half2*>(&u);
-    return __half22float2(h);
+    const uint16_t a = (uint16_t)(HI ? w >> 16 : w & 0xffffu);
+    float d;
+    if (ISBF) asm("add.rn.f32.bf16 %0, %1, %2;" : "=f"(d) : "h"(a), "f"(c));
+    else asm("add.rn.f32.f16 %0, %1, %2;" : "=f"(d) : "h"(a), "f"(c));
+    return d;
 }
+template <int ISBF, int HI>
+__device__ __forceinline__ float half_minus(uint32_t w, float c)
+{
+    const uint16_t a = (uint16_t)(HI ? w >> 16 : w & 0xffffu);
+    float d;
+    if (ISBF) asm("sub.rn.f32.bf16 %0, %1, %2;" : "=f"(d) : "h"(a), "f"(c));
+    else asm("sub.rn.f32.f16 %0, %1, %2;" : "=f"(d) : "h"(a), "f"(c));
+    return d;
+}
+// the value itself: a + (-0) is a for every a, its sign of zero included
+template <int ISBF, int HI>
+__device__ __forceinline__ float half_value(uint32_t w)
+{
+    return add_half<ISBF, HI>(w, -0.f);
+}
+template <int ISBF>
+__device__ __forceinline__ float2 halves(uint32_t w)
+{
+    return make_float2(half_value<ISBF, 0>(w), half_value<ISBF, 1>(w));
+}
+__device__ __forceinline__ float2 h2f(uint32_t u, int isbf) { return isbf ? halves<1>(u) : halves<0>(u); }
 
 __device__ __forceinline__ uint32_t f2h(float a, float b, int isbf)
 {

@@ -192,29 +192,165 @@ __device__ __forceinline__ void su3_mul_half(const R u[18], const R h[12], R w[1
     }
 }
 
-// One hop of the sum for the neighbour spinor v: forward (BWD false)
-// (1 - g_mu) U_mu(x) v, backward (1 + g_mu) U_mu(x - mu)^dag v (projectors
-// swapped by DAG); the link is U_mu at checkerboard index lidx of parity
-// lpar; flip: the hop crosses the antiperiodic t boundary.
-template <int PG, int RECON, int MU, bool DAG, bool BWD, bool PACK, class R>
-__device__ __forceinline__ void hop_product(const DslashArgs& A, const R v[24], bool flip, int lpar, int lidx, R w[12])
-{
-    constexpr int S = (BWD != DAG) ? +1 : -1;
-    R h[12], u[18];
-    project<MU, S>(v, h);
-    if (flip) {
+// ---- the neighbour's spinor of a hop, as it is stored
+// load(), then project<MU, S>() onto the two colour vectors, and, after the
+// link product, add<MU, S>() into the sum.  flip: the hop crosses the
+// antiperiodic t boundary.
+template <int PS>
+struct HopSpinor {
+    typedef typename RealT<PS>::type R;
+    R v[24];
+    bool flip;
+    __device__ __forceinline__ void load(const void* base, int stride, int j) { SpinorIO<PS>::load(base, stride, j, v); }
+    template <int MU, int S>
+    __device__ __forceinline__ void project_to(R h[12]) const
+    {
+        project<MU, S>(v, h);
+        if (flip) {
 #pragma unroll
-        for (int k = 0; k < 12; ++k) h[k] = -h[k];
+            for (int k = 0; k < 12; ++k) h[k] = -h[k];
+        }
     }
+    template <int MU, int S>
+    __device__ __forceinline__ void add(R acc[24], const R w[12]) const
+    {
+        accumulate<MU, S>(acc, w);
+    }
+    __device__ __forceinline__ R scale() const { return (R)1; }
+};
+
+// Half precision: 12 packed complex values q and the site's norm n.  The
+// projection is formed from the packed halves (two mixed-precision adds a
+// value), and the norm, with the boundary sign, multiplies the products where
+// they are added to the sum (a multiply-add instead of an add): 48 instructions
+// of the FMA pipe a hop where decoding, scaling and projecting took 84.
+template <int MU, int S>
+__device__ __forceinline__ void accumulate_scaled(float acc[24], const float w[12], float n)
+{
+    const float f = S * n;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const float w0r = w[2 * c], w0i = w[2 * c + 1], w1r = w[2 * (3 + c)], w1i = w[2 * (3 + c) + 1];
+        float* const a0 = acc + 2 * c;
+        float* const a1 = acc + 2 * (3 + c);
+        float* const a2 = acc + 2 * (6 + c);
+        float* const a3 = acc + 2 * (9 + c);
+        a0[0] += n * w0r;
+        a0[1] += n * w0i;
+        a1[0] += n * w1r;
+        a1[1] += n * w1i;
+        if (MU == 0) {
+            a2[0] += f * w1i;
+            a2[1] -= f * w1r;
+            a3[0] += f * w0i;
+            a3[1] -= f * w0r;
+        } else if (MU == 1) {
+            a2[0] += f * w1r;
+            a2[1] += f * w1i;
+            a3[0] -= f * w0r;
+            a3[1] -= f * w0i;
+        } else if (MU == 2) {
+            a2[0] += f * w0i;
+            a2[1] -= f * w0r;
+            a3[0] -= f * w1i;
+            a3[1] += f * w1r;
+        } else {
+            a2[0] += f * w0r;
+            a2[1] += f * w0i;
+            a3[0] += f * w1r;
+            a3[1] += f * w1i;
+        }
+    }
+}
+
+template <int ISBF>
+struct HopSpinorHalf {
+    uint32_t q[12];
+    float n;
+    bool flip;
+    __device__ __forceinline__ void set(const uint4 s[3])
+    {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            q[4 * k] = s[k].x; q[4 * k + 1] = s[k].y; q[4 * k + 2] = s[k].z; q[4 * k + 3] = s[k].w;
+        }
+    }
+    __device__ __forceinline__ void load(const void* base, int stride, int j)
+    {
+        const uint4* p = static_cast<const uint4*>(base);
+        n = __ldg(reinterpret_cast<const float*>(p + (size_t)3 * stride) + j);
+        uint4 s[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s[k] = __ldg(p + (size_t)k * stride + j);
+        set(s);
+    }
+    // h0 = q0 + e0 q_a, h1 = q1 + e1 q_b with e = +-1 (REAL) or +-i
+    template <bool PLUS>
+    __device__ __forceinline__ static void real_pair(uint32_t x, uint32_t y, float& re, float& im)
+    {
+        const float yr = half_value<ISBF, 0>(y), yi = half_value<ISBF, 1>(y);
+        re = PLUS ? add_half<ISBF, 0>(x, yr) : half_minus<ISBF, 0>(x, yr);
+        im = PLUS ? add_half<ISBF, 1>(x, yi) : half_minus<ISBF, 1>(x, yi);
+    }
+    template <bool PLUS>
+    __device__ __forceinline__ static void imag_pair(uint32_t x, uint32_t y, float& re, float& im)
+    {
+        const float yr = half_value<ISBF, 0>(y), yi = half_value<ISBF, 1>(y);
+        re = PLUS ? half_minus<ISBF, 0>(x, yi) : add_half<ISBF, 0>(x, yi);
+        im = PLUS ? add_half<ISBF, 1>(x, yr) : half_minus<ISBF, 1>(x, yr);
+    }
+    template <int MU, int S>
+    __device__ __forceinline__ void project_to(float h[12]) const
+    {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const uint32_t p0 = q[c], p1 = q[3 + c], p2 = q[6 + c], p3 = q[9 + c];
+            float* const h0 = h + 2 * c;
+            float* const h1 = h + 2 * (3 + c);
+            if (MU == 0) {  // p0 + S i p3, p1 + S i p2
+                imag_pair<(S > 0)>(p0, p3, h0[0], h0[1]);
+                imag_pair<(S > 0)>(p1, p2, h1[0], h1[1]);
+            } else if (MU == 1) {  // p0 - S p3, p1 + S p2
+                real_pair<(S < 0)>(p0, p3, h0[0], h0[1]);
+                real_pair<(S > 0)>(p1, p2, h1[0], h1[1]);
+            } else if (MU == 2) {  // p0 + S i p2, p1 - S i p3
+                imag_pair<(S > 0)>(p0, p2, h0[0], h0[1]);
+                imag_pair<(S < 0)>(p1, p3, h1[0], h1[1]);
+            } else {  // p0 + S p2, p1 + S p3
+                real_pair<(S > 0)>(p0, p2, h0[0], h0[1]);
+                real_pair<(S > 0)>(p1, p3, h1[0], h1[1]);
+            }
+        }
+    }
+    template <int MU, int S>
+    __device__ __forceinline__ void add(float acc[24], const float w[12]) const
+    {
+        accumulate_scaled<MU, S>(acc, w, scale());
+    }
+    __device__ __forceinline__ float scale() const { return flip ? -n : n; }
+};
+template <> struct HopSpinor<P16> : HopSpinorHalf<0> {};
+template <> struct HopSpinor<PB16> : HopSpinorHalf<1> {};
+
+// w = U P q (backward: U^dag P q) for the neighbour's spinor q: forward hops
+// (BWD false) use (1 - g_mu), backward ones (1 + g_mu), swapped by DAG; the
+// link is U_mu at checkerboard index lidx of parity lpar.  hop_term adds it.
+template <int PG, int PS, int RECON, int MU, bool DAG, bool BWD, bool PACK>
+__device__ __forceinline__ void hop_product(const DslashArgs& A, const HopSpinor<PS>& q, int lpar, int lidx,
+                                            typename RealT<PS>::type w[12])
+{
+    typename RealT<PS>::type h[12], u[18];
+    q.template project_to<MU, (BWD != DAG) ? +1 : -1>(h);
     GaugeIO<PG, RECON>::load(A.gauge, A.g.stride, lpar, MU, lidx, u);
     su3_mul_half<BWD, PACK>(u, h, w);
 }
-template <int PG, int RECON, int MU, bool DAG, bool BWD, bool PACK, class R>
-__device__ __forceinline__ void hop_term(const DslashArgs& A, const R v[24], bool flip, int lpar, int lidx, R acc[24])
+template <int PG, int PS, int RECON, int MU, bool DAG, bool BWD, bool PACK>
+__device__ __forceinline__ void hop_term(const DslashArgs& A, const HopSpinor<PS>& q, int lpar, int lidx,
+                                         typename RealT<PS>::type acc[24])
 {
-    R w[12];
-    hop_product<PG, RECON, MU, DAG, BWD, PACK>(A, v, flip, lpar, lidx, w);
-    accumulate<MU, (BWD != DAG) ? +1 : -1>(acc, w);
+    typename RealT<PS>::type w[12];
+    hop_product<PG, PS, RECON, MU, DAG, BWD, PACK>(A, q, lpar, lidx, w);
+    q.template add<MU, (BWD != DAG) ? +1 : -1>(acc, w);
 }
 
 // PG: storage of links and clover; PS: storage of spinor fields; the
@@ -225,20 +361,21 @@ template <int PG, int PS, int RECON, int MU, bool DAG, bool HALO = false, bool P
 __device__ __forceinline__ void hop_dir(const DslashArgs& A, const char* in, int i, int full, const int c[4],
                                         int stepmu, typename RealT<PS>::type acc[24])
 {
-    typedef typename RealT<PS>::type R;
     const int L = A.g.L[MU];
     const int fwd = (c[MU] == L - 1) ? full - (L - 1) * stepmu : full + stepmu;
     const int bwd = (c[MU] == 0) ? full + (L - 1) * stepmu : full - stepmu;
     const bool tb = (MU == 3) && A.g.tanti;
     const bool cut = HALO && ((A.g.part >> MU) & 1);
-    R v[24];
+    HopSpinor<PS> q;
     if (!(cut && c[MU] == L - 1)) {
-        SpinorIO<PS>::load(in, A.g.stride, fwd >> 1, v);
-        hop_term<PG, RECON, MU, DAG, false, PACK>(A, v, tb && c[3] == L - 1, A.par, i, acc);
+        q.load(in, A.g.stride, fwd >> 1);
+        q.flip = tb && c[3] == L - 1;
+        hop_term<PG, PS, RECON, MU, DAG, false, PACK>(A, q, A.par, i, acc);
     }
     if (!(cut && c[MU] == 0)) {
-        SpinorIO<PS>::load(in, A.g.stride, bwd >> 1, v);
-        hop_term<PG, RECON, MU, DAG, true, PACK>(A, v, tb && c[3] == 0, 1 - A.par, bwd >> 1, acc);
+        q.load(in, A.g.stride, bwd >> 1);
+        q.flip = tb && c[3] == 0;
+        hop_term<PG, PS, RECON, MU, DAG, true, PACK>(A, q, 1 - A.par, bwd >> 1, acc);
     }
 }
 
@@ -286,38 +423,29 @@ __device__ __forceinline__ void load_half_hop(const char* in, const void* gauge,
 }
 
 template <int ISBF, int RECON, int MU, bool BWD, bool DAG, bool PACK>
-__device__ __forceinline__ void half_hop_product(const HalfHopRaw<RECON>& r, bool flip, float w[12])
+__device__ __forceinline__ void half_hop_product(const HalfHopRaw<RECON>& r, HopSpinorHalf<ISBF>& q, bool flip, float w[12])
 {
-    float v[24], h[12], u[18];
-    // decode without the norm: the projection is linear, so the norm (and the
-    // boundary sign) scale the 12 projected values instead of the 24 inputs
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const uint4 c = r.s[k];
-        const float2 a = h2f(c.x, ISBF), b = h2f(c.y, ISBF), d = h2f(c.z, ISBF), e = h2f(c.w, ISBF);
-        v[8 * k + 0] = a.x; v[8 * k + 1] = a.y; v[8 * k + 2] = b.x; v[8 * k + 3] = b.y;
-        v[8 * k + 4] = d.x; v[8 * k + 5] = d.y; v[8 * k + 6] = e.x; v[8 * k + 7] = e.y;
-    }
+    float h[12], u[18];
+    q.set(r.s);
+    q.n = r.n;
+    q.flip = flip;
 #pragma unroll
     for (int k = 0; k < (RECON == 12 ? 6 : 9); ++k) {
-        const float2 a = h2f(r.u[k], ISBF);
+        const float2 a = halves<ISBF>(r.u[k]);
         u[2 * k] = a.x;
         u[2 * k + 1] = a.y;
     }
     if constexpr (RECON == 12) reconstruct_row2(u);
-    constexpr int S = (BWD != DAG) ? +1 : -1;  // forward (1 - g), backward (1 + g); swapped by DAG
-    project<MU, S>(v, h);
-    const float scale = flip ? -r.n : r.n;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) h[k] *= scale;
+    q.template project_to<MU, (BWD != DAG) ? +1 : -1>(h);
     su3_mul_half<BWD, PACK>(u, h, w);
 }
 template <int ISBF, int RECON, int MU, bool BWD, bool DAG, bool PACK>
 __device__ __forceinline__ void compute_half_hop(const HalfHopRaw<RECON>& r, bool flip, float acc[24])
 {
+    HopSpinorHalf<ISBF> q;
     float w[12];
-    half_hop_product<ISBF, RECON, MU, BWD, DAG, PACK>(r, flip, w);
-    accumulate<MU, (BWD != DAG) ? +1 : -1>(acc, w);
+    half_hop_product<ISBF, RECON, MU, BWD, DAG, PACK>(r, q, flip, w);
+    q.template add<MU, (BWD != DAG) ? +1 : -1>(acc, w);
 }
 
 template <int ISBF, int RECON, bool DAG, bool PACK, int H>
@@ -568,10 +696,20 @@ template <class R> struct Pair;
 template <> struct Pair<float> { typedef float2 type; };
 template <> struct Pair<double> { typedef double2 type; };
 
-// The product of hop H (2 mu + backward) at site i into ws[6 H + q][lane].
+// The products of the eight hops (two colour vectors each) of the block's 32
+// sites, the neighbours' norms (half precision) and what the epilogue warps exchange.
+template <int PS>
+struct WideShared {
+    typedef typename RealT<PS>::type R;
+    typename Pair<R>::type w[8 * 6][32];
+    float n[PS == P16 || PS == PB16 ? 8 : 1][32];
+    R ex[3][32];
+};
+
+// The product of hop H (2 mu + backward) at site i.
 template <int PG, int PS, int RECON, bool DAG, bool PACK, int H>
 __device__ __forceinline__ void wide_hop(const DslashArgs& A, const char* in, int i, int full, const int c[4],
-                                         typename Pair<typename RealT<PS>::type>::type* ws)
+                                         WideShared<PS>& sh)
 {
     typedef typename RealT<PS>::type R;
     constexpr int MU = H / 2;
@@ -582,6 +720,7 @@ __device__ __forceinline__ void wide_hop(const DslashArgs& A, const char* in, in
     const int nb = BWD ? (edge ? full + (L - 1) * step : full - step) : (edge ? full - (L - 1) * step : full + step);
     const int j = nb >> 1;
     const bool flip = MU == 3 && A.g.tanti && edge;
+    HopSpinor<PS> q;
     R w[12];
     if constexpr ((PS == P16 || PS == PB16) && PG == PS) {
         HopPlan hp;
@@ -589,42 +728,47 @@ __device__ __forceinline__ void wide_hop(const DslashArgs& A, const char* in, in
         hp.lidx[H] = BWD ? j : i;
         HalfHopRaw<RECON> raw;
         load_half_hop<RECON>(in, A.gauge, A.g.stride, A.par, hp, H, raw);
-        half_hop_product<PS == PB16 ? 1 : 0, RECON, MU, BWD, DAG, PACK>(raw, flip, w);
+        half_hop_product<PS == PB16 ? 1 : 0, RECON, MU, BWD, DAG, PACK>(raw, q, flip, w);
     } else {
-        R v[24];
-        SpinorIO<PS>::load(in, A.g.stride, j, v);
-        hop_product<PG, RECON, MU, DAG, BWD, PACK>(A, v, flip, BWD ? 1 - A.par : A.par, BWD ? j : i, w);
+        q.load(in, A.g.stride, j);
+        q.flip = flip;
+        hop_product<PG, PS, RECON, MU, DAG, BWD, PACK>(A, q, BWD ? 1 - A.par : A.par, BWD ? j : i, w);
     }
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        ws[(6 * H + q) * 32 + lane].x = w[2 * q];
-        ws[(6 * H + q) * 32 + lane].y = w[2 * q + 1];
+    for (int k = 0; k < 6; ++k) {
+        sh.w[6 * H + k][lane].x = w[2 * k];
+        sh.w[6 * H + k][lane].y = w[2 * k + 1];
     }
+    if constexpr (PS == P16 || PS == PB16) sh.n[H][lane] = q.scale();
 }
 
 // both hops of direction MU
 template <int PG, int PS, int RECON, bool DAG, bool PACK, int MU>
 __device__ __forceinline__ void wide_hops(const DslashArgs& A, const char* in, int i, int full, const int c[4],
-                                          typename Pair<typename RealT<PS>::type>::type* ws)
+                                          WideShared<PS>& sh)
 {
-    wide_hop<PG, PS, RECON, DAG, PACK, 2 * MU>(A, in, i, full, c, ws);
-    wide_hop<PG, PS, RECON, DAG, PACK, 2 * MU + 1>(A, in, i, full, c, ws);
+    wide_hop<PG, PS, RECON, DAG, PACK, 2 * MU>(A, in, i, full, c, sh);
+    wide_hop<PG, PS, RECON, DAG, PACK, 2 * MU + 1>(A, in, i, full, c, sh);
 }
 
-template <bool DAG, int B, int H, class R>
-__device__ __forceinline__ void wide_sum(const typename Pair<R>::type* ws, R acc[24])
+template <int PS, bool DAG, int H>
+__device__ __forceinline__ void wide_sum(const WideShared<PS>& sh, typename RealT<PS>::type acc[24])
 {
+    typedef typename RealT<PS>::type R;
+    constexpr int S = ((H & 1) != 0) != DAG ? +1 : -1;
     const int lane = threadIdx.x & 31;
     R w[12];
 #pragma unroll
     for (int q = 0; q < 6; ++q) {
-        const typename Pair<R>::type t = ws[(6 * H + q) * 32 + lane];
+        const typename Pair<R>::type t = sh.w[6 * H + q][lane];
         w[2 * q] = t.x;
         w[2 * q + 1] = t.y;
     }
-    accumulate<H / 2, (((H & 1) != 0) != DAG) ? +1 : -1>(acc, w);  // (the other half is dead code)
-    if constexpr (H < 7) wide_sum<DAG, B, H + 1>(ws, acc);
+    // (of acc the caller uses one half; the other is dead code)
+    if constexpr (PS == P16 || PS == PB16) accumulate_scaled<H / 2, S>(acc, w, sh.n[H][lane]);
+    else accumulate<H / 2, S>(acc, w);
+    if constexpr (H < 7) wide_sum<PS, DAG, H + 1>(sh, acc);
 }
 
 // What an epilogue warp holds before the barrier, for its half B of the site.
@@ -670,13 +814,12 @@ __device__ __forceinline__ void wide_operands(const DslashArgs& A, int rhs, int 
 }
 
 // Sum, epilogue and store of half B; both epilogue warps run this together
-// (they exchange the half's norm and largest component through ex[2][32]).
+// (they exchange the half's norm and largest component).
 // Returns the site's |out|^2 (|r|^2) in the thread of half 1: its FP32 sum
 // runs over the 24 components in order, so half 1 continues from half 0's.
 template <int PG, int PS, bool DAG, int EPI, bool RED, int B>
 __device__ __forceinline__ double wide_finish(const DslashArgs& A, int rhs, int i, bool live,
-                                              const typename Pair<typename RealT<PS>::type>::type* ws,
-                                              WideOperands<PS, EPI>& o, typename RealT<PS>::type (*ex)[32])
+                                              WideShared<PS>& sh, WideOperands<PS, EPI>& o)
 {
     typedef typename RealT<PS>::type R;
     typedef typename RealT<AccumP<PS>::value>::type RA;
@@ -686,7 +829,7 @@ __device__ __forceinline__ double wide_finish(const DslashArgs& A, int rhs, int 
     R full[24], out[12];
 #pragma unroll
     for (int k = 0; k < 24; ++k) full[k] = 0;
-    wide_sum<DAG, B, 0, R>(ws, full);
+    wide_sum<PS, DAG, 0>(sh, full);
     const R* acc = full + 12 * B;
     const R a = (R)A.a;
     if constexpr (EPI == EPI_NONE) {
@@ -724,24 +867,24 @@ __device__ __forceinline__ double wide_finish(const DslashArgs& A, int rhs, int 
     if constexpr (HALF && EPI != EPI_CG) {
 #pragma unroll
         for (int k = 0; k < 12; ++k) big = fmaxf(big, fabsf(out[k]));
-        ex[B][lane] = big;
+        sh.ex[B][lane] = big;
     }
     if constexpr (NORM) {
         if (B == 0) {
 #pragma unroll
             for (int k = 0; k < 12; ++k) n += EPI == EPI_CG ? (R)o.r[k] * (R)o.r[k] : out[k] * out[k];
-            ex[2][lane] = n;
+            sh.ex[2][lane] = n;
         }
     }
     if constexpr ((HALF && EPI != EPI_CG) || NORM) asm volatile("bar.sync 1, 64;" ::: "memory");
     if constexpr (HALF && EPI != EPI_CG) {
-        big = fmaxf(big, ex[1 - B][lane]);
+        big = fmaxf(big, sh.ex[1 - B][lane]);
         if (live)
             SpinorIO<PS>::template store_half<B>(static_cast<char*>(A.out) + rhs * A.out_rb, A.g.stride, i, out, big);
     }
     if constexpr (NORM) {
         if (B == 1) {
-            n = ex[2][lane];
+            n = sh.ex[2][lane];
 #pragma unroll
             for (int k = 0; k < 12; ++k) n += EPI == EPI_CG ? (R)o.r[k] * (R)o.r[k] : out[k] * out[k];
         }
@@ -754,10 +897,7 @@ __device__ __forceinline__ double wide_finish(const DslashArgs& A, int rhs, int 
 template <int PG, int PS, int RECON, bool DAG, int EPI, bool RED>
 __global__ void __launch_bounds__(WIDE_THREADS, (PG == P64 ? 1 : 3)) dslash_wide_kernel(const DslashArgs A)
 {
-    typedef typename RealT<PS>::type R;
-    typedef typename Pair<R>::type R2;
-    __shared__ R2 ws[8 * 6 * 32];
-    __shared__ R ex[3][32];
+    __shared__ WideShared<PS> sh;
     const int rhs = (int)(blockIdx.x % (unsigned)A.nrhs);
     const int sb = (int)(blockIdx.x / (unsigned)A.nrhs), nsb = (int)(gridDim.x / (unsigned)A.nrhs);
     constexpr bool PACK = !(RED || EPI == EPI_CG);  // the gathering kernel's choice per launch class
@@ -774,10 +914,10 @@ __global__ void __launch_bounds__(WIDE_THREADS, (PG == P64 ? 1 : 3)) dslash_wide
         if (live) {
             const char* in = static_cast<const char*>(A.in) + rhs * A.in_rb;
             switch (warp) {
-            case 0: wide_hops<PG, PS, RECON, DAG, PACK, 0>(A, in, i, full, c, ws); break;
-            case 1: wide_hops<PG, PS, RECON, DAG, PACK, 1>(A, in, i, full, c, ws); break;
-            case 2: wide_hops<PG, PS, RECON, DAG, PACK, 2>(A, in, i, full, c, ws); break;
-            default: wide_hops<PG, PS, RECON, DAG, PACK, 3>(A, in, i, full, c, ws); break;
+            case 0: wide_hops<PG, PS, RECON, DAG, PACK, 0>(A, in, i, full, c, sh); break;
+            case 1: wide_hops<PG, PS, RECON, DAG, PACK, 1>(A, in, i, full, c, sh); break;
+            case 2: wide_hops<PG, PS, RECON, DAG, PACK, 2>(A, in, i, full, c, sh); break;
+            default: wide_hops<PG, PS, RECON, DAG, PACK, 3>(A, in, i, full, c, sh); break;
             }
         }
     } else if (live) {
@@ -786,8 +926,8 @@ __global__ void __launch_bounds__(WIDE_THREADS, (PG == P64 ? 1 : 3)) dslash_wide
     }
     __syncthreads();
     double nrm = 0.0;
-    if (warp == 4) nrm = wide_finish<PG, PS, DAG, EPI, RED, 0>(A, rhs, i, live, ws, o, ex);
-    else if (warp == 5) nrm = wide_finish<PG, PS, DAG, EPI, RED, 1>(A, rhs, i, live, ws, o, ex);
+    if (warp == 4) nrm = wide_finish<PG, PS, DAG, EPI, RED, 0>(A, rhs, i, live, sh, o);
+    else if (warp == 5) nrm = wide_finish<PG, PS, DAG, EPI, RED, 1>(A, rhs, i, live, sh, o);
     pdl_start_next();
     if constexpr (RED || EPI == EPI_CG) {
         double v[1] = {nrm};
@@ -879,39 +1019,26 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src)
 }
 
 // A staged spinor (row-major staging rows, the field's chunk order).
-template <int PS> struct SpinorSmem;
-template <> struct SpinorSmem<P32> {
-    __device__ __forceinline__ static void load(const unsigned char* sm, int ns, int j, float v[24])
-    {
-        const float4* p = reinterpret_cast<const float4*>(sm);
+__device__ __forceinline__ void load_staged(const unsigned char* sm, int ns, int j, HopSpinor<P32>& q)
+{
+    const float4* p = reinterpret_cast<const float4*>(sm);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            const float4 c = p[k * ns + j];
-            v[4 * k] = c.x;
-            v[4 * k + 1] = c.y;
-            v[4 * k + 2] = c.z;
-            v[4 * k + 3] = c.w;
-        }
+    for (int k = 0; k < 6; ++k) {
+        const float4 c = p[k * ns + j];
+        q.v[4 * k] = c.x;
+        q.v[4 * k + 1] = c.y;
+        q.v[4 * k + 2] = c.z;
+        q.v[4 * k + 3] = c.w;
     }
-};
-template <int ISBF> struct SpinorSmemHalf {
-    __device__ __forceinline__ static void load(const unsigned char* sm, int ns, int j, float v[24])
-    {
-        const uint4* p = reinterpret_cast<const uint4*>(sm);
-        const float n = reinterpret_cast<const float*>(p + 3 * ns)[j];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const uint4 c = p[k * ns + j];
-            const float2 a = h2f(c.x, ISBF), b = h2f(c.y, ISBF), d = h2f(c.z, ISBF), e = h2f(c.w, ISBF);
-            v[8 * k + 0] = a.x * n; v[8 * k + 1] = a.y * n;
-            v[8 * k + 2] = b.x * n; v[8 * k + 3] = b.y * n;
-            v[8 * k + 4] = d.x * n; v[8 * k + 5] = d.y * n;
-            v[8 * k + 6] = e.x * n; v[8 * k + 7] = e.y * n;
-        }
-    }
-};
-template <> struct SpinorSmem<P16> : SpinorSmemHalf<0> {};
-template <> struct SpinorSmem<PB16> : SpinorSmemHalf<1> {};
+}
+template <int ISBF>
+__device__ __forceinline__ void load_staged(const unsigned char* sm, int ns, int j, HopSpinorHalf<ISBF>& q)
+{
+    const uint4* p = reinterpret_cast<const uint4*>(sm);
+    q.n = reinterpret_cast<const float*>(p + 3 * ns)[j];
+    const uint4 s[3] = {p[j], p[ns + j], p[2 * ns + j]};
+    q.set(s);
+}
 
 // One hop direction of the staged kernel: the neighbours' staging indices
 // jf, jb, the backward link's checkerboard index bwd_cb.
@@ -919,11 +1046,13 @@ template <int PG, int PS, int RECON, int MU, bool DAG>
 __device__ __forceinline__ void hop_dir_staged(const DslashArgs& A, const unsigned char* sm, int ns, int i, int jf,
                                                int jb, int bwd_cb, bool flipf, bool flipb, float acc[24])
 {
-    float v[24];
-    SpinorSmem<PS>::load(sm, ns, jf, v);
-    hop_term<PG, RECON, MU, DAG, false, true>(A, v, flipf, A.par, i, acc);
-    SpinorSmem<PS>::load(sm, ns, jb, v);
-    hop_term<PG, RECON, MU, DAG, true, true>(A, v, flipb, 1 - A.par, bwd_cb, acc);
+    HopSpinor<PS> q;
+    load_staged(sm, ns, jf, q);
+    q.flip = flipf;
+    hop_term<PG, PS, RECON, MU, DAG, false, true>(A, q, A.par, i, acc);
+    load_staged(sm, ns, jb, q);
+    q.flip = flipb;
+    hop_term<PG, PS, RECON, MU, DAG, true, true>(A, q, 1 - A.par, bwd_cb, acc);
 }
 
 // Block b: right-hand side b % nrhs, tile b / nrhs (y fastest, then z, t);

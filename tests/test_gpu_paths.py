@@ -224,3 +224,31 @@ def test_training_loss(lq, scale, batch):
     d = (flat(y) - flat(e)).astype(np.float64)  # the difference is taken in FP32
     want = np.mean((d ** 2).sum(1) / (flat(e).astype(np.float64) ** 2).sum(1))
     assert abs(net.train_step(r, e, batch, lr=0.0) / want - 1.0) < 1e-12
+
+
+@pytest.mark.parametrize("prec", ["f16spinors", "f16"])
+@pytest.mark.parametrize("block", [128, 96])
+def test_hop_reads_subnormal_halves(lq, prec, block):
+    """A site whose components span more than FP16's normal range: with unit
+    links colour 1 carries only values that are subnormal in units of the
+    site's norm, and one step of that grid is 2^-24 (flushed to zero they
+    would be 2^-15 off)."""
+    dims = (4, 4, 4, 4)
+    U = np.zeros((4, 4, 4, 4, 4, 3, 3), dtype=complex)
+    U[...] = np.eye(3)
+    psi = np.zeros((4, 4, 4, 4, 4, 3), dtype=complex)
+    psi[1, 2, 1, 3, :, 0] = 1.0 + 0.5j  # t + z + y + x odd
+    psi[1, 2, 1, 3, :, 1] = np.array([1, -2, 5, 11]) * 2.0 ** -18 + 1j * np.array([3, 7, -1, 2]) * 2.0 ** -20
+    lat = lq.Lattice(dims, precisions=("f64", "f32", prec))
+    lat.gauge_load(on_device(U))
+    lq.lqcd_tune_set(lat.ctx, prec, (block,) * 4)
+    fin, fout = lat.new_field(prec), lat.new_field(prec)
+    lat.pack(fin, on_device(psi), 1, prec)
+    lat.dslash(fout, fin, 0, prec=prec)
+    out = lat.canonical_spinor()
+    lat.unpack(out, fout, 0, prec)
+    lat.sync()
+    got, want = out.cpu().numpy()[..., 1], hop_ref(U, psi, dims, 0)[..., 1]
+    norm = np.abs(hop_ref(U, psi, dims, 0)).max()
+    assert np.abs(want).max() > 2.0 ** -17 * norm  # well above a step, far below the normal range
+    assert np.abs(got - want).max() < 2.0 ** -23 * norm
