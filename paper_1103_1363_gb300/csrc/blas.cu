@@ -74,9 +74,14 @@ __global__ void cg_p_kernel(Geom g, char* p, size_t p_rb, const char* r, size_t 
     const int rhs = blockIdx.y;
     pdl_wait();
     if (skip && skip[rhs]) return;
-    const double* sc = scal + rhs * SC_PER_RHS;
-    const double bden = sc[den] + sc[den + 1];  // 0 once the residual has vanished
-    const RR beta = bden > 0.0 ? (RR)((sc[num] + sc[num + 1]) / bden) : (RR)0;
+    __shared__ RR beta_s;  // one FP64 division a block (see cg_alpha)
+    if (threadIdx.x == 0) {
+        const double* sc = scal + rhs * SC_PER_RHS;
+        const double bden = sc[den] + sc[den + 1];  // 0 once the residual has vanished
+        beta_s = bden > 0.0 ? (RR)((sc[num] + sc[num + 1]) / bden) : (RR)0;
+    }
+    __syncthreads();
+    const RR beta = beta_s;
     const size_t fp = spinor_field_bytes(PP, g.stride), fr = spinor_field_bytes(PR, g.stride);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.Vh; i += gridDim.x * blockDim.x)
         for (int f = 0; f < nf; ++f) {

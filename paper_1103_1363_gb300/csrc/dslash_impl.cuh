@@ -493,11 +493,25 @@ __device__ __forceinline__ void hop_all_half(const DslashArgs& A, const char* in
 #define DSLASH_MAX_BLOCK 128
 #define DSLASH_WIDE 2    // internal: the warp-per-direction kernel
 #define DSLASH_STAGED 1  // a "block size" that selects the shared-memory staged kernel (LQCD_BLOCK_STAGED)
+// The CG step alpha = |r|^2 / |Mp|^2; once r is exactly zero (an exact
+// solution inside a check interval) both vanish: no step instead of 0/0.  An
+// FP64 division is some fifteen instructions of a pipe with 1/63 of FP32's
+// rate, so it is done once a block, not once a site (CG iteration at 16^4, 12 FP16-spinor rhs:
+// 206 -> 202 us; 32^3 x 64 FP32 746 -> 740).
+template <int PS>
+__device__ __forceinline__ typename RealT<AccumP<PS>::value>::type cg_alpha(const DslashArgs& A, int rhs)
+{
+    typedef typename RealT<AccumP<PS>::value>::type RA;
+    const double* sc = A.scal + rhs * A.scal_rs;
+    const double den = sc[A.s_den] + sc[A.s_den2];
+    return den > 0.0 ? (RA)((sc[A.s_num] + sc[A.s_num2]) / den) : (RA)0;
+}
+
 // Epilogue at output site i of right-hand side rhs for the hopping term
-// acc; nrm accumulates |out|^2 (|r|^2 for EPI_CG).
+// acc; nrm accumulates |out|^2 (|r|^2 for EPI_CG, whose step is alpha).
 template <int PG, int PS, bool DAG, int EPI, bool RED>
 __device__ __forceinline__ void dslash_epilogue(const DslashArgs& A, int rhs, int i, typename RealT<PS>::type acc[24],
-                                                double& nrm)
+                                                double& nrm, typename RealT<AccumP<PS>::value>::type alpha)
 {
     typedef typename RealT<PS>::type R;
     const R a = (R)A.a;
@@ -528,11 +542,6 @@ __device__ __forceinline__ void dslash_epilogue(const DslashArgs& A, int rhs, in
     }
     if constexpr (EPI == EPI_CG) {
         typedef typename RealT<AccumP<PS>::value>::type RA;
-        const double* sc = A.scal + rhs * A.scal_rs;
-        // alpha = |r|^2 / |Mp|^2; once r is exactly zero (an exact solution
-        // inside a check interval) both vanish: no step instead of 0/0
-        const double den = sc[A.s_den] + sc[A.s_den2];
-        const RA alpha = den > 0.0 ? (RA)((sc[A.s_num] + sc[A.s_num2]) / den) : (RA)0;
         R pv[24];
         RA xv[24], rv[24];
         SpinorIO<PS>::load(static_cast<const char*>(A.p) + rhs * A.p_rb, A.g.stride, i, pv);
@@ -561,6 +570,17 @@ __device__ __forceinline__ void dslash_epilogue(const DslashArgs& A, int rhs, in
     }
 }
 
+// Packed link products: in the launches that neither reduce nor update, and
+// with all operands in 16 bits in every launch.  In the reducing launches the
+// packed form is slower with FP32 links (CG iteration 24^3 x 48, us: FP32 263
+// scalar, 271 packed; FP16 spinors 232 / 253) and faster with 16-bit ones
+// (FP16 217 / 198, 12 rhs 2079 / 2041).  The results are the same.
+template <int PG, int PS, int EPI, bool RED>
+__host__ __device__ constexpr bool packed_products()
+{
+    return !(RED || EPI == EPI_CG) || ((PG == P16 || PG == PB16) && PS == PG);
+}
+
 // True if site c of a sub-domain has a neighbour across a cut boundary.
 __device__ __forceinline__ bool on_cut_face(const Geom& g, const int c[4])
 {
@@ -576,7 +596,8 @@ __device__ __forceinline__ bool on_cut_face(const Geom& g, const int c[4])
 // sub-domain; a site with a neighbour across a cut boundary stores its
 // partial sum unfinished (no epilogue) for the face pass to complete.
 template <int PG, int PS, int RECON, bool DAG, int EPI, bool RED, bool HALO = false>
-__device__ __forceinline__ void dslash_site(const DslashArgs& A, int rhs, int i, double& nrm)
+__device__ __forceinline__ void dslash_site(const DslashArgs& A, int rhs, int i, double& nrm,
+                                            typename RealT<AccumP<PS>::value>::type alpha)
 {
     typedef typename RealT<PS>::type R;
     int c[4];
@@ -586,9 +607,7 @@ __device__ __forceinline__ void dslash_site(const DslashArgs& A, int rhs, int i,
     R acc[24];
 #pragma unroll
     for (int k = 0; k < 24; ++k) acc[k] = 0;
-    // packed link products in the launches that neither reduce nor update
-    // (measured faster there; slower in the reducing launches of the solver)
-    constexpr bool PACK = !(RED || EPI == EPI_CG);
+    constexpr bool PACK = packed_products<PG, PS, EPI, RED>();
     if constexpr ((PS == P16 || PS == PB16) && PG == PS) {
         static_assert(!HALO, "sub-domain hops use the generic gather");
         hop_all_half<PS == PB16 ? 1 : 0, RECON, DAG, PACK>(A, in, i, full, c, acc);
@@ -602,7 +621,7 @@ __device__ __forceinline__ void dslash_site(const DslashArgs& A, int rhs, int i,
         SpinorIO<PS>::store(static_cast<char*>(A.out) + rhs * A.out_rb, A.g.stride, i, acc);
         return;
     }
-    dslash_epilogue<PG, PS, DAG, EPI, RED>(A, rhs, i, acc, nrm);
+    dslash_epilogue<PG, PS, DAG, EPI, RED>(A, rhs, i, acc, nrm, alpha);
 }
 
 // One-dimensional grid: block b serves right-hand side b % nrhs and site
@@ -620,17 +639,24 @@ __global__ void __launch_bounds__(DSLASH_MAX_BLOCK, (PG == P64 ? 1 : LQCD_DSLASH
     pdl_wait();
     if (A.skip && A.skip[rhs]) return;  // uniform over the rhs: no block of it reduces
     double nrm = 0.0;
+    typename RealT<AccumP<PS>::value>::type alpha = 0;
+    if constexpr (EPI == EPI_CG) {
+        __shared__ typename RealT<AccumP<PS>::value>::type alpha_s;
+        if (threadIdx.x == 0) alpha_s = cg_alpha<PS>(A, rhs);
+        __syncthreads();
+        alpha = alpha_s;
+    }
     if constexpr (RED || EPI == EPI_CG) {
         // grid-stride: the launcher runs one wave of blocks, so that each
         // block's partial sum covers many sites
         for (int i = sb * blockDim.x + threadIdx.x; i < A.g.Vh; i += nsb * blockDim.x)
-            dslash_site<PG, PS, RECON, DAG, EPI, RED>(A, rhs, i, nrm);
+            dslash_site<PG, PS, RECON, DAG, EPI, RED>(A, rhs, i, nrm, alpha);
         pdl_start_next();
         double v[1] = {nrm};
         block_reduce_finalize<1>(v, A.partials + rhs * A.part_rs, A.tickets + rhs, A.red + rhs * A.red_rs, sb, nsb);
     } else {
         const int i = sb * blockDim.x + threadIdx.x;
-        if (i < A.g.Vh) dslash_site<PG, PS, RECON, DAG, EPI, RED>(A, rhs, i, nrm);
+        if (i < A.g.Vh) dslash_site<PG, PS, RECON, DAG, EPI, RED>(A, rhs, i, nrm, alpha);
         pdl_start_next();
     }
 }
@@ -802,11 +828,8 @@ __device__ __forceinline__ void wide_operands(const DslashArgs& A, int rhs, int 
         }
     }
     if constexpr (EPI == EPI_CG) {
-        typedef typename RealT<AccumP<PS>::value>::type RA;
         constexpr int PA = AccumP<PS>::value;
-        const double* sc = A.scal + rhs * A.scal_rs;
-        const double den = sc[A.s_den] + sc[A.s_den2];
-        o.alpha = den > 0.0 ? (RA)((sc[A.s_num] + sc[A.s_num2]) / den) : (RA)0;
+        o.alpha = cg_alpha<PS>(A, rhs);
         SpinorIO<PS>::template load_half<B>(static_cast<const char*>(A.p) + rhs * A.p_rb, A.g.stride, i, o.p);
         SpinorIO<PA>::template load_half<B>(static_cast<const char*>(A.x) + rhs * A.acc_rb, A.g.stride, i, o.x);
         SpinorIO<PA>::template load_half<B>(static_cast<const char*>(A.r) + rhs * A.acc_rb, A.g.stride, i, o.r);
@@ -900,7 +923,7 @@ __global__ void __launch_bounds__(WIDE_THREADS, (PG == P64 ? 1 : 3)) dslash_wide
     __shared__ WideShared<PS> sh;
     const int rhs = (int)(blockIdx.x % (unsigned)A.nrhs);
     const int sb = (int)(blockIdx.x / (unsigned)A.nrhs), nsb = (int)(gridDim.x / (unsigned)A.nrhs);
-    constexpr bool PACK = !(RED || EPI == EPI_CG);  // the gathering kernel's choice per launch class
+    constexpr bool PACK = packed_products<PG, PS, EPI, RED>();  // the gathering kernel's choice
     const int warp = threadIdx.x >> 5;
     const int i = sb * WIDE_SITES + (threadIdx.x & 31);
     const bool live = i < A.g.Vh;
@@ -1134,7 +1157,7 @@ __global__ void __launch_bounds__(STG_NIN * STG_MAXLXH, 2) dslash_staged_kernel(
                                               tb && c[3] == 0, acc);
     }
     double nrm = 0.0;
-    dslash_epilogue<PG, PS, DAG, EPI, false>(A, rhs, i, acc, nrm);
+    dslash_epilogue<PG, PS, DAG, EPI, false>(A, rhs, i, acc, nrm, 0);
 }
 
 template <int PG, int PS, int RECON, bool DAG, int EPI>

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(128) halo_faces_kernel(const DslashArgs A, con
     add_faces<P, RECON, 2, DAG>(A, rv, hs, i, c, acc);
     add_faces<P, RECON, 3, DAG>(A, rv, hs, i, c, acc);
     double nrm = 0.0;
-    dslash_epilogue<P, P, DAG, EPI, false>(A, rhs, i, acc, nrm);
+    dslash_epilogue<P, P, DAG, EPI, false>(A, rhs, i, acc, nrm, 0);
 }
 
 // Interior pass: the hopping kernel with the hops across cut boundaries left out.
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(DSLASH_MAX_BLOCK) halo_interior_kernel(const D
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int rhs = blockIdx.y;
     double nrm = 0.0;
-    if (i < A.g.Vh) dslash_site<P, P, RECON, DAG, EPI, false, true>(A, rhs, i, nrm);
+    if (i < A.g.Vh) dslash_site<P, P, RECON, DAG, EPI, false, true>(A, rhs, i, nrm, 0);
 }
 
 HaloSeg halo_segments(const lqcd_ctx* c, int P)

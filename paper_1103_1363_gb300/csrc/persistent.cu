@@ -123,9 +123,10 @@ __device__ __forceinline__ void hop_stage(const PersistArgs& P, int stage, int j
         if (A.skip && A.skip[rhs]) continue;        // uniform over the block
         const int tl = t - P.tile0[q];
         double nrm = 0.0;
+        const float alpha = EPI == EPI_CG ? cg_alpha<PS>(A, rhs) : 0.f;
         for (int k = 0; k < L.spt; ++k) {
             const int i = (tl * L.spt + k) * PERSIST_THREADS + threadIdx.x;
-            if (i < A.g.Vh) dslash_site<PG, PS, RECON, DAG, EPI, RED>(A, rhs, i, nrm);
+            if (i < A.g.Vh) dslash_site<PG, PS, RECON, DAG, EPI, RED>(A, rhs, i, nrm, alpha);
         }
         if (RED) {
             double v[1] = {nrm};
