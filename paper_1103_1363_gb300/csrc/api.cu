@@ -95,7 +95,7 @@ static double launch_bytes_per_site(const lqcd_ctx* c, const DslashArgs& A, int 
     case EPI_NONE: per_rhs += S; break;
     case EPI_CLOVINV: per_rhs += S; break;
     case EPI_XPAY: per_rhs += 2 * S; break;
-    default: per_rhs += 2 * S + 4 * Acc; break;  // y, p read; x, r read and written
+    default: per_rhs += S + 2 * Acc + (A.x ? S + 2 * Acc : 0.0); break;  // y read, r read and written; p, x likewise
     }
     return nrhs * per_rhs + 8 * L + (epi == EPI_NONE ? 0.0 : Cl);
 }

@@ -63,10 +63,10 @@ __global__ void xmy_norm_kernel(Geom g, char* out, const char* b, const char* a,
     block_reduce_finalize<1>(vv, partials + rhs * part_rs, tickets + rhs, red + rhs * SC_PER_RHS);
 }
 
-// p = r + beta p, beta = (scal[num] + scal[num + 1]) / (scal[den] + scal[den + 1])
+// p_out = r + beta p, beta = (scal[num] + scal[num + 1]) / (scal[den] + scal[den + 1])
 // (the two slots hold the even- and odd-parity parts of |r|^2)
 template <int PP, int PR>
-__global__ void cg_p_kernel(Geom g, char* p, size_t p_rb, const char* r, size_t r_rb, int nf, const double* scal,
+__global__ void cg_p_kernel(Geom g, char* p_out, const char* p, size_t p_rb, const char* r, size_t r_rb, int nf, const double* scal,
                             int num, int den, const int* skip)
 {
     typedef typename RealT<PP>::type RP;
@@ -91,8 +91,45 @@ __global__ void cg_p_kernel(Geom g, char* p, size_t p_rb, const char* r, size_t 
             SpinorIO<PR>::load(r + rhs * r_rb + f * fr, g.stride, i, vr);
 #pragma unroll
             for (int k = 0; k < 24; ++k) vp[k] = (RP)(vr[k] + beta * (RR)vp[k]);
-            SpinorIO<PP>::store(p + rhs * p_rb + f * fp, g.stride, i, vp);
+            SpinorIO<PP>::store(p_out + rhs * p_rb + f * fp, g.stride, i, vp);
         }
+    pdl_start_next();
+}
+
+// x += alpha_j p_j for the iterations j0 <= j < j1 of a block, in order, with
+// p_j in direction slot j % slots and alpha_j from the block's scalar slots
+// (as cg_alpha).  One parity.
+template <int PP>
+__global__ void __launch_bounds__(256) cg_x_kernel(Geom g, char* x, size_t x_rb, const char* p, size_t p_rb, size_t slot_bytes,
+                                                   int j0, int j1, int slots, const double* scal, const int* skip)
+{
+    __shared__ float alpha[SC_RING];
+    const int rhs = blockIdx.y;
+    pdl_wait();
+    if (skip && skip[rhs]) return;
+    const int n = j1 - j0;
+    if ((int)threadIdx.x < n) {
+        const double* sc = scal + rhs * SC_PER_RHS;
+        const int num = rr_slot(j0 + threadIdx.x), den = pap_slot(j0 + threadIdx.x);
+        const double d = sc[den] + sc[den + 1];
+        alpha[threadIdx.x] = d > 0.0 ? (float)((sc[num] + sc[num + 1]) / d) : 0.f;
+    }
+    __syncthreads();
+    char* xr = x + rhs * x_rb;
+    const char* pr = p + rhs * p_rb;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.Vh; i += gridDim.x * blockDim.x) {
+        float vx[24];
+        SpinorIO<P32>::load(xr, g.stride, i, vx);
+#pragma unroll 2
+        for (int k = 0; k < n; ++k) {
+            float vp[24];
+            SpinorIO<PP>::load(pr + (size_t)((j0 + k) % slots) * slot_bytes, g.stride, i, vp);
+            const float a = alpha[k];
+#pragma unroll
+            for (int q = 0; q < 24; ++q) vx[q] += a * vp[q];
+        }
+        SpinorIO<P32>::store(xr, g.stride, i, vx);
+    }
     pdl_start_next();
 }
 
@@ -174,21 +211,43 @@ lqcd_status blas_xmy_norm(lqcd_ctx* c, void* out, const void* b, const void* a, 
     return LQCD_OK;
 }
 
-lqcd_status blas_cg_p_update(lqcd_ctx* c, void* p, int Pp, const void* r, int Pr, int nrhs, size_t p_rb,
+lqcd_status blas_cg_p_update(lqcd_ctx* c, void* p_out, const void* p, int Pp, const void* r, int Pr, int nrhs, size_t p_rb,
                              size_t r_rb, int nf, int s_num, int s_den)
 {
     const int block = 256;
     dim3 grid(blas_grid(c, block), nrhs);
-    char* pp = static_cast<char*>(p);
+    char* po = static_cast<char*>(p_out);
+    const char* pp = static_cast<const char*>(p);
     const char* rr = static_cast<const char*>(r);
     const bool small = (long)c->g.Vh * nrhs + own_capture.other_sites <= 12288;  // as the iteration's reducing hops
     if (Pr == P64) {
         if (Pp != P64) return fail(LQCD_ERR_INVALID, "cg_p_update: FP64 r needs FP64 p");
-        LQ_CUDA(launch_dependent(cg_p_kernel<P64, P64>, small, grid, block, c->stream, 0, c->g, pp, p_rb, rr, r_rb, nf,
+        LQ_CUDA(launch_dependent(cg_p_kernel<P64, P64>, small, grid, block, c->stream, 0, c->g, po, pp, p_rb, rr, r_rb, nf,
                                  c->scal, s_num, s_den, c->skip));
     } else {
-        LQ_SWITCH_P(Pp, LQ_CUDA(launch_dependent(cg_p_kernel<PT, P32>, small, grid, block, c->stream, 0, c->g, pp, p_rb, rr,
+        LQ_SWITCH_P(Pp, LQ_CUDA(launch_dependent(cg_p_kernel<PT, P32>, small, grid, block, c->stream, 0, c->g, po, pp, p_rb, rr,
                                                  r_rb, nf, c->scal, s_num, s_den, c->skip)));
+    }
+    c->launches++;
+    return LQCD_OK;
+}
+
+lqcd_status blas_cg_x_update(lqcd_ctx* c, void* x, size_t x_rb, const void* p, int Pp, size_t p_rb, size_t slot_bytes,
+                             int nrhs, int j0, int j1, int slots)
+{
+    const int block = 256;
+    dim3 grid(blas_grid(c, block), nrhs);
+    char* xx = static_cast<char*>(x);
+    const char* pp = static_cast<const char*>(p);
+    const bool small = (long)c->g.Vh * nrhs + own_capture.other_sites <= 12288;
+    switch (Pp) {
+    case P32: LQ_CUDA(launch_dependent(cg_x_kernel<P32>, small, grid, block, c->stream, 0, c->g, xx, x_rb, pp, p_rb,
+                                       slot_bytes, j0, j1, slots, c->scal, c->skip)); break;
+    case P16: LQ_CUDA(launch_dependent(cg_x_kernel<P16>, small, grid, block, c->stream, 0, c->g, xx, x_rb, pp, p_rb,
+                                       slot_bytes, j0, j1, slots, c->scal, c->skip)); break;
+    case PB16: LQ_CUDA(launch_dependent(cg_x_kernel<PB16>, small, grid, block, c->stream, 0, c->g, xx, x_rb, pp, p_rb,
+                                        slot_bytes, j0, j1, slots, c->scal, c->skip)); break;
+    default: return fail(LQCD_ERR_INVALID, "cg_x_update: inner vectors in FP32 or 16 bits");
     }
     c->launches++;
     return LQCD_OK;

@@ -17,7 +17,7 @@
 //   EPI_NONE     out = a * D
 //   EPI_CLOVINV  out = a * Cl D                  (Cl = A^{-1} of the output parity)
 //   EPI_XPAY     out = Cl y + a * D               (Cl = A, or 1 without clover)
-//   EPI_CG       s = Cl y + a * D; x += alpha p; r -= alpha s  (s never stored)
+//   EPI_CG       s = Cl y + a * D; r -= alpha s  (s never stored); x += alpha p unless A.x is null
 // and optionally (RED) the grid sum of |out|^2 (|r|^2 for EPI_CG) in FP64.
 #pragma once
 #include "core.cuh"
@@ -542,23 +542,27 @@ __device__ __forceinline__ void dslash_epilogue(const DslashArgs& A, int rhs, in
     }
     if constexpr (EPI == EPI_CG) {
         typedef typename RealT<AccumP<PS>::value>::type RA;
-        R pv[24];
-        RA xv[24], rv[24];
-        SpinorIO<PS>::load(static_cast<const char*>(A.p) + rhs * A.p_rb, A.g.stride, i, pv);
-        char* xb = static_cast<char*>(A.x) + rhs * A.acc_rb;
+        RA rv[24];
         char* rb = static_cast<char*>(A.r) + rhs * A.acc_rb;
-        SpinorIO<AccumP<PS>::value>::load(xb, A.g.stride, i, xv);
         SpinorIO<AccumP<PS>::value>::load(rb, A.g.stride, i, rv);
         RA n = 0;
 #pragma unroll
         for (int k = 0; k < 24; ++k) {
-            xv[k] += alpha * (RA)pv[k];
             rv[k] -= alpha * (RA)acc[k];
             n += rv[k] * rv[k];
         }
         nrm += (double)n;
-        SpinorIO<AccumP<PS>::value>::store(xb, A.g.stride, i, xv);
         SpinorIO<AccumP<PS>::value>::store(rb, A.g.stride, i, rv);
+        if (A.x) {  // (uniform; a deferred x is added by cg_x_kernel)
+            R pv[24];
+            RA xv[24];
+            SpinorIO<PS>::load(static_cast<const char*>(A.p) + rhs * A.p_rb, A.g.stride, i, pv);
+            char* xb = static_cast<char*>(A.x) + rhs * A.acc_rb;
+            SpinorIO<AccumP<PS>::value>::load(xb, A.g.stride, i, xv);
+#pragma unroll
+            for (int k = 0; k < 24; ++k) xv[k] += alpha * (RA)pv[k];
+            SpinorIO<AccumP<PS>::value>::store(xb, A.g.stride, i, xv);
+        }
     } else {
         SpinorIO<PS>::store(static_cast<char*>(A.out) + rhs * A.out_rb, A.g.stride, i, acc);
         if (RED) {
@@ -830,8 +834,10 @@ __device__ __forceinline__ void wide_operands(const DslashArgs& A, int rhs, int 
     if constexpr (EPI == EPI_CG) {
         constexpr int PA = AccumP<PS>::value;
         o.alpha = cg_alpha<PS>(A, rhs);
-        SpinorIO<PS>::template load_half<B>(static_cast<const char*>(A.p) + rhs * A.p_rb, A.g.stride, i, o.p);
-        SpinorIO<PA>::template load_half<B>(static_cast<const char*>(A.x) + rhs * A.acc_rb, A.g.stride, i, o.x);
+        if (A.x) {
+            SpinorIO<PS>::template load_half<B>(static_cast<const char*>(A.p) + rhs * A.p_rb, A.g.stride, i, o.p);
+            SpinorIO<PA>::template load_half<B>(static_cast<const char*>(A.x) + rhs * A.acc_rb, A.g.stride, i, o.x);
+        }
         SpinorIO<PA>::template load_half<B>(static_cast<const char*>(A.r) + rhs * A.acc_rb, A.g.stride, i, o.r);
     }
 }
@@ -874,13 +880,14 @@ __device__ __forceinline__ double wide_finish(const DslashArgs& A, int rhs, int 
     }
     if constexpr (EPI == EPI_CG) {
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            o.x[k] += o.alpha * (RA)o.p[k];
-            o.r[k] -= o.alpha * (RA)out[k];
-        }
+        for (int k = 0; k < 12; ++k) o.r[k] -= o.alpha * (RA)out[k];
         if (live) {
             constexpr int PA = AccumP<PS>::value;
-            SpinorIO<PA>::template store_half<B>(static_cast<char*>(A.x) + rhs * A.acc_rb, A.g.stride, i, o.x);
+            if (A.x) {
+#pragma unroll
+                for (int k = 0; k < 12; ++k) o.x[k] += o.alpha * (RA)o.p[k];
+                SpinorIO<PA>::template store_half<B>(static_cast<char*>(A.x) + rhs * A.acc_rb, A.g.stride, i, o.x);
+            }
             SpinorIO<PA>::template store_half<B>(static_cast<char*>(A.r) + rhs * A.acc_rb, A.g.stride, i, o.r);
         }
     } else if constexpr (!HALF) {

@@ -78,8 +78,8 @@ enum {
     SC_TMP = 128,       // scratch reductions [128, 160)
     SC_PER_RHS = 160
 };
-inline int rr_slot(int k) { return SC_RR + 2 * (k % SC_RING); }
-inline int pap_slot(int k) { return SC_PAP + 2 * (k % SC_RING); }
+__host__ __device__ inline int rr_slot(int k) { return SC_RR + 2 * (k % SC_RING); }
+__host__ __device__ inline int pap_slot(int k) { return SC_PAP + 2 * (k % SC_RING); }
 
 // dslash launch (dispatch by precision); block = threads per block
 cudaError_t dslash_dispatch_f64(const DslashArgs&, int, bool, int, bool, int, int, cudaStream_t);
@@ -252,7 +252,9 @@ lqcd_status clover_build(lqcd_ctx* c, double kappa, double csw);
 lqcd_status blas_norm2(lqcd_ctx* c, const void* x, int P, int nrhs, size_t rb, int nf, int slot);
 lqcd_status blas_xmy_norm(lqcd_ctx* c, void* out, const void* b, const void* a, int P, int nrhs, size_t rb, int nf,
                           int slot);
-lqcd_status blas_cg_p_update(lqcd_ctx* c, void* p, int Pp, const void* r, int Pr, int nrhs, size_t p_rb,
+lqcd_status blas_cg_x_update(lqcd_ctx* c, void* x, size_t x_rb, const void* p, int Pp, size_t p_rb, size_t slot_bytes,
+                             int nrhs, int j0, int j1, int slots);
+lqcd_status blas_cg_p_update(lqcd_ctx* c, void* p_out, const void* p, int Pp, const void* r, int Pr, int nrhs, size_t p_rb,
                              size_t r_rb, int nf, int s_num, int s_den);
 lqcd_status blas_accumulate_x(lqcd_ctx* c, void* xhi, const void* xlo, int Plo, int nrhs, size_t hi_rb,
                               size_t lo_rb, int nf);

@@ -34,10 +34,15 @@ struct Cg {
     bool eo;
     size_t fb64, rb64, fbi, rbi, fba, rba;
     char *B, *X, *T1, *BH, *RH, *T2;  // FP64 full fields (rhs stride rb64)
-    char *Pv, *Qv;                    // inner precision full fields (rhs stride rbi)
+    char *Pv, *Qv;                    // inner precision full fields (rhs stride rbi); even-odd: Qv alone
+    // the search direction on the solved sites: `slots` of them, slot_bytes
+    // apart, right-hand sides p_rb apart (see set_directions)
+    char* P0;
+    size_t slot_bytes, p_rb;
+    int slots;
     char *XLO, *RV;                   // accumulation precision full fields (rhs stride rba)
     int nf;                           // 1 (odd parity only) or 2 (full lattice)
-    size_t o64, oi, oa;               // byte offset of the solved parity in each field
+    size_t o64, oa;                   // byte offset of the solved parity in each field
     long reliable = 0, checks = 0;
 };
 
@@ -49,25 +54,66 @@ static const void* clov_or_null(lqcd_ctx* c, int P, int parity, bool inverse)
     return base + parity * c->clov_parity_bytes(pg);
 }
 
+// Deferred x.  With one direction slot, x += alpha p is part of the fused CG
+// launch: x is read and written and p read once more in every iteration,
+// 192 + 52 (FP16 spinors) of the 3800 bytes a site that an iteration moves.
+// With more, the directions of up to `slots` iterations stay where they are
+// and one pass adds them to x in the same order with the same steps (the same
+// bits): per iteration 52 bytes and a share of x's 192.  The directions take
+// what the inner vectors' room leaves beside q (ten in FP32, twenty in 16
+// bits).
+static void set_directions(Cg& s, bool defer)
+{
+    lqcd_ctx* c = s.c;
+    const size_t room = (size_t)NVLO * 2 * c->field_bytes(P64);  // per right-hand side
+    if (s.eo) {  // q_e, q_o, then the directions on the odd sites
+        s.Qv = c->veclo;
+        s.P0 = c->veclo + (size_t)s.R * s.rbi;
+        s.p_rb = s.fbi;
+        s.slots = defer ? (int)((room - s.rbi) / s.fbi) : 1;
+        if (s.slots > SC_RING - 2) s.slots = SC_RING - 2;
+        s.Pv = nullptr;
+    } else {
+        s.Pv = s.P0 = c->veclo;
+        s.Qv = c->veclo + (size_t)s.R * s.rbi;
+        s.p_rb = s.rbi;
+        s.slots = 1;
+    }
+    s.slot_bytes = (size_t)s.R * s.p_rb;
+}
+
+// Is x deferred?  Only in mixed even-odd solves (not by the persistent kernel,
+// and not in FP64, which its pipe bounds), and where the iteration streams
+// from HBM: per iteration, x in the launch against deferred, FP32 and FP16
+// spinors, us: 32768 sites (times right-hand sides) 37.4 / 35.8 against 38.1 /
+// 35.9, 65536 55.1 / 58.4 against 56.0 / 58.2, 165888 164 / 149 against 162 /
+// 145, 331776 259 / 248 against 254 / 241, 1048576 737 / 653 against 714 / 629.
+// Below, everything stays in L2 and the ring of directions only takes room there.
+static bool defer_x(const Cg& s, bool persistent)
+{
+    return s.eo && s.Pi != P64 && !persistent && (long)s.c->g.Vh * s.R >= 131072;
+}
+
 // The four hopping launches of an even-odd CG iteration j (block-relative
-// scalar slots):
+// scalar slots), p_o in direction slot `slot`:
 //   D1: t_e = A_ee^{-1} H_eo p_o
 //   D2: q_o = A_oo p_o - kappa^2 H_oe t_e,               |q_o|^2 -> pap slot j
 //   D3: t_e = A_ee^{-1} H_eo^dag q_o
 //   D4: s = A_oo q_o - kappa^2 H_oe^dag t_e; x += alpha p; r -= alpha s,
 //       alpha = |r|^2 / |q|^2 from slots j,                |r|^2 -> rr slot j + 1
 // (D1, D3: EPI_CLOVINV; D2: EPI_XPAY with the norm; D4: EPI_CG, dagger for D3, D4.)
-void eo_stage_args(const Cg& s, int j, DslashArgs d[4])
+void eo_stage_args(const Cg& s, int j, int slot, DslashArgs d[4])
 {
     lqcd_ctx* c = s.c;
     const int P = s.Pi;
+    char* const p = s.P0 + slot * s.slot_bytes;
     DslashArgs A = base_args(c, P);
     A.skip = c->skip;
     A.par = 0;
     A.out = s.Qv;
     A.out_rb = s.rbi;
-    A.in = s.Pv + s.fbi;
-    A.in_rb = s.rbi;
+    A.in = p;
+    A.in_rb = s.p_rb;
     A.clov = clov_or_null(c, P, 0, true);
     A.a = 1.0;
     d[0] = A;
@@ -79,12 +125,13 @@ void eo_stage_args(const Cg& s, int j, DslashArgs d[4])
     B.in = s.Qv;
     B.in_rb = s.rbi;
     B.clov = clov_or_null(c, P, 1, false);
-    B.y = s.Pv + s.fbi;
-    B.y_rb = s.rbi;
+    B.y = p;
+    B.y_rb = s.p_rb;
     B.a = -c->kappa * c->kappa;
     B.red = c->scal + pap_slot(j) + 1;
     d[1] = B;
     A.in = s.Qv + s.fbi;
+    A.in_rb = s.rbi;
     d[2] = A;
     DslashArgs D = base_args(c, P);
     D.skip = c->skip;
@@ -95,11 +142,11 @@ void eo_stage_args(const Cg& s, int j, DslashArgs d[4])
     D.y = s.Qv + s.fbi;
     D.y_rb = s.rbi;
     D.a = -c->kappa * c->kappa;
-    D.x = s.XLO + s.fba;
+    D.x = s.slots > 1 ? nullptr : s.XLO + s.fba;  // nullptr: x is added later
     D.r = s.RV + s.fba;
     D.acc_rb = s.rba;
-    D.p = s.Pv + s.fbi;
-    D.p_rb = s.rbi;
+    D.p = p;
+    D.p_rb = s.p_rb;
     D.s_num = rr_slot(j);
     D.s_num2 = rr_slot(j) + 1;
     D.s_den = pap_slot(j);
@@ -112,13 +159,13 @@ namespace {
 
 // One inner CG iteration j of a block: q = K p, x += alpha p, r -= alpha K^dag q
 // with K = Mhat (eo) or M (full), |r|^2 into block slot j + 1.
-lqcd_status cg_iteration(Cg& s, int j)
+lqcd_status cg_iteration(Cg& s, int j, int slot)
 {
     lqcd_ctx* c = s.c;
     const int P = s.Pi;
     if (s.eo) {
         DslashArgs d[4];
-        eo_stage_args(s, j, d);
+        eo_stage_args(s, j, slot, d);
         LQ_TRY(launch_dslash(c, d[0], P, false, EPI_CLOVINV, false, s.R));
         LQ_TRY(launch_dslash(c, d[1], P, false, EPI_XPAY, true, s.R));
         LQ_TRY(launch_dslash(c, d[2], P, true, EPI_CLOVINV, false, s.R));
@@ -227,11 +274,19 @@ lqcd_status reliable_update(Cg& s, int j)
 // the last direction update; ends by moving slot n to slot 0.
 lqcd_status run_block(Cg& s, int n, bool ru_at_end)
 {
+    int first = 0;  // first iteration whose step is not yet in x
     for (int j = 0; j < n; ++j) {
-        LQ_TRY(cg_iteration(s, j));
-        if (ru_at_end && j == n - 1) LQ_TRY(reliable_update(s, j + 1));
-        LQ_TRY(blas_cg_p_update(s.c, s.Pv + s.oi, mode_ps(s.Pi), s.RV + s.oa, s.PA, s.R, s.rbi, s.rba, s.nf, rr_slot(j + 1),
-                                rr_slot(j)));
+        const int slot = j % s.slots, last = j == n - 1;
+        LQ_TRY(cg_iteration(s, j, slot));
+        if (s.slots > 1 && (last || slot == s.slots - 1)) {
+            LQ_TRY(blas_cg_x_update(s.c, s.XLO + s.oa, s.rba, s.P0, mode_ps(s.Pi), s.p_rb, s.slot_bytes, s.R, first, j + 1,
+                                    s.slots));
+            first = j + 1;
+        }
+        if (ru_at_end && last) LQ_TRY(reliable_update(s, j + 1));
+        // every block starts from slot 0 (x holds all earlier steps by then)
+        LQ_TRY(blas_cg_p_update(s.c, s.P0 + (last ? 0 : (j + 1) % s.slots) * s.slot_bytes, s.P0 + slot * s.slot_bytes,
+                                mode_ps(s.Pi), s.RV + s.oa, s.PA, s.R, s.p_rb, s.rba, s.nf, rr_slot(j + 1), rr_slot(j)));
     }
     return blas_copy_scalar_pair(s.c, rr_slot(0), rr_slot(n), s.R);
 }
@@ -331,12 +386,10 @@ lqcd_status cg_setup(CgRun& run, lqcd_ctx* c, double* x, const double* b, double
     s.BH = vec64_field(c, 3, 0);
     s.RH = vec64_field(c, 4, 0);
     s.T2 = vec64_field(c, 5, 0);
-    s.Pv = c->veclo;
-    s.Qv = c->veclo + (size_t)R * s.rbi;
+    set_directions(s, defer_x(s, p->persistent != 0));
     s.XLO = c->vecacc;
     s.RV = c->vecacc + (size_t)R * s.rba;
     s.o64 = s.eo ? s.fb64 : 0;
-    s.oi = s.eo ? s.fbi : 0;
     s.oa = s.eo ? s.fba : 0;
     if (p->residual_prec != LQCD_F64) return fail(LQCD_ERR_INVALID, "lqcd_solve: residual_prec must be LQCD_F64");
     const size_t canon_rb = (size_t)c->volume * 192;
@@ -367,7 +420,7 @@ lqcd_status cg_setup(CgRun& run, lqcd_ctx* c, double* x, const double* b, double
                       s.rb64, -1));
         // r0 = Mhat^dag bhat_o (x0 = 0)
         LQ_TRY(normal_residual_eo(s, s.BH + s.fb64, rr_slot(0) + 1));
-        LQ_TRY(convert_field(c, s.Pv + s.fbi, mode_ps(s.Pi), s.RV + s.fba, s.PA, R, s.rbi, s.rba, 1, -1));
+        LQ_TRY(convert_field(c, s.P0, mode_ps(s.Pi), s.RV + s.fba, s.PA, R, s.p_rb, s.rba, 1, -1));
     } else {
         LQ_TRY(op_full(c, s.RH, s.B, P64, true, R, s.rb64));
         LQ_TRY(convert_field(c, s.RV, s.PA, s.RH, P64, R, s.rba, s.rb64, 1, rr_slot(0)));
@@ -411,9 +464,8 @@ lqcd_status fall_back_to_f32(CgRun& run)
     s.Pi = LQCD_F32;
     s.fbi = c->field_bytes(s.Pi);
     s.rbi = 2 * s.fbi;
-    s.Qv = c->veclo + (size_t)s.R * s.rbi;
-    s.oi = s.eo ? s.fbi : 0;
-    if (s.eo) LQ_TRY(convert_field(c, s.Pv + s.fbi, P32, s.RV + s.fba, s.PA, s.R, s.rbi, s.rba, 1, -1));
+    set_directions(s, s.slots > 1);
+    if (s.eo) LQ_TRY(convert_field(c, s.P0, P32, s.RV + s.fba, s.PA, s.R, s.p_rb, s.rba, 1, -1));
     else LQ_TRY(convert_field(c, s.Pv, P32, s.RV, s.PA, s.R, s.rbi, s.rba, 2, -1));
     run.fell_back = true;
     run.rebuild_graphs = true;
@@ -584,7 +636,7 @@ lqcd_status run_block_persistent(std::vector<CgRun*>& runs, unsigned long long m
             lqcd_ctx* c = s.c;
             PersistLattice& L = P.lat[P.nlat++];
             for (int jj = 0; jj < 2; ++jj) {
-                eo_stage_args(s, jj, L.d[jj]);
+                eo_stage_args(s, jj, 0, L.d[jj]);
                 L.d[jj][3].red = c->scal + rr_slot((jj + 1) & 1) + 1;  // the ring of two
                 for (int k = 0; k < 4; ++k) {
                     L.d[jj][k].nrhs = s.R;
@@ -606,8 +658,8 @@ lqcd_status run_block_persistent(std::vector<CgRun*>& runs, unsigned long long m
                 P.npairs++;
                 ntiles += L.ntiles;
             }
-            L.p = s.Pv + s.fbi;
-            L.p_rb = s.rbi;
+            L.p = s.P0;
+            L.p_rb = s.p_rb;
             L.r = s.RV + s.fba;
             L.r_rb = s.rba;
             L.scal = c->scal;
@@ -642,7 +694,7 @@ lqcd_status run_block_persistent(std::vector<CgRun*>& runs, unsigned long long m
             if (!(mask >> i & 1)) continue;
             Cg& s = runs[i]->s;
             LQ_TRY(reliable_update(s, jn));
-            LQ_TRY(blas_cg_p_update(s.c, s.Pv + s.oi, mode_ps(s.Pi), s.RV + s.oa, s.PA, s.R, s.rbi, s.rba, s.nf,
+            LQ_TRY(blas_cg_p_update(s.c, s.P0, s.P0, mode_ps(s.Pi), s.RV + s.oa, s.PA, s.R, s.p_rb, s.rba, s.nf,
                                     rr_slot(jn), rr_slot(jp)));
             if (jn) LQ_TRY(blas_copy_scalar_pair(s.c, rr_slot(0), rr_slot(1), s.R));
         }

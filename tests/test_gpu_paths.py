@@ -252,3 +252,44 @@ def test_hop_reads_subnormal_halves(lq, prec, block):
     norm = np.abs(hop_ref(U, psi, dims, 0)).max()
     assert np.abs(want).max() > 2.0 ** -17 * norm  # well above a step, far below the normal range
     assert np.abs(got - want).max() < 2.0 ** -23 * norm
+
+
+@pytest.mark.parametrize("inner", ["f32", "f16spinors", "f16"])
+@pytest.mark.parametrize("graph", [0, 1])
+@pytest.mark.parametrize("check,every,maxiter", [(10, 0, 25), (30, 0, 60), (30, 7, 33), (1, 2, 5)])
+def test_deferred_solution_updates(lq, inner, graph, check, every, maxiter):
+    """Two right-hand sides of 65536 sites take the deferred x (ring of ten or
+    twenty directions: wrapped, cut short by a replacement or by maxiter), one
+    the fused update; the steps are the same, so the iterates are equal."""
+    import torch
+    dims = (16, 16, 16, 32)
+    lat = lq.Lattice(dims, precisions=("f64", "f32", inner), max_nrhs=2, stream=torch.cuda.Stream())
+    lat.gauge_load(on_device(synth.gauge_field(dims, "smooth", 31, eps=0.5)))
+    lat.clover_compute(0.13, 1.0)
+    b = on_device(np.stack([synth.gaussian_spinor(dims, 32 + r) for r in range(2)]))
+    x2, x1 = torch.zeros_like(b), torch.zeros_like(b)
+    torch.cuda.synchronize()
+    kw = dict(raise_on_error=False, inner_prec=inner, use_graph=graph, check_interval=check, reliable_interval=every,
+              reliable_delta=0.0, maxiter=maxiter)
+    lat.solve(x2, b, 1e-30, nrhs=2, **kw)
+    for r in range(2):
+        lat.solve(x1[r], b[r], 1e-30, nrhs=1, **kw)
+    assert torch.equal(x1, x2)
+
+
+def test_deferred_solve(lq):
+    """A deferred solve whose right-hand sides converge at different times."""
+    import torch
+    dims = (16, 16, 16, 32)
+    U = synth.gauge_field(dims, "smooth", 33, eps=0.5)
+    lat = lq.Lattice(dims, precisions=("f64", "f32"), max_nrhs=3)
+    lat.gauge_load(on_device(U))
+    lat.clover_compute(0.125, 1.0)
+    A = oracle.clover(U, 0.125, 1.0)
+    b = np.stack([synth.gaussian_spinor(dims, 34), np.zeros((32, 16, 16, 16, 4, 3), complex), synth.gaussian_spinor(dims, 35)])
+    b[2, 1:] = 0.0
+    x = torch.zeros(b.shape, dtype=torch.complex128, device="cuda")
+    lat.solve(x, on_device(b), 1e-10, nrhs=3, inner_prec="f16spinors")
+    assert not x[1].any()
+    for r in (0, 2):
+        assert oracle.true_residual(U, A, 0.125, b[r], x[r].cpu().numpy()) <= 1e-10
