@@ -455,8 +455,7 @@ lqcd_status lqcd_gauge_load(lqcd_ctx* c, const double* links)
     const int Lt = c->g.L[3];
     const size_t per_t = (size_t)c->volume / Lt * 72;  // doubles per t slice
     if (is_device_ptr(links)) {
-        for (int P = 0; P < 4; ++P)
-            if (c->holds(P)) LQ_TRY(gauge_pack(c, links, 0, Lt, P));
+        LQ_TRY(gauge_pack(c, links, 0, Lt));
     } else {
         int nt = (int)(c->staging_bytes / (per_t * sizeof(double)));
         if (nt < 1) return fail(LQCD_ERR_NOMEM, "lqcd_gauge_load: staging too small");
@@ -464,8 +463,7 @@ lqcd_status lqcd_gauge_load(lqcd_ctx* c, const double* links)
             const int t1 = t0 + nt < Lt ? t0 + nt : Lt;
             LQ_CUDA(cudaMemcpyAsync(c->staging, links + (size_t)t0 * per_t, (size_t)(t1 - t0) * per_t * sizeof(double),
                                     cudaMemcpyHostToDevice, c->stream));
-            for (int P = 0; P < 4; ++P)
-                if (c->holds(P)) LQ_TRY(gauge_pack(c, static_cast<const double*>(c->staging), t0, t1, P));
+            LQ_TRY(gauge_pack(c, static_cast<const double*>(c->staging), t0, t1));
         }
         LQ_CUDA(cudaStreamSynchronize(c->stream));  // staging is reused by the next call
     }

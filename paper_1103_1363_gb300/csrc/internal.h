@@ -242,7 +242,7 @@ lqcd_status pack_difference(lqcd_ctx* c, void* internal, const double* a, const 
                             size_t internal_rb, size_t canon_rb);
 lqcd_status unpack_spinor_f32(lqcd_ctx* c, float* canon, const void* internal, int nrhs, size_t internal_rb,
                               size_t canon_rb);
-lqcd_status gauge_pack(lqcd_ctx* c, const double* canon_dev_slice, int t0, int t1, int P);
+lqcd_status gauge_pack(lqcd_ctx* c, const double* canon_dev_slice, int t0, int t1);  // every held precision
 lqcd_status convert_field(lqcd_ctx* c, void* out, int Pout, const void* in, int Pin, int nrhs, size_t out_rb,
                           size_t in_rb, int nf, int norm_slot /* -1: no norm */);
 // clover.cu

@@ -293,3 +293,62 @@ def test_deferred_solve(lq):
     assert not x[1].any()
     for r in (0, 2):
         assert oracle.true_residual(U, A, 0.125, b[r], x[r].cpu().numpy()) <= 1e-10
+
+
+@pytest.mark.parametrize("dims,nrhs", [((2, 2, 2, 2), 1), ((4, 2, 6, 6), 3), ((8, 4, 8, 10), 2)])  # 8, 144, 1280 sites a parity
+@pytest.mark.parametrize("prec,eps", [("f64", 0.0), ("f32", 2.0 ** -24), ("f16", 2.0 ** -10), ("bf16spinors", 2.0 ** -7)])
+def test_pack_and_unpack(lq, dims, nrhs, prec, eps):
+    """Canonical spinors to internal fields and back, one parity and both, from
+    host and device: each component within the storage's rounding of the site's
+    largest, untouched sites of a one-parity unpack left alone."""
+    import torch
+    psi = np.stack([synth.gaussian_spinor(dims, 41 + r) for r in range(nrhs)])
+    big = np.abs(psi).max(axis=(-2, -1), keepdims=True)
+    par = np.indices(psi.shape[1:5]).sum(axis=0) % 2
+    lat = lq.Lattice(dims, precisions=("f64", "f32", prec), max_nrhs=nrhs)
+    for parity in (-1, 0, 1):
+        for host in (False, True):
+            f = lat.new_field(prec, nrhs, parity < 0)
+            src = torch.from_numpy(psi) if host else on_device(psi)
+            lat.pack(f, src, parity, prec, nrhs)
+            out = torch.full(psi.shape, 7.0, dtype=torch.complex128, device="cpu" if host else "cuda")
+            lat.unpack(out, f, parity, prec, nrhs)
+            lat.sync()
+            got = out.cpu().numpy()
+            on = np.ones_like(par, bool) if parity < 0 else par == parity
+            assert (np.abs(got - psi)[:, on] <= 1.5 * eps * big[:, on]).all()
+            if not host:  # (a host copy comes back whole, with the staging area's other sites)
+                assert (got[:, ~on] == 7.0).all()
+
+
+@pytest.mark.parametrize("recon", [12, 18])
+def test_gauge_load_sources(lq, recon):
+    """Links from the host, the device, and a device buffer that starts at an
+    odd double: the same fields in every precision."""
+    import torch
+    dims = (4, 6, 2, 10)  # 24 sites a parity and slice, blocks of 32
+    U = synth.gauge_field(dims, "smooth", 45, eps=0.5)
+    psi = on_device(synth.gaussian_spinor(dims, 46))
+    odd = torch.empty(2 * U.size + 1, dtype=torch.float64, device="cuda")[1:]
+    odd.copy_(torch.view_as_real(torch.from_numpy(U)).reshape(-1))
+    assert odd.data_ptr() % 16 == 8
+    outs = []
+    for links in (on_device(U), odd, torch.from_numpy(U)):
+        lat = lq.Lattice(dims, recon=recon)
+        lat.gauge_load(links)
+        fields = []
+        for prec in ("f64", "f32", "f16", "bf16"):
+            fin, fout = lat.new_field(prec), lat.new_field(prec)
+            fout.zero_()
+            lat.pack(fin, psi, 1, prec)
+            lat.dslash(fout, fin, 0, prec=prec)
+            fields.append(fout)
+        lat.sync()
+        outs.append(fields)
+    for fields in outs[1:]:
+        for a, b in zip(outs[0], fields):
+            assert torch.equal(a, b)
+    got = lat.canonical_spinor()
+    lat.unpack(got, outs[0][0], 0, "f64")
+    lat.sync()
+    assert rel(got.cpu().numpy(), hop_ref(U, psi.cpu().numpy(), dims, 0)) < 1e-13
