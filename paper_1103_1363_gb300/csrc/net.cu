@@ -498,6 +498,132 @@ struct ItemCursor {
     }
 };
 
+// ---- one hop of a one-channel FP32 activation, its loads apart from its arithmetic
+// fetch() issues the loads of the link and of the neighbour's spinor, finish()
+// forms the transported channel, so that a thread has the loads of several hops
+// in flight instead of one round trip to L2 per hop.
+template <int RECON>
+struct HopFetch {
+    float lk[RECON == 12 ? 12 : 18];
+    float p[24];
+    float sign;
+    int h;
+    bool fwd, live;
+    // hop hh at site x (coordinates c0..c3; live: x < V) of the activation act
+    __device__ __forceinline__ void fetch(const NetLayerArgs& a, const float* act, int x, int c0, int c1, int c2, int c3,
+                                          bool inside, int hh)
+    {
+        h = hh;
+        live = inside;
+        sign = 1.f;
+        fwd = (h & 1) != 0;
+        const int y = live ? hop_neighbour(a, x, c0, c1, c2, c3, h) : -1;
+        if (live && h > 0) {
+            const int mu = (h - 1) / 2;
+            if (a.tanti && mu == 3 && (fwd ? c3 == a.L[3] - 1 : c3 == 0)) sign = -1.f;
+            // forward: U_mu(x); backward: U_mu(y)^dag, y of the other parity (all extents are even)
+            const int par = (c0 + c1 + c2 + c3 + (fwd ? 0 : 1)) & 1, i = (fwd ? x : y) >> 1;
+            if constexpr (RECON == 12) {
+                const float4* q = static_cast<const float4*>(a.gauge) + (size_t)((par * 4 + mu) * 3) * a.stride + i;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const float4 v = __ldg(q + (size_t)k * a.stride);
+                    lk[4 * k] = v.x; lk[4 * k + 1] = v.y; lk[4 * k + 2] = v.z; lk[4 * k + 3] = v.w;
+                }
+            } else {
+                const float2* q = static_cast<const float2*>(a.gauge) + (size_t)((par * 4 + mu) * 9) * a.stride + i;
+#pragma unroll
+                for (int k = 0; k < 9; ++k) {
+                    const float2 v = __ldg(q + (size_t)k * a.stride);
+                    lk[2 * k] = v.x; lk[2 * k + 1] = v.y;
+                }
+            }
+        }
+        load_channel(act, a.V, 0, y, p);
+    }
+    // w[colour][spin]: the transported channel, rounded to BF16 (zero past the lattice)
+    __device__ __forceinline__ void finish(uint32_t w[3][4]) const
+    {
+        if (h == 0 || !live) {  // (past the lattice p is zero)
+#pragma unroll
+            for (int ca = 0; ca < 3; ++ca)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) w[ca][r] = pack_bf16x2(p[2 * (3 * r + ca)], p[2 * (3 * r + ca) + 1]);
+            return;
+        }
+        float u[18];
+#pragma unroll
+        for (int k = 0; k < (RECON == 12 ? 12 : 18); ++k) u[k] = lk[k];
+        if constexpr (RECON == 12) reconstruct_row2(u);
+        if (!fwd) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+#pragma unroll
+                for (int j = i; j < 3; ++j) {
+                    const float ar = u[2 * (3 * i + j)], ai = u[2 * (3 * i + j) + 1];
+                    const float br = u[2 * (3 * j + i)], bi = u[2 * (3 * j + i) + 1];
+                    u[2 * (3 * i + j)] = br; u[2 * (3 * i + j) + 1] = -bi;
+                    u[2 * (3 * j + i)] = ar; u[2 * (3 * j + i) + 1] = -ai;
+                }
+        }
+#pragma unroll
+        for (int k = 0; k < 18; ++k) u[k] = sign * u[k];
+#pragma unroll
+        for (int ca = 0; ca < 3; ++ca)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                float re = 0.f, im = 0.f;
+#pragma unroll
+                for (int cb = 0; cb < 3; ++cb) {  // one multiply-add per real product
+                    const float ur = u[2 * (3 * ca + cb)], ui = u[2 * (3 * ca + cb) + 1];
+                    const float pr = p[2 * (3 * r + cb)], pi = p[2 * (3 * r + cb) + 1];
+                    re += ur * pr;
+                    re -= ui * pi;
+                    im += ur * pi;
+                    im += ui * pr;
+                }
+                w[ca][r] = pack_bf16x2(re, im);
+            }
+    }
+};
+
+// Coordinates of canonical site x.
+struct SiteCoords {
+    int c0, c1, c2, c3;
+    __device__ __forceinline__ SiteCoords(const NetLayerArgs& a, int x)
+    {
+        c0 = x % a.L[0];
+        x /= a.L[0];
+        c1 = x % a.L[1];
+        x /= a.L[1];
+        c2 = x % a.L[2];
+        c3 = x / a.L[2];
+    }
+};
+
+// Channels first, first + G, ... of BF16 activations at site y (-1: zero), as
+// they are, into the rows dst + colour * pitch + channel * 128; all loads are
+// issued before the first store, and between() after them.
+template <int G, class F>
+__device__ __forceinline__ void put_channels(const NetLayerArgs& a, const void* act, int ch, int b, int y, int first,
+                                             unsigned char* dst, uint32_t pitch, F between)
+{
+    constexpr int N = (NET_MAXC + G - 1) / G;
+    uint32_t raw[N][12];
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+        if (first + G * j < ch) load_raw_bf16(act, a.V, ch, b, first + G * j, y, raw[j]);
+    between();
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        if (first + G * j >= ch) break;
+#pragma unroll
+        for (int ca = 0; ca < 3; ++ca)
+            *reinterpret_cast<uint4*>(dst + ca * pitch + (first + G * j) * 128) =
+                make_uint4(raw[j][ca], raw[j][3 + ca], raw[j][6 + ca], raw[j][9 + ca]);
+    }
+}
+
 // Default bound of a wait on the kernels' own MMAs and copies (a hop's MMAs
 // take microseconds); an expired wait sets ERRW_TIMEOUT and the CTA stops,
 // after waiting (with this bound) for its own operations in flight and
@@ -772,49 +898,23 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_layer_c1_kernel(const NetL
     auto gather = [&](int t, int s) {
         const int b = t / ntiles, x = (t - b * ntiles) * NTC_TS + sl;
         unsigned char* xrow = smem + s * xbytes + (sl >> 3) * sbo + (sl & 7) * 16;
-        for (int h = grp; h < 9; h += NTC_THREADS / NTC_TS) {
-            float u[18], p[24];
-            float sign = 1.f;
-            int y = -1;
+        const float* act = a.in + (size_t)b * a.V * 24;
+        const SiteCoords q(a, x);
+        auto put = [&](const HopFetch<RECON>& f) {
+            uint32_t w[3][4];
+            f.finish(w);
 #pragma unroll
-            for (int k = 0; k < 18; ++k) u[k] = 0.f;  // padding sites: zero link, zero input
-            if (x < a.V) {
-                if (h > 0) {
-                    y = hop_link<RECON>(a, x, h, u, sign);
-#pragma unroll
-                    for (int k = 0; k < 18; ++k) u[k] = sign * u[k];
-                } else {
-                    y = x;
-                }
-            }
-            load_act(a.in, a.in_bf16, a.V, 1, b, 0, y, p);
-#pragma unroll
-            for (int ca = 0; ca < 3; ++ca) {
-                uint32_t w[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    float re, im;
-                    if (h == 0) {
-                        re = p[2 * (3 * r + ca)];
-                        im = p[2 * (3 * r + ca) + 1];
-                    } else {
-                        re = 0.f;
-                        im = 0.f;
-#pragma unroll
-                        for (int cb = 0; cb < 3; ++cb) {  // one multiply-add per real product
-                            const float ur = u[2 * (3 * ca + cb)], ui = u[2 * (3 * ca + cb) + 1];
-                            const float pr = p[2 * (3 * r + cb)], pi = p[2 * (3 * r + cb) + 1];
-                            re += ur * pr;
-                            re -= ui * pi;
-                            im += ur * pi;
-                            im += ui * pr;
-                        }
-                    }
-                    w[r] = pack_bf16x2(re, im);
-                }
-                *reinterpret_cast<uint4*>(xrow + ca * blk + h * 128) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        }
+            for (int ca = 0; ca < 3; ++ca)
+                *reinterpret_cast<uint4*>(xrow + ca * blk + f.h * 128) = make_uint4(w[ca][0], w[ca][1], w[ca][2], w[ca][3]);
+        };
+        // hops grp and grp + 4 together, then hop 8 (group 0)
+        HopFetch<RECON> f0, f1;
+        f0.fetch(a, act, x, q.c0, q.c1, q.c2, q.c3, x < a.V, grp);
+        f1.fetch(a, act, x, q.c0, q.c1, q.c2, q.c3, x < a.V, grp + 4);
+        put(f0);
+        if (grp == 0) f0.fetch(a, act, x, q.c0, q.c1, q.c2, q.c3, x < a.V, 8);
+        put(f1);
+        if (grp == 0) put(f0);
     };
 
     bool failed = false;
@@ -944,64 +1044,28 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_c1_kernel(const NetL
         const int b = t / ntiles, x = (t - b * ntiles) * NTC_TS + sl;
         // the operand tiles are free once the MMAs of tile k - 1 have completed
         if (k >= 1 && !wait_failed) wait_failed = !tc::mbar_wait(mma_bar, (k - 1) & 1, a.wait_ns);
-        // X: the transported input of hops grp, grp + 4, grp + 8 at M rows 8 h .. 8 h + 7
-        for (int h = grp; h < 9; h += G4) {
-            float u[18], p[24];
-            float sign = 1.f;
-            int y = -1;
+        // X: the transported input of hops grp, grp + 4, grp + 8 at M rows 8 h .. 8 h + 7;
+        // G: output-gradient channels grp, grp + 4, ... at the site (their
+        // loads first: they are used first)
+        const float* act = a.in + (size_t)b * a.V * 24;
+        const SiteCoords q(a, x);
+        auto put = [&](const HopFetch<RECON>& f) {
+            uint32_t w[3][4];
+            f.finish(w);
 #pragma unroll
-            for (int q = 0; q < 18; ++q) u[q] = 0.f;  // padding sites: zero link, zero input
-            if (x < a.V) {
-                if (h > 0) {
-                    y = hop_link<RECON>(a, x, h, u, sign);
-#pragma unroll
-                    for (int q = 0; q < 18; ++q) u[q] = sign * u[q];
-                } else {
-                    y = x;
-                }
-            }
-            load_act(a.in, a.in_bf16, a.V, 1, b, 0, y, p);
-#pragma unroll
-            for (int ca = 0; ca < 3; ++ca) {
-                uint32_t w[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    float re, im;
-                    if (h == 0) {
-                        re = p[2 * (3 * r + ca)];
-                        im = p[2 * (3 * r + ca) + 1];
-                    } else {
-                        re = 0.f;
-                        im = 0.f;
-#pragma unroll
-                        for (int cb = 0; cb < 3; ++cb) {  // one multiply-add per real product
-                            const float ur = u[2 * (3 * ca + cb)], ui = u[2 * (3 * ca + cb) + 1];
-                            const float pr = p[2 * (3 * r + cb)], pi = p[2 * (3 * r + cb) + 1];
-                            re += ur * pr;
-                            re -= ui * pi;
-                            im += ur * pi;
-                            im += ui * pr;
-                        }
-                    }
-                    w[r] = pack_bf16x2(re, im);
-                }
-                *reinterpret_cast<uint4*>(Xs + ca * blkx + (sl >> 3) * sbox + h * 128 + rowoff) =
-                    make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        }
-        // G: output-gradient channels grp, grp + 4, ... at the site
-        for (int co = grp; co < a.cout; co += G4) {
-            float p[24];
-            load_act(gout, a.gout_bf16, a.V, a.cout, b, co, x < a.V ? x : -1, p);
-#pragma unroll
-            for (int ca = 0; ca < 3; ++ca) {
-                uint32_t w[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) w[r] = pack_bf16x2(p[2 * (3 * r + ca)], p[2 * (3 * r + ca) + 1]);
-                *reinterpret_cast<uint4*>(Gs + ca * blkg + (sl >> 3) * sbog + co * 128 + rowoff) =
-                    make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        }
+            for (int ca = 0; ca < 3; ++ca)
+                *reinterpret_cast<uint4*>(Xs + ca * blkx + (sl >> 3) * sbox + f.h * 128 + rowoff) =
+                    make_uint4(w[ca][0], w[ca][1], w[ca][2], w[ca][3]);
+        };
+        HopFetch<RECON> f0, f1;
+        put_channels<G4>(a, gout, a.cout, b, x < a.V ? x : -1, grp, Gs + (sl >> 3) * sbog + rowoff, blkg, [&]() {
+            f0.fetch(a, act, x, q.c0, q.c1, q.c2, q.c3, x < a.V, grp);
+        });
+        f1.fetch(a, act, x, q.c0, q.c1, q.c2, q.c3, x < a.V, grp + 4);
+        put(f0);
+        if (grp == 0) f0.fetch(a, act, x, q.c0, q.c1, q.c2, q.c3, x < a.V, 8);
+        put(f1);
+        if (grp == 0) put(f0);
         tc::fence_proxy_async();
         if (__syncthreads_or(wait_failed)) {
             failed = true;
@@ -1101,64 +1165,42 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_wgrad_o1_kernel(const NetL
     for (int t = blockIdx.x; t < total; t += gridDim.x, ++k) {
         const int b = t / ntiles, y = (t - b * ntiles) * NTC_TS + sl;
         if (k >= 1 && !wait_failed) wait_failed = !tc::mbar_wait(mma_bar, (k - 1) & 1, a.wait_ns);
-        // A: the input channels grp, grp + 4, ... at the site, untransported
-        for (int ci = grp; ci < a.cin; ci += G4) {
-            float p[24];
-            load_act(a.in, a.in_bf16, a.V, a.cin, b, ci, y < a.V ? y : -1, p);
-#pragma unroll
-            for (int ca = 0; ca < 3; ++ca) {
-                uint32_t w[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) w[r] = pack_bf16x2(p[2 * (3 * r + ca)], p[2 * (3 * r + ca) + 1]);
-                *reinterpret_cast<uint4*>(Xs + ca * blkx + (sl >> 3) * sbox + ci * 128 + rowoff) =
-                    make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        }
+        // A: the input channels grp, grp + 4, ... at the site, untransported;
         // B: the output gradient brought to the site by the adjoint of hops grp, grp + 4, grp + 8
-        for (int h = grp; h < 9; h += G4) {
-            float u[18], p[24];
-            float sign = 1.f;
-            int src = -1;
+        const float* act = gout + (size_t)b * a.V * 24;
+        const SiteCoords q(a, y);
+        auto put = [&](const HopFetch<RECON>& f, int h) {
+            uint32_t w[3][4];
+            f.finish(w);
 #pragma unroll
-            for (int q = 0; q < 18; ++q) u[q] = 0.f;  // padding sites: zero link, zero input
-            if (y < a.V) {
-                if (h > 0) {
-                    src = hop_link<RECON>(a, y, adj_hop(h), u, sign);
-#pragma unroll
-                    for (int q = 0; q < 18; ++q) u[q] = sign * u[q];
-                } else {
-                    src = y;
-                }
-            }
-            load_act(gout, a.gout_bf16, a.V, 1, b, 0, src, p);
-#pragma unroll
-            for (int ca = 0; ca < 3; ++ca) {
-                uint32_t w[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    float re, im;
-                    if (h == 0) {
-                        re = p[2 * (3 * r + ca)];
-                        im = p[2 * (3 * r + ca) + 1];
-                    } else {
-                        re = 0.f;
-                        im = 0.f;
-#pragma unroll
-                        for (int cb = 0; cb < 3; ++cb) {  // one multiply-add per real product
-                            const float ur = u[2 * (3 * ca + cb)], ui = u[2 * (3 * ca + cb) + 1];
-                            const float pr = p[2 * (3 * r + cb)], pi = p[2 * (3 * r + cb) + 1];
-                            re += ur * pr;
-                            re -= ui * pi;
-                            im += ur * pi;
-                            im += ui * pr;
-                        }
-                    }
-                    w[r] = pack_bf16x2(re, im);
-                }
+            for (int ca = 0; ca < 3; ++ca)
                 *reinterpret_cast<uint4*>(Gs + ca * blkg + (sl >> 3) * sbog + h * 128 + rowoff) =
-                    make_uint4(w[0], w[1], w[2], w[3]);
+                    make_uint4(w[ca][0], w[ca][1], w[ca][2], w[ca][3]);
+        };
+        HopFetch<RECON> f0, f1;
+        if (a.in_bf16) {
+            put_channels<G4>(a, a.in, a.cin, b, y < a.V ? y : -1, grp, Xs + (sl >> 3) * sbox + rowoff, blkx, [&]() {
+                f0.fetch(a, act, y, q.c0, q.c1, q.c2, q.c3, y < a.V, adj_hop(grp));
+            });
+        } else {  // a layer from one channel to one: the input is FP32
+            if (grp == 0) {
+                float p[24];
+                load_channel(a.in + (size_t)b * a.V * 24, a.V, 0, y < a.V ? y : -1, p);
+#pragma unroll
+                for (int ca = 0; ca < 3; ++ca) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) w[r] = pack_bf16x2(p[2 * (3 * r + ca)], p[2 * (3 * r + ca) + 1]);
+                    *reinterpret_cast<uint4*>(Xs + ca * blkx + (sl >> 3) * sbox + rowoff) = make_uint4(w[0], w[1], w[2], w[3]);
+                }
             }
+            f0.fetch(a, act, y, q.c0, q.c1, q.c2, q.c3, y < a.V, adj_hop(grp));
         }
+        f1.fetch(a, act, y, q.c0, q.c1, q.c2, q.c3, y < a.V, adj_hop(grp + 4));
+        put(f0, grp);
+        if (grp == 0) f0.fetch(a, act, y, q.c0, q.c1, q.c2, q.c3, y < a.V, adj_hop(8));
+        put(f1, grp + 4);
+        if (grp == 0) put(f0, 8);
         tc::fence_proxy_async();
         if (__syncthreads_or(wait_failed)) {
             failed = true;

@@ -352,3 +352,41 @@ def test_gauge_load_sources(lq, recon):
     lat.unpack(got, outs[0][0], 0, "f64")
     lat.sync()
     assert rel(got.cpu().numpy(), hop_ref(U, psi.cpu().numpy(), dims, 0)) < 1e-13
+
+
+@pytest.mark.parametrize("channels", [(1, 1), (1, 2, 1), (1, 12, 12, 1), (1, 11, 5, 1)])
+@pytest.mark.parametrize("dims,batch,recon", [((2, 2, 2, 2), 1, 12), ((4, 4, 6, 6), 3, 18), ((4, 2, 6, 10), 2, 12)])
+def test_network_kernels_by_shape(lq, channels, dims, batch, recon):
+    """The BF16 network's layers, adjoints and weight gradients against the
+    FP32 network's, for every kernel that a shape selects (one input channel,
+    one output channel, both, neither; odd channel counts) and lattices with a
+    ragged last tile.  BF16 operands, and activations between layers, have unit
+    roundoff 2^-9; sums are FP32: 5e-3 of the norm, as for single layers."""
+    import torch
+    lat = lq.Lattice(dims, precisions=("f64", "f32"), recon=recon)
+    lat.gauge_load(on_device(synth.gauge_field(dims, "smooth", 51, eps=0.5)))
+    rng = np.random.default_rng(52)
+    nets = [lq.Net(lat, channels, bf16=bf, max_batch=batch) for bf in (True, False)]
+    w = (rng.standard_normal(nets[0].num_weights) + 1j * rng.standard_normal(nets[0].num_weights)).astype(np.complex64)
+    for n in nets:
+        n.set_weights(w)
+
+    def act(ch):
+        shape = (batch, dims[3], dims[2], dims[1], dims[0], ch, 4, 3)
+        return on_device((rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64))
+
+    at = 0
+    for l, (cin, cout) in enumerate(zip(channels, channels[1:])):
+        x, g = act(cin), act(cout)
+        size = 9 * 16 * cin * cout
+        res = []
+        for n in nets:
+            y, z = torch.empty_like(g), torch.empty_like(x)
+            n.layer_apply(l, y, x, batch)
+            n.layer_apply(l, z, g, batch, adjoint=True)
+            n.layer_wgrad(l, x, g, batch)
+            lat.sync()
+            res.append((y.cpu().numpy(), z.cpu().numpy(), n.get_weights(grad=True)[1][at:at + size].numpy()))
+        for got, want in zip(*res):
+            assert rel(got, want) < 5e-3, (l, cin, cout)
+        at += size
