@@ -672,6 +672,7 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_layer_tc_kernel(const NetL
     __syncthreads();
     tc::fence_after();
     const uint32_t tmem = *tslot;
+    pdl_wait();  // (shared memory keeps a predecessor of this kind off this SM, so the allocation did not wait for it)
 
     const int ntiles = (a.V + NTC_TS - 1) / NTC_TS;
     const int total = ntiles * a.batch;
@@ -827,6 +828,7 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_layer_tc_kernel(const NetL
         tc::fence_before();
         __syncthreads();  // tensor memory read before the next tile's first MMA overwrites it
     }
+    pdl_start_next();
     if (failed) {  // bounded waits for this CTA's own operations in flight, then free the tensor memory
         if (copies > 0) {
             const uint32_t gc = (uint32_t)copies - 1;
@@ -874,17 +876,18 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_layer_c1_kernel(const NetL
     // B[n2][8 h + k] = B_h[n2][k] for the 8 real K of each hop (K2p = 16)
     for (uint32_t e = tid; e < 2 * xbytes / 16; e += NTC_THREADS)
         reinterpret_cast<uint4*>(smem)[e] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) {
+        tc::mbar_init(&mma_bar[0], 1);
+        tc::mbar_init(&mma_bar[1], 1);
+    }
+    if (warp == 0) tc::tmem_alloc(tslot, ncols);
+    pdl_wait();
     for (int e = tid; e < NC1_KG * N2p; e += NTC_THREADS) {
         const int h = e / N2p, n2 = e - h * N2p;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         if (h < 9) v = *reinterpret_cast<const uint4*>(a.Bh + (size_t)h * N2p * 16 + (n2 / 8) * 128 + (n2 % 8) * 8);
         *reinterpret_cast<uint4*>(Bs + ((size_t)(n2 / 8) * NC1_KG * 64 + h * 64 + (n2 % 8) * 8) * 2) = v;
     }
-    if (tid == 0) {
-        tc::mbar_init(&mma_bar[0], 1);
-        tc::mbar_init(&mma_bar[1], 1);
-    }
-    if (warp == 0) tc::tmem_alloc(tslot, ncols);
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -989,6 +992,7 @@ __global__ void __launch_bounds__(NTC_THREADS, 1) net_layer_c1_kernel(const NetL
             }
         }
     }
+    pdl_start_next();
     if (failed) {  // bounded wait for the MMAs of tile k (issued, not seen complete), then free the tensor memory
         tc::mbar_wait(&mma_bar[k & 1], (k >> 1) & 1u, NTC_WAIT_NS);
         if (tid == 0) atomicOr(a.errw, ERRW_TIMEOUT);
@@ -1628,6 +1632,7 @@ template <int RECON>
 __global__ void __launch_bounds__(128) net_gather_transport_kernel(const NetLayerArgs a, const void* z, float* out)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
+    pdl_wait();
     if (x >= a.V) return;
     float acc[24];
     load_act(z, 1, a.V, 9, b, 0, x, acc);
@@ -1657,6 +1662,7 @@ __global__ void __launch_bounds__(128) net_gather_transport_kernel(const NetLaye
     float4* o = reinterpret_cast<float4*>(out) + (size_t)b * a.V * 6;
 #pragma unroll
     for (int q = 0; q < 6; ++q) o[plane4(a.V, 0, q) + x] = make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+    pdl_start_next();
 }
 
 // Canonical complex spinor (Cin = 1 activation) <-> internal FP32 full field.
@@ -1664,6 +1670,7 @@ __global__ void net_from_internal_kernel(Geom g, const char* in, size_t in_rb, f
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int par = blockIdx.y % 2, b = blockIdx.y / 2;
+    pdl_wait();
     if (i >= g.Vh || b >= nb) return;
     int c[4];
     cb_coords(g, i, par, c);
@@ -1673,12 +1680,14 @@ __global__ void net_from_internal_kernel(Geom g, const char* in, size_t in_rb, f
     float4* dst = reinterpret_cast<float4*>(act) + (size_t)b * V * 6 + full_index(g, c);
 #pragma unroll
     for (int k = 0; k < 6; ++k) dst[(size_t)k * V] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+    pdl_start_next();
 }
 
 __global__ void net_to_internal_kernel(Geom g, char* out, size_t out_rb, const float* act, int nb)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int par = blockIdx.y % 2, b = blockIdx.y / 2;
+    pdl_wait();
     if (i >= g.Vh || b >= nb) return;
     int c[4];
     cb_coords(g, i, par, c);
@@ -1691,6 +1700,7 @@ __global__ void net_to_internal_kernel(Geom g, char* out, size_t out_rb, const f
         v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
     }
     SpinorIO<P32>::store(out + b * out_rb + par * spinor_field_bytes(P32, g.stride), g.stride, i, v);
+    pdl_start_next();
 }
 
 // Canonical [b][site][ch][4][3] complex <-> planar activations of nb batch
@@ -1698,6 +1708,7 @@ __global__ void net_to_internal_kernel(Geom g, char* out, size_t out_rb, const f
 // order, so the planar side is coalesced.
 __global__ void net_layout_kernel(const float4* src, float4* dst, int V, int ch, int nb, int to_planar)
 {
+    pdl_wait();
     const size_t per = (size_t)V * ch * 6, total = per * nb;
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
         const size_t b = e / per, r = e - b * per;
@@ -1706,12 +1717,14 @@ __global__ void net_layout_kernel(const float4* src, float4* dst, int V, int ch,
         if (to_planar) dst[e] = src[can];
         else dst[can] = src[e];
     }
+    pdl_start_next();
 }
 
 // Canonical FP32 <-> BF16 planar: plane q of channel c holds complex 4q .. 4q+3
 // (two canonical float4) of every site, as eight BF16 values.
 __global__ void net_layout_bf16_kernel(const void* src, void* dst, int V, int ch, int nb, int to_planar)
 {
+    pdl_wait();
     const size_t per = (size_t)V * ch * 3, total = per * nb;
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
         const size_t b = e / per, r = e - b * per;
@@ -1731,6 +1744,7 @@ __global__ void net_layout_bf16_kernel(const void* src, void* dst, int V, int ch
                                       __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xffff0000u));
         }
     }
+    pdl_start_next();
 }
 
 // Running sum in two FP32 words (value hi + lo), good to about 2^-46: FP64
@@ -1993,24 +2007,24 @@ lqcd_status run_layer(lqcd_net* n, const NetLayerArgs& a0, int batch, int prof_i
             const size_t sm1 = (size_t)2 * 3 * NTC_TS * NC1_K * 2 + (size_t)t.N2p * NC1_K * 2 + 2 * 8 + 16;
             if (c->cfg.recon == 12) {
                 LQ_CUDA(cudaFuncSetAttribute(net_layer_c1_kernel<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
-                net_layer_c1_kernel<12><<<grid, NTC_THREADS, sm1, c->stream>>>(t);
+                LQ_CUDA(launch_dependent(net_layer_c1_kernel<12>, false, dim3(grid), dim3(NTC_THREADS), c->stream, sm1, t));
             } else {
                 LQ_CUDA(cudaFuncSetAttribute(net_layer_c1_kernel<18>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
-                net_layer_c1_kernel<18><<<grid, NTC_THREADS, sm1, c->stream>>>(t);
+                LQ_CUDA(launch_dependent(net_layer_c1_kernel<18>, false, dim3(grid), dim3(NTC_THREADS), c->stream, sm1, t));
             }
         } else if (c->cfg.recon == 12) {
             LQ_CUDA(cudaFuncSetAttribute(net_layer_tc_kernel<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-            net_layer_tc_kernel<12><<<grid, NTC_THREADS, sm, c->stream>>>(t);
+            LQ_CUDA(launch_dependent(net_layer_tc_kernel<12>, false, dim3(grid), dim3(NTC_THREADS), c->stream, sm, t));
         } else {
             LQ_CUDA(cudaFuncSetAttribute(net_layer_tc_kernel<18>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-            net_layer_tc_kernel<18><<<grid, NTC_THREADS, sm, c->stream>>>(t);
+            LQ_CUDA(launch_dependent(net_layer_tc_kernel<18>, false, dim3(grid), dim3(NTC_THREADS), c->stream, sm, t));
         }
         if (stack) {  // then the transport of the four colour vectors per hop
             LQ_CUDA(cudaGetLastError());
             c->launches++;
             dim3 g2((a.V + 127) / 128, batch);
-            if (c->cfg.recon == 12) net_gather_transport_kernel<12><<<g2, 128, 0, c->stream>>>(a, n->zbuf, a.out);
-            else net_gather_transport_kernel<18><<<g2, 128, 0, c->stream>>>(a, n->zbuf, a.out);
+            const auto gather = c->cfg.recon == 12 ? net_gather_transport_kernel<12> : net_gather_transport_kernel<18>;
+            LQ_CUDA(launch_dependent(gather, false, g2, dim3(128), c->stream, 0, a, n->zbuf, a.out));
         }
     } else {
         const size_t sm = layer_smem_f32(a);
@@ -2059,10 +2073,12 @@ lqcd_status convert_layout(lqcd_net* n, const float* src, float* dst, int ch, in
     const size_t total = (size_t)V * ch * 6 * batch;
     const int grid = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
     if (n->bf16 && ch > 1)
-        net_layout_bf16_kernel<<<grid, 256, 0, c->stream>>>(src, dst, V, ch, batch, to_planar ? 1 : 0);
+        LQ_CUDA(launch_dependent(net_layout_bf16_kernel, false, dim3(grid), dim3(256), c->stream, 0, src, dst, V, ch, batch,
+                                 to_planar ? 1 : 0));
     else
-        net_layout_kernel<<<grid, 256, 0, c->stream>>>(reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst),
-                                                       V, ch, batch, to_planar ? 1 : 0);
+        LQ_CUDA(launch_dependent(net_layout_kernel, false, dim3(grid), dim3(256), c->stream, 0,
+                                 reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst), V, ch, batch,
+                                 to_planar ? 1 : 0));
     LQ_CUDA(cudaGetLastError());
     c->launches++;
     return LQCD_OK;
@@ -2199,10 +2215,12 @@ lqcd_status net_apply_internal(lqcd_net* n, void* z, const void* r, size_t rb)
 {
     lqcd_ctx* c = n->ctx;
     dim3 grid((c->g.Vh + 127) / 128, 2);
-    net_from_internal_kernel<<<grid, 128, 0, c->stream>>>(c->g, static_cast<const char*>(r), rb, n->act[0], 0, 1);
+    LQ_CUDA(launch_dependent(net_from_internal_kernel, false, grid, dim3(128), c->stream, 0, c->g,
+                             static_cast<const char*>(r), rb, n->act[0], 0, 1));
     LQ_CUDA(cudaGetLastError());
     LQ_TRY(net_forward_all(n, 1));
-    net_to_internal_kernel<<<grid, 128, 0, c->stream>>>(c->g, static_cast<char*>(z), rb, n->act[n->nlayers], 1);
+    LQ_CUDA(launch_dependent(net_to_internal_kernel, false, grid, dim3(128), c->stream, 0, c->g, static_cast<char*>(z), rb,
+                             n->act[n->nlayers], 1));
     LQ_CUDA(cudaGetLastError());
     c->launches += 2;
     return LQCD_OK;
