@@ -643,56 +643,89 @@ __device__ __forceinline__ void clover_apply_site(const void* base, int stride, 
 // block to finish (atomic ticket) adds the partials in block order.  The
 // result never depends on scheduling.
 
+// Sums of v[0 .. NV) over the warp, NV a power of two, to out[0 .. NV).  A
+// step of the tree adds lane pairs 16, 8, 4, .. apart; while more than one
+// value is left, the two lanes of a pair take half of the values each, so
+// that a lane does NV - 1 + 5 - log2(NV) FP64 additions instead of 5 NV, in
+// the same order (8 values: 9 for 40).  FP64 additions bound these
+// reductions: a warp's addition holds the SM's FP64 pipe for 16 cycles.
+template <int NV>
+__device__ __forceinline__ void warp_sums(double (&v)[NV], int lane, double* out)
+{
+    static_assert(NV >= 1 && NV <= 32 && (NV & (NV - 1)) == 0, "a power of two");
+    int o = 16, k = 0;
+#pragma unroll
+    for (int n = NV / 2; n > 0; n >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int j = 0; j < n; ++j) {
+            const double give = up ? v[j] : v[j + n], keep = up ? v[j + n] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+        if (up) k += n;
+    }
+    const int writers = o;  // 2 o lanes hold the same value
+#pragma unroll
+    for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    if ((lane & (2 * writers - 1)) == 0) out[k] = v[0];
+}
+
+// The same for any NV, in power-of-two parts.
+template <int NV, int OFF = 0>
+__device__ __forceinline__ void warp_sums_any(const double (&v)[NV], int lane, double* out)
+{
+    if constexpr (OFF < NV) {
+        constexpr int left = NV - OFF;
+        constexpr int n = left >= 16 ? 16 : left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
+        double part[n];
+#pragma unroll
+        for (int j = 0; j < n; ++j) part[j] = v[OFF + j];
+        warp_sums<n>(part, lane, out + OFF);
+        warp_sums_any<NV, OFF + n>(v, lane, out);
+    }
+}
+
 // Block bidx of the nblk blocks that reduce into `result`.
 template <int NV>
 __device__ __forceinline__ void block_reduce_finalize(double (&v)[NV], double* partials, unsigned* ticket,
                                                       double* result, int bidx, int nblk)
 {
+    static_assert(NV <= 32, "one lane of the first warp per value");
     __shared__ double sm[32][NV];
     __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nwarps = (blockDim.x + 31) >> 5;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        double x = v[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (lane == 0) sm[warp][k] = x;
-    }
+    warp_sums_any<NV>(v, lane, sm[warp]);
     __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
+    if (warp == 0) {
+        if (lane < NV) {
             double s = 0.0;
-            for (int w = 0; w < nwarps; ++w) s += sm[w][k];
-            partials[(size_t)bidx * NV + k] = s;
+            for (int w = 0; w < nwarps; ++w) s += sm[w][lane];
+            partials[(size_t)bidx * NV + lane] = s;
+            __threadfence();
         }
-        __threadfence();
-        const unsigned t = atomicAdd(ticket, 1u);
-        last = (t == (unsigned)nblk - 1);
+        __syncwarp();
+        if (lane == 0) last = (atomicAdd(ticket, 1u) == (unsigned)nblk - 1);
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
     const volatile double* vp = partials;
+    double x[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        double x = 0.0;
-        for (int b = threadIdx.x; b < nblk; b += blockDim.x) x += vp[(size_t)b * NV + k];
+    for (int k = 0; k < NV; ++k) x[k] = 0.0;
+    for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (lane == 0) sm[warp][k] = x;
+        for (int k = 0; k < NV; ++k) x[k] += vp[(size_t)b * NV + k];
     }
+    warp_sums_any<NV>(x, lane, sm[warp]);
     __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            double s = 0.0;
-            for (int w = 0; w < nwarps; ++w) s += sm[w][k];
-            result[k] = s;
-        }
-        *ticket = 0u;  // ready for the next launch on this slot
+    if (threadIdx.x < NV) {
+        double s = 0.0;
+        for (int w = 0; w < nwarps; ++w) s += sm[w][threadIdx.x];
+        result[threadIdx.x] = s;
     }
+    if (threadIdx.x == 0) *ticket = 0u;  // ready for the next launch on this slot
 }
 
 template <int NV>

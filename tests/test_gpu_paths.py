@@ -390,3 +390,41 @@ def test_network_kernels_by_shape(lq, channels, dims, batch, recon):
         for got, want in zip(*res):
             assert rel(got, want) < 5e-3, (l, cin, cout)
         at += size
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 4, 10, 2), (8, 6, 4, 10)])
+@pytest.mark.parametrize("nkrylov,steps", [(1, 3), (4, 4), (5, 5), (9, 9), (24, 24), (4, 9)])
+def test_fgcr_steps(lq, dims, nkrylov, steps):
+    """The residual after a number of FGCR(nkrylov) steps against the smallest
+    one over each cycle's Krylov space (the dots run in chunks of four vectors
+    per parity).  The directions are FP32, each off by some 1e-7; 1e-5 of |b|
+    covers 24 of them."""
+    U = synth.gauge_field(dims, "smooth", 31, eps=0.5)
+    A = oracle.clover(U, 0.12, 1.0)
+    b = synth.gaussian_spinor(dims, 32)
+    r, left = b.reshape(-1), steps
+    while left:  # a cycle: min |r - M K y|, K = (r, M r, ..), by orthonormal vectors
+        n = min(left, nkrylov)
+        Q = np.zeros((n, r.size), complex)
+        v = r
+        for k in range(n):
+            v = oracle.wilson_clover(U, A, 0.12, v.reshape(b.shape)).reshape(-1)
+            for _ in range(2):
+                v = v - Q[:k].T @ (Q[:k].conj() @ v)
+            v = v / np.linalg.norm(v)
+            Q[k] = v
+        r = r - Q.T @ (Q.conj() @ r)
+        left -= n
+    want = np.linalg.norm(r) / np.linalg.norm(b)
+    lat = lq.Lattice(dims, precisions=("f64", "f32"), gcr_nkrylov=24)
+    lat.gauge_load(on_device(U))
+    lat.clover_compute(0.12, 1.0)
+    x = lat.canonical_spinor()
+    _, st = lat.solve(x, on_device(b), 1e-30, solver=lq.SOLVER_FGCR, inner_prec="f32", nkrylov=nkrylov,
+                      maxiter=steps, raise_on_error=False)
+    assert st["iterations"] <= steps
+    got = oracle.true_residual(U, A, 0.12, b, x.cpu().numpy())
+    if st["iterations"] == steps:
+        assert abs(got - want) <= 1e-5
+    else:  # a cycle ended early at FP32's resolution, and so did the exact one
+        assert got <= want + 1e-5
