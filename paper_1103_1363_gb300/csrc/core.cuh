@@ -685,9 +685,10 @@ __device__ __forceinline__ void warp_sums_any(const double (&v)[NV], int lane, d
     }
 }
 
-// Block bidx of the nblk blocks that reduce into `result`.
+// Block bidx of the nblk blocks that reduce into `result`; true in the block
+// that wrote it.
 template <int NV>
-__device__ __forceinline__ void block_reduce_finalize(double (&v)[NV], double* partials, unsigned* ticket,
+__device__ __forceinline__ bool block_reduce_finalize(double (&v)[NV], double* partials, unsigned* ticket,
                                                       double* result, int bidx, int nblk)
 {
     static_assert(NV <= 32, "one lane of the first warp per value");
@@ -708,7 +709,7 @@ __device__ __forceinline__ void block_reduce_finalize(double (&v)[NV], double* p
         if (lane == 0) last = (atomicAdd(ticket, 1u) == (unsigned)nblk - 1);
     }
     __syncthreads();
-    if (!last) return;
+    if (!last) return false;
     __threadfence();
     const volatile double* vp = partials;
     double x[NV];
@@ -726,13 +727,14 @@ __device__ __forceinline__ void block_reduce_finalize(double (&v)[NV], double* p
         result[threadIdx.x] = s;
     }
     if (threadIdx.x == 0) *ticket = 0u;  // ready for the next launch on this slot
+    return true;
 }
 
 template <int NV>
-__device__ __forceinline__ void block_reduce_finalize(double (&v)[NV], double* partials, unsigned* ticket,
+__device__ __forceinline__ bool block_reduce_finalize(double (&v)[NV], double* partials, unsigned* ticket,
                                                       double* result)
 {
-    block_reduce_finalize<NV>(v, partials, ticket, result, (int)blockIdx.x, (int)gridDim.x);
+    return block_reduce_finalize<NV>(v, partials, ticket, result, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // --------------------------------------------------------------- geometry

@@ -8,8 +8,8 @@
 // residual is recomputed in double precision at each restart (Sec. 5).
 //
 // Here w_k is orthogonalised against the earlier w_j by classical
-// Gram-Schmidt: one kernel forms <w_j, w_k>, <w_k, r> and |w_k|^2, the host
-// forms c_j = <w_j, w_k>/|w_j|^2 and the step a = <w_k, r>/|w^_k|^2 with
+// Gram-Schmidt: one kernel forms <w_j, w_k>, <w_k, r> and |w_k|^2 and from
+// them c_j = <w_j, w_k>/|w_j|^2 and the step a = <w_k, r>/|w^_k|^2 with
 // |w^_k|^2 = |w_k|^2 - sum_j |<w_j, w_k>|^2/|w_j|^2, and one fused kernel
 // writes w^_k = w_k - sum_j c_j w_j and r -= a w^_k.  When that estimate
 // shows cancellation (|w^_k|^2 < |w_k|^2 / 2, the "twice is enough"
@@ -41,6 +41,7 @@ lqcd_status net_apply_internal(lqcd_net* n, void* z, const void* r, size_t rb);
 
 enum { GCR_KMAX = 24, GCR_NDOT = 2 * GCR_KMAX + 8 };  // the last chunk writes 8 values at 2 GCR_KMAX
 constexpr double GCR_CYCLE_REDUCTION = 1e-5;
+constexpr size_t GCR_RECORD_BYTES = 2048;
 
 // out[2j, 2j+1] = <w_j, w_k> (j < k), out[2 KMAX, 2 KMAX + 1] = <w_k, r>,
 // out[2 KMAX + 2] = |w_k|^2.  The dots are split over blockIdx.y in chunks
@@ -54,9 +55,50 @@ constexpr double GCR_CYCLE_REDUCTION = 1e-5;
 // now 4.20.
 enum { GCR_CH = 4 };
 
-__global__ void gcr_dots_kernel(Geom g, const char* W, size_t fld, int k, const char* wk, const char* r,
-                                double* partials, unsigned* tickets, double* out)
+// Device record of a solve's recursion, read back once per Gram-Schmidt pass.
+// (The step was formed on the host between the two kernels before: a second
+// copy and wait per pass; a 16^4 solve with SAP took 4.20 ms, now 4.07.)
+enum { GCR_USE = 0, GCR_AGAIN = 1, GCR_STOP = 2 };  // what the update does: full, projection only, nothing
+
+struct GcrRecord {
+    double dots[GCR_NDOT];      // of the last dots kernel
+    double ar, ai;              // the step a
+    double rw[2 * GCR_KMAX];    // |r|^2 and |w^_k|^2 after the update of direction k
+    int status, pad;
+    float2 c[GCR_KMAX], a;      // as the update applies them
+};
+
+// c_j, a and the status from the dots, by one warp.  `first` is |w_k|^2 before
+// the first pass (negative in that pass).
+__device__ void gcr_step(GcrRecord* rec, int k, double first)
 {
+    const int lane = threadIdx.x & 31;
+    const volatile double* dots = rec->dots;
+    double share = 0.0;
+    if (lane < k) {
+        const double re = dots[2 * lane], im = dots[2 * lane + 1], wn = rec->rw[2 * lane + 1];
+        rec->c[lane] = make_float2((float)(re / wn), (float)(im / wn));
+        share = (re * re + im * im) / wn;
+    }
+    const double ww = dots[2 * GCR_KMAX + 2], ww0 = first < 0.0 ? ww : first;
+    double what2 = ww;
+    for (int j = 0; j < k; ++j) what2 -= __shfl_sync(0xffffffffu, share, j);
+    if (lane != 0) return;
+    // nothing new in w_k (also catches NaN): do not use it
+    if (!(what2 > 1e-10 * ww0) || !isfinite(ww)) {
+        rec->status = GCR_STOP;
+        return;
+    }
+    rec->status = first < 0.0 && k > 0 && what2 < 0.5 * ww ? GCR_AGAIN : GCR_USE;
+    rec->ar = dots[2 * GCR_KMAX] / what2;
+    rec->ai = dots[2 * GCR_KMAX + 1] / what2;
+    rec->a = make_float2((float)rec->ar, (float)rec->ai);
+}
+
+__global__ void gcr_dots_kernel(Geom g, const char* W, size_t fld, int k, const char* wk, const char* r,
+                                double* partials, unsigned* tickets, GcrRecord* rec, double first)
+{
+    double* out = rec->dots;
     const int c = blockIdx.y, nch_j = (k + GCR_CH - 1) / GCR_CH;
     const bool with_r = c == nch_j;
     const int j0 = c * GCR_CH, cnt = with_r ? 0 : min(GCR_CH, k - j0);
@@ -102,20 +144,36 @@ __global__ void gcr_dots_kernel(Geom g, const char* W, size_t fld, int k, const 
 #pragma unroll
     for (int j = 0; j < 2 * GCR_CH; ++j) d[j] = acc[j];
     const int nblk = 2 * gridDim.x;
-    block_reduce_finalize<2 * GCR_CH>(d, partials + (size_t)c * nblk * 2 * GCR_CH, tickets + c,
-                                      out + (with_r ? 2 * GCR_KMAX : 2 * j0), par * gridDim.x + blockIdx.x, nblk);
+    if (!block_reduce_finalize<2 * GCR_CH>(d, partials + (size_t)c * nblk * 2 * GCR_CH, tickets + c,
+                                           out + (with_r ? 2 * GCR_KMAX : 2 * j0), par * gridDim.x + blockIdx.x, nblk))
+        return;
+    // the chunk that is done last forms the step
+    __shared__ bool all;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned* t = tickets + GCR_KMAX;
+        all = atomicAdd(t, 1u) == gridDim.y - 1;
+        if (all) *t = 0u;
+    }
+    __syncthreads();
+    if (!all || threadIdx.x >= 32) return;
+    __threadfence();
+    gcr_step(rec, k, first);
 }
 
-struct GcrStep {
-    float2 c[GCR_KMAX];  // w_k -= sum_j c_j w_j
-    float2 a;            // r -= a w_k (after the projection)
-    int update_r;
-};
-
-// w_k -= sum_j c_j w_j; if update_r: r -= a w_k.  out[0] = |r|^2, out[1] = |w_k|^2.
-__global__ void gcr_orth_update_kernel(Geom g, const char* W, size_t fld, int k, char* wk, char* r, GcrStep st,
-                                       double* partials, unsigned* ticket, double* out)
+// w_k -= sum_j c_j w_j and, unless a second pass follows, r -= a w_k.
+// rec->rw[2k] = |r|^2 (0 without the r update), rec->rw[2k + 1] = |w_k|^2.
+__global__ void gcr_orth_update_kernel(Geom g, const char* W, size_t fld, int k, char* wk, char* r, GcrRecord* rec,
+                                       double* partials, unsigned* ticket)
 {
+    __shared__ float2 cj[GCR_KMAX];
+    const int status = rec->status;
+    if (status == GCR_STOP) return;  // uniform over the grid
+    const bool update_r = status == GCR_USE;
+    const float2 step = rec->a;
+    if (threadIdx.x < k) cj[threadIdx.x] = rec->c[threadIdx.x];
+    __syncthreads();
     // blockIdx.y = (parity, float4 chunk), a thread per site: the update is
     // elementwise, so six threads share a site, each running the chain of k
     // loads for its chunk (six times the loads in flight of a thread per site)
@@ -128,7 +186,7 @@ __global__ void gcr_orth_update_kernel(Geom g, const char* W, size_t fld, int k,
 #pragma unroll 4
         for (int j = 0; j < k; ++j) {
             const float4 w = __ldg(reinterpret_cast<const float4*>(W + j * fld + off));
-            const float xr = st.c[j].x, xi = st.c[j].y;
+            const float xr = cj[j].x, xi = cj[j].y;
             a.x -= xr * w.x - xi * w.y;
             a.y -= xr * w.y + xi * w.x;
             a.z -= xr * w.z - xi * w.w;
@@ -137,20 +195,22 @@ __global__ void gcr_orth_update_kernel(Geom g, const char* W, size_t fld, int k,
         if (k > 0) *reinterpret_cast<float4*>(wk + off) = a;
         const float nw = a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
         float nr = 0.f;
-        if (st.update_r) {
+        if (update_r) {
             float4 rv = *reinterpret_cast<const float4*>(r + off);
-            rv.x -= st.a.x * a.x - st.a.y * a.y;
-            rv.y -= st.a.x * a.y + st.a.y * a.x;
-            rv.z -= st.a.x * a.z - st.a.y * a.w;
-            rv.w -= st.a.x * a.w + st.a.y * a.z;
+            rv.x -= step.x * a.x - step.y * a.y;
+            rv.y -= step.x * a.y + step.y * a.x;
+            rv.z -= step.x * a.z - step.y * a.w;
+            rv.w -= step.x * a.w + step.y * a.z;
             *reinterpret_cast<float4*>(r + off) = rv;
             nr = rv.x * rv.x + rv.y * rv.y + rv.z * rv.z + rv.w * rv.w;
         }
         acc[0] += nr;
         acc[1] += nw;
     }
-    block_reduce_finalize<2>(acc, partials, ticket, out, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+    block_reduce_finalize<2>(acc, partials, ticket, rec->rw + 2 * k, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
 }
+
+static_assert(sizeof(GcrRecord) <= GCR_RECORD_BYTES, "the record fits before the tickets");
 
 struct GcrCombine {
     float2 beta[GCR_KMAX];
@@ -210,10 +270,9 @@ lqcd_status solve_fgcr(lqcd_ctx* c, lqcd_net* net, double* x, const double* b, d
     char* Wb = Zb + (size_t)K * fld;
     char* R32 = Wb + (size_t)K * fld;
     char* X32 = R32 + fld;
-    double* dev = reinterpret_cast<double*>(X32 + fld);  // scalars of the recursion
-    double* dots = dev;                                    // [GCR_NDOT]
-    double* upd = dev + 64;                                // [2]
-    unsigned* tick = reinterpret_cast<unsigned*>(upd + 4); // [0]: updates, [1 + c]: dot chunk c
+    GcrRecord* rec = reinterpret_cast<GcrRecord*>(X32 + fld);
+    unsigned* tick = reinterpret_cast<unsigned*>(X32 + fld + GCR_RECORD_BYTES);  // [0]: updates, [1 + c]: dot chunk c,
+                                                                               // [1 + KMAX]: chunks done
     double* parts = reinterpret_cast<double*>(reinterpret_cast<char*>(tick) + 256);
     const size_t canon_rb = (size_t)c->volume * 192;
 
@@ -248,25 +307,18 @@ lqcd_status solve_fgcr(lqcd_ctx* c, lqcd_net* net, double* x, const double* b, d
     lqcd_status status = LQCD_OK;
     typedef std::complex<double> cd;
     std::vector<cd> alpha(K), coef((size_t)K * K);  // coef[j * K + k] = c_jk
-    std::vector<double> wn(K);                       // |w^_j|^2
-    std::vector<double> hd(GCR_NDOT);
-    auto launch_dots = [&](int k, const char* wk) -> lqcd_status {
+    GcrRecord hrec;
+    // one Gram-Schmidt pass of w_k, up to the update that its status asks for
+    auto launch_pass = [&](int k, char* wk, double first) -> lqcd_status {
         const dim3 gd(grid.x, (k + GCR_CH - 1) / GCR_CH + 1, 2);
-        gcr_dots_kernel<<<gd, block, 0, c->stream>>>(c->g, Wb, fld, k, wk, R32, parts, tick + 1, dots);
+        gcr_dots_kernel<<<gd, block, 0, c->stream>>>(c->g, Wb, fld, k, wk, R32, parts, tick + 1, rec, first);
         LQ_CUDA(cudaGetLastError());
-        c->launches++;
-        return read(dots, hd.data(), GCR_NDOT);
-    };
-    auto launch_update = [&](int k, char* wk, const cd* cj, cd a, bool update_r, double out[2]) -> lqcd_status {
-        GcrStep st;
-        memset(&st, 0, sizeof st);
-        for (int j = 0; j < k; ++j) st.c[j] = make_float2((float)cj[j].real(), (float)cj[j].imag());
-        st.a = make_float2((float)a.real(), (float)a.imag());
-        st.update_r = update_r ? 1 : 0;
-        gcr_orth_update_kernel<<<gu, block, 0, c->stream>>>(c->g, Wb, fld, k, wk, R32, st, parts, tick, upd);
+        gcr_orth_update_kernel<<<gu, block, 0, c->stream>>>(c->g, Wb, fld, k, wk, R32, rec, parts, tick);
         LQ_CUDA(cudaGetLastError());
-        c->launches++;
-        return read(upd, out, 2);
+        c->launches += 2;
+        LQ_CUDA(cudaMemcpyAsync(&hrec, rec, sizeof hrec, cudaMemcpyDeviceToHost, c->stream));
+        LQ_CUDA(cudaStreamSynchronize(c->stream));
+        return LQCD_OK;
     };
     while (true) {
         // restart: r = b - M x in FP64; stop on the true residual
@@ -301,46 +353,27 @@ lqcd_status solve_fgcr(lqcd_ctx* c, lqcd_net* net, double* x, const double* b, d
             sap_ready = sap;
             LQ_TRY(op_full(c, wk, zk, mode, false, 1, fld));
             // classical Gram-Schmidt, a second pass when the first cancels
-            std::vector<cd> ck(k, cd(0.0, 0.0)), cj(k);
-            double out[2] = {0.0, 0.0};
-            cd a(0.0, 0.0);
-            double what2 = 0.0, ww0 = 0.0;
+            std::vector<cd> ck(k, cd(0.0, 0.0));
             bool used = false;
-            for (int pass = 0; pass < 2; ++pass) {
-                LQ_TRY(launch_dots(k, wk));
-                const double ww = hd[2 * GCR_KMAX + 2];
-                if (pass == 0) ww0 = ww;
-                what2 = ww;
-                for (int j = 0; j < k; ++j) {
-                    const cd d(hd[2 * j], hd[2 * j + 1]);
-                    cj[j] = d / wn[j];
-                    what2 -= std::norm(d) / wn[j];
-                }
-                const cd wr(hd[2 * GCR_KMAX], hd[2 * GCR_KMAX + 1]);
-                // nothing new in w_k (also catches NaN): do not use it
-                if (!(what2 > 1e-10 * ww0) || !std::isfinite(ww)) break;
-                for (int j = 0; j < k; ++j) ck[j] += cj[j];
-                if (pass == 0 && k > 0 && what2 < 0.5 * ww) {
-                    LQ_TRY(launch_update(k, wk, cj.data(), cd(0.0, 0.0), false, out));
-                    continue;
-                }
-                a = wr / what2;
-                LQ_TRY(launch_update(k, wk, cj.data(), a, true, out));
-                used = true;
-                break;
+            double first = -1.0;
+            for (int pass = 0; pass < 2 && !used; ++pass) {
+                LQ_TRY(launch_pass(k, wk, first));
+                if (hrec.status == GCR_STOP) break;
+                for (int j = 0; j < k; ++j) ck[j] += cd(hrec.dots[2 * j], hrec.dots[2 * j + 1]) / hrec.rw[2 * j + 1];
+                first = hrec.dots[2 * GCR_KMAX + 2];
+                used = hrec.status == GCR_USE;
             }
             if (!used) {
                 // w_k lies in the span of the earlier w_j: end the cycle without it
                 if (k == 0) status = LQCD_ERR_BREAKDOWN;
                 break;
             }
-            if (!std::isfinite(out[0])) { status = LQCD_ERR_BREAKDOWN; break; }
-            wn[k] = out[1];
-            alpha[k] = a;
+            const double r2 = hrec.rw[2 * k];
+            if (!std::isfinite(r2)) { status = LQCD_ERR_BREAKDOWN; break; }
+            alpha[k] = cd(hrec.ar, hrec.ai);
             for (int j = 0; j < k; ++j) coef[(size_t)j * K + k] = ck[j];
             m = k + 1;
             ++iters;
-            const double r2 = out[0];
             if (log) fprintf(stderr, "[lqcd] fgcr iter %d |r|/|b| %.3e\n", iters, std::sqrt(r2 / bn2));
             if (std::sqrt(r2 / bn2) <= 0.5 * tol) break;
             if (r2 <= GCR_CYCLE_REDUCTION * GCR_CYCLE_REDUCTION * r2_cycle) break;
