@@ -486,9 +486,9 @@ lqcd_status lqcd_sync(lqcd_ctx* ctx);
  * reduction) at 128, 96, 64 and 32 threads per block on this context's
  * lattice and keep, for each of the four classes, the fastest (a smaller
  * block must win by 2 %) for every later launch of that class.  128 is the
- * library's default: the gathering kernel with 128 threads per block, or, for
- * launches of few sites, a kernel with a warp per direction (same results).  For the
- * plain classes of the modes with FP32 links (LQCD_F32, LQCD_F16_SPINORS,
+ * library's default: the gathering kernel with 128 threads per block (plain
+ * FP64 launches: 32), or, for launches of few sites, a kernel with a warp per
+ * direction (same results).  For the plain classes of the modes with FP32 links (LQCD_F32, LQCD_F16_SPINORS,
  * LQCD_BF16_SPINORS) with recon-12 the candidates also include the
  * shared-memory staged kernel (LQCD_BLOCK_STAGED below), which must win by
  * 2 % as well.  Reducing

@@ -116,6 +116,14 @@ static bool wide_default(int mode, bool reducing, long sites)
     return sites <= (mode == P64 ? 8192 : reducing ? 12288 : 16384);
 }
 
+// FP64 launches without a sum run blocks of one warp: the FP64 pipe bounds
+// them, so the launch ends when the SM with the most sites does, and single
+// warps spread more evenly.  Schur operator in us, blocks of 128 -> 32: 12^4 2
+// rhs 161 -> 121, 16^4 163 -> 145, 24^4 2 rhs 1418 -> 1401, 16^3 x 32 322 ->
+// 322.  (The reducing launches are one wave of grid-stride blocks and lose 1 %
+// with four times the partial sums; FP32 and 16 bits are the same within 1 %.)
+enum { F64_BLOCK = 32 };
+
 lqcd_status launch_dslash(lqcd_ctx* c, const DslashArgs& A0, int P, bool dag, int epi, bool red, int nrhs)
 {
     DslashArgs A = A0;
@@ -125,6 +133,8 @@ lqcd_status launch_dslash(lqcd_ctx* c, const DslashArgs& A0, int P, bool dag, in
     const bool reducing = red || epi == EPI_CG;
     if (block == DSLASH_MAX_BLOCK && A.sites_per_thread == 0 && wide_default(P, reducing, (long)c->g.Vh * nrhs + own_capture.other_sites))
         block = DSLASH_WIDE;
+    else if (block == DSLASH_MAX_BLOCK && P == P64 && !reducing)
+        block = F64_BLOCK;
     const int rc = c->recon_of(mode_pg(P));
     Profiler* pr = c->prof;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
