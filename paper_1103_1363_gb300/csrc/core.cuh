@@ -711,13 +711,13 @@ __device__ __forceinline__ bool block_reduce_finalize(double (&v)[NV], double* p
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    const volatile double* vp = partials;
     double x[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k) x[k] = 0.0;
+#pragma unroll 4
     for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
 #pragma unroll
-        for (int k = 0; k < NV; ++k) x[k] += vp[(size_t)b * NV + k];
+        for (int k = 0; k < NV; ++k) x[k] += __ldcg(partials + (size_t)b * NV + k);
     }
     warp_sums_any<NV>(x, lane, sm[warp]);
     __syncthreads();

@@ -52,12 +52,12 @@ constexpr size_t GCR_RECORD_BYTES = 2048;
 // threads.  The vectors of a 16^4 solve are in L2, where FP64 additions and
 // too few blocks bound these kernels: with a block for both parities and 5
 // additions a value in the reduction, a 16^4 solve with SAP took 4.28 ms,
-// now 4.20.
+// without 4.20.
 enum { GCR_CH = 4 };
 
 // Device record of a solve's recursion, read back once per Gram-Schmidt pass.
 // (The step was formed on the host between the two kernels before: a second
-// copy and wait per pass; a 16^4 solve with SAP took 4.20 ms, now 4.07.)
+// copy and wait per pass; a 16^4 solve with SAP took 4.20 ms, without 4.07.)
 enum { GCR_USE = 0, GCR_AGAIN = 1, GCR_STOP = 2 };  // what the update does: full, projection only, nothing
 
 struct GcrRecord {
@@ -174,38 +174,48 @@ __global__ void gcr_orth_update_kernel(Geom g, const char* W, size_t fld, int k,
     const float2 step = rec->a;
     if (threadIdx.x < k) cj[threadIdx.x] = rec->c[threadIdx.x];
     __syncthreads();
-    // blockIdx.y = (parity, float4 chunk), a thread per site: the update is
-    // elementwise, so six threads share a site, each running the chain of k
-    // loads for its chunk (six times the loads in flight of a thread per site)
+    // blockIdx.y = (parity, q), a thread per site and chunks q and q + 3: the
+    // update is elementwise, so three threads share a site, each running two
+    // chains of k loads (16^4: one wave of 768 blocks, 15.8 us on average; 1536
+    // blocks of one chunk 20.5)
     double acc[2] = {0.0, 0.0};
     const size_t fb = fld / 2;
-    const int par = blockIdx.y / 6, q = blockIdx.y % 6;
+    const int par = blockIdx.y / 3, q = blockIdx.y % 3;
+    const size_t apart = (size_t)3 * g.stride * sizeof(float4);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.Vh; i += gridDim.x * blockDim.x) {
         const size_t off = par * fb + ((size_t)q * g.stride + i) * sizeof(float4);
-        float4 a = *reinterpret_cast<const float4*>(wk + off);
+        float4 a[2], rv[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            a[h] = *reinterpret_cast<const float4*>(wk + off + h * apart);
+            if (update_r) rv[h] = *reinterpret_cast<const float4*>(r + off + h * apart);
+        }
 #pragma unroll 4
         for (int j = 0; j < k; ++j) {
-            const float4 w = __ldg(reinterpret_cast<const float4*>(W + j * fld + off));
             const float xr = cj[j].x, xi = cj[j].y;
-            a.x -= xr * w.x - xi * w.y;
-            a.y -= xr * w.y + xi * w.x;
-            a.z -= xr * w.z - xi * w.w;
-            a.w -= xr * w.w + xi * w.z;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float4 w = __ldg(reinterpret_cast<const float4*>(W + j * fld + off + h * apart));
+                a[h].x -= xr * w.x - xi * w.y;
+                a[h].y -= xr * w.y + xi * w.x;
+                a[h].z -= xr * w.z - xi * w.w;
+                a[h].w -= xr * w.w + xi * w.z;
+            }
         }
-        if (k > 0) *reinterpret_cast<float4*>(wk + off) = a;
-        const float nw = a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
-        float nr = 0.f;
-        if (update_r) {
-            float4 rv = *reinterpret_cast<const float4*>(r + off);
-            rv.x -= step.x * a.x - step.y * a.y;
-            rv.y -= step.x * a.y + step.y * a.x;
-            rv.z -= step.x * a.z - step.y * a.w;
-            rv.w -= step.x * a.w + step.y * a.z;
-            *reinterpret_cast<float4*>(r + off) = rv;
-            nr = rv.x * rv.x + rv.y * rv.y + rv.z * rv.z + rv.w * rv.w;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 v = a[h];
+            if (k > 0) *reinterpret_cast<float4*>(wk + off + h * apart) = v;
+            acc[1] += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+            if (!update_r) continue;
+            float4 s = rv[h];
+            s.x -= step.x * v.x - step.y * v.y;
+            s.y -= step.x * v.y + step.y * v.x;
+            s.z -= step.x * v.z - step.y * v.w;
+            s.w -= step.x * v.w + step.y * v.z;
+            *reinterpret_cast<float4*>(r + off + h * apart) = s;
+            acc[0] += s.x * s.x + s.y * s.y + s.z * s.z + s.w * s.w;
         }
-        acc[0] += nr;
-        acc[1] += nw;
     }
     block_reduce_finalize<2>(acc, partials, ticket, rec->rw + 2 * k, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
 }
@@ -298,8 +308,8 @@ lqcd_status solve_fgcr(lqcd_ctx* c, lqcd_net* net, double* x, const double* b, d
     const double bn2 = h[SC_TMP + 0];
     const int block = 256;
     const dim3 grid(gcr_grid(c, block));
-    // the elementwise update: a block row per (parity, float4 chunk), about 10 blocks per SM
-    const dim3 gu(grid.x < 128 ? grid.x : 128, 12);
+    // the elementwise update: a block row per parity and pair of float4 chunks, at most 8 blocks per SM
+    const dim3 gu(grid.x < 8 * 152 / 6 ? grid.x : 8 * 152 / 6, 6);
     bool sap = !net && c->sap_on, sap_ready = false;
     if (sap) LQ_TRY(sap_check(c, c->sap_bs));
     int iters = 0, restarts = 0, fallback = 0;
