@@ -277,13 +277,13 @@ lqcd_status solve_batch(lqcd_ctx* const* ctxs, int n, double* const* x, const do
                         const lqcd_solver_params* p, lqcd_solver_stats* st);
 // fgcr.cu
 // sap.cu: z = SAP(r) on FP32 full internal fields; rho_buf and dlt_buf are
-// two FP32 full fields of scratch (block residuals and corrections); uses
-// veclo for the clover term in block order, which have_clover says an earlier
-// call with this block shape has left there (nothing else of a flexible solve
-// writes it)
+// two FP64 full fields of scratch (block residuals and z; corrections); uses
+// veclo for the links and the clover term in block order, which have_copies
+// says an earlier call with this block shape has left there (nothing else of
+// a flexible solve writes it)
 lqcd_status sap_check(const lqcd_ctx* c, const int bs[4]);
 lqcd_status sap_apply(lqcd_ctx* c, void* z, const void* r, const int bs[4], int ncycle, int nmr, char* rho_buf,
-                      char* dlt_buf, bool have_clover);
+                      char* dlt_buf, bool have_copies);
 lqcd_status solve_fgcr(lqcd_ctx* c, lqcd_net* net, double* x, const double* b, double tol,
                        const lqcd_solver_params* p, lqcd_solver_stats* st, bool host_io);
 // fgmres.cu

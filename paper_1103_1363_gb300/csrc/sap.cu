@@ -22,10 +22,11 @@
 //
 // Blocks of at most SAP_THREADS sites run one site per thread with q and
 // delta in registers, the block's links staged in shared memory once per
-// block solve and the clover term read from a copy in block order; larger
-// blocks (up to 1024 sites, e.g. the paper's 8x4x8x4) stride over the sites
-// with q in shared memory, delta accumulated in dlt and the links read
-// through L1/L2.
+// block solve; the links and the clover term are read from copies in block
+// order, and rho, delta and z are kept in block order between the launches.
+// Larger blocks (up to 1024 sites, e.g. the paper's 8x4x8x4) stride over the
+// sites with q in shared memory, delta accumulated in dlt and the links read
+// through L1/L2, all in the fields' order.
 #include <cmath>
 #include <cstring>
 
@@ -46,8 +47,14 @@ struct SapArgs {
     const void* gauge;  // FP32 links
     const char* clov;   // FP32 clover A, parity p at clov + p * clov_pb; nullptr: A = 1
     size_t clov_pb;
-    const float4* clovb;  // the clover term in block order (one thread per site)
     float kappa;
+    // one thread per site: arrays in block order, planes of vol sites
+    const float4* clovb;  // the clover term [block][18][vol]
+    const float4* linkb;  // the links, as a block's links lie in shared memory
+    float4* rhob;         // residual, correction and z [block][6][vol]
+    float4* dltb;
+    float4* zb;
+    int first, last;      // first cycle: rho from rho_in, z = delta; last: z to the field, rho not kept
     const char* rho_in; // residual on the solved sites before the neighbours' last correction
     char* rho_out;      // final block residual on the solved sites (may equal rho_in)
     char* dlt;          // corrections: read at other-colour sites, written at solved sites
@@ -318,18 +325,20 @@ template <> struct SmemLinks<18> {
 // One thread per site (blocks of at most SAP_THREADS sites): q and delta in
 // registers, the block's links staged in shared memory behind rho, two CTAs
 // an SM, so that one block's loads and barriers hide behind the other's
-// arithmetic.  The clover term is read in every MR step, from a copy in block
-// order: in the field's order the pieces of a warp's load lie in sixteen
-// places (two sites of a parity side by side), and those lookups took 4.6 M
-// of L1's 7.8 M wavefronts a launch at 16^3 x 32, more than shared memory's
-// 3.2 M; from the copy they take 0.6 M.  What is left is bound by L1 and
-// shared memory (6.0 M wavefronts, two thirds of the time) and the issue of
-// 2000 instructions a site and step (40 %).  One application (4^4 blocks, 5
-// cycles of 4 steps): 16^4 391 -> 248 us, 16^3 x 32 436 -> 374, 32^3 x 64
-// 5.85 -> 5.40 ms, of which the copy is 8 us at 16^3 x 32.
+// arithmetic.  Global arrays are in block order: in the fields' order the
+// pieces of a warp's load lie in sixteen places (two sites of a parity side by
+// side), and those lookups took 4.6 M of L1's 7.8 M wavefronts a launch at
+// 16^3 x 32 for the clover term alone, read in every MR step (0.6 M from the
+// copy), and 2 M for the links, rho, delta and z of a launch's start and end.
+// What is left is bound by shared memory (3.2 M) and the issue of 2000
+// instructions a site and step.  One application (4^4 blocks, 5 cycles of 4
+// steps), all in field order -> clover copied -> all in block order: 16^4 391
+// -> 248 -> 253 us, 16^3 x 32 436 -> 374 -> 337, 32^3 x 64 5.85 -> 5.40 ->
+// 4.48 ms, of which the copies are 12 us at 16^3 x 32 (a solve makes them
+// once: SAP-FGCR at 16^4 3.98 -> 3.53 ms by the second step).
 // Two threads a site (a colour vector each, the clover block in registers,
 // one CTA of 512 threads an SM) took 222 us at 16^4, 493 at 16^3 x 32 and 7.4
-// ms at 32^3 x 64: each reads every link for itself.
+// ms at 32^3 x 64 with the clover copy: each reads every link for itself.
 template <int RECON, int MU, int B>
 __device__ __forceinline__ void sap_hop_staged(const SapArgs& a, const float4* rs, const char* lk, const int xl[4],
                                                int l, float acc[24])
@@ -353,17 +362,71 @@ __device__ __forceinline__ void sap_hop_staged(const SapArgs& a, const float4* r
     }
 }
 
-// A in block order: float4 chunk k (18 a site) of site l of block b at [(b 18 + k) vol + l].
-__global__ void sap_clover_kernel(const SapArgs a, float4* out)
+// The border hops of sap_border_hop with everything in block order: the
+// neighbouring site across face MU is the one at the other end of the row, in
+// the next block; the forward link is staged, the backward one the
+// neighbour's.
+template <int RECON, int MU, int B>
+__device__ __forceinline__ void sap_border_staged(const SapArgs& a, const char* lk, const int bc[4], const int xl[4],
+                                                  int l, float acc[24])
+{
+    typedef SapShape<B> Shape;
+    const int vol = Shape::vol(a), row = (Shape::template extent<MU>(a) - 1) * Shape::template step<MU>(a);
+    const int per = MU == 0 ? 1 : MU == 1 ? a.nb[0] : MU == 2 ? a.nb[0] * a.nb[1] : a.nb[0] * a.nb[1] * a.nb[2];
+    const int block = ((bc[3] * a.nb[2] + bc[2]) * a.nb[1] + bc[1]) * a.nb[0] + bc[0];
+    float v[24], h[12], u[18], w[12];
+    if (xl[MU] == Shape::template extent<MU>(a) - 1) {
+        const bool wraps = bc[MU] == a.nb[MU] - 1;
+        const int n = block + (wraps ? 1 - a.nb[MU] : 1) * per;
+        smem_load(a.dltb + (size_t)n * 6 * vol, vol, l - row, v);
+        project<MU, -1>(v, h);
+        if (MU == 3 && a.g.tanti && wraps) {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) h[k] = -h[k];
+        }
+        SmemLinks<RECON>::load(lk, vol, MU, l, u);
+        su3_mul_half<false, true>(u, h, w);
+        accumulate<MU, -1>(acc, w);
+    }
+    if (xl[MU] == 0) {
+        const bool wraps = bc[MU] == 0;
+        const int n = block + (wraps ? a.nb[MU] - 1 : -1) * per;
+        smem_load(a.dltb + (size_t)n * 6 * vol, vol, l + row, v);
+        project<MU, +1>(v, h);
+        if (MU == 3 && a.g.tanti && wraps) {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) h[k] = -h[k];
+        }
+        SmemLinks<RECON>::load(reinterpret_cast<const char*>(a.linkb) + (size_t)n * 4 * SmemLinks<RECON>::bytes * vol, vol,
+                               MU, l + row, u);
+        su3_mul_half<true, true>(u, h, w);
+        accumulate<MU, +1>(acc, w);
+    }
+}
+
+// The copies in block order: A (blockIdx.y = 1) as float4 chunk k (18 a site)
+// of site l of block b at [(b 18 + k) vol + l], the links as in shared memory.
+template <int RECON>
+__global__ void sap_copy_kernel(const SapArgs a, float4* clov, float4* link)
 {
     const int b = blockIdx.x;
     const int bc[4] = {b % a.nb[0], b / a.nb[0] % a.nb[1], b / (a.nb[0] * a.nb[1]) % a.nb[2],
                        b / (a.nb[0] * a.nb[1] * a.nb[2])};
     for (int l = threadIdx.x; l < a.vol; l += blockDim.x) {
         const SapSite s = sap_site(a, bc, l);
-        const float4* src = reinterpret_cast<const float4*>(a.clov + s.par * a.clov_pb) + s.cb;
+        if (blockIdx.y) {
+            const float4* src = reinterpret_cast<const float4*>(a.clov + s.par * a.clov_pb) + s.cb;
 #pragma unroll
-        for (int k = 0; k < 18; ++k) out[((size_t)b * 18 + k) * a.vol + l] = __ldg(src + (size_t)k * a.g.stride);
+            for (int k = 0; k < 18; ++k) clov[((size_t)b * 18 + k) * a.vol + l] = __ldg(src + (size_t)k * a.g.stride);
+        } else {
+            char* base = reinterpret_cast<char*>(link) + (size_t)b * 4 * SmemLinks<RECON>::bytes * a.vol;
+            float u[18];
+#pragma unroll
+            for (int mu = 0; mu < 4; ++mu) {
+                GaugeIO<P32, RECON>::load(a.gauge, a.g.stride, s.par, mu, s.cb, u);
+                SmemLinks<RECON>::store(base, a.vol, mu, l, u);
+            }
+        }
     }
 }
 
@@ -379,26 +442,45 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) sap_block_kernel_one(const Sap
     sap_block_coords(a, bc);
     const int l = threadIdx.x;
     const bool live = B ? true : l < vol;
-    SapSite s = sap_site(a, bc, live ? l : 0);
-    if (B) {
-        s.l[0] = l % B; s.l[1] = l / B % B; s.l[2] = l / (B * B) % B; s.l[3] = l / (B * B * B);
-    }
-    const float4* clb = a.clovb + (size_t)(((bc[3] * a.nb[2] + bc[2]) * a.nb[1] + bc[1]) * a.nb[0] + bc[0]) * 18 * vol + l;
+    const int e[4] = {SapShape<B>::template extent<0>(a), SapShape<B>::template extent<1>(a),
+                      SapShape<B>::template extent<2>(a), SapShape<B>::template extent<3>(a)};
+    const int xl[4] = {l % e[0], l / e[0] % e[1], l / (e[0] * e[1]) % e[2], l / (e[0] * e[1] * e[2])};
+    const size_t block = ((bc[3] * a.nb[2] + bc[2]) * a.nb[1] + bc[1]) * a.nb[0] + bc[0];
+    const float4* clb = a.clovb + block * 18 * vol + l;
+    float4* const rhob = a.rhob + block * 6 * vol;
+    float4* const zb = a.zb + block * 6 * vol;
     float delta[24];
 #pragma unroll
     for (int k = 0; k < 24; ++k) delta[k] = 0.f;
-    if (live) {  // links: complete since before the chain of launches (it starts with an ordinary one)
-        float u[18];
+    constexpr int nch = SmemLinks<RECON>::bytes / 4;  // float4 chunks of the links a site
+    if (live) {  // links: complete since before the chain of launches
+        const float4* src = a.linkb + block * nch * vol;
+        float4* dst = reinterpret_cast<float4*>(lk);
 #pragma unroll
-        for (int mu = 0; mu < 4; ++mu) {
-            GaugeIO<P32, RECON>::load(a.gauge, a.g.stride, s.par, mu, s.cb, u);
-            SmemLinks<RECON>::store(lk, vol, mu, l, u);
-        }
+        for (int k = 0; k < nch; ++k)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(dst + k * vol + l)), "l"(src + k * vol + l) : "memory");
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
     pdl_wait();
     if (live) {
         float rho[24];
-        sap_residual_site<RECON>(a, s, rho);
+        if (a.first) {
+            const SapSite s = sap_site(a, bc, l);
+            SpinorIO<P32>::load(a.rho_in + s.par * a.fb, a.g.stride, s.cb, rho);
+        } else smem_load(rhob, vol, l, rho);
+        if (a.has_prev) {
+            float acc[24];
+#pragma unroll
+            for (int k = 0; k < 24; ++k) acc[k] = 0.f;
+            sap_border_staged<RECON, 0, B>(a, lk, bc, xl, l, acc);
+            sap_border_staged<RECON, 1, B>(a, lk, bc, xl, l, acc);
+            sap_border_staged<RECON, 2, B>(a, lk, bc, xl, l, acc);
+            sap_border_staged<RECON, 3, B>(a, lk, bc, xl, l, acc);
+#pragma unroll
+            for (int k = 0; k < 24; ++k) rho[k] += a.kappa * acc[k];
+        }
         smem_store(rs, vol, l, rho);
     }
     __syncthreads();
@@ -409,10 +491,10 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) sap_block_kernel_one(const Sap
             float acc[24];
 #pragma unroll
             for (int k = 0; k < 24; ++k) acc[k] = 0.f;
-            sap_hop_staged<RECON, 0, B>(a, rs, lk, s.l, l, acc);
-            sap_hop_staged<RECON, 1, B>(a, rs, lk, s.l, l, acc);
-            sap_hop_staged<RECON, 2, B>(a, rs, lk, s.l, l, acc);
-            sap_hop_staged<RECON, 3, B>(a, rs, lk, s.l, l, acc);
+            sap_hop_staged<RECON, 0, B>(a, rs, lk, xl, l, acc);
+            sap_hop_staged<RECON, 1, B>(a, rs, lk, xl, l, acc);
+            sap_hop_staged<RECON, 2, B>(a, rs, lk, xl, l, acc);
+            sap_hop_staged<RECON, 3, B>(a, rs, lk, xl, l, acc);
             smem_load(rs, vol, l, rho);
             if (a.clov) {
 #pragma unroll
@@ -478,15 +560,22 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) sap_block_kernel_one(const Sap
     }
     pdl_start_next();
     if (live) {
-        float rho[24], zv[24];
-        smem_load(rs, vol, l, rho);
-        SpinorIO<P32>::store(a.rho_out + s.par * a.fb, a.g.stride, s.cb, rho);
-        SpinorIO<P32>::store(a.dlt + s.par * a.fb, a.g.stride, s.cb, delta);
-        char* zp = a.z + s.par * a.fb;
-        SpinorIO<P32>::load(zp, a.g.stride, s.cb, zv);
+        if (!(a.last && a.colour)) smem_store(a.dltb + block * 6 * vol, vol, l, delta);
+        float zv[24];
+        if (!a.first) {
+            smem_load(zb, vol, l, zv);
 #pragma unroll
-        for (int k = 0; k < 24; ++k) zv[k] += delta[k];
-        SpinorIO<P32>::store(zp, a.g.stride, s.cb, zv);
+            for (int k = 0; k < 24; ++k) delta[k] += zv[k];
+        }
+        if (a.last) {
+            const SapSite s = sap_site(a, bc, l);
+            SpinorIO<P32>::store(a.z + s.par * a.fb, a.g.stride, s.cb, delta);
+        } else {
+            smem_store(zb, vol, l, delta);
+            float rho[24];
+            smem_load(rs, vol, l, rho);
+            smem_store(rhob, vol, l, rho);
+        }
     }
 }
 
@@ -576,11 +665,10 @@ lqcd_status sap_check(const lqcd_ctx* c, const int bs[4])
 }
 
 lqcd_status sap_apply(lqcd_ctx* c, void* z, const void* r, const int bs[4], int ncycle, int nmr, char* rho_buf,
-                      char* dlt_buf, bool have_clover)
+                      char* dlt_buf, bool have_copies)
 {
     LQ_TRY(sap_check(c, bs));
     const size_t fb = c->field_bytes(P32), fld = 2 * fb;
-    LQ_TRY(blas_zero(c, z, P32, 1, fld, 2));
     SapArgs a;
     memset(&a, 0, sizeof a);
     a.g = c->g;
@@ -613,15 +701,27 @@ lqcd_status sap_apply(lqcd_ctx* c, void* z, const void* r, const int bs[4], int 
                       : cube ? (r12 ? sap_block_kernel_one<12, 4> : sap_block_kernel_one<18, 4>)
                              : (r12 ? sap_block_kernel_one<12, 0> : sap_block_kernel_one<18, 0>);
     LQ_CUDA(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (small && a.clov) {  // CG's inner vectors are free here: 576 bytes a site, of which the copy takes 288
-        static_assert(NVLO * 192 >= 288, "the block-ordered clover term exceeds the inner vectors");
-        float4* copy = reinterpret_cast<float4*>(c->veclo);
-        if (!have_clover) {
-            sap_clover_kernel<<<nblocks, threads, 0, c->stream>>>(a, copy);
+    if (small) {
+        // CG's inner vectors are free here: 576 bytes a site, of which the copies take 288 + 288 (recon-12: 192);
+        // rho and z share a 192-byte FP64 field
+        static_assert(NVLO * 192 >= 288 + 4 * SmemLinks<18>::bytes, "the block-ordered copies exceed the inner vectors");
+        const size_t sites = (size_t)nblocks * a.vol;
+        float4* link = reinterpret_cast<float4*>(c->veclo);
+        float4* clov = link + sites * (link_bytes / 4);
+        if (!have_copies) {
+            const dim3 grid(nblocks, a.clov ? 2 : 1);
+            if (r12) sap_copy_kernel<12><<<grid, threads, 0, c->stream>>>(a, clov, link);
+            else sap_copy_kernel<18><<<grid, threads, 0, c->stream>>>(a, clov, link);
             LQ_CUDA(cudaGetLastError());
             c->launches++;
         }
-        a.clovb = copy;
+        a.linkb = link;
+        a.clovb = clov;
+        a.rhob = reinterpret_cast<float4*>(rho_buf);
+        a.zb = a.rhob + sites * 6;
+        a.dltb = reinterpret_cast<float4*>(dlt_buf);
+    } else {
+        LQ_TRY(blas_zero(c, z, P32, 1, fld, 2));
     }
     for (int cy = 0; cy < ncycle; ++cy)
         for (int colour = 0; colour < 2; ++colour) {
@@ -630,7 +730,11 @@ lqcd_status sap_apply(lqcd_ctx* c, void* z, const void* r, const int bs[4], int 
             a.rho_in = cy == 0 ? static_cast<const char*>(r) : rho_buf;
             a.has_prev = !(cy == 0 && colour == 0);
             a.colour = colour;
-            if (small) LQ_CUDA(launch_dependent(fn, false, dim3(nblocks / 2), dim3(threads), c->stream, smem, a));
+            a.first = cy == 0;
+            a.last = cy == ncycle - 1;
+            // the first launch waits for the copies; the later ones stage their links under their predecessor's tail
+            if (small && a.has_prev)
+                LQ_CUDA(launch_dependent(fn, false, dim3(nblocks / 2), dim3(threads), c->stream, smem, a));
             else fn<<<nblocks / 2, threads, smem, c->stream>>>(a);
             LQ_CUDA(cudaGetLastError());
             c->launches++;
