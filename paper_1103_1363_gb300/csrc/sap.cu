@@ -35,6 +35,7 @@
 namespace lqcd {
 
 enum { SAP_THREADS = 256, SAP_MAX_SITES = 1024 };
+constexpr size_t SAP_ALONE_BYTES = 120 * 1024;  // more than half of an SM's shared memory
 
 struct SapArgs {
     Geom g;
@@ -333,7 +334,7 @@ template <> struct SmemLinks<18> {
 // What is left is bound by shared memory (3.2 M) and the issue of 2000
 // instructions a site and step.  One application (4^4 blocks, 5 cycles of 4
 // steps), all in field order -> clover copied -> all in block order: 16^4 391
-// -> 248 -> 253 us, 16^3 x 32 436 -> 374 -> 337, 32^3 x 64 5.85 -> 5.40 ->
+// -> 248 -> 253 us (197: ALONE below), 16^3 x 32 436 -> 374 -> 337, 32^3 x 64 5.85 -> 5.40 ->
 // 4.48 ms, of which the copies are 12 us at 16^3 x 32 (a solve makes them
 // once: SAP-FGCR at 16^4 3.98 -> 3.53 ms by the second step).
 // Two threads a site (a colour vector each, the clover block in registers,
@@ -430,7 +431,21 @@ __global__ void sap_copy_kernel(const SapArgs a, float4* clov, float4* link)
     }
 }
 
-template <int RECON, int B>
+__device__ __forceinline__ void sap_stage16(float4* dst, const float4* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+// ALONE: one CTA an SM, with the clover term in shared memory as well.  For
+// launches of at most one CTA for each SM: there a second one would share its
+// SM with a CTA of the same launch while other SMs idle, since the next
+// launch's CTAs are placed while the preceding one's still run.  One
+// application at 16^4 253 -> 197 us (203 by the placement alone), 8 x 16^3 195
+// -> 185, 8^4 187 -> 180; with more CTAs than SMs it loses (16^3 x 32 337 ->
+// 443).  A launch is 5.8 us of start, border and end, and 3.1 us a step, of
+// which issue is half: two warps a scheduler wait for each other's latencies.
+template <int RECON, int B, bool ALONE>
 __global__ void __launch_bounds__(SAP_THREADS, 2) sap_block_kernel_one(const SapArgs a)
 {
     extern __shared__ float4 sap_smem[];
@@ -453,15 +468,20 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) sap_block_kernel_one(const Sap
 #pragma unroll
     for (int k = 0; k < 24; ++k) delta[k] = 0.f;
     constexpr int nch = SmemLinks<RECON>::bytes / 4;  // float4 chunks of the links a site
-    if (live) {  // links: complete since before the chain of launches
+    float4* const cs = sap_smem + (6 + nch) * vol + l;  // ALONE: clover [18][vol]
+    if (live) {  // the copies: complete since before the chain of launches
         const float4* src = a.linkb + block * nch * vol;
         float4* dst = reinterpret_cast<float4*>(lk);
 #pragma unroll
-        for (int k = 0; k < nch; ++k)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                             (unsigned)__cvta_generic_to_shared(dst + k * vol + l)), "l"(src + k * vol + l) : "memory");
+        for (int k = 0; k < nch; ++k) sap_stage16(dst + k * vol + l, src + k * vol + l);
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (ALONE && live && a.clov) {  // a thread reads its own site's only: waits in the first step
+#pragma unroll
+        for (int k = 0; k < 18; ++k) sap_stage16(cs + k * vol, clb + k * vol);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
     pdl_wait();
     if (live) {
@@ -497,12 +517,13 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) sap_block_kernel_one(const Sap
             sap_hop_staged<RECON, 3, B>(a, rs, lk, xl, l, acc);
             smem_load(rs, vol, l, rho);
             if (a.clov) {
+                if (ALONE && it == 0) asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
                     float c[36];
 #pragma unroll
                     for (int k = 0; k < 9; ++k) {
-                        const float4 v = __ldg(clb + (9 * b + k) * vol);
+                        const float4 v = ALONE ? cs[(9 * b + k) * vol] : __ldg(clb + (9 * b + k) * vol);
                         c[4 * k] = v.x; c[4 * k + 1] = v.y; c[4 * k + 2] = v.z; c[4 * k + 3] = v.w;
                     }
                     hermitian6_apply<float>(c, rho + 12 * b, q + 12 * b);
@@ -693,13 +714,17 @@ lqcd_status sap_apply(lqcd_ctx* c, void* z, const void* r, const int bs[4], int 
     const bool r12 = c->cfg.recon == 12;
     const int threads = small ? (a.vol + 31) / 32 * 32 : SAP_THREADS;
     const size_t link_bytes = r12 ? SmemLinks<12>::bytes : SmemLinks<18>::bytes;
-    const size_t smem = small ? (size_t)a.vol * (6 * sizeof(float4) + 4 * link_bytes)
-                              : (size_t)a.vol * 2 * 6 * sizeof(float4);
+    const bool alone = small && nblocks / 2 <= 152;  // CTAs of a launch, SMs
+    size_t smem = small ? (size_t)a.vol * ((alone ? 24 : 6) * sizeof(float4) + 4 * link_bytes)
+                        : (size_t)a.vol * 2 * 6 * sizeof(float4);
+    if (alone && smem < SAP_ALONE_BYTES) smem = SAP_ALONE_BYTES;
     const bool cube = bs[0] == 4 && bs[1] == 4 && bs[2] == 4 && bs[3] == 4;
     typedef void (*Kernel)(const SapArgs);
     const Kernel fn = !small ? (r12 ? sap_block_kernel_strided<12> : sap_block_kernel_strided<18>)
-                      : cube ? (r12 ? sap_block_kernel_one<12, 4> : sap_block_kernel_one<18, 4>)
-                             : (r12 ? sap_block_kernel_one<12, 0> : sap_block_kernel_one<18, 0>);
+                      : alone ? (cube ? (r12 ? sap_block_kernel_one<12, 4, true> : sap_block_kernel_one<18, 4, true>)
+                                      : (r12 ? sap_block_kernel_one<12, 0, true> : sap_block_kernel_one<18, 0, true>))
+                      : cube ? (r12 ? sap_block_kernel_one<12, 4, false> : sap_block_kernel_one<18, 4, false>)
+                             : (r12 ? sap_block_kernel_one<12, 0, false> : sap_block_kernel_one<18, 0, false>);
     LQ_CUDA(cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (small) {
         // CG's inner vectors are free here: 576 bytes a site, of which the copies take 288 + 288 (recon-12: 192);

@@ -150,6 +150,8 @@ def test_small_solves(lq, dims, inner, graph):
     ((4, 12, 8, 4), (2, 6, 4, 2), 12, 1.0),   # 96 sites a block: a whole number of warps, fewer than the CTA's most
     ((12, 12, 4, 4), (6, 6, 2, 2), 18, 1.0),  # 144: idle lanes
     ((8, 8, 8, 8), (4, 4, 4, 4), 12, 0.0),    # no clover term
+    ((8, 16, 16, 40), (4, 4, 4, 4), 12, 1.0),  # more blocks of a colour than SMs: two on one
+    ((8, 8, 12, 16), (2, 2, 2, 2), 18, 1.0),   # the same, 16 sites a block
 ])
 def test_sap_block_kernel(lq, dims, block, recon, csw):
     """SAP of blocks of at most 256 sites against the oracle (FP32 sums of
