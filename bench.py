@@ -57,8 +57,9 @@ FALLBACK_HBM_GBS = 6800.0
 # DRAM bytes (read + write) per output site of the inner hopping kernels,
 # from one ncu capture of a CG iteration on 24^3x48 (the four launches of an
 # iteration: Mhat sweeps with A^-1 and x-pay + norm epilogues, Mhat^dag sweeps
-# with A^-1 and the fused CG update); traffic grows with the sites processed.
-DRAM_BYTES_PER_SITE = {"f16spinors": (765.3 + 820.3 + 765.6 + 1151.4) / 4}
+# with A^-1 and the fused CG update, the solution's update deferred); traffic
+# grows with the sites processed.
+DRAM_BYTES_PER_SITE = {"f16spinors": (756.6 + 813.2 + 757.0 + 937.1) / 4}
 STORAGE = {
     "f32": "f32 spinors, links (recon-12) and clover",
     "f16": "f16 spinors (per-site norm), links (recon-12) and clover",
