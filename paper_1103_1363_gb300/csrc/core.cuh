@@ -121,9 +121,11 @@ __device__ __forceinline__ uint32_t f2h(float a, float b, int isbf)
 // ---- programmatic dependent launch
 // A kernel launched with launch_dependent() may start while its predecessor
 // in the stream finishes: it computes its indices, then pdl_wait() holds it
-// until the predecessor has completed and its writes are visible.  Before
-// pdl_wait() it reads kernel parameters only, and every thread calls it, so
-// that a kernel's completion implies its predecessor's.  pdl_start_next()
+// until the predecessor has completed and its writes are visible.  Every
+// thread calls it, so that a kernel's completion implies its predecessor's.
+// Before it a kernel reads its parameters only, or data that was complete when
+// the first launch of the chain, a plain one, started (SAP's copies of links
+// and clover).  pdl_start_next()
 // stands where a block has done its sites, before the reduction: called at
 // the top, the next kernel's blocks fill the slots that happen to be free
 // and share SMs unevenly (CG iteration at 16^4, FP32: 50.9 us, as without;
@@ -137,6 +139,28 @@ __device__ __forceinline__ uint32_t f2h(float a, float b, int isbf)
 // user's capture sees plain launches.
 __device__ __forceinline__ void pdl_start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Loads from global memory.  The read-only path (ld.global.nc) is for data that
+// nothing writes from a kernel's start to its end.  A kernel that starts under
+// its predecessor's tail runs while that one still writes its spinors,
+// activations or (first launch after a new gauge field) links, and some kernels
+// update their fields in place: those arrays are read by ordinary loads, which
+// also stay behind pdl_wait().  (Read-only loads here cost registers besides:
+// the reducing hops with FP16 spinors and recon-12 links spilled 12 to 60
+// bytes, now none; 24^3 x 48 Schur operator, 12 rhs, 576 -> 565 us, the other
+// operators and solves within 1 %.)
+template <class T>
+__device__ __forceinline__ T ld_plain(const T* p)
+{
+    return *p;
+}
+// Data complete before the chain's first launch, or read by a plain launch that
+// does not write it.
+template <class T>
+__device__ __forceinline__ T ld_fixed(const T* p)
+{
+    return __ldg(p);
+}
 
 // What this thread is capturing: an iteration block of the library, and the
 // sites (times right-hand sides) of the other lattices on parallel branches
@@ -182,7 +206,7 @@ template <> struct SpinorIO<P64> {
         const double2* p = static_cast<const double2*>(base);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            double2 c = __ldg(p + (size_t)k * stride + i);
+            double2 c = ld_plain(p + (size_t)k * stride + i);
             v[2 * k] = c.x;
             v[2 * k + 1] = c.y;
         }
@@ -200,7 +224,7 @@ template <> struct SpinorIO<P64> {
         const double2* p = static_cast<const double2*>(base) + (size_t)(6 * B) * stride + i;
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            double2 c = __ldg(p + (size_t)k * stride);
+            double2 c = ld_plain(p + (size_t)k * stride);
             v[2 * k] = c.x;
             v[2 * k + 1] = c.y;
         }
@@ -221,7 +245,7 @@ template <> struct SpinorIO<P32> {
         const float4* p = static_cast<const float4*>(base);
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            float4 c = __ldg(p + (size_t)k * stride + i);
+            float4 c = ld_plain(p + (size_t)k * stride + i);
             v[4 * k] = c.x;
             v[4 * k + 1] = c.y;
             v[4 * k + 2] = c.z;
@@ -241,7 +265,7 @@ template <> struct SpinorIO<P32> {
         const float4* p = static_cast<const float4*>(base) + (size_t)(3 * B) * stride + i;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            float4 c = __ldg(p + (size_t)k * stride);
+            float4 c = ld_plain(p + (size_t)k * stride);
             v[4 * k] = c.x;
             v[4 * k + 1] = c.y;
             v[4 * k + 2] = c.z;
@@ -264,10 +288,10 @@ template <int ISBF> struct SpinorHalfIO {
     __device__ __forceinline__ static void load(const void* base, int stride, int i, float v[24])
     {
         const uint4* p = static_cast<const uint4*>(base);
-        const float n = __ldg(reinterpret_cast<const float*>(p + (size_t)3 * stride) + i);
+        const float n = ld_plain(reinterpret_cast<const float*>(p + (size_t)3 * stride) + i);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            uint4 c = __ldg(p + (size_t)k * stride + i);
+            uint4 c = ld_plain(p + (size_t)k * stride + i);
             float2 a = h2f(c.x, ISBF), b = h2f(c.y, ISBF), d = h2f(c.z, ISBF), e = h2f(c.w, ISBF);
             v[8 * k + 0] = a.x * n; v[8 * k + 1] = a.y * n;
             v[8 * k + 2] = b.x * n; v[8 * k + 3] = b.y * n;
@@ -302,9 +326,9 @@ template <int ISBF> struct SpinorHalfIO {
     __device__ __forceinline__ static void load_half(const void* base, int stride, int i, float v[12])
     {
         const uint4* p = static_cast<const uint4*>(base);
-        const float n = __ldg(reinterpret_cast<const float*>(p + (size_t)3 * stride) + i);
-        const uint4 c = __ldg(p + (size_t)(2 * B) * stride + i);
-        const uint2 m = __ldg(reinterpret_cast<const uint2*>(p + (size_t)stride + i) + B);
+        const float n = ld_plain(reinterpret_cast<const float*>(p + (size_t)3 * stride) + i);
+        const uint4 c = ld_plain(p + (size_t)(2 * B) * stride + i);
+        const uint2 m = ld_plain(reinterpret_cast<const uint2*>(p + (size_t)stride + i) + B);
         const uint32_t w[6] = {B ? m.x : c.x, B ? m.y : c.y, B ? c.x : c.z, B ? c.y : c.w, B ? c.z : m.x, B ? c.w : m.y};
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
@@ -378,7 +402,7 @@ template <int RECON> struct GaugeIO<P64, RECON> {
         const double2* p = static_cast<const double2*>(base) + (size_t)((par * 4 + mu) * nchunk) * stride + i;
 #pragma unroll
         for (int k = 0; k < nchunk; ++k) {
-            double2 c = __ldg(p + (size_t)k * stride);
+            double2 c = ld_plain(p + (size_t)k * stride);
             u[2 * k] = c.x;
             u[2 * k + 1] = c.y;
         }
@@ -401,7 +425,7 @@ template <> struct GaugeIO<P32, 18> {
         const float2* p = static_cast<const float2*>(base) + (size_t)((par * 4 + mu) * 9) * stride + i;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            float2 c = __ldg(p + (size_t)k * stride);
+            float2 c = ld_plain(p + (size_t)k * stride);
             u[2 * k] = c.x;
             u[2 * k + 1] = c.y;
         }
@@ -422,7 +446,7 @@ template <> struct GaugeIO<P32, 12> {
         const float4* p = static_cast<const float4*>(base) + (size_t)((par * 4 + mu) * 3) * stride + i;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            float4 c = __ldg(p + (size_t)k * stride);
+            float4 c = ld_plain(p + (size_t)k * stride);
             u[4 * k] = c.x;
             u[4 * k + 1] = c.y;
             u[4 * k + 2] = c.z;
@@ -449,7 +473,7 @@ template <int ISBF, int RECON> struct GaugeHalfIO {
             const uint2* p = static_cast<const uint2*>(base) + (size_t)((par * 4 + mu) * 3) * stride + i;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                uint2 c = __ldg(p + (size_t)k * stride);
+                uint2 c = ld_plain(p + (size_t)k * stride);
                 float2 a = h2f(c.x, ISBF), b = h2f(c.y, ISBF);
                 u[4 * k] = a.x; u[4 * k + 1] = a.y; u[4 * k + 2] = b.x; u[4 * k + 3] = b.y;
             }
@@ -458,7 +482,7 @@ template <int ISBF, int RECON> struct GaugeHalfIO {
             const uint32_t* p = static_cast<const uint32_t*>(base) + (size_t)((par * 4 + mu) * 9) * stride + i;
 #pragma unroll
             for (int k = 0; k < 9; ++k) {
-                float2 a = h2f(__ldg(p + (size_t)k * stride), ISBF);
+                float2 a = h2f(ld_plain(p + (size_t)k * stride), ISBF);
                 u[2 * k] = a.x; u[2 * k + 1] = a.y;
             }
         }
@@ -504,7 +528,7 @@ template <> struct CloverIO<P64> {
         const double2* p = static_cast<const double2*>(base) + (size_t)(18 * blk) * stride + i;
 #pragma unroll
         for (int k = 0; k < 18; ++k) {
-            double2 v = __ldg(p + (size_t)k * stride);
+            double2 v = ld_plain(p + (size_t)k * stride);
             c[2 * k] = v.x;
             c[2 * k + 1] = v.y;
         }
@@ -524,7 +548,7 @@ template <> struct CloverIO<P32> {
         const float4* p = static_cast<const float4*>(base) + (size_t)(9 * blk) * stride + i;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            float4 v = __ldg(p + (size_t)k * stride);
+            float4 v = ld_plain(p + (size_t)k * stride);
             c[4 * k] = v.x; c[4 * k + 1] = v.y; c[4 * k + 2] = v.z; c[4 * k + 3] = v.w;
         }
     }
@@ -546,7 +570,7 @@ template <int ISBF> struct CloverHalfIO {
         const uint4* p = static_cast<const uint4*>(base) + i;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            uint4 v = __ldg(p + (size_t)k * stride);
+            uint4 v = ld_plain(p + (size_t)k * stride);
             float2 a = h2f(v.x, ISBF), b = h2f(v.y, ISBF), d = h2f(v.z, ISBF), e = h2f(v.w, ISBF);
             c[8 * k] = a.x; c[8 * k + 1] = a.y; c[8 * k + 2] = b.x; c[8 * k + 3] = b.y;
             c[8 * k + 4] = d.x; c[8 * k + 5] = d.y; c[8 * k + 6] = e.x; c[8 * k + 7] = e.y;
@@ -559,7 +583,7 @@ template <int ISBF> struct CloverHalfIO {
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             const int piece = 9 * b + k;
-            const uint2 v = __ldg(p + ((size_t)(piece >> 1) * stride + i) * 2 + (piece & 1));
+            const uint2 v = ld_plain(p + ((size_t)(piece >> 1) * stride + i) * 2 + (piece & 1));
             const float2 x = h2f(v.x, ISBF), y = h2f(v.y, ISBF);
             c[4 * k] = x.x; c[4 * k + 1] = x.y; c[4 * k + 2] = y.x; c[4 * k + 3] = y.y;
         }

@@ -335,10 +335,10 @@ struct HopSpinorHalf {
     __device__ __forceinline__ void load(const void* base, int stride, int j)
     {
         const uint4* p = static_cast<const uint4*>(base);
-        n = __ldg(reinterpret_cast<const float*>(p + (size_t)3 * stride) + j);
+        n = ld_plain(reinterpret_cast<const float*>(p + (size_t)3 * stride) + j);
         uint4 s[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) s[k] = __ldg(p + (size_t)k * stride + j);
+        for (int k = 0; k < 3; ++k) s[k] = ld_plain(p + (size_t)k * stride + j);
         set(s);
     }
     // h0 = q0 + e0 q_a, h1 = q1 + e1 q_b with e = +-1 (REAL) or +-i
@@ -488,22 +488,22 @@ __device__ __forceinline__ void load_half_hop(const char* in, const void* gauge,
 {
     const uint4* sp = reinterpret_cast<const uint4*>(in);
     const int j = hp.nb[h];
-    r.n = __ldg(reinterpret_cast<const float*>(sp + (size_t)3 * stride) + j);
+    r.n = ld_plain(reinterpret_cast<const float*>(sp + (size_t)3 * stride) + j);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) r.s[k] = __ldg(sp + (size_t)k * stride + j);
+    for (int k = 0; k < 3; ++k) r.s[k] = ld_plain(sp + (size_t)k * stride + j);
     const int mu = h >> 1, lpar = (h & 1) ? 1 - par : par;
     if constexpr (RECON == 12) {
         const uint2* lp = static_cast<const uint2*>(gauge) + (size_t)((lpar * 4 + mu) * 3) * stride + hp.lidx[h];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const uint2 q = __ldg(lp + (size_t)k * stride);
+            const uint2 q = ld_plain(lp + (size_t)k * stride);
             r.u[2 * k] = q.x;
             r.u[2 * k + 1] = q.y;
         }
     } else {
         const uint32_t* lp = static_cast<const uint32_t*>(gauge) + (size_t)((lpar * 4 + mu) * 9) * stride + hp.lidx[h];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) r.u[k] = __ldg(lp + (size_t)k * stride);
+        for (int k = 0; k < 9; ++k) r.u[k] = ld_plain(lp + (size_t)k * stride);
     }
 }
 

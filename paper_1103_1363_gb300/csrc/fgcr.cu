@@ -195,7 +195,7 @@ __global__ void gcr_orth_update_kernel(Geom g, const char* W, size_t fld, int k,
             const float xr = cj[j].x, xi = cj[j].y;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const float4 w = __ldg(reinterpret_cast<const float4*>(W + j * fld + off + h * apart));
+                const float4 w = ld_fixed(reinterpret_cast<const float4*>(W + j * fld + off + h * apart));
                 a[h].x -= xr * w.x - xi * w.y;
                 a[h].y -= xr * w.y + xi * w.x;
                 a[h].z -= xr * w.z - xi * w.w;

@@ -108,7 +108,7 @@ __global__ void arn_update_kernel(Geom g, const char* V, size_t fld, int n, cons
             for (int j = 0; j < n; ++j) {
                 float v[24];
                 SpinorIO<P32>::load(V + (size_t)j * fld + par * fb, g.stride, i, v);
-                const float2 c = __ldg(coef + j);
+                const float2 c = ld_fixed(coef + j);
 #pragma unroll
                 for (int q = 0; q < 12; ++q) {
                     a[2 * q] -= c.x * v[2 * q] - c.y * v[2 * q + 1];
@@ -158,7 +158,7 @@ __global__ void arn_lincomb_kernel(Geom g, char* out, const char* in, size_t fld
 #pragma unroll
             for (int l = 0; l < KO; ++l) {
                 if (l >= kout) break;
-                const float2 c = __ldg(P + j + (size_t)l * n);
+                const float2 c = ld_fixed(P + j + (size_t)l * n);
                 acc[l][0].x += c.x * v.x - c.y * v.y;
                 acc[l][0].y += c.x * v.y + c.y * v.x;
                 acc[l][1].x += c.x * v.z - c.y * v.w;

@@ -158,8 +158,8 @@ __global__ void __launch_bounds__(4 * GAUGE_SITES) gauge_pack_kernel(Geom g, con
         const int site = e / 36, k = e - site * 36;
         if (full[site] < 0) continue;
         const size_t at = (size_t)full[site] * 36 + k;
-        if (aligned) st[site][k] = __ldg(reinterpret_cast<const double2*>(slice) + at);
-        else st[site][k] = make_double2(__ldg(slice + 2 * at), __ldg(slice + 2 * at + 1));
+        if (aligned) st[site][k] = ld_fixed(reinterpret_cast<const double2*>(slice) + at);
+        else st[site][k] = make_double2(ld_fixed(slice + 2 * at), ld_fixed(slice + 2 * at + 1));
     }
     __syncthreads();
     const int site = threadIdx.x % GAUGE_SITES, mu = threadIdx.x / GAUGE_SITES;

@@ -349,7 +349,7 @@ __device__ __forceinline__ void load_channel_bf16(const uint4* in_b, int V, int 
         const uint4* src = in_b + (size_t)ci * 3 * V + y;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const uint4 v = __ldg(src + (size_t)q * V);
+            const uint4 v = ld_plain(src + (size_t)q * V);
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
@@ -370,7 +370,7 @@ __device__ __forceinline__ void load_channel(const float* in_b, int V, int ci, i
         const float4* src = reinterpret_cast<const float4*>(in_b) + plane4(V, ci, 0) + y;
 #pragma unroll
         for (int q = 0; q < 6; ++q) {
-            const float4 v = __ldg(src + (size_t)q * V);
+            const float4 v = ld_plain(src + (size_t)q * V);
             p[4 * q] = v.x; p[4 * q + 1] = v.y; p[4 * q + 2] = v.z; p[4 * q + 3] = v.w;
         }
     } else {
@@ -405,7 +405,7 @@ __device__ __forceinline__ void load_raw_bf16(const void* act, int V, int ch, in
                            (size_t)ci * 3 * V + y;
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const uint4 v = __ldg(src + (size_t)q * V);
+            const uint4 v = ld_plain(src + (size_t)q * V);
             raw[4 * q] = v.x; raw[4 * q + 1] = v.y; raw[4 * q + 2] = v.z; raw[4 * q + 3] = v.w;
         }
     } else {
@@ -527,14 +527,14 @@ struct HopFetch {
                 const float4* q = static_cast<const float4*>(a.gauge) + (size_t)((par * 4 + mu) * 3) * a.stride + i;
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    const float4 v = __ldg(q + (size_t)k * a.stride);
+                    const float4 v = ld_plain(q + (size_t)k * a.stride);
                     lk[4 * k] = v.x; lk[4 * k + 1] = v.y; lk[4 * k + 2] = v.z; lk[4 * k + 3] = v.w;
                 }
             } else {
                 const float2* q = static_cast<const float2*>(a.gauge) + (size_t)((par * 4 + mu) * 9) * a.stride + i;
 #pragma unroll
                 for (int k = 0; k < 9; ++k) {
-                    const float2 v = __ldg(q + (size_t)k * a.stride);
+                    const float2 v = ld_plain(q + (size_t)k * a.stride);
                     lk[2 * k] = v.x; lk[2 * k + 1] = v.y;
                 }
             }

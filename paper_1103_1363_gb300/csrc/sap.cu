@@ -418,7 +418,7 @@ __global__ void sap_copy_kernel(const SapArgs a, float4* clov, float4* link)
         if (blockIdx.y) {
             const float4* src = reinterpret_cast<const float4*>(a.clov + s.par * a.clov_pb) + s.cb;
 #pragma unroll
-            for (int k = 0; k < 18; ++k) clov[((size_t)b * 18 + k) * a.vol + l] = __ldg(src + (size_t)k * a.g.stride);
+            for (int k = 0; k < 18; ++k) clov[((size_t)b * 18 + k) * a.vol + l] = ld_fixed(src + (size_t)k * a.g.stride);
         } else {
             char* base = reinterpret_cast<char*>(link) + (size_t)b * 4 * SmemLinks<RECON>::bytes * a.vol;
             float u[18];
@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(SAP_THREADS, 2) sap_block_kernel_one(const Sap
                     float c[36];
 #pragma unroll
                     for (int k = 0; k < 9; ++k) {
-                        const float4 v = ALONE ? cs[(9 * b + k) * vol] : __ldg(clb + (9 * b + k) * vol);
+                        const float4 v = ALONE ? cs[(9 * b + k) * vol] : ld_fixed(clb + (9 * b + k) * vol);
                         c[4 * k] = v.x; c[4 * k + 1] = v.y; c[4 * k + 2] = v.z; c[4 * k + 3] = v.w;
                     }
                     hermitian6_apply<float>(c, rho + 12 * b, q + 12 * b);
