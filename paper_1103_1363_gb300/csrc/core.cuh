@@ -104,6 +104,13 @@ __device__ __forceinline__ float2 halves(uint32_t w)
     return make_float2(half_value<ISBF, 0>(w), half_value<ISBF, 1>(w));
 }
 __device__ __forceinline__ float2 h2f(uint32_t u, int isbf) { return isbf ? halves<1>(u) : halves<0>(u); }
+// the same by the conversion instructions
+template <int ISBF>
+__device__ __forceinline__ float2 converted(uint32_t w)
+{
+    if (ISBF) return __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&w));
+    return __half22float2(*reinterpret_cast<__half2*>(&w));
+}
 
 __device__ __forceinline__ uint32_t f2h(float a, float b, int isbf)
 {
@@ -467,6 +474,8 @@ template <int ISBF, int RECON> struct GaugeHalfIO {
     // recon-12: 3 chunks of uint2 (two complex each); recon-18: 9 chunks of one half2
     static constexpr int nchunk = RECON == 12 ? 3 : 9;
     static constexpr int bytes_per_link = RECON == 12 ? 24 : 36;
+    // CONVERT: decoded by conversions, otherwise by adds (the same values)
+    template <bool CONVERT = false>
     __device__ __forceinline__ static void load(const void* base, int stride, int par, int mu, int i, float u[18])
     {
         if (RECON == 12) {
@@ -474,7 +483,7 @@ template <int ISBF, int RECON> struct GaugeHalfIO {
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 uint2 c = ld_plain(p + (size_t)k * stride);
-                float2 a = h2f(c.x, ISBF), b = h2f(c.y, ISBF);
+                float2 a = decode<CONVERT>(c.x), b = decode<CONVERT>(c.y);
                 u[4 * k] = a.x; u[4 * k + 1] = a.y; u[4 * k + 2] = b.x; u[4 * k + 3] = b.y;
             }
             reconstruct_row2(u);
@@ -482,10 +491,15 @@ template <int ISBF, int RECON> struct GaugeHalfIO {
             const uint32_t* p = static_cast<const uint32_t*>(base) + (size_t)((par * 4 + mu) * 9) * stride + i;
 #pragma unroll
             for (int k = 0; k < 9; ++k) {
-                float2 a = h2f(ld_plain(p + (size_t)k * stride), ISBF);
+                float2 a = decode<CONVERT>(ld_plain(p + (size_t)k * stride));
                 u[2 * k] = a.x; u[2 * k + 1] = a.y;
             }
         }
+    }
+    template <bool CONVERT>
+    __device__ __forceinline__ static float2 decode(uint32_t w)
+    {
+        return CONVERT ? converted<ISBF>(w) : halves<ISBF>(w);
     }
     __device__ __forceinline__ static void store(void* base, int stride, int par, int mu, int i, const float u[18])
     {

@@ -392,13 +392,22 @@ template <> struct HopSpinor<PB16> : HopSpinorHalf<1> {};
 // w = U P q (backward: U^dag P q) for the neighbour's spinor q: forward hops
 // (BWD false) use (1 - g_mu), backward ones (1 + g_mu), swapped by DAG; the
 // link is U_mu at checkerboard index lidx of parity lpar.  hop_term adds it.
+// 16-bit links with FP32 spinors are decoded by conversions in the forward
+// operator and by adds in its adjoint (and with BF16 recon-18): the values are
+// the same and neither pipe is full, but the compiler's schedules differ by
+// several per cent.  42 x 32^2 x 48, 4 rhs, us, by adds / by conversions: BF16
+// recon-12 hop 265 / 250, Schur operator 658 / 642, adjoint full operator 555 /
+// 576; BF16 recon-18 hop 281 / 284; FP16 recon-18 full operator 646 / 604,
+// adjoint 600 / 605; FP16 recon-12 Schur operator 658 / 622, adjoint 641 / 648.
 template <int PG, int PS, int RECON, int MU, bool DAG, bool BWD, bool PACK>
 __device__ __forceinline__ void hop_product(const DslashArgs& A, const HopSpinor<PS>& q, int lpar, int lidx,
                                             typename RealT<PS>::type w[12])
 {
     typename RealT<PS>::type h[12], u[18];
     q.template project_to<MU, (BWD != DAG) ? +1 : -1>(h);
-    GaugeIO<PG, RECON>::load(A.gauge, A.g.stride, lpar, MU, lidx, u);
+    if constexpr (PG == P16 || PG == PB16)
+        GaugeIO<PG, RECON>::template load<!DAG && (PG == P16 || RECON == 12)>(A.gauge, A.g.stride, lpar, MU, lidx, u);
+    else GaugeIO<PG, RECON>::load(A.gauge, A.g.stride, lpar, MU, lidx, u);
     su3_mul_half<BWD, PACK>(u, h, w);
 }
 template <int PG, int PS, int RECON, int MU, bool DAG, bool BWD, bool PACK>
