@@ -1747,29 +1747,55 @@ __global__ void net_layout_bf16_kernel(const void* src, void* dst, int V, int ch
     pdl_start_next();
 }
 
-// Running sum in two FP32 words (value hi + lo), good to about 2^-46: FP64
-// additions would be bound by the FP64 pipe (five of its instructions an
-// element took 211 us for 16 spinors of 16^4, at 1/63 of the FP32 rate).
-// Components whose square FP32 cannot hold to its last bit (and infinities,
-// NaN) go to an FP64 sum as before.
-struct TwoFloat {
-    float hi = 0.f, lo = 0.f;
+// Running sum in three FP32 words (value hi + mid + lo): hi and mid take each
+// addend without loss (Knuth's sum: the error of a + b is exact), lo collects
+// what mid could not hold, so that a thread's sum is good to about 2^-70 and
+// is rounded to FP64 once, where FP64 additions round each time.  Those would
+// be bound by the FP64 pipe (five of its instructions an element took 211 us
+// for 16 spinors of 16^4, at 1/63 of the FP32 rate; 58 now).  Components
+// whose square FP32 cannot hold to its last bit (and infinities, NaN) go to an
+// FP64 sum.
+struct ThreeFloat {
+    float hi = 0.f, mid = 0.f, lo = 0.f;
     double rest = 0.0;
-    // + a^2, the square exact as s + fma(a, a, -s) (sum of Knuth: the error of hi + s is exact)
+    // a = a + b rounded; returns the error
+    __device__ __forceinline__ static float add(float& a, float b)
+    {
+        const float t = __fadd_rn(a, b), z = __fadd_rn(t, -a);
+        const float r = __fadd_rn(__fadd_rn(a, -__fadd_rn(t, -z)), __fadd_rn(b, -z));
+        a = t;
+        return r;
+    }
+    // + a^2, the square exact as s + fma(a, a, -s)
     __device__ __forceinline__ void add_square(float a)
     {
-        const float m = fabsf(a);
-        if (!(m >= 0x1p-48f && m <= 0x1p50f)) {
-            if (a != 0.f) rest += (double)a * a;
-            return;
-        }
         const float s = __fmul_rn(a, a), e = __fmaf_rn(a, a, -s);
-        const float t = __fadd_rn(hi, s), z = __fadd_rn(t, -hi);
-        const float r = __fadd_rn(__fadd_rn(hi, -__fadd_rn(t, -z)), __fadd_rn(s, -z));
-        hi = t;
-        lo = __fadd_rn(lo, __fadd_rn(r, e));
+        const float r = add(mid, add(hi, s)), q = add(mid, e);
+        lo = __fadd_rn(lo, __fadd_rn(r, q));
     }
-    __device__ __forceinline__ double value() const { return rest + ((double)hi + (double)lo); }
+    __device__ __forceinline__ static bool holds(float a) { return a >= 0x1p-48f && a <= 0x1p50f; }
+    __device__ __forceinline__ void add_squares(float a, float b, float c, float d)
+    {
+        const float v[4] = {fabsf(a), fabsf(b), fabsf(c), fabsf(d)};
+        bool all = true;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool h = holds(v[k]);
+            all = all && h;
+            add_square(h ? v[k] : 0.f);
+        }
+        if (all) return;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double x = holds(v[k]) ? 0.f : v[k];
+            rest += x * x;
+        }
+    }
+    __device__ __forceinline__ double value() const
+    {
+        const double sum = (double)hi + ((double)mid + (double)lo);
+        return rest == 0.0 ? sum : rest + sum;
+    }
 };
 
 // Loss L = (1/B) sum_b |y_b - e_b|^2 / |e_b|^2; gout_b = 2 (y_b - e_b) / (B |e_b|^2).
@@ -1778,19 +1804,13 @@ __global__ void net_loss_reduce_kernel(const float4* y, const float4* e, size_t 
                                        unsigned* tickets, double* red)
 {
     const int b = blockIdx.y;
-    TwoFloat d2, e2;
+    ThreeFloat d2, e2;
     const float4* yb = y + (size_t)b * n_per;
     const float4* eb = e + (size_t)b * n_per;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_per; i += (size_t)gridDim.x * blockDim.x) {
         const float4 p = yb[i], q = eb[i];
-        d2.add_square(p.x - q.x);
-        d2.add_square(p.y - q.y);
-        d2.add_square(p.z - q.z);
-        d2.add_square(p.w - q.w);
-        e2.add_square(q.x);
-        e2.add_square(q.y);
-        e2.add_square(q.z);
-        e2.add_square(q.w);
+        d2.add_squares(p.x - q.x, p.y - q.y, p.z - q.z, p.w - q.w);
+        e2.add_squares(q.x, q.y, q.z, q.w);
     }
     double v[2] = {d2.value(), e2.value()};
     block_reduce_finalize<2>(v, partials + b * part_rs, tickets + b, red + b * 2);

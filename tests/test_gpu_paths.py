@@ -228,6 +228,32 @@ def test_training_loss(lq, scale, batch):
     assert abs(net.train_step(r, e, batch, lr=0.0) / want - 1.0) < 1e-12
 
 
+@pytest.mark.parametrize("c", ["0x1.64fa88p+0", "0x1.fbaef8p+0"])
+def test_training_loss_of_a_constant_target(lq, c):
+    """Every component of the target is the same number, so that every thread's
+    96 additions round alike and their errors do not average out.  A loss of
+    FP64 sums of positive terms: at most 30 roundings of 2^-53 each in a sum
+    (a thread's sum, the block's tree, the blocks) and the division."""
+    import math
+    import torch
+    dims = (16, 16, 16, 16)
+    lat = lq.Lattice(dims, precisions=("f64", "f32"))
+    lat.gauge_load(on_device(synth.gauge_field(dims, "smooth", 23, eps=0.5)))
+    net = lq.Net(lat, (1, 3, 1), bf16=True, max_batch=1)
+    rng = np.random.default_rng(24)
+    net.set_weights((0.1 * (rng.standard_normal(net.num_weights) + 1j * rng.standard_normal(net.num_weights))).astype(np.complex64))
+    shape = (1, dims[3], dims[2], dims[1], dims[0], 4, 3)
+    c = float.fromhex(c)
+    r = on_device((rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64))
+    e = torch.full(shape, complex(c, c), dtype=torch.complex64, device="cuda")
+    y = torch.empty_like(r)
+    net.forward(y, r, 1)
+    lat.sync()
+    d = (torch.view_as_real(y) - torch.view_as_real(e)).reshape(-1).cpu().numpy().astype(np.float64)
+    want = math.fsum(d * d) / (d.size * c * c)  # squares of 24-bit numbers and the products are exact
+    assert abs(net.train_step(r, e, 1, lr=0.0) / want - 1.0) < 2 * 31 * 2.0 ** -53
+
+
 @pytest.mark.parametrize("prec", ["f16spinors", "f16"])
 @pytest.mark.parametrize("block", [128, 96])
 def test_hop_reads_subnormal_halves(lq, prec, block):
