@@ -702,10 +702,9 @@ __device__ __forceinline__ void warp_sums(double (&v)[NV], int lane, double* out
         }
         if (up) k += n;
     }
-    const int writers = o;  // 2 o lanes hold the same value
 #pragma unroll
     for (; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
-    if ((lane & (2 * writers - 1)) == 0) out[k] = v[0];
+    if ((lane & (32 / NV - 1)) == 0) out[k] = v[0];  // 32 / NV lanes hold the same value
 }
 
 // The same for any NV, in power-of-two parts.
