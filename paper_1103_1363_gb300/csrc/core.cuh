@@ -602,19 +602,6 @@ template <int ISBF> struct CloverHalfIO {
             c[4 * k] = x.x; c[4 * k + 1] = x.y; c[4 * k + 2] = y.x; c[4 * k + 3] = y.y;
         }
     }
-    __device__ __forceinline__ static void store_all(void* base, int stride, int i, const float c[72])
-    {
-        uint4* p = static_cast<uint4*>(base) + i;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            uint4 v;
-            v.x = f2h(c[8 * k], c[8 * k + 1], ISBF);
-            v.y = f2h(c[8 * k + 2], c[8 * k + 3], ISBF);
-            v.z = f2h(c[8 * k + 4], c[8 * k + 5], ISBF);
-            v.w = f2h(c[8 * k + 6], c[8 * k + 7], ISBF);
-            p[(size_t)k * stride] = v;
-        }
-    }
 };
 template <> struct CloverIO<P16> : CloverHalfIO<0> {};
 template <> struct CloverIO<PB16> : CloverHalfIO<1> {};

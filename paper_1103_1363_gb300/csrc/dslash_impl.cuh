@@ -273,7 +273,6 @@ struct HopSpinor {
     {
         accumulate<MU, S>(acc, w);
     }
-    __device__ __forceinline__ R scale() const { return (R)1; }
 };
 
 // Half precision: 12 packed complex values q and the site's norm n.  The
