@@ -1,5 +1,6 @@
 // C ABI entry points (include/lqcd.h): context and workspace management,
 // gauge and clover set-up, packing, operator application.
+#include <atomic>
 #include <chrono>
 #include <cstdio>
 #include <cstdlib>
@@ -100,6 +101,18 @@ static double launch_bytes_per_site(const lqcd_ctx* c, const DslashArgs& A, int 
     return nrhs * per_rhs + 8 * L + (epi == EPI_NONE ? 0.0 : Cl);
 }
 
+int sm_count()
+{
+    static std::atomic<int> known{0};
+    int sms = known.load(std::memory_order_relaxed), dev = 0;
+    if (sms == 0) {
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            sms = 0;
+        known.store(sms, std::memory_order_relaxed);
+    }
+    return sms;
+}
+
 // Does the warp-per-direction kernel take a launch of `sites` (sites per
 // parity times right-hand sides) by default?  Measured, gathering kernel
 // against it (schur / CG iteration in plain launches, us): FP32 2048 sites
@@ -113,7 +126,7 @@ static double launch_bytes_per_site(const lqcd_ctx* c, const DslashArgs& A, int 
 // 145, 10368 86 / 188 against 89 / 210.
 static bool wide_default(int mode, bool reducing, long sites)
 {
-    return sites <= (mode == P64 ? 8192 : reducing ? 12288 : 16384);
+    return sites <= (mode == P64 ? 8192 : reducing ? (long)SMALL_ITERATION_SITES : 16384);
 }
 
 // FP64 launches without a sum run blocks of one warp: the FP64 pipe bounds

@@ -219,7 +219,7 @@ lqcd_status blas_cg_p_update(lqcd_ctx* c, void* p_out, const void* p, int Pp, co
     char* po = static_cast<char*>(p_out);
     const char* pp = static_cast<const char*>(p);
     const char* rr = static_cast<const char*>(r);
-    const bool small = (long)c->g.Vh * nrhs + own_capture.other_sites <= 12288;  // as the iteration's reducing hops
+    const bool small = (long)c->g.Vh * nrhs + own_capture.other_sites <= SMALL_ITERATION_SITES;
     if (Pr == P64) {
         if (Pp != P64) return fail(LQCD_ERR_INVALID, "cg_p_update: FP64 r needs FP64 p");
         LQ_CUDA(launch_dependent(cg_p_kernel<P64, P64>, small, grid, block, c->stream, 0, c->g, po, pp, p_rb, rr, r_rb, nf,
@@ -239,7 +239,7 @@ lqcd_status blas_cg_x_update(lqcd_ctx* c, void* x, size_t x_rb, const void* p, i
     dim3 grid(blas_grid(c, block), nrhs);
     char* xx = static_cast<char*>(x);
     const char* pp = static_cast<const char*>(p);
-    const bool small = (long)c->g.Vh * nrhs + own_capture.other_sites <= 12288;
+    const bool small = (long)c->g.Vh * nrhs + own_capture.other_sites <= SMALL_ITERATION_SITES;
     switch (Pp) {
     case P32: LQ_CUDA(launch_dependent(cg_x_kernel<P32>, small, grid, block, c->stream, 0, c->g, xx, x_rb, pp, p_rb,
                                        slot_bytes, j0, j1, slots, c->scal, c->skip)); break;

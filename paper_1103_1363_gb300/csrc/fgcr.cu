@@ -25,6 +25,7 @@
 // or when a new direction lies numerically in the span of the earlier ones:
 // past FP32's resolution of the starting residual the recursion only adds
 // rounding, and the rebuilt solution would no longer match it.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <complex>
@@ -309,7 +310,9 @@ lqcd_status solve_fgcr(lqcd_ctx* c, lqcd_net* net, double* x, const double* b, d
     const int block = 256;
     const dim3 grid(gcr_grid(c, block));
     // the elementwise update: a block row per parity and pair of float4 chunks, at most 8 blocks per SM
-    const dim3 gu(grid.x < 8 * 152 / 6 ? grid.x : 8 * 152 / 6, 6);
+    const int sms = sm_count();
+    if (sms <= 0) return fail(LQCD_ERR_CUDA, "lqcd_solve: no SM count");
+    const dim3 gu(std::min(grid.x, 8u * sms / 6), 6);
     bool sap = !net && c->sap_on, sap_ready = false;
     if (sap) LQ_TRY(sap_check(c, c->sap_bs));
     int iters = 0, restarts = 0, fallback = 0;

@@ -230,6 +230,14 @@ inline char* vec64_field(lqcd_ctx* c, int which, int rhs)
     return c->vec64 + ((size_t)which * c->cfg.max_nrhs + rhs) * 2 * c->field_bytes(P64);
 }
 
+// SMs of the GPU, 0 if the query fails (api.cu)
+int sm_count();
+
+// sites (times right-hand sides) up to which a CG iteration counts as small:
+// its reducing hops take the warp-per-direction kernel (wide_default, where
+// both sides are measured), its vector kernels programmatic edges under capture
+enum : long { SMALL_ITERATION_SITES = 12288 };
+
 // ---- launchers exported by the translation units (all asynchronous on s)
 // fields.cu
 lqcd_status pack_spinor(lqcd_ctx* c, void* internal, const double* canon_dev, int parity, int P, int nrhs,

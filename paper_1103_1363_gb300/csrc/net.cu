@@ -1957,17 +1957,6 @@ size_t layer_smem_f32(const NetLayerArgs& a)
     return (size_t)NET_ROWS * (a.K2p + 4) * 4 + (size_t)a.K2 * (a.N2p + 4) * 4;
 }
 
-int sm_count()
-{
-    static int sms = 0;
-    if (sms == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            sms = 0;
-    }
-    return sms;
-}
-
 // Algorithmic work of one layer launch over `batch` items: the channel
 // contraction (8 real flops per complex multiply-add, 4 C_out x 4 C_in x 3
 // colours x 9 hops per site) and the compulsory bytes (input activations,

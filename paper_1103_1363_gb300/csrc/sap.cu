@@ -714,7 +714,9 @@ lqcd_status sap_apply(lqcd_ctx* c, void* z, const void* r, const int bs[4], int 
     const bool r12 = c->cfg.recon == 12;
     const int threads = small ? (a.vol + 31) / 32 * 32 : SAP_THREADS;
     const size_t link_bytes = r12 ? SmemLinks<12>::bytes : SmemLinks<18>::bytes;
-    const bool alone = small && nblocks / 2 <= 152;  // CTAs of a launch, SMs
+    const int sms = sm_count();
+    if (sms <= 0) return fail(LQCD_ERR_CUDA, "SAP: no SM count");
+    const bool alone = small && nblocks / 2 <= sms;  // CTAs of a launch, SMs
     size_t smem = small ? (size_t)a.vol * ((alone ? 24 : 6) * sizeof(float4) + 4 * link_bytes)
                         : (size_t)a.vol * 2 * 6 * sizeof(float4);
     if (alone && smem < SAP_ALONE_BYTES) smem = SAP_ALONE_BYTES;
