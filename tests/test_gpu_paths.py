@@ -456,3 +456,68 @@ def test_fgcr_steps(lq, dims, nkrylov, steps):
         assert abs(got - want) <= 1e-5
     else:  # a cycle ended early at FP32's resolution, and so did the exact one
         assert got <= want + 1e-5
+
+
+@pytest.mark.parametrize("kappa,steps", [(0.12, 8), (0.2, 5), (0.2, 8), (0.5, 2), (0.5, 12)])
+def test_fgcr_second_passes(lq, kappa, steps):
+    """At large kappa most of w_k lies in the span of the earlier w_j, and the
+    device asks for a second Gram-Schmidt pass: as many of them, counted by
+    their two launches each, as directions whose orthogonal part the exact
+    recursion finds below half of |w_k|^2; and the residual of that recursion
+    (FP32 directions, 1e-5 of |b| as for the steps above)."""
+    dims = (4, 4, 4, 4)
+    U = synth.gauge_field(dims, "smooth", 31, eps=0.5)
+    A = oracle.clover(U, kappa, 0.0)
+    b = synth.gaussian_spinor(dims, 32)
+    r, Q, part = b.reshape(-1), [], []
+    for k in range(steps):
+        w = oracle.wilson_clover(U, A, kappa, r.reshape(b.shape)).reshape(-1)
+        ww = np.vdot(w, w).real
+        for _ in range(2):
+            for q in Q:
+                w = w - q * np.vdot(q, w)
+        part.append(np.vdot(w, w).real / ww)
+        Q.append(w / np.linalg.norm(w))
+        r = r - Q[-1] * np.vdot(Q[-1], r)
+    part = np.array(part)
+    assert np.abs(part - 0.5).min() > 0.05  # on one side or the other beyond FP32's doubt
+    lat = lq.Lattice(dims, precisions=("f64", "f32"), gcr_nkrylov=24)
+    lat.gauge_load(on_device(U))
+    lat.clover_compute(kappa, 0.0)
+    launches = []
+    for n in (1, steps):  # within one cycle; a further direction: identity, operator (2), one or two passes (2 each)
+        x = lat.canonical_spinor()
+        _, st = lat.solve(x, on_device(b), 1e-30, solver=lq.SOLVER_FGCR, inner_prec="f32", nkrylov=24, maxiter=n,
+                          raise_on_error=False)
+        assert st["iterations"] == n and st["restarts"] == 1
+        launches.append(st["kernel_launches"])
+    assert launches[1] - launches[0] - 5 * (steps - 1) == 2 * np.sum(part < 0.5)
+    want = np.linalg.norm(r) / np.linalg.norm(b)
+    assert abs(oracle.true_residual(U, A, kappa, b, x.cpu().numpy()) - want) <= 1e-5
+
+
+def test_fgcr_ends_a_cycle_without_a_dependent_direction(lq):
+    """A preconditioner of rank two (spins 0 and 1 alone) on constant spinors,
+    which M = 1 - 8 kappa keeps: the third direction lies in the span of the
+    first two.  The cycle ends with those, the next one takes the identity (the
+    residual has not halved) and solves."""
+    import torch
+    dims, kappa = (4, 4, 4, 4), 0.1
+    lat = lq.Lattice(dims, t_antiperiodic=0, precisions=("f64", "f32"), gcr_nkrylov=20)
+    U = np.zeros((4, 4, 4, 4, 4, 3, 3), dtype=complex)
+    U[...] = np.eye(3)
+    lat.gauge_load(on_device(U))
+    lat.clover_compute(kappa, 0.0)
+    net = lq.Net(lat, (1, 1), bf16=False)
+    W = np.zeros((9, 4, 4), complex)
+    W[0] = np.diag([1.0, 0.3, 0.0, 0.0])
+    net.set_weights(W.reshape(-1).astype(np.complex64))
+    net.use_as_preconditioner()
+    b = np.zeros((4, 4, 4, 4, 4, 3), complex)
+    b[..., 0] = [0.7 + 0.2j, 0.9 - 0.4j, 1.1 + 0.3j, -0.8 + 0.6j]
+    x = lat.canonical_spinor()
+    _, st = lat.solve(x, on_device(b), 1e-10, solver=lq.SOLVER_FGCR, inner_prec="f32", nkrylov=20, maxiter=12)
+    # without the early end the first cycle would go on to maxiter
+    assert st["preconditioner_fallback"] == 1 and 2 <= st["restarts"] and 3 <= st["iterations"] < 12
+    assert rel(x.cpu().numpy(), b / (1.0 - 8.0 * kappa)) < 1e-9
+    net.use_as_preconditioner(False)
