@@ -317,7 +317,9 @@ lqcd_status lqcd_create(const lqcd_config* cfg, void* stream, lqcd_ctx** out)
     c->g.tfirst = (part >> 3) & 1 ? (cfg->coord[3] == 0) : 1;
     c->g.tlast = (part >> 3) & 1 ? (cfg->coord[3] == cfg->part[3] - 1) : 1;
     c->block = DSLASH_MAX_BLOCK;
-    if (const char* eb = getenv("LQCD_DSLASH_BLOCK")) {  // experiments: threads per dslash block
+    // experiments: threads per dslash block (128, as unset and as in lqcd_tune_set, leaves the
+    // kernel and its block to launch_dslash's rules)
+    if (const char* eb = getenv("LQCD_DSLASH_BLOCK")) {
         const int b = atoi(eb);
         if (b >= 32 && b <= DSLASH_MAX_BLOCK && b % 32 == 0) c->block = b;
     }

@@ -589,8 +589,10 @@ __device__ __forceinline__ void hop_all_half(const DslashArgs& A, const char* in
 // The CG step alpha = |r|^2 / |Mp|^2; once r is exactly zero (an exact
 // solution inside a check interval) both vanish: no step instead of 0/0.  An
 // FP64 division is some fifteen instructions of a pipe with 1/63 of FP32's
-// rate, so it is done once a block, not once a site (CG iteration at 16^4, 12 FP16-spinor rhs:
-// 206 -> 202 us; 32^3 x 64 FP32 746 -> 740).
+// rate, so the gathering kernel does it once a block, not once a site (CG
+// iteration at 16^4, 12 FP16-spinor rhs: 206 -> 202 us; 32^3 x 64 FP32 746 ->
+// 740).  The warp-per-direction kernel does it in its epilogue threads, beside
+// the hops and before the barrier, the persistent kernel once a tile and thread.
 template <int PS>
 __device__ __forceinline__ typename RealT<AccumP<PS>::value>::type cg_alpha(const DslashArgs& A, int rhs)
 {
