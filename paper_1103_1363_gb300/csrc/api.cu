@@ -148,6 +148,15 @@ lqcd_status launch_dslash(lqcd_ctx* c, const DslashArgs& A0, int P, bool dag, in
         block = DSLASH_WIDE;
     else if (block == DSLASH_MAX_BLOCK && P == P64 && !reducing)
         block = F64_BLOCK;
+    // The kernels read links and clover as data that nothing writes while they
+    // run, so the first launch behind a load on this stream is a plain one; later
+    // ones start under the tail of a kernel that has waited for the load.
+    A.plain = c->links_new;
+    if (c->links_new) {
+        cudaStreamCaptureStatus now = cudaStreamCaptureStatusNone;
+        if (c->stream) LQ_CUDA(cudaStreamIsCapturing(c->stream, &now));
+        if (now == cudaStreamCaptureStatusNone) c->links_new = 0;  // (a captured launch has not run yet)
+    }
     const int rc = c->recon_of(mode_pg(P));
     Profiler* pr = c->prof;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -493,6 +502,7 @@ lqcd_status lqcd_gauge_load(lqcd_ctx* c, const double* links)
         LQ_CUDA(cudaStreamSynchronize(c->stream));  // staging is reused by the next call
     }
     c->gauge_loaded = 1;
+    c->links_new = 1;
     c->clover_state = 0;
     c->csw = 0.0;
     return LQCD_OK;
@@ -517,6 +527,7 @@ lqcd_status lqcd_clover_compute(lqcd_ctx* c, double kappa, double csw)
         return LQCD_OK;
     }
     LQ_CUDA(cudaMemsetAsync(c->errw, 0, sizeof(int), c->stream));
+    c->links_new = 1;
     LQ_TRY(clover_build(c, kappa, csw));
     int err = 0;
     LQ_CUDA(cudaMemcpyAsync(&err, c->errw, sizeof(int), cudaMemcpyDeviceToHost, c->stream));

@@ -149,24 +149,25 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 // Loads from global memory.  The read-only path (ld.global.nc) is for data that
 // nothing writes from a kernel's start to its end.  A kernel that starts under
-// its predecessor's tail runs while that one still writes its spinors,
-// activations or (first launch after a new gauge field) links, and some kernels
-// update their fields in place: those arrays are read by ordinary loads, which
-// also stay behind pdl_wait().  (Read-only loads here cost registers besides:
-// the reducing hops with FP16 spinors and recon-12 links spilled 12 to 60
-// bytes, now none; 24^3 x 48 Schur operator, 12 rhs, 576 -> 565 us, the other
-// operators and solves within 1 %.)
+// its predecessor's tail runs while that one still writes its spinors or
+// activations, and some kernels update their fields in place: those arrays are
+// read by ordinary loads, which also stay behind pdl_wait().  Links and clover
+// are complete by then (the first hopping launch after a load is a plain one,
+// see launch_dslash), and so are the copies that SAP's plain launch waited for.
+template <bool FIXED, class T>
+__device__ __forceinline__ T ld(const T* p)
+{
+    return FIXED ? __ldg(p) : *p;
+}
 template <class T>
 __device__ __forceinline__ T ld_plain(const T* p)
 {
-    return *p;
+    return ld<false>(p);
 }
-// Data complete before the chain's first launch, or read by a plain launch that
-// does not write it.
 template <class T>
 __device__ __forceinline__ T ld_fixed(const T* p)
 {
-    return __ldg(p);
+    return ld<true>(p);
 }
 
 // What this thread is capturing: an iteration block of the library, and the
@@ -403,13 +404,14 @@ template <int P, int RECON> struct GaugeIO;
 template <int RECON> struct GaugeIO<P64, RECON> {
     static constexpr int nchunk = RECON == 12 ? 6 : 9;
     static constexpr int bytes_per_link = nchunk * 16;
+    template <bool FIXED = false>
     __device__ __forceinline__ static void load(const void* base, int stride, int par, int mu, int i,
                                                 double u[18])
     {
         const double2* p = static_cast<const double2*>(base) + (size_t)((par * 4 + mu) * nchunk) * stride + i;
 #pragma unroll
         for (int k = 0; k < nchunk; ++k) {
-            double2 c = ld_plain(p + (size_t)k * stride);
+            double2 c = ld<FIXED>(p + (size_t)k * stride);
             u[2 * k] = c.x;
             u[2 * k + 1] = c.y;
         }
@@ -427,12 +429,13 @@ template <int RECON> struct GaugeIO<P64, RECON> {
 template <> struct GaugeIO<P32, 18> {
     static constexpr int nchunk = 9;
     static constexpr int bytes_per_link = 72;
+    template <bool FIXED = false>
     __device__ __forceinline__ static void load(const void* base, int stride, int par, int mu, int i, float u[18])
     {
         const float2* p = static_cast<const float2*>(base) + (size_t)((par * 4 + mu) * 9) * stride + i;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            float2 c = ld_plain(p + (size_t)k * stride);
+            float2 c = ld<FIXED>(p + (size_t)k * stride);
             u[2 * k] = c.x;
             u[2 * k + 1] = c.y;
         }
@@ -448,12 +451,13 @@ template <> struct GaugeIO<P32, 18> {
 template <> struct GaugeIO<P32, 12> {
     static constexpr int nchunk = 3;
     static constexpr int bytes_per_link = 48;
+    template <bool FIXED = false>
     __device__ __forceinline__ static void load(const void* base, int stride, int par, int mu, int i, float u[18])
     {
         const float4* p = static_cast<const float4*>(base) + (size_t)((par * 4 + mu) * 3) * stride + i;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            float4 c = ld_plain(p + (size_t)k * stride);
+            float4 c = ld<FIXED>(p + (size_t)k * stride);
             u[4 * k] = c.x;
             u[4 * k + 1] = c.y;
             u[4 * k + 2] = c.z;
@@ -475,14 +479,14 @@ template <int ISBF, int RECON> struct GaugeHalfIO {
     static constexpr int nchunk = RECON == 12 ? 3 : 9;
     static constexpr int bytes_per_link = RECON == 12 ? 24 : 36;
     // CONVERT: decoded by conversions, otherwise by adds (the same values)
-    template <bool CONVERT = false>
+    template <bool FIXED = false, bool CONVERT = false>
     __device__ __forceinline__ static void load(const void* base, int stride, int par, int mu, int i, float u[18])
     {
         if (RECON == 12) {
             const uint2* p = static_cast<const uint2*>(base) + (size_t)((par * 4 + mu) * 3) * stride + i;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                uint2 c = ld_plain(p + (size_t)k * stride);
+                uint2 c = ld<FIXED>(p + (size_t)k * stride);
                 float2 a = decode<CONVERT>(c.x), b = decode<CONVERT>(c.y);
                 u[4 * k] = a.x; u[4 * k + 1] = a.y; u[4 * k + 2] = b.x; u[4 * k + 3] = b.y;
             }
@@ -491,7 +495,7 @@ template <int ISBF, int RECON> struct GaugeHalfIO {
             const uint32_t* p = static_cast<const uint32_t*>(base) + (size_t)((par * 4 + mu) * 9) * stride + i;
 #pragma unroll
             for (int k = 0; k < 9; ++k) {
-                float2 a = decode<CONVERT>(ld_plain(p + (size_t)k * stride));
+                float2 a = decode<CONVERT>(ld<FIXED>(p + (size_t)k * stride));
                 u[2 * k] = a.x; u[2 * k + 1] = a.y;
             }
         }
@@ -537,12 +541,13 @@ template <int P> struct CloverIO;
 
 template <> struct CloverIO<P64> {
     static constexpr int bytes_per_site = 576;
+    template <bool FIXED = false>
     __device__ __forceinline__ static void load_block(const void* base, int stride, int i, int blk, double c[36])
     {
         const double2* p = static_cast<const double2*>(base) + (size_t)(18 * blk) * stride + i;
 #pragma unroll
         for (int k = 0; k < 18; ++k) {
-            double2 v = ld_plain(p + (size_t)k * stride);
+            double2 v = ld<FIXED>(p + (size_t)k * stride);
             c[2 * k] = v.x;
             c[2 * k + 1] = v.y;
         }
@@ -557,12 +562,13 @@ template <> struct CloverIO<P64> {
 
 template <> struct CloverIO<P32> {
     static constexpr int bytes_per_site = 288;
+    template <bool FIXED = false>
     __device__ __forceinline__ static void load_block(const void* base, int stride, int i, int blk, float c[36])
     {
         const float4* p = static_cast<const float4*>(base) + (size_t)(9 * blk) * stride + i;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            float4 v = ld_plain(p + (size_t)k * stride);
+            float4 v = ld<FIXED>(p + (size_t)k * stride);
             c[4 * k] = v.x; c[4 * k + 1] = v.y; c[4 * k + 2] = v.z; c[4 * k + 3] = v.w;
         }
     }
@@ -579,25 +585,27 @@ template <> struct CloverIO<P32> {
 // both blocks are read together.
 template <int ISBF> struct CloverHalfIO {
     static constexpr int bytes_per_site = 144;
+    template <bool FIXED = false>
     __device__ __forceinline__ static void load_all(const void* base, int stride, int i, float c[72])
     {
         const uint4* p = static_cast<const uint4*>(base) + i;
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-            uint4 v = ld_plain(p + (size_t)k * stride);
+            uint4 v = ld<FIXED>(p + (size_t)k * stride);
             float2 a = h2f(v.x, ISBF), b = h2f(v.y, ISBF), d = h2f(v.z, ISBF), e = h2f(v.w, ISBF);
             c[8 * k] = a.x; c[8 * k + 1] = a.y; c[8 * k + 2] = b.x; c[8 * k + 3] = b.y;
             c[8 * k + 4] = d.x; c[8 * k + 5] = d.y; c[8 * k + 6] = e.x; c[8 * k + 7] = e.y;
         }
     }
     // block b alone: nine 8-byte pieces, two to a chunk
+    template <bool FIXED = false>
     __device__ __forceinline__ static void load_block(const void* base, int stride, int i, int b, float c[36])
     {
         const uint2* p = static_cast<const uint2*>(base);
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             const int piece = 9 * b + k;
-            const uint2 v = ld_plain(p + ((size_t)(piece >> 1) * stride + i) * 2 + (piece & 1));
+            const uint2 v = ld<FIXED>(p + ((size_t)(piece >> 1) * stride + i) * 2 + (piece & 1));
             const float2 x = h2f(v.x, ISBF), y = h2f(v.y, ISBF);
             c[4 * k] = x.x; c[4 * k + 1] = x.y; c[4 * k + 2] = y.x; c[4 * k + 3] = y.y;
         }
@@ -641,7 +649,7 @@ __device__ __forceinline__ void hermitian6_apply(const R c[36], const R v[12], R
 }
 
 // Full-site clover application in the compute precision of P.
-template <int P>
+template <int P, bool FIXED = false>
 __device__ __forceinline__ void clover_apply_site(const void* base, int stride, int i,
                                                   const typename RealT<P>::type in[24],
                                                   typename RealT<P>::type out[24])
@@ -651,12 +659,12 @@ __device__ __forceinline__ void clover_apply_site(const void* base, int stride, 
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
             R c[36];
-            CloverIO<P>::load_block(base, stride, i, b, c);
+            CloverIO<P>::template load_block<FIXED>(base, stride, i, b, c);
             hermitian6_apply<R>(c, in + 12 * b, out + 12 * b);
         }
     } else {
         float c[72];
-        CloverIO<P>::load_all(base, stride, i, c);
+        CloverIO<P>::template load_all<FIXED>(base, stride, i, c);
         hermitian6_apply<float>(c, in, out);
         hermitian6_apply<float>(c + 36, in + 12, out + 12);
     }

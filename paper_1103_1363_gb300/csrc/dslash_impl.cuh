@@ -57,6 +57,7 @@ struct DslashArgs {
     const int* skip;         // per rhs: nonzero = converged, do nothing (may be nullptr)
     int sites_per_thread;    // reducing launches: grid of Vh / (block * this); 0 = one wave of blocks
     int nrhs;                // right-hand sides of the launch (set by the launcher)
+    int plain;               // not under the predecessor's tail (see launch_dslash)
 };
 
 // ---- spin projection (1 + S g_mu), S = -1 or +1, onto two colour vectors
@@ -388,6 +389,19 @@ struct HopSpinorHalf {
 template <> struct HopSpinor<P16> : HopSpinorHalf<0> {};
 template <> struct HopSpinor<PB16> : HopSpinorHalf<1> {};
 
+// Are links read through the read-only path?  The two kinds of load give the
+// compiler different schedules: read-only ones are faster with links and
+// spinors in the same storage (CG iteration at 24^3 x 48, FP32, us, plain /
+// read-only: recon-12 292 / 285; FP16 hop 23.1 / 22.7) and with 16-bit spinors
+// and recon-18 (a CG solve by 1 to 2 %); with 16-bit spinors and recon-12 plain
+// ones are, where the others spill (241 / 244; 16^4 by 3 %), and with 16-bit
+// links and FP32 spinors (FP16 recon-12 hop by 3 %).
+template <int PG, int PS, int RECON>
+__host__ __device__ constexpr bool fixed_links()
+{
+    return (PG == PS && PG != P64) || (PG == P32 && RECON == 18);
+}
+
 // w = U P q (backward: U^dag P q) for the neighbour's spinor q: forward hops
 // (BWD false) use (1 - g_mu), backward ones (1 + g_mu), swapped by DAG; the
 // link is U_mu at checkerboard index lidx of parity lpar.  hop_term adds it.
@@ -404,9 +418,10 @@ __device__ __forceinline__ void hop_product(const DslashArgs& A, const HopSpinor
 {
     typename RealT<PS>::type h[12], u[18];
     q.template project_to<MU, (BWD != DAG) ? +1 : -1>(h);
+    constexpr bool FIXED = fixed_links<PG, PS, RECON>();
     if constexpr (PG == P16 || PG == PB16)
-        GaugeIO<PG, RECON>::template load<!DAG && (PG == P16 || RECON == 12)>(A.gauge, A.g.stride, lpar, MU, lidx, u);
-    else GaugeIO<PG, RECON>::load(A.gauge, A.g.stride, lpar, MU, lidx, u);
+        GaugeIO<PG, RECON>::template load<FIXED, !DAG && (PG == P16 || RECON == 12)>(A.gauge, A.g.stride, lpar, MU, lidx, u);
+    else GaugeIO<PG, RECON>::template load<FIXED>(A.gauge, A.g.stride, lpar, MU, lidx, u);
     su3_mul_half<BWD, PACK>(u, h, w);
 }
 template <int PG, int PS, int RECON, int MU, bool DAG, bool BWD, bool PACK>
@@ -504,14 +519,14 @@ __device__ __forceinline__ void load_half_hop(const char* in, const void* gauge,
         const uint2* lp = static_cast<const uint2*>(gauge) + (size_t)((lpar * 4 + mu) * 3) * stride + hp.lidx[h];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const uint2 q = ld_plain(lp + (size_t)k * stride);
+            const uint2 q = ld_fixed(lp + (size_t)k * stride);
             r.u[2 * k] = q.x;
             r.u[2 * k + 1] = q.y;
         }
     } else {
         const uint32_t* lp = static_cast<const uint32_t*>(gauge) + (size_t)((lpar * 4 + mu) * 9) * stride + hp.lidx[h];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) r.u[k] = ld_plain(lp + (size_t)k * stride);
+        for (int k = 0; k < 9; ++k) r.u[k] = ld_fixed(lp + (size_t)k * stride);
     }
 }
 
@@ -616,7 +631,7 @@ __device__ __forceinline__ void dslash_epilogue(const DslashArgs& A, int rhs, in
     } else if (EPI == EPI_CLOVINV) {
         if (A.clov) {
             R t[24];
-            clover_apply_site<PG>(A.clov, A.g.stride, i, acc, t);
+            clover_apply_site<PG, PG == PS>(A.clov, A.g.stride, i, acc, t);
 #pragma unroll
             for (int k = 0; k < 24; ++k) acc[k] = a * t[k];
         } else {
@@ -627,7 +642,7 @@ __device__ __forceinline__ void dslash_epilogue(const DslashArgs& A, int rhs, in
         R yv[24], t[24];
         SpinorIO<PS>::load(static_cast<const char*>(A.y) + rhs * A.y_rb, A.g.stride, i, yv);
         if (A.clov) {
-            clover_apply_site<PG>(A.clov, A.g.stride, i, yv, t);
+            clover_apply_site<PG, PG == PS>(A.clov, A.g.stride, i, yv, t);
         } else {
 #pragma unroll
             for (int k = 0; k < 24; ++k) t[k] = yv[k];
@@ -793,6 +808,10 @@ cudaError_t launch_dslash_t(const DslashArgs& A, int nrhs, int block, cudaStream
     if ((long)gx * nrhs > 0x7fffffffL) return cudaErrorInvalidConfiguration;
     DslashArgs Ar = A;
     Ar.nrhs = nrhs;
+    if (A.plain) {
+        dslash_kernel<PG, PS, RECON, DAG, EPI, RED><<<gx * nrhs, block, 0, s>>>(Ar);
+        return cudaGetLastError();
+    }
     return launch_dependent(dslash_kernel<PG, PS, RECON, DAG, EPI, RED>, false, gx * nrhs, block, s, 0, Ar);
 }
 
@@ -938,14 +957,14 @@ __device__ __forceinline__ void wide_operands(const DslashArgs& A, int rhs, int 
 {
     typedef typename RealT<PS>::type R;
     if constexpr (EPI == EPI_CLOVINV) {
-        if (A.clov) CloverIO<PG>::load_block(A.clov, A.g.stride, i, B, o.cl);
+        if (A.clov) CloverIO<PG>::template load_block<PG == PS>(A.clov, A.g.stride, i, B, o.cl);
     }
     if constexpr (EPI >= EPI_XPAY) {
         R yv[12];
         SpinorIO<PS>::template load_half<B>(static_cast<const char*>(A.y) + rhs * A.y_rb, A.g.stride, i, yv);
         if (A.clov) {
             R cl[36];
-            CloverIO<PG>::load_block(A.clov, A.g.stride, i, B, cl);
+            CloverIO<PG>::template load_block<PG == PS>(A.clov, A.g.stride, i, B, cl);
             hermitian6_apply<R>(cl, yv, o.t);
         } else {
 #pragma unroll
@@ -1094,6 +1113,10 @@ cudaError_t launch_wide_t(const DslashArgs& A, int nrhs, cudaStream_t s)
     if (blocks > 0x7fffffffL) return cudaErrorInvalidConfiguration;
     DslashArgs Ar = A;
     Ar.nrhs = nrhs;
+    if (A.plain) {
+        dslash_wide_kernel<PG, PS, RECON, DAG, EPI, RED><<<(unsigned)blocks, WIDE_THREADS, 0, s>>>(Ar);
+        return cudaGetLastError();
+    }
     return launch_dependent(dslash_wide_kernel<PG, PS, RECON, DAG, EPI, RED>, true, (unsigned)blocks, WIDE_THREADS, s, 0, Ar);
 }
 

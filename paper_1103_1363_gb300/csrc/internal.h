@@ -187,6 +187,7 @@ struct lqcd_ctx {
 
     // state
     int gauge_loaded;
+    int links_new;           // links or clover written, no hopping launch behind that yet
     int clover_state;        // 0 none, 1 built
     double kappa, csw;
     int block;               // threads per block of the dslash kernels

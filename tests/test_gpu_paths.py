@@ -521,3 +521,33 @@ def test_fgcr_ends_a_cycle_without_a_dependent_direction(lq):
     assert st["preconditioner_fallback"] == 1 and 2 <= st["restarts"] and 3 <= st["iterations"] < 12
     assert rel(x.cpu().numpy(), b / (1.0 - 8.0 * kappa)) < 1e-9
     net.use_as_preconditioner(False)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32", "f16", "f16spinors"])
+def test_hop_right_behind_a_load(lq, prec):
+    """Links loaded from the device and a hop on them, time after time with
+    another field and without a wait between: the hop of a settled context,
+    bit for bit (a wide and a gathering launch)."""
+    import torch
+    for dims in ((4, 4, 4, 6), (16, 16, 16, 16)):
+        links = [on_device(synth.gauge_field(dims, "smooth", 41 + k, eps=0.5)) for k in range(2)]
+        psi = on_device(synth.gaussian_spinor(dims, 43))
+        lat = lq.Lattice(dims, precisions=("f64", "f32", prec))
+        fin = lat.new_field(prec)
+        lat.pack(fin, psi, 1, prec)
+        want = []
+        for u in links:
+            want.append(torch.zeros_like(fin))
+            lat.gauge_load(u)
+            lat.sync()
+            for _ in range(2):
+                lat.dslash(want[-1], fin, 0, prec=prec)
+            lat.sync()
+        assert not torch.equal(*want)
+        got = [torch.zeros_like(fin) for _ in range(40)]
+        for k, f in enumerate(got):
+            lat.gauge_load(links[k % 2])
+            lat.dslash(f, fin, 0, prec=prec)
+        lat.sync()
+        for k, f in enumerate(got):
+            assert torch.equal(f, want[k % 2]), (dims, k)
