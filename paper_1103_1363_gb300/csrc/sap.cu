@@ -658,11 +658,11 @@ __global__ void __launch_bounds__(SAP_THREADS) sap_block_kernel_strided(const Sa
     for (int l = threadIdx.x; l < a.vol; l += blockDim.x) {
         const SapSite s = sap_site(a, bc, l);
         float rho[24], dv[24], zv[24];
+        char* zp = a.z + s.par * a.fb;
+        SpinorIO<P32>::load(a.dlt + s.par * a.fb, a.g.stride, s.cb, dv);  // (no load stands behind a store)
+        SpinorIO<P32>::load(zp, a.g.stride, s.cb, zv);
         smem_load(rs, a.vol, l, rho);
         SpinorIO<P32>::store(a.rho_out + s.par * a.fb, a.g.stride, s.cb, rho);
-        SpinorIO<P32>::load(a.dlt + s.par * a.fb, a.g.stride, s.cb, dv);
-        char* zp = a.z + s.par * a.fb;
-        SpinorIO<P32>::load(zp, a.g.stride, s.cb, zv);
 #pragma unroll
         for (int k = 0; k < 24; ++k) zv[k] += dv[k];
         SpinorIO<P32>::store(zp, a.g.stride, s.cb, zv);
